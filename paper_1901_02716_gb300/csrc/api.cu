@@ -115,12 +115,12 @@ maclab_status ensure_staging(maclab_ctx* h, size_t bytes) {
 
 size_t state_bytes(const maclab_ctx* h) { return (size_t)(h->g.d + 1) * (size_t)h->g.n * h->elem; }
 
-// Copy the current buffer onto the other one so that both hold the same wall
-// values (wall nodes are never written by the step kernels).
-maclab_status mirror_buffers(maclab_ctx* h) {
-  CUDA_TRY(cudaMemcpyAsync(h->buf[h->cur ^ 1], h->buf[h->cur], state_bytes(h),
-                           cudaMemcpyDeviceToDevice, h->stream),
-           "mirror state");
+// Put the current buffer's wall values into the other one as well (wall nodes
+// are never written by the step kernels; every fluid node of a buffer is
+// written by the step that fills it, so nothing else needs to be copied).
+maclab_status mirror_walls(maclab_ctx* h) {
+  CUDA_TRY(launch_copy_walls(h->g, h->precision, h->d_node_type, h->buf[h->cur], h->buf[h->cur ^ 1], h->stream),
+           "mirror wall values");
   return MACLAB_OK;
 }
 
@@ -432,10 +432,8 @@ maclab_status maclab_set_state(maclab_handle h, const void* rho, const void* u, 
     v = st + nb;
   }
   CUDA_TRY(launch_set_physical(h->g, h->precision, r, v, dtype, h->rho0, h->e, h->d_node_type,
-                               h->d_wall_lat, h->n_wall_ids, h->buf[h->cur], h->stream),
+                               h->d_wall_lat, h->n_wall_ids, h->buf[h->cur], h->buf[h->cur ^ 1], h->stream),
            "set_state kernel");
-  maclab_status s = mirror_buffers(h);
-  if (s != MACLAB_OK) return s;
   h->steps = 0;
   h->prev_valid = false;
   if (where == MACLAB_HOST) CUDA_TRY(cudaStreamSynchronize(h->stream), "set_state sync");
@@ -527,7 +525,7 @@ maclab_status maclab_set_lattice_state(maclab_handle h, const void* state, int32
                            where == MACLAB_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice,
                            h->stream),
            "set_lattice_state");
-  maclab_status s = mirror_buffers(h);
+  maclab_status s = mirror_walls(h);
   if (s != MACLAB_OK) return s;
   h->prev_valid = false;
   if (where == MACLAB_HOST) CUDA_TRY(cudaStreamSynchronize(h->stream), "set_lattice_state sync");

@@ -329,13 +329,15 @@ void batch_items(int inst, const Geometry& g, int rows, int depth, std::vector<i
 cudaError_t launch_set_physical(const Geometry& g, int precision, const void* rho,
                                 const void* u, int dtype, double rho0, double e,
                                 const uint8_t* node_type, const double* wall_lat,
-                                int n_wall_ids, void* state, cudaStream_t stream);
+                                int n_wall_ids, void* state, void* other, cudaStream_t stream);
 cudaError_t launch_get_physical(const Geometry& g, int precision, const void* state,
                                 void* rho, void* u, int dtype, double rho0, double e,
                                 cudaStream_t stream);
 cudaError_t launch_set_wall_values(const Geometry& g, int precision, const void* rho, const void* u,
                                    int dtype, double rho0, double e, const uint8_t* node_type, void* s0,
                                    void* s1, cudaStream_t stream);
+cudaError_t launch_copy_walls(const Geometry& g, int precision, const uint8_t* node_type, const void* src,
+                              void* dst, cudaStream_t stream);
 cudaError_t launch_fill_walls(const Geometry& g, int precision, const uint8_t* node_type,
                               const double* wall_lat, int n_wall_ids, void* state,
                               cudaStream_t stream);

@@ -2,47 +2,177 @@
 //
 // Physical (rho, u) <-> stored lattice state (drho = rho / rho0 - 1, ut = u / e)
 // with e = 6 nu / dx (Eq. (6)).  Wall nodes take their wall id's values
-// (procedure step (iv): physical variables are retained on walls).  The maps
-// are computed in FP64 and rounded once to the storage type.  User arrays are
-// in logical order; the state and the device node-type copy in storage order.
+// (procedure step (iv): physical variables are retained on walls).  User
+// arrays are in logical order; the state and the device node-type copy in
+// storage order.
+//
+// The maps are defined in FP64 and rounded once to the arithmetic type.  Done
+// literally that costs two FP64 operations and two conversions per value on a
+// pipe of two lanes per SM: it bounded these kernels (512^3 FP32: 3.18 ms for
+// 4.3 GB in and out, 20 % of the copy bandwidth).  With 32-bit user arrays and 32-bit
+// arithmetic the same values come from the FP32 pipe (UnitMap):
+//  * rho0 a power of two: v / rho0 - 1 and rho0 (1 + drho) are one exact
+//    scaling and one FP32 rounding, as from FP64;
+//  * e and 1 / e as a sum of two floats (48 bits): the leading product's error
+//    is exact from an fma, so the one rounding that counts is the last, and
+//    only a value within 2^-23 ulp of a rounding boundary can differ.
+// Other rho0, an e whose two floats would leave the normal range, and FP64
+// arrays or storage keep the FP64 form.
+// Now bound by memory: 512^3 FP32 set 0.77 ms, get 0.61 ms (5.6 and 7.0 TB/s);
+// setting no longer copies the state to the other buffer either (0.64 ms more).
+
+#include <math.h>
+
+#include <type_traits>
 
 #include "common.cuh"
 
 namespace maclab {
 
+// The unit maps: stored = v * inv_rho0 - 1 and v * inv_e; physical = rho0 (1 + v) and e v.
+struct UnitMap {
+  double rho0, e, inv_rho0, inv_e;
+  float f_rho0, f_inv_rho0;      // exact (rho0 a power of two)
+  float e_hi, e_lo, ie_hi, ie_lo;  // e and 1 / e as sums of two floats
+};
+
+// Whether the FP32 forms above apply.
+static bool unit_map(double rho0, double e, UnitMap* m) {
+  m->rho0 = rho0;
+  m->e = e;
+  m->inv_rho0 = 1.0 / rho0;
+  m->inv_e = 1.0 / e;
+  m->f_rho0 = (float)rho0;
+  m->f_inv_rho0 = (float)m->inv_rho0;
+  m->e_hi = (float)e;
+  m->e_lo = (float)(e - (double)m->e_hi);
+  m->ie_hi = (float)m->inv_e;
+  m->ie_lo = (float)(m->inv_e - (double)m->ie_hi);
+  int x = 0;
+  const bool pow2 = frexp(rho0, &x) == 0.5 && x > -60 && x < 60;
+  return pow2 && e > 0x1p-60 && e < 0x1p60;
+}
+
+// v (hi + lo), rounded once; infinities and NaN as in v * hi.
+__device__ __forceinline__ float mul_pair(float v, float hi, float lo) {
+  const float p = __fmul_rn(v, hi);
+  const float s = __fadd_rn(p, __fmaf_rn(v, lo, __fmaf_rn(v, hi, -p)));
+  return s == s ? s : p;
+}
+
+// FAST: 32-bit values and the FP32 forms.
+template <typename S, bool FAST>
+struct Map {
+  using C = typename Store<S>::C;
+  template <typename T>
+  __device__ __forceinline__ static S rho_in(T v, const UnitMap& m) {
+    if constexpr (FAST) return Store<S>::to(__fmaf_rn(v, m.f_inv_rho0, -1.0f));
+    else return Store<S>::to(C((double)v * m.inv_rho0 - 1.0));
+  }
+  template <typename T>
+  __device__ __forceinline__ static S u_in(T v, const UnitMap& m) {
+    if constexpr (FAST) return Store<S>::to(mul_pair(v, m.ie_hi, m.ie_lo));
+    else return Store<S>::to(C((double)v * m.inv_e));
+  }
+  template <typename T>
+  __device__ __forceinline__ static T rho_out(S v, const UnitMap& m) {
+    if constexpr (FAST) return __fmul_rn(m.f_rho0, __fadd_rn(1.0f, Store<S>::from(v)));
+    else return (T)(m.rho0 * (1.0 + (double)Store<S>::from(v)));
+  }
+  template <typename T>
+  __device__ __forceinline__ static T u_out(S v, const UnitMap& m) {
+    if constexpr (FAST) return mul_pair(Store<S>::from(v), m.e_hi, m.e_lo);
+    else return (T)(m.e * (double)Store<S>::from(v));
+  }
+};
+
 template <typename T>
-__device__ __forceinline__ double ld_user(const T* p, int64_t i) {
-  return (double)p[i];
-}
+struct alignas(2 * sizeof(T)) Two {
+  T x, y;
+};
+template <typename S>
+struct alignas(4 * sizeof(S) > 16 ? 16 : 4 * sizeof(S)) Four {
+  S v[4];
+};
 
-// User arrays are in logical order (x fastest); the state in storage order.
-// The maps walk the user arrays in order (a warp touches one contiguous run of
+// The kernels walk the user arrays in order (a warp touches contiguous runs of
 // each user array, which may be page-locked host memory read or written over
-// the host link) and place each node at its storage index.
-__device__ __forceinline__ int64_t storage_index(const Geometry& g, int64_t j) {
-  const int64_t row = j / g.nx;
-  return row * g.nx + mem_x(g, (int)(j - row * g.nx));
-}
-
-template <typename S, typename T>
-__global__ void set_physical_k(Geometry g, int d, int64_t N, const T* __restrict__ rho, const T* __restrict__ u,
-                               double inv_rho0, double inv_e, const uint8_t* __restrict__ node_type,
-                               const double* __restrict__ wall_lat, int n_wall_ids,
-                               S* __restrict__ state) {
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < N;
-       j += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = storage_index(g, j);
-    const int k = node_type ? (int)node_type[i] : 0;
-    if (k > 0 && k <= n_wall_ids) {
-      const double* w = wall_lat + 4 * (k - 1);
-      state[i] = Store<S>::to(typename Store<S>::C(w[0]));
-      for (int c = 0; c < d; ++c) state[(1 + c) * N + i] = Store<S>::to(typename Store<S>::C(w[1 + c]));
+// the host link).  QUAD (interleaved rows, nx % 4 == 0, user arrays aligned to
+// two values): a thread takes one storage quad, the nodes (2t, 2t + H,
+// 2t + 1, 2t + 1 + H) of a row, i.e. two runs of two user values per field and
+// one wide store, so a warp moves whole sectors on both sides; otherwise a
+// thread takes one node.  I: index type (32 bits wherever the count allows, as
+// the division by the row length is the largest integer cost).
+template <typename I, bool QUAD, typename Fn>
+__device__ __forceinline__ void for_units(const Geometry& g, Fn&& fn) {
+  const I per_row = (I)(QUAD ? g.nx / 4 : g.nx);
+  const I units = (I)(QUAD ? g.n / 4 : g.n);
+  for (I k = (I)blockIdx.x * blockDim.x + threadIdx.x; k < units; k += (I)gridDim.x * blockDim.x) {
+    const I row = k / per_row;
+    const int t = (int)(k - row * per_row);
+    if constexpr (QUAD) {
+      fn((int64_t)4 * k, (int64_t)row * g.nx + 2 * t);
     } else {
-      state[i] = Store<S>::to(typename Store<S>::C(ld_user(rho, j) * inv_rho0 - 1.0));
-      for (int c = 0; c < d; ++c)
-        state[(1 + c) * N + i] = Store<S>::to(typename Store<S>::C(ld_user(u, c * N + j) * inv_e));
+      fn((int64_t)row * g.nx + mem_x(g, t), (int64_t)k);
     }
   }
+}
+
+// Both state buffers are given: wall nodes are written into both (the step
+// kernels never write them), fluid nodes into s0 only, as every step writes
+// all fluid nodes of the buffer it fills.
+template <typename S, typename T, bool FAST, typename I, bool QUAD>
+__global__ void __launch_bounds__(256) set_physical_k(Geometry g, const T* __restrict__ rho, const T* __restrict__ u,
+                                                      UnitMap m, const uint8_t* __restrict__ node_type,
+                                                      const double* __restrict__ wall_lat, int n_wall_ids,
+                                                      S* __restrict__ s0, S* __restrict__ s1) {
+  using MP = Map<S, FAST>;
+  const int64_t N = g.n;
+  const int d = g.d;
+  for_units<I, QUAD>(g, [&](int64_t i, int64_t j) {
+    if constexpr (QUAD) {
+      Four<S> q[4];
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        if (f > d) continue;
+        const T* src = f == 0 ? rho : u + (f - 1) * N;
+        const Two<T> a = *reinterpret_cast<const Two<T>*>(src + j);
+        const Two<T> b = *reinterpret_cast<const Two<T>*>(src + j + g.hx);
+        const T v[4] = {a.x, b.x, a.y, b.y};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) q[f].v[c] = f == 0 ? MP::rho_in(v[c], m) : MP::u_in(v[c], m);
+      }
+      bool any = false;
+      if (node_type) {
+        const uchar4 k4 = *reinterpret_cast<const uchar4*>(node_type + i);
+        const int k[4] = {k4.x, k4.y, k4.z, k4.w};
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (k[c] > 0 && k[c] <= n_wall_ids) {
+            any = true;
+            const double* w = wall_lat + 4 * (k[c] - 1);
+#pragma unroll
+            for (int f = 0; f < 4; ++f)
+              if (f <= d) q[f].v[c] = Store<S>::to(typename Store<S>::C(w[f]));
+          }
+      }
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        if (f > d) continue;
+        *reinterpret_cast<Four<S>*>(s0 + f * N + i) = q[f];
+        if (any) *reinterpret_cast<Four<S>*>(s1 + f * N + i) = q[f];
+      }
+    } else {
+      const int k = node_type ? (int)node_type[i] : 0;
+      if (k > 0 && k <= n_wall_ids) {
+        const double* w = wall_lat + 4 * (k - 1);
+        for (int f = 0; f <= d; ++f) s0[f * N + i] = s1[f * N + i] = Store<S>::to(typename Store<S>::C(w[f]));
+      } else {
+        s0[i] = MP::rho_in(rho[j], m);
+        for (int c = 0; c < d; ++c) s0[(1 + c) * N + i] = MP::u_in(u[c * N + j], m);
+      }
+    }
+  });
 }
 
 template <typename S>
@@ -64,101 +194,174 @@ __global__ void fill_walls_k(int d, int64_t N, const uint8_t* __restrict__ node_
 // physical (rho, u), in both state buffers (the step kernels never write a
 // wall node, so whichever buffer is current reads them); fluid entries of the
 // arrays are not read.
-template <typename S, typename T>
-__global__ void set_walls_k(Geometry g, int d, int64_t N, const T* __restrict__ rho, const T* __restrict__ u,
-                            double inv_rho0, double inv_e, const uint8_t* __restrict__ node_type,
-                            S* __restrict__ s0, S* __restrict__ s1) {
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < N;
-       j += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = storage_index(g, j);
-    if (node_type[i] == 0) continue;
-    const S r = Store<S>::to(typename Store<S>::C(ld_user(rho, j) * inv_rho0 - 1.0));
-    s0[i] = r;
-    s1[i] = r;
-    for (int c = 0; c < d; ++c) {
-      const S v = Store<S>::to(typename Store<S>::C(ld_user(u, c * N + j) * inv_e));
-      s0[(1 + c) * N + i] = v;
-      s1[(1 + c) * N + i] = v;
+template <typename S, typename T, bool FAST, typename I>
+__global__ void __launch_bounds__(256) set_walls_k(Geometry g, const T* __restrict__ rho, const T* __restrict__ u,
+                                                   UnitMap m, const uint8_t* __restrict__ node_type,
+                                                   S* __restrict__ s0, S* __restrict__ s1) {
+  using MP = Map<S, FAST>;
+  const int64_t N = g.n;
+  for_units<I, false>(g, [&](int64_t i, int64_t j) {
+    if (node_type[i] == 0) return;
+    s0[i] = s1[i] = MP::rho_in(rho[j], m);
+    for (int c = 0; c < g.d; ++c) s0[(1 + c) * N + i] = s1[(1 + c) * N + i] = MP::u_in(u[c * N + j], m);
+  });
+}
+
+// The wall nodes of one raw state into the other buffer.
+template <typename S>
+__global__ void __launch_bounds__(256) copy_walls_k(int d, int64_t N, const uint8_t* __restrict__ node_type,
+                                                    const S* __restrict__ src, S* __restrict__ dst) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
+    if (node_type[i] != 0)
+      for (int f = 0; f <= d; ++f) dst[f * N + i] = src[f * N + i];
+}
+
+template <typename S, typename T, bool FAST, typename I, bool QUAD>
+__global__ void __launch_bounds__(256) get_physical_k(Geometry g, const S* __restrict__ state, UnitMap m,
+                                                      T* __restrict__ rho, T* __restrict__ u) {
+  using MP = Map<S, FAST>;
+  const int64_t N = g.n;
+  const int d = g.d;
+  for_units<I, QUAD>(g, [&](int64_t i, int64_t j) {
+    if constexpr (QUAD) {
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        if (f > d) continue;
+        const Four<S> q = *reinterpret_cast<const Four<S>*>(state + f * N + i);
+        T v[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          v[c] = f == 0 ? MP::template rho_out<T>(q.v[c], m) : MP::template u_out<T>(q.v[c], m);
+        T* dst = f == 0 ? rho : u + (f - 1) * N;
+        *reinterpret_cast<Two<T>*>(dst + j) = Two<T>{v[0], v[2]};
+        *reinterpret_cast<Two<T>*>(dst + j + g.hx) = Two<T>{v[1], v[3]};
+      }
+    } else {
+      rho[j] = MP::template rho_out<T>(state[i], m);
+      for (int c = 0; c < d; ++c) u[c * N + j] = MP::template u_out<T>(state[(1 + c) * N + i], m);
     }
-  }
+  });
 }
 
-template <typename S, typename T>
-__global__ void get_physical_k(Geometry g, int d, int64_t N, const S* __restrict__ state, double rho0,
-                               double e, T* __restrict__ rho, T* __restrict__ u) {
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < N;
-       j += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = storage_index(g, j);
-    rho[j] = (T)(rho0 * (1.0 + (double)Store<S>::from(state[i])));
-    for (int c = 0; c < d; ++c) u[c * N + j] = (T)(e * (double)Store<S>::from(state[(1 + c) * N + i]));
-  }
-}
-
+// Blocks of 256 threads for n threads' worth of units, at most 2^20 (each
+// thread then takes several): a thread's few loads are all it has in flight,
+// so the block scheduler, not a loop, keeps the SMs full.
 static unsigned grid_for(int64_t n) {
   int64_t b = (n + 255) / 256;
-  if (b > 4096) b = 4096;
+  if (b > (1 << 20)) b = 1 << 20;
   return (unsigned)(b < 1 ? 1 : b);
 }
 
+// 32-bit unit indices where neither the count nor a grid stride past it overflows.
+static bool small_index(int64_t units) { return units < ((int64_t)1 << 31); }
+
+static bool aligned_to(const void* a, const void* b, size_t bytes) {
+  return (reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) % bytes == 0;
+}
+
+template <typename S, typename T, bool FAST, typename I, bool QUAD>
+static cudaError_t set_launch(const Geometry& g, const void* rho, const void* u, const UnitMap& m, const uint8_t* nt,
+                              const double* wl, int nw, void* s0, void* s1, cudaStream_t st) {
+  set_physical_k<S, T, FAST, I, QUAD><<<grid_for(QUAD ? g.n / 4 : g.n), 256, 0, st>>>(
+      g, (const T*)rho, (const T*)u, m, nt, wl, nw, (S*)s0, (S*)s1);
+  return cudaGetLastError();
+}
+
+template <typename S, typename T, bool FAST>
+static cudaError_t set_t(const Geometry& g, const void* rho, const void* u, const UnitMap& m, const uint8_t* nt,
+                         const double* wl, int nw, void* s0, void* s1, cudaStream_t st) {
+  const bool small = small_index(g.n);
+  if (g.ilv && aligned_to(rho, u, 2 * sizeof(T)))
+    return small ? set_launch<S, T, FAST, uint32_t, true>(g, rho, u, m, nt, wl, nw, s0, s1, st)
+                 : set_launch<S, T, FAST, int64_t, true>(g, rho, u, m, nt, wl, nw, s0, s1, st);
+  return small ? set_launch<S, T, FAST, uint32_t, false>(g, rho, u, m, nt, wl, nw, s0, s1, st)
+               : set_launch<S, T, FAST, int64_t, false>(g, rho, u, m, nt, wl, nw, s0, s1, st);
+}
+
 template <typename S>
-static cudaError_t set_t(const Geometry& g, const void* rho, const void* u, int dtype, double rho0,
-                         double e, const uint8_t* nt, const double* wl, int nw, void* state,
+static cudaError_t set_s(const Geometry& g, const void* rho, const void* u, int dtype, double rho0, double e,
+                         const uint8_t* nt, const double* wl, int nw, void* s0, void* s1, cudaStream_t st) {
+  UnitMap m;
+  const bool fast = unit_map(rho0, e, &m);
+  if (dtype == MACLAB_DTYPE_F64) return set_t<S, double, false>(g, rho, u, m, nt, wl, nw, s0, s1, st);
+  if constexpr (!std::is_same<S, double>::value)
+    if (fast) return set_t<S, float, true>(g, rho, u, m, nt, wl, nw, s0, s1, st);
+  return set_t<S, float, false>(g, rho, u, m, nt, wl, nw, s0, s1, st);
+}
+
+cudaError_t launch_set_physical(const Geometry& g, int precision, const void* rho, const void* u, int dtype,
+                                double rho0, double e, const uint8_t* nt, const double* wl, int nw, void* state,
+                                void* other, cudaStream_t st) {
+  switch (precision) {
+    case MACLAB_F64: return set_s<double>(g, rho, u, dtype, rho0, e, nt, wl, nw, state, other, st);
+    case MACLAB_F32: return set_s<float>(g, rho, u, dtype, rho0, e, nt, wl, nw, state, other, st);
+    case MACLAB_BF16_STORE: return set_s<__nv_bfloat16>(g, rho, u, dtype, rho0, e, nt, wl, nw, state, other, st);
+    case MACLAB_F16_STORE: return set_s<__half>(g, rho, u, dtype, rho0, e, nt, wl, nw, state, other, st);
+  }
+  return cudaErrorInvalidValue;
+}
+
+template <typename S, typename T, bool FAST, typename I, bool QUAD>
+static cudaError_t get_launch(const Geometry& g, const void* state, const UnitMap& m, void* rho, void* u,
+                              cudaStream_t st) {
+  get_physical_k<S, T, FAST, I, QUAD><<<grid_for(QUAD ? g.n / 4 : g.n), 256, 0, st>>>(g, (const S*)state, m, (T*)rho,
+                                                                                     (T*)u);
+  return cudaGetLastError();
+}
+
+template <typename S, typename T, bool FAST>
+static cudaError_t get_t(const Geometry& g, const void* state, const UnitMap& m, void* rho, void* u, cudaStream_t st) {
+  const bool small = small_index(g.n);
+  if (g.ilv && aligned_to(rho, u, 2 * sizeof(T)))
+    return small ? get_launch<S, T, FAST, uint32_t, true>(g, state, m, rho, u, st)
+                 : get_launch<S, T, FAST, int64_t, true>(g, state, m, rho, u, st);
+  return small ? get_launch<S, T, FAST, uint32_t, false>(g, state, m, rho, u, st)
+               : get_launch<S, T, FAST, int64_t, false>(g, state, m, rho, u, st);
+}
+
+template <typename S>
+static cudaError_t get_s(const Geometry& g, const void* state, void* rho, void* u, int dtype, double rho0, double e,
                          cudaStream_t st) {
-  if (dtype == MACLAB_DTYPE_F64)
-    set_physical_k<S, double><<<grid_for(g.n), 256, 0, st>>>(
-        g, g.d, g.n, (const double*)rho, (const double*)u, 1.0 / rho0, 1.0 / e, nt, wl, nw, (S*)state);
-  else
-    set_physical_k<S, float><<<grid_for(g.n), 256, 0, st>>>(
-        g, g.d, g.n, (const float*)rho, (const float*)u, 1.0 / rho0, 1.0 / e, nt, wl, nw, (S*)state);
-  return cudaGetLastError();
+  UnitMap m;
+  const bool fast = unit_map(rho0, e, &m);
+  if (dtype == MACLAB_DTYPE_F64) return get_t<S, double, false>(g, state, m, rho, u, st);
+  if constexpr (!std::is_same<S, double>::value)
+    if (fast) return get_t<S, float, true>(g, state, m, rho, u, st);
+  return get_t<S, float, false>(g, state, m, rho, u, st);
 }
 
-template <typename S>
-static cudaError_t get_t(const Geometry& g, const void* state, void* rho, void* u, int dtype,
-                         double rho0, double e, cudaStream_t st) {
-  if (dtype == MACLAB_DTYPE_F64)
-    get_physical_k<S, double><<<grid_for(g.n), 256, 0, st>>>(g, g.d, g.n, (const S*)state, rho0, e,
-                                                            (double*)rho, (double*)u);
-  else
-    get_physical_k<S, float><<<grid_for(g.n), 256, 0, st>>>(g, g.d, g.n, (const S*)state, rho0, e,
-                                                           (float*)rho, (float*)u);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_set_physical(const Geometry& g, int precision, const void* rho, const void* u,
-                                int dtype, double rho0, double e, const uint8_t* nt,
-                                const double* wl, int nw, void* state, cudaStream_t st) {
+cudaError_t launch_get_physical(const Geometry& g, int precision, const void* state, void* rho, void* u, int dtype,
+                                double rho0, double e, cudaStream_t st) {
   switch (precision) {
-    case MACLAB_F64: return set_t<double>(g, rho, u, dtype, rho0, e, nt, wl, nw, state, st);
-    case MACLAB_F32: return set_t<float>(g, rho, u, dtype, rho0, e, nt, wl, nw, state, st);
-    case MACLAB_BF16_STORE:
-      return set_t<__nv_bfloat16>(g, rho, u, dtype, rho0, e, nt, wl, nw, state, st);
-    case MACLAB_F16_STORE: return set_t<__half>(g, rho, u, dtype, rho0, e, nt, wl, nw, state, st);
+    case MACLAB_F64: return get_s<double>(g, state, rho, u, dtype, rho0, e, st);
+    case MACLAB_F32: return get_s<float>(g, state, rho, u, dtype, rho0, e, st);
+    case MACLAB_BF16_STORE: return get_s<__nv_bfloat16>(g, state, rho, u, dtype, rho0, e, st);
+    case MACLAB_F16_STORE: return get_s<__half>(g, state, rho, u, dtype, rho0, e, st);
   }
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_get_physical(const Geometry& g, int precision, const void* state, void* rho,
-                                void* u, int dtype, double rho0, double e, cudaStream_t st) {
-  switch (precision) {
-    case MACLAB_F64: return get_t<double>(g, state, rho, u, dtype, rho0, e, st);
-    case MACLAB_F32: return get_t<float>(g, state, rho, u, dtype, rho0, e, st);
-    case MACLAB_BF16_STORE: return get_t<__nv_bfloat16>(g, state, rho, u, dtype, rho0, e, st);
-    case MACLAB_F16_STORE: return get_t<__half>(g, state, rho, u, dtype, rho0, e, st);
-  }
-  return cudaErrorInvalidValue;
+template <typename S, typename T, bool FAST>
+static cudaError_t walls_t(const Geometry& g, const void* rho, const void* u, const UnitMap& m, const uint8_t* nt,
+                           void* s0, void* s1, cudaStream_t st) {
+  if (small_index(g.n))
+    set_walls_k<S, T, FAST, uint32_t><<<grid_for(g.n), 256, 0, st>>>(g, (const T*)rho, (const T*)u, m, nt, (S*)s0,
+                                                                    (S*)s1);
+  else
+    set_walls_k<S, T, FAST, int64_t><<<grid_for(g.n), 256, 0, st>>>(g, (const T*)rho, (const T*)u, m, nt, (S*)s0,
+                                                                   (S*)s1);
+  return cudaGetLastError();
 }
 
 template <typename S>
-static cudaError_t walls_t(const Geometry& g, const void* rho, const void* u, int dtype, double rho0,
-                           double e, const uint8_t* nt, void* s0, void* s1, cudaStream_t st) {
-  if (dtype == MACLAB_DTYPE_F64)
-    set_walls_k<S, double><<<grid_for(g.n), 256, 0, st>>>(g, g.d, g.n, (const double*)rho, (const double*)u,
-                                                         1.0 / rho0, 1.0 / e, nt, (S*)s0, (S*)s1);
-  else
-    set_walls_k<S, float><<<grid_for(g.n), 256, 0, st>>>(g, g.d, g.n, (const float*)rho, (const float*)u,
-                                                        1.0 / rho0, 1.0 / e, nt, (S*)s0, (S*)s1);
-  return cudaGetLastError();
+static cudaError_t walls_s(const Geometry& g, const void* rho, const void* u, int dtype, double rho0, double e,
+                           const uint8_t* nt, void* s0, void* s1, cudaStream_t st) {
+  UnitMap m;
+  const bool fast = unit_map(rho0, e, &m);
+  if (dtype == MACLAB_DTYPE_F64) return walls_t<S, double, false>(g, rho, u, m, nt, s0, s1, st);
+  if constexpr (!std::is_same<S, double>::value)
+    if (fast) return walls_t<S, float, true>(g, rho, u, m, nt, s0, s1, st);
+  return walls_t<S, float, false>(g, rho, u, m, nt, s0, s1, st);
 }
 
 cudaError_t launch_set_wall_values(const Geometry& g, int precision, const void* rho, const void* u,
@@ -166,12 +369,25 @@ cudaError_t launch_set_wall_values(const Geometry& g, int precision, const void*
                                    void* s1, cudaStream_t st) {
   if (!nt) return cudaSuccess;
   switch (precision) {
-    case MACLAB_F64: return walls_t<double>(g, rho, u, dtype, rho0, e, nt, s0, s1, st);
-    case MACLAB_F32: return walls_t<float>(g, rho, u, dtype, rho0, e, nt, s0, s1, st);
-    case MACLAB_BF16_STORE: return walls_t<__nv_bfloat16>(g, rho, u, dtype, rho0, e, nt, s0, s1, st);
-    case MACLAB_F16_STORE: return walls_t<__half>(g, rho, u, dtype, rho0, e, nt, s0, s1, st);
+    case MACLAB_F64: return walls_s<double>(g, rho, u, dtype, rho0, e, nt, s0, s1, st);
+    case MACLAB_F32: return walls_s<float>(g, rho, u, dtype, rho0, e, nt, s0, s1, st);
+    case MACLAB_BF16_STORE: return walls_s<__nv_bfloat16>(g, rho, u, dtype, rho0, e, nt, s0, s1, st);
+    case MACLAB_F16_STORE: return walls_s<__half>(g, rho, u, dtype, rho0, e, nt, s0, s1, st);
   }
   return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_copy_walls(const Geometry& g, int precision, const uint8_t* nt, const void* src, void* dst,
+                              cudaStream_t st) {
+  if (!nt) return cudaSuccess;
+  const unsigned grid = grid_for(g.n);
+  switch (storage_bytes(precision)) {
+    case 8: copy_walls_k<double><<<grid, 256, 0, st>>>(g.d, g.n, nt, (const double*)src, (double*)dst); break;
+    case 4: copy_walls_k<float><<<grid, 256, 0, st>>>(g.d, g.n, nt, (const float*)src, (float*)dst); break;
+    case 2: copy_walls_k<uint16_t><<<grid, 256, 0, st>>>(g.d, g.n, nt, (const uint16_t*)src, (uint16_t*)dst); break;
+    default: return cudaErrorInvalidValue;
+  }
+  return cudaGetLastError();
 }
 
 cudaError_t launch_fill_walls(const Geometry& g, int precision, const uint8_t* nt, const double* wl,
