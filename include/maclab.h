@@ -188,7 +188,12 @@ maclab_status maclab_step(maclab_handle h, int64_t n);
  * passes through global memory once per ty steps; a run of n steps ends with
  * a one-step launch (the previous state is step n - 1).  Its sums run in the
  * tiled kernel's order: identical bits.  The default for FP32 and FP64 D2Q9
- * grids of up to 131,072 node pairs (512^2). */
+ * grids of up to 131,072 node pairs (512^2).
+ * The default also takes these kernels where a choice by hand is refused: a
+ * closed x axis of at least 17 nodes whose width is not a multiple of 4 is
+ * stored in rows padded to one (the raw state keeps its (d + 1) * N values),
+ * and the two-rows and folded kernels run on row counts that their tiles do not
+ * divide (at least one tile of rows). */
 #define MACLAB_KERNEL_AUTO 0
 #define MACLAB_KERNEL_REFERENCE 1
 #define MACLAB_KERNEL_TILED 2
@@ -291,7 +296,7 @@ maclab_status maclab_set_graph(maclab_handle h, int32_t steps);
 /* ---------------------------------------------------------------- batches
  * Many independent domains advanced together: every maclab_batch_step is one
  * kernel launch over the work items of all domains (D2Q9 domains whose nx is a
- * multiple of 4), or one launch per domain otherwise, and runs of steps are
+ * multiple of 4, or at least 17 with a closed x axis), or one launch per domain otherwise, and runs of steps are
  * captured in CUDA graphs.  Domains may differ in size, dx, nu, walls and
  * force; they must share lattice, precision, device and stream. */
 typedef struct maclab_batch_ctx *maclab_batch;

@@ -95,6 +95,7 @@ void free_ctx(maclab_ctx* h) {
   cudaFree(h->buf[0]);
   cudaFree(h->buf[1]);
   cudaFree(h->d_node_type);
+  cudaFree(h->d_node_type_raw);
   cudaFree(h->d_wall_lat);
   cudaFree(h->d_staging);
   delete h;
@@ -113,7 +114,9 @@ maclab_status ensure_staging(maclab_ctx* h, size_t bytes) {
   return MACLAB_OK;
 }
 
-size_t state_bytes(const maclab_ctx* h) { return (size_t)(h->g.d + 1) * (size_t)h->g.n * h->elem; }
+size_t state_bytes(const maclab_ctx* h) { return (size_t)(h->g.d + 1) * (size_t)h->raw.n * h->elem; }
+// one of the two state buffers
+size_t buffer_bytes(const maclab_ctx* h) { return (size_t)(h->g.d + 1) * (size_t)h->g.n * h->elem; }
 
 // Put the current buffer's wall values into the other one as well (wall nodes
 // are never written by the step kernels; every fluid node of a buffer is
@@ -301,10 +304,18 @@ maclab_status maclab_create(const maclab_config* cfg, maclab_handle* out) {
   }
   h->n_fluid = N - n_wall;
   g.wall_mode = n_wall == 0 ? kWallNone : (box ? kWallBox : kWallMask);
+  h->raw = g;
+  if (!(g.periodic & 1u) && nx % 4 != 0 && nx >= kMinPadWidth) {  // interleaved rows with padding (Geometry)
+    g.pad = (int)(4 - nx % 4);
+    g.nx += g.pad;
+    g.n = (int64_t)g.nx * ny * nz;
+    g.ilv = 1;
+    g.hx = g.nx / 2;
+  }
 
   DeviceGuard dg(h->device);
-  const size_t sb = state_bytes(h);
-  h->diag_nblocks = diag_blocks(N);
+  const size_t sb = buffer_bytes(h);
+  h->diag_nblocks = diag_blocks(g.n);
   if (cudaMalloc(&h->buf[0], sb) != cudaSuccess || cudaMalloc(&h->buf[1], sb) != cudaSuccess ||
       cudaMalloc(&h->d_partial, sizeof(double) * (kDiagOut * h->diag_nblocks + 1)) != cudaSuccess ||
       cudaMalloc(&h->d_diag, sizeof(double) * kDiagOut) != cudaSuccess ||
@@ -325,18 +336,21 @@ maclab_status maclab_create(const maclab_config* cfg, maclab_handle* out) {
     return fail(MACLAB_ERR_CUDA, "diagnostics scratch initialisation failed");
   }
   if (n_wall > 0) {
-    if (cudaMalloc(&h->d_node_type, (size_t)N) != cudaSuccess ||
+    if (cudaMalloc(&h->d_node_type, (size_t)g.n) != cudaSuccess ||
+        (g.pad && cudaMalloc(&h->d_node_type_raw, (size_t)N) != cudaSuccess) ||
         cudaMalloc(&h->d_wall_lat, sizeof(double) * h->wall_lat.size()) != cudaSuccess) {
       cudaGetLastError();
       free_ctx(h);
       return fail(MACLAB_ERR_OOM, "mask allocation failed");
     }
-    // device copy in storage order
-    std::vector<uint8_t> nt_mem((size_t)N);
+    // device copy in storage order (padding: wall)
+    std::vector<uint8_t> nt_mem((size_t)g.n, g.pad ? 1 : 0);
     for (int64_t row = 0; row < N / nx; ++row)
       for (int64_t x = 0; x < nx; ++x)
-        nt_mem[(size_t)(row * nx + mem_x(g, (int)x))] = cfg->node_type[row * nx + x];
-    cudaError_t e1 = cudaMemcpy(h->d_node_type, nt_mem.data(), (size_t)N, cudaMemcpyHostToDevice);
+        nt_mem[(size_t)(row * g.nx + mem_x(g, (int)x))] = cfg->node_type[row * nx + x];
+    cudaError_t e1 = cudaMemcpy(h->d_node_type, nt_mem.data(), (size_t)g.n, cudaMemcpyHostToDevice);
+    if (e1 == cudaSuccess && g.pad)
+      e1 = cudaMemcpy(h->d_node_type_raw, cfg->node_type, (size_t)N, cudaMemcpyHostToDevice);
     cudaError_t e2 = cudaMemcpy(h->d_wall_lat, h->wall_lat.data(),
                                 sizeof(double) * h->wall_lat.size(), cudaMemcpyHostToDevice);
     if (e1 != cudaSuccess || e2 != cudaSuccess) {
@@ -345,6 +359,7 @@ maclab_status maclab_create(const maclab_config* cfg, maclab_handle* out) {
     }
   }
   g.mask = g.wall_mode == kWallMask ? h->d_node_type : nullptr;
+  h->raw.mask = g.wall_mode == kWallMask ? (g.pad ? h->d_node_type_raw : h->d_node_type) : nullptr;
 
   // rest state with the wall values in place, in both buffers
   cudaError_t e = cudaMemsetAsync(h->buf[0], 0, sb, h->stream);
@@ -413,7 +428,7 @@ maclab_status maclab_set_state(maclab_handle h, const void* rho, const void* u, 
   if (where != MACLAB_HOST && where != MACLAB_DEVICE) return fail(MACLAB_ERR_INVALID, "bad where");
   DeviceGuard dg(h->device);
   const size_t es = dtype == MACLAB_DTYPE_F64 ? 8 : 4;
-  const size_t nb = (size_t)h->g.n * es;
+  const size_t nb = (size_t)h->raw.n * es;
   const void* r = rho;
   const void* v = u;
   const void* pr = where == MACLAB_HOST ? pinned_device_ptr(rho, h->device) : nullptr;
@@ -450,7 +465,7 @@ maclab_status maclab_set_wall_state(maclab_handle h, const void* rho, const void
   if (!h->d_node_type) return MACLAB_OK;  // no wall nodes
   DeviceGuard dg(h->device);
   const size_t es = dtype == MACLAB_DTYPE_F64 ? 8 : 4;
-  const size_t nb = (size_t)h->g.n * es;
+  const size_t nb = (size_t)h->raw.n * es;
   const void* r = rho;
   const void* v = u;
   const void* pr = where == MACLAB_HOST ? pinned_device_ptr(rho, h->device) : nullptr;
@@ -483,7 +498,7 @@ maclab_status maclab_get_state(maclab_handle h, void* rho, void* u, int32_t wher
   if (where != MACLAB_HOST && where != MACLAB_DEVICE) return fail(MACLAB_ERR_INVALID, "bad where");
   DeviceGuard dg(h->device);
   const size_t es = dtype == MACLAB_DTYPE_F64 ? 8 : 4;
-  const size_t nb = (size_t)h->g.n * es;
+  const size_t nb = (size_t)h->raw.n * es;
   void* pr = where == MACLAB_HOST ? pinned_device_ptr(rho, h->device) : nullptr;
   void* pu = pr ? pinned_device_ptr(u, h->device) : nullptr;
   if (where == MACLAB_DEVICE || (pr && pu)) {
@@ -505,14 +520,37 @@ maclab_status maclab_get_state(maclab_handle h, void* rho, void* u, int32_t wher
   return MACLAB_OK;
 }
 
+// Planes of the march axis.
+static int64_t march_planes(const maclab_ctx* h) { return h->g.d == 3 ? h->g.nz : h->g.ny; }
+
+// The current state of padded rows in the raw layout: into `device` (a buffer
+// of the handle's device) or, where that is null, the staging buffer.
+static maclab_status stage_raw(maclab_ctx* h, void* device, const void** out) {
+  if (!device || reinterpret_cast<uintptr_t>(device) % h->elem != 0) {
+    maclab_status s = ensure_staging(h, state_bytes(h));
+    if (s != MACLAB_OK) return s;
+    device = h->d_staging;
+  }
+  CUDA_TRY(launch_repack(h->g, h->precision, h->buf[h->cur], device, 0, march_planes(h), true, h->stream),
+           "raw state repack");
+  *out = device;
+  return MACLAB_OK;
+}
+
 maclab_status maclab_get_lattice_state(maclab_handle h, void* state, int32_t where) {
   if (!h || !state) return fail(MACLAB_ERR_INVALID, "NULL argument");
   if (where != MACLAB_HOST && where != MACLAB_DEVICE) return fail(MACLAB_ERR_INVALID, "bad where");
   DeviceGuard dg(h->device);
-  CUDA_TRY(cudaMemcpyAsync(state, h->buf[h->cur], state_bytes(h),
-                           where == MACLAB_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice,
-                           h->stream),
-           "get_lattice_state");
+  const void* src = h->buf[h->cur];
+  if (h->g.pad) {
+    maclab_status s = stage_raw(h, where == MACLAB_DEVICE ? state : nullptr, &src);
+    if (s != MACLAB_OK) return s;
+  }
+  if (src != state)
+    CUDA_TRY(cudaMemcpyAsync(state, src, state_bytes(h),
+                             where == MACLAB_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice,
+                             h->stream),
+             "get_lattice_state");
   CUDA_TRY(cudaStreamSynchronize(h->stream), "get_lattice_state sync");
   return MACLAB_OK;
 }
@@ -521,10 +559,25 @@ maclab_status maclab_set_lattice_state(maclab_handle h, const void* state, int32
   if (!h || !state) return fail(MACLAB_ERR_INVALID, "NULL argument");
   if (where != MACLAB_HOST && where != MACLAB_DEVICE) return fail(MACLAB_ERR_INVALID, "bad where");
   DeviceGuard dg(h->device);
-  CUDA_TRY(cudaMemcpyAsync(h->buf[h->cur], state, state_bytes(h),
-                           where == MACLAB_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice,
+  if (h->g.pad) {
+    const void* raw = state;
+    if (where == MACLAB_HOST || reinterpret_cast<uintptr_t>(state) % h->elem != 0) {
+      maclab_status s = ensure_staging(h, state_bytes(h));
+      if (s != MACLAB_OK) return s;
+      CUDA_TRY(cudaMemcpyAsync(h->d_staging, state, state_bytes(h),
+                               where == MACLAB_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, h->stream),
+               "set_lattice_state staging");
+      raw = h->d_staging;
+    }
+    CUDA_TRY(launch_repack(h->g, h->precision, h->buf[h->cur], const_cast<void*>(raw), 0, march_planes(h), false,
                            h->stream),
-           "set_lattice_state");
+             "set_lattice_state repack");
+  } else {
+    CUDA_TRY(cudaMemcpyAsync(h->buf[h->cur], state, state_bytes(h),
+                             where == MACLAB_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice,
+                             h->stream),
+             "set_lattice_state");
+  }
   maclab_status s = mirror_walls(h);
   if (s != MACLAB_OK) return s;
   h->prev_valid = false;
@@ -586,7 +639,7 @@ static int device_sms() {
 static maclab_status segment_persist_prepare(maclab_ctx* h) {
   if (h->seg_persist_blocks > 0 || h->seg_depth != 2) return MACLAB_OK;
   int capacity = 0;
-  if (batch_persist_capacity(h->precision, &capacity) != cudaSuccess || capacity < 1) {
+  if (batch_persist_capacity(h->precision, (h->g.pad & 1) != 0, &capacity) != cudaSuccess || capacity < 1) {
     cudaGetLastError();
     return MACLAB_OK;  // the form is unavailable; stepping uses graphs of launches
   }
@@ -706,7 +759,7 @@ maclab_status maclab_step(maclab_handle h, int64_t n) {
     const int sweeps = pairs > (1 << 30) ? (1 << 30) : (int)pairs;
     CUDA_TRY(launch_batch_step2_persist(h->precision, h->d_seg_inst, h->d_seg_items, h->seg_n_items, h->cur,
                                         h->seg_persist_blocks, sweeps, h->d_seg_deps, h->d_seg_done,
-                                        step_status(), h->wait_limit, h->stream),
+                                        step_status(), h->wait_limit, (h->g.pad & 1) != 0, h->stream),
              "persistent step launch");
     if (sweeps & 1) h->cur ^= 1;
     done += 2 * (int64_t)sweeps;
@@ -746,14 +799,14 @@ maclab_status maclab_set_graph(maclab_handle h, int32_t steps) {
 }
 
 static size_t adjoint_bytes(const maclab_ctx* h) {
-  return (size_t)(h->g.d + 1) * (size_t)h->g.n * (h->precision == MACLAB_F64 ? 8 : 4);
+  return (size_t)(h->raw.d + 1) * (size_t)h->raw.n * (h->precision == MACLAB_F64 ? 8 : 4);
 }
 
 // records: the per-node (L_r, L_m) buffer that only the reference kernels use
 static maclab_status ensure_adjoint(maclab_ctx* h, bool records = false) {
   if (records && !h->d_adj_scratch) {
     // one 4-value record per node
-    const size_t rec = 4 * (size_t)h->g.n * (h->precision == MACLAB_F64 ? 8 : 4);
+    const size_t rec = 4 * (size_t)h->raw.n * (h->precision == MACLAB_F64 ? 8 : 4);
     if (cudaMalloc(&h->d_adj_scratch, rec) != cudaSuccess) {
       cudaGetLastError();
       h->d_adj_scratch = nullptr;
@@ -783,15 +836,15 @@ maclab_status maclab_adjoint_step(maclab_handle h, const void* state_n, const vo
   if (lam_n == lam_np1) return fail(MACLAB_ERR_INVALID, "lam_n must not alias lam_np1");
   DeviceGuard dg(h->device);
   // the tiled reverse step where it is built (unless the reference kernel was chosen)
-  const bool tiled = h->kernel != MACLAB_KERNEL_REFERENCE && tiled_adjoint_supported(h->g, h->precision);
+  const bool tiled = h->kernel != MACLAB_KERNEL_REFERENCE && tiled_adjoint_supported(h->raw, h->precision);
   maclab_status s = ensure_adjoint(h, !tiled);
   if (s != MACLAB_OK) return s;
   if (tiled) {
-    CUDA_TRY(launch_tiled_adjoint(h->g, h->precision, state_n, state_np1, lam_np1, lam_n,
+    CUDA_TRY(launch_tiled_adjoint(h->raw, h->precision, state_n, state_np1, lam_np1, lam_n,
                                   h->force_lat, grad_force, h->overlap, h->stream),
              "adjoint step");
   } else {
-    CUDA_TRY(launch_adjoint_step(h->g, h->precision, state_n, state_np1, lam_np1, lam_n,
+    CUDA_TRY(launch_adjoint_step(h->raw, h->precision, state_n, state_np1, lam_np1, lam_n,
                                  h->d_adj_scratch, h->force_lat, grad_force, h->stream),
              "adjoint step");
   }
@@ -804,14 +857,14 @@ maclab_status maclab_adjoint_nu_term(maclab_handle h, const void* state_n, const
   if (!h || !state_n || !lam_np1 || !acc) return fail(MACLAB_ERR_INVALID, "NULL argument");
   DeviceGuard dg(h->device);
   auto aligned = [](const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; };
-  if (state_np1 && h->kernel != MACLAB_KERNEL_REFERENCE && rows2_nu_supported(h->g, h->precision) &&
+  if (state_np1 && h->kernel != MACLAB_KERNEL_REFERENCE && rows2_nu_supported(h->raw, h->precision) &&
       aligned(state_n) && aligned(state_np1) && aligned(lam_np1)) {
-    CUDA_TRY(launch_rows2_nu(h->g, state_n, state_np1, static_cast<const float*>(lam_np1), h->force_lat, acc,
+    CUDA_TRY(launch_rows2_nu(h->raw, state_n, state_np1, static_cast<const float*>(lam_np1), h->force_lat, acc,
                              h->overlap, h->stream),
              "adjoint nu term (two-rows kernel)");
     return MACLAB_OK;
   }
-  CUDA_TRY(launch_adjoint_nu_term(h->g, h->precision, state_n, lam_np1, h->force_lat, acc, h->stream),
+  CUDA_TRY(launch_adjoint_nu_term(h->raw, h->precision, state_n, lam_np1, h->force_lat, acc, h->stream),
            "adjoint nu term");
   return MACLAB_OK;
 }
@@ -824,7 +877,7 @@ maclab_status maclab_adjoint_seed(maclab_handle h, const void* grad_rho, const v
   maclab_status s = ensure_adjoint(h);
   if (s != MACLAB_OK) return s;
   CUDA_TRY(cudaMemsetAsync(h->d_adj_red, 0, sizeof(double), h->stream), "adjoint seed");
-  CUDA_TRY(launch_adjoint_seed(h->g, h->precision, grad_rho, grad_u, dtype, state_T, h->rho0, h->e,
+  CUDA_TRY(launch_adjoint_seed(h->raw, h->precision, grad_rho, grad_u, dtype, state_T, h->rho0, h->e,
                                lam_T, h->d_adj_red, h->stream),
            "adjoint seed");
   double dot = 0;
@@ -846,7 +899,8 @@ maclab_status maclab_adjoint_finish(maclab_handle h, const void* lam_0, const vo
   if (s != MACLAB_OK) return s;
   const size_t nred = 1 + 4 * (size_t)h->n_wall_ids;
   CUDA_TRY(cudaMemsetAsync(h->d_adj_red, 0, sizeof(double) * nred, h->stream), "adjoint finish");
-  CUDA_TRY(launch_adjoint_finish(h->g, h->precision, lam_0, state_0, h->d_node_type, h->n_wall_ids,
+  CUDA_TRY(launch_adjoint_finish(h->raw, h->precision, lam_0, state_0,
+                                 h->g.pad ? h->d_node_type_raw : h->d_node_type, h->n_wall_ids,
                                  h->rho0, h->e, grad_rho0, grad_u0, dtype,
                                  h->n_wall_ids ? h->d_adj_red + 1 : nullptr, h->d_adj_red, h->stream),
            "adjoint finish");
@@ -932,9 +986,9 @@ static maclab_status planes_args(maclab_ctx* h, int64_t p0, int64_t count, const
                                  size_t* plane_bytes) {
   if (!h || !buf) return fail(MACLAB_ERR_INVALID, "NULL argument");
   if (where != MACLAB_HOST && where != MACLAB_DEVICE) return fail(MACLAB_ERR_INVALID, "bad where");
-  const int64_t np = h->g.d == 3 ? h->g.nz : h->g.ny;
+  const int64_t np = march_planes(h);
   if (count < 1 || p0 < 0 || p0 + count > np) return fail(MACLAB_ERR_INVALID, "plane range outside the domain");
-  *plane_bytes = (size_t)(h->g.n / np) * h->elem;
+  *plane_bytes = (size_t)(h->raw.n / np) * h->elem;
   return MACLAB_OK;
 }
 
@@ -944,6 +998,16 @@ maclab_status maclab_get_planes(maclab_handle h, int64_t p0, int64_t count, void
   maclab_status s = planes_args(h, p0, count, dst, where, &pb);
   if (s != MACLAB_OK) return s;
   DeviceGuard dg(h->device);
+  if (h->g.pad) {  // packed into the staging buffer, then one copy (dst may be on another device)
+    const size_t bytes = (size_t)(h->g.d + 1) * count * pb;
+    s = ensure_staging(h, bytes);
+    if (s != MACLAB_OK) return s;
+    CUDA_TRY(launch_repack(h->g, h->precision, h->buf[h->cur], h->d_staging, p0, count, true, h->stream),
+             "get_planes repack");
+    CUDA_TRY(cudaMemcpyAsync(dst, h->d_staging, bytes, cudaMemcpyDefault, h->stream), "get_planes copy");
+    if (where == MACLAB_HOST) CUDA_TRY(cudaStreamSynchronize(h->stream), "get_planes sync");
+    return MACLAB_OK;
+  }
   const size_t field = (size_t)h->g.n * h->elem;
   for (int f = 0; f <= h->g.d; ++f)
     CUDA_TRY(cudaMemcpyAsync((char*)dst + f * count * pb, (const char*)h->buf[h->cur] + f * field + p0 * pb,
@@ -959,6 +1023,16 @@ maclab_status maclab_set_planes(maclab_handle h, int64_t p0, int64_t count, cons
   maclab_status s = planes_args(h, p0, count, src, where, &pb);
   if (s != MACLAB_OK) return s;
   DeviceGuard dg(h->device);
+  if (h->g.pad) {
+    const size_t bytes = (size_t)(h->g.d + 1) * count * pb;
+    s = ensure_staging(h, bytes);
+    if (s != MACLAB_OK) return s;
+    CUDA_TRY(cudaMemcpyAsync(h->d_staging, src, bytes, cudaMemcpyDefault, h->stream), "set_planes copy");
+    CUDA_TRY(launch_repack(h->g, h->precision, h->buf[h->cur], h->d_staging, p0, count, false, h->stream),
+             "set_planes repack");
+    if (where == MACLAB_HOST) CUDA_TRY(cudaStreamSynchronize(h->stream), "set_planes sync");
+    return MACLAB_OK;
+  }
   const size_t field = (size_t)h->g.n * h->elem;
   for (int f = 0; f <= h->g.d; ++f)
     CUDA_TRY(cudaMemcpyAsync((char*)h->buf[h->cur] + f * field + p0 * pb, (const char*)src + f * count * pb,
@@ -1040,7 +1114,9 @@ maclab_status maclab_set_kernel(maclab_handle h, int32_t kernel) {
   if (kernel != MACLAB_KERNEL_REFERENCE && kernel != MACLAB_KERNEL_TILED && kernel != MACLAB_KERNEL_FOLDED &&
       kernel != MACLAB_KERNEL_SEGMENT && kernel != MACLAB_KERNEL_ROWS2 && kernel != MACLAB_KERNEL_BLOCK)
     return fail(MACLAB_ERR_INVALID, "unknown kernel id");
-  if (!step_kernel_supported(h->g, h->precision, kernel))
+  // chosen by hand, a kernel takes the caller's row length and whole tiles only
+  // (padded rows and ragged last tiles are the library's own choice)
+  if (!step_kernel_supported(h->raw, h->precision, kernel))
     return fail(MACLAB_ERR_UNSUPPORTED, "kernel does not support this domain");
   h->kernel = kernel;
   // a tile shape the new kernel lacks falls back to its default
@@ -1068,14 +1144,19 @@ maclab_status maclab_get_launch_overlap(maclab_handle h, int32_t* on) {
 maclab_status maclab_set_tile(maclab_handle h, int32_t ty, int32_t tz) {
   if (!h) return fail(MACLAB_ERR_INVALID, "NULL handle");
   if (ty < 0 || tz < 0 || tz > (1 << 20)) return fail(MACLAB_ERR_INVALID, "bad tile shape");
-  const bool ok = h->kernel == MACLAB_KERNEL_FOLDED    ? fold_supported(h->g, h->precision, ty)
-                  : h->kernel == MACLAB_KERNEL_ROWS2   ? rows2_supported(h->g, h->precision, ty)
+  if (h->g.pad) return fail(MACLAB_ERR_UNSUPPORTED, "no built tiled instance has this shape");
+  bool ok = h->kernel == MACLAB_KERNEL_FOLDED          ? fold_supported(h->g, h->precision, ty, true)
+                  : h->kernel == MACLAB_KERNEL_ROWS2   ? rows2_supported(h->g, h->precision, ty, true)
                   : h->kernel == MACLAB_KERNEL_BLOCK   ? block_supported(h->g, h->precision, ty)  // ty: steps
                   : h->kernel == MACLAB_KERNEL_SEGMENT
                       ? (ty <= 1 || segment_depth(h->g, h->precision, ty) == 2)  // ty: steps per launch, tz: rows
                                                        : tiled_supported(h->g, h->precision, ty, tz);
-  if (!ok) return fail(MACLAB_ERR_UNSUPPORTED, "no built tiled instance has this shape");
+  // a ragged ny that the library serves with another kernel: the tiled kernel's shapes stay available
+  const bool to_tiled = !ok && !step_kernel_supported(h->g, h->precision, h->kernel) &&
+                        tiled_supported(h->g, h->precision, ty, tz);
+  if (!ok && !to_tiled) return fail(MACLAB_ERR_UNSUPPORTED, "no built tiled instance has this shape");
   drop_graphs(h);
+  if (to_tiled) h->kernel = MACLAB_KERNEL_TILED;
   h->ty = ty;
   h->tz = tz;
   return MACLAB_OK;
@@ -1175,7 +1256,8 @@ maclab_status maclab_set_wait_limit(maclab_handle h, int64_t polls) {
 struct maclab_batch_ctx {
   std::vector<maclab_ctx*> members;
   int lattice = 0, precision = 0;
-  bool one_launch = false;     // all D2Q9 with nx % 4 == 0: one launch per step
+  bool one_launch = false;     // all D2Q9 with rows of whole quads (nx % 4 == 0 or padded): one launch per step
+  bool odd_pad = false;        // some member's rows have odd padding
   void* d_insts = nullptr;
   void* d_items = nullptr;
   int n_items = 0;
@@ -1287,7 +1369,7 @@ maclab_status batch_persist_prepare(maclab_batch_ctx* b) {
   if (b->persist_blocks > 0) return MACLAB_OK;
   if (b->depth != 2) return fail(MACLAB_ERR_INVALID, "the persistent form needs the two-step work list");
   int capacity = 0;
-  if (batch_persist_capacity(b->precision, &capacity) != cudaSuccess || capacity < 1) {
+  if (batch_persist_capacity(b->precision, b->odd_pad, &capacity) != cudaSuccess || capacity < 1) {
     cudaGetLastError();
     return fail(MACLAB_ERR_UNSUPPORTED, "the persistent launch does not fit on this device");
   }
@@ -1318,17 +1400,17 @@ maclab_status batch_persist_prepare(maclab_batch_ctx* b) {
 // `sweeps` two-step sweeps from buffer c in one persistent launch.
 cudaError_t batch_launch_persist(maclab_batch_ctx* b, int c, int sweeps, cudaStream_t st) {
   return launch_batch_step2_persist(b->precision, b->d_insts, b->d_items, b->n_items, c, b->persist_blocks, sweeps,
-                                    b->d_deps, b->d_done, step_status(), b->wait_limit, st);
+                                    b->d_deps, b->d_done, step_status(), b->wait_limit, b->odd_pad, st);
 }
 
 // One launch of `steps` time steps (1, or b->depth) from buffer c.
 cudaError_t batch_launch_steps(maclab_batch_ctx* b, int c, int steps, cudaStream_t st) {
   if (b->one_launch && steps == 2)
-    return launch_batch_step2(b->precision, b->d_insts, b->d_items, b->n_items, c, b->blocks, st,
+    return launch_batch_step2(b->precision, b->d_insts, b->d_items, b->n_items, c, b->blocks, b->odd_pad, st,
                               b->overlap);
   if (b->one_launch)
     return launch_batch_step(b->precision, b->d_insts, b->d_items, b->n_items, c, b->blocks,
-                             b->depth == 2 ? kBatchSegW2 : kBatchSegW1, st, b->overlap);
+                             b->depth == 2 ? kBatchSegW2 : kBatchSegW1, b->odd_pad, st, b->overlap);
   for (maclab_ctx* m : b->members) {
     StepLaunch sl = step_launch(m, c);
     sl.seg_steps = 1;  // one step per member launch (the block kernel's one-step form)
@@ -1406,7 +1488,10 @@ maclab_status maclab_batch_create(const maclab_config* cfgs, int32_t count, macl
     }
   DeviceGuard dg(b->device);
   b->one_launch = b->lattice == MACLAB_D2Q9;
-  for (maclab_ctx* m : b->members) b->one_launch = b->one_launch && m->g.ilv == 1;
+  for (maclab_ctx* m : b->members) {
+    b->one_launch = b->one_launch && m->g.ilv == 1;
+    b->odd_pad = b->odd_pad || (m->g.pad & 1) != 0;
+  }
   // one launch per member and step: the segment kernel's work list is not
   // built, and the block kernel would take one step per launch
   if (!b->one_launch)
@@ -1553,7 +1638,7 @@ maclab_status maclab_batch_info(maclab_batch b, int64_t out[7]) {
   if (!b || !out) return fail(MACLAB_ERR_INVALID, "NULL argument");
   int64_t nodes = 0, fluid = 0;
   for (maclab_ctx* m : b->members) {
-    nodes += m->g.n;
+    nodes += m->raw.n;
     fluid += m->n_fluid;
   }
   out[0] = (int64_t)b->members.size();
@@ -1583,9 +1668,9 @@ bool shape_supported(const maclab_ctx* h, int kernel, int ty, int tz) {
   if (kernel == MACLAB_KERNEL_SEGMENT)
     return step_kernel_supported(h->g, h->precision, MACLAB_KERNEL_SEGMENT) &&
            (ty <= 1 || segment_depth(h->g, h->precision, ty) == 2);
-  if (kernel == MACLAB_KERNEL_ROWS2) return rows2_supported(h->g, h->precision, ty);
+  if (kernel == MACLAB_KERNEL_ROWS2) return rows2_supported(h->g, h->precision, ty, true);
   if (kernel == MACLAB_KERNEL_BLOCK) return block_supported(h->g, h->precision, ty);
-  return kernel == MACLAB_KERNEL_FOLDED ? fold_supported(h->g, h->precision, ty)
+  return kernel == MACLAB_KERNEL_FOLDED ? fold_supported(h->g, h->precision, ty, true)
                                         : tiled_supported(h->g, h->precision, ty, tz);
 }
 
@@ -1612,7 +1697,7 @@ std::string device_tag(int device) {
 
 std::string tune_key(const maclab_ctx* h) {
   char buf[160];
-  snprintf(buf, sizeof(buf), "%d/%d/%d/%d/%d/%u/%d/", h->g.lattice, h->precision, h->g.nx, h->g.ny,
+  snprintf(buf, sizeof(buf), "%d/%d/%d/%d/%d/%u/%d/", h->g.lattice, h->precision, h->raw.nx, h->g.ny,
            h->g.nz, h->g.periodic, h->g.wall_mode);
   return buf + device_tag(h->device);
 }
@@ -1707,14 +1792,14 @@ maclab_status maclab_tune(maclab_handle h, int32_t out[2]) {
   bool any = false;
   for (int kernel : {MACLAB_KERNEL_TILED, MACLAB_KERNEL_FOLDED, MACLAB_KERNEL_SEGMENT, MACLAB_KERNEL_ROWS2,
                      MACLAB_KERNEL_BLOCK})
-    any = any || step_kernel_supported(h->g, h->precision, kernel);
+    any = any || shape_supported(h, kernel, 0, 0);
   if (!any) {
     if (out) { out[0] = 0; out[1] = 0; }
     return MACLAB_OK;  // only the reference kernel serves this domain
   }
   // save the state
   void* saved = nullptr;
-  const size_t sb = state_bytes(h);
+  const size_t sb = buffer_bytes(h);
   if (cudaMalloc(&saved, sb) != cudaSuccess) {
     cudaGetLastError();
     return fail(MACLAB_ERR_OOM, "tuning buffer allocation failed");
@@ -1790,7 +1875,7 @@ maclab_status maclab_tune(maclab_handle h, int32_t out[2]) {
       ms = time_ms(h->stream, 1, [&]() {
              launch_batch_step2_persist(h->precision, h->d_seg_inst, h->d_seg_items, h->seg_n_items, h->cur,
                                         h->seg_persist_blocks, 32, h->d_seg_deps, h->d_seg_done, step_status(),
-                                        kWaitLimit, h->stream);
+                                        kWaitLimit, (h->g.pad & 1) != 0, h->stream);
            }) / 64.f;
     } else {
       ms = graph_ms(8);
@@ -1870,12 +1955,12 @@ maclab_status maclab_batch_tune(maclab_batch b, int32_t* rows_out) {
   std::vector<void*> saved(b->members.size(), nullptr);
   for (size_t i = 0; i < b->members.size(); ++i) {
     maclab_ctx* m = b->members[i];
-    if (cudaMalloc(&saved[i], state_bytes(m)) != cudaSuccess) {
+    if (cudaMalloc(&saved[i], buffer_bytes(m)) != cudaSuccess) {
       cudaGetLastError();
       for (void* p : saved) cudaFree(p);
       return fail(MACLAB_ERR_OOM, "tuning buffer allocation failed");
     }
-    cudaMemcpyAsync(saved[i], m->buf[m->cur], state_bytes(m), cudaMemcpyDeviceToDevice, b->stream);
+    cudaMemcpyAsync(saved[i], m->buf[m->cur], buffer_bytes(m), cudaMemcpyDeviceToDevice, b->stream);
   }
   // rows per work item x time steps per launch, compared per time step on a
   // captured graph of 8 launches, or 64 where 8 take under 0.5 ms (stepping
@@ -1954,8 +2039,8 @@ maclab_status maclab_batch_tune(maclab_batch b, int32_t* rows_out) {
   b->cur = 0;
   for (size_t i = 0; i < b->members.size(); ++i) {
     maclab_ctx* m = b->members[i];
-    cudaMemcpyAsync(m->buf[0], saved[i], state_bytes(m), cudaMemcpyDeviceToDevice, b->stream);
-    cudaMemcpyAsync(m->buf[1], saved[i], state_bytes(m), cudaMemcpyDeviceToDevice, b->stream);
+    cudaMemcpyAsync(m->buf[0], saved[i], buffer_bytes(m), cudaMemcpyDeviceToDevice, b->stream);
+    cudaMemcpyAsync(m->buf[1], saved[i], buffer_bytes(m), cudaMemcpyDeviceToDevice, b->stream);
     m->cur = 0;
     m->prev_valid = false;
   }

@@ -36,6 +36,8 @@ struct BatchInst {
   int nx, ny;            // nx % 4 == 0
   int px, py;            // periodic flags
   int wall_mode;
+  int pad;               // storage positions of a row beyond the domain (Geometry)
+  int hi_quad;           // quad of the domain's last node (hi_wall_quad)
   float force[2];        // lattice-unit force increment (FP32 arithmetic)
   double force64[2];     // the same for FP64 storage
 };
@@ -120,12 +122,12 @@ __device__ __forceinline__ void batch_row_update(const typename Pair<C>::P (&st)
 
 // Store of one final row (Eq. (5): u' = M / (36 + R) + F).  In box mode every
 // lane stores its whole quad: a lane whose quad holds one x-wall node (a.x at
-// x = 0, b.y at x = nx - 1) puts that node's unchanged fields wk in place of
+// x = 0, b.y, or a.y with odd padding, at the domain's last node) puts that node's unchanged fields wk in place of
 // the computed ones, so the warp never splits into per-node stores.  Masks,
 // and a quad holding both x-walls (nx = 4), store node by node.
-template <typename S>
+template <typename S, bool HIA>
 __device__ __forceinline__ void batch_store(S* out, int64_t n, int64_t off, const uint8_t* mask, int wall_mode,
-                                            bool x_lo_wall, bool x_hi_wall,
+                                            bool x_lo_wall, bool x_hi_wall, bool hi_a,
                                             const typename Store<S>::C (&wk)[3],
                                             const typename Pair<typename Store<S>::C>::P (&acc)[2][3],
                                             const typename Pair<typename Store<S>::C>::P (&force)[2]) {
@@ -142,7 +144,7 @@ __device__ __forceinline__ void batch_store(S* out, int64_t n, int64_t off, cons
     v[2][q] = O::fma(acc[q][2], inv, force[1]);
   }
   if (wall_mode == kWallMask || (x_lo_wall && x_hi_wall)) {
-    bool wall[4] = {x_lo_wall, false, false, x_hi_wall};
+    bool wall[4] = {x_lo_wall, x_hi_wall && hi_a, false, x_hi_wall && !hi_a};
     if (wall_mode == kWallMask) {
       const uchar4 m = *reinterpret_cast<const uchar4*>(mask + off);
       wall[0] = m.x != 0; wall[1] = m.y != 0; wall[2] = m.z != 0; wall[3] = m.w != 0;
@@ -164,14 +166,21 @@ __device__ __forceinline__ void batch_store(S* out, int64_t n, int64_t off, cons
 #pragma unroll
   for (int f = 0; f < K; ++f) {
     if (x_lo_wall) v[f][0].x = wk[f];
-    if (x_hi_wall) v[f][1].y = wk[f];
+    if constexpr (HIA) {
+      if (x_hi_wall && !hi_a) v[f][1].y = wk[f];
+      if (x_hi_wall && hi_a) v[f][0].y = wk[f];
+    } else {
+      if (x_hi_wall) v[f][1].y = wk[f];
+    }
     Quad<S>::st(out + f * n + off, v[f][0], v[f][1]);
   }
 }
 
 // segw: quads per work item's segment (30, or fewer when the work list was cut
-// for two steps per launch)
-template <typename S>
+// for two steps per launch).  HIA: some domain's rows have odd padding (its
+// right wall is lane a.y of its quad instead of b.y; an instance of its own, as
+// the run-time choice costs 6 % at 1024^2).
+template <typename S, bool HIA>
 __global__ void __launch_bounds__(256) batch_step_d2q9(const BatchInst* __restrict__ insts,
                                                        const BatchItem* __restrict__ items,
                                                        int n_items, int cur, int segw) {
@@ -213,7 +222,8 @@ __global__ void __launch_bounds__(256) batch_step_d2q9(const BatchInst* __restri
       force[1] = O::splat(C(I.force[1]));
     }
     const bool x_lo_wall = d_wall == kWallBox && !d_px && t == 0 && interior;
-    const bool x_hi_wall = d_wall == kWallBox && !d_px && t == nq - 1 && interior;
+    const bool x_hi_wall = d_wall == kWallBox && !d_px && t == I.hi_quad && interior;
+    const bool hi_a = HIA && (I.pad & 1) != 0;  // the right wall is lane a.y of its quad instead of b.y
     C wk[K] = {C(0), C(0), C(0)};  // x-wall lanes: the wall node's fields in the row stored next
 
     auto row_exists = [&](int y) { return (y >= 0 && y < d_ny) || d_py; };
@@ -239,7 +249,7 @@ __global__ void __launch_bounds__(256) batch_step_d2q9(const BatchInst* __restri
       if (!interior) return;
       if (!d_py && (y == 0 || y == d_ny - 1)) return;
       const int64_t off = (int64_t)y * d_nx + 4 * t;
-      batch_store<S>(out, n, off, d_mask, d_wall, x_lo_wall, x_hi_wall, wk, acc, force);
+      batch_store<S, HIA>(out, n, off, d_mask, d_wall, x_lo_wall, x_hi_wall, hi_a, wk, acc, force);
     };
 
     P R0[2][K], R1[2][K], R2[2][K];
@@ -265,7 +275,7 @@ __global__ void __launch_bounds__(256) batch_step_d2q9(const BatchInst* __restri
       batch_row_update<C, kMid>(st, A, B, N);
       if (y - 1 >= y0) store(y - 1, A);
 #pragma unroll
-      for (int f = 0; f < K; ++f) wk[f] = x_lo_wall ? st[f][0].x : st[f][1].y;  // row y, stored next
+      for (int f = 0; f < K; ++f) wk[f] = x_lo_wall ? st[f][0].x : (hi_a ? st[f][0].y : st[f][1].y);  // row y, stored next
 #pragma unroll
       for (int q = 0; q < 2; ++q)
 #pragma unroll
@@ -376,7 +386,7 @@ __device__ __forceinline__ void zero_sums(P (&a)[2][3]) {
 // Two updates of every work item, reading buffer cur and writing cur ^ 1:
 // the work of one launch of batch_step2_d2q9 (and of one sweep of the
 // persistent kernel below).
-template <typename S>
+template <typename S, bool HIA>
 __device__ __forceinline__ void batch2_sweep(const BatchInst* __restrict__ insts,
                                              const BatchItem* __restrict__ items, int n_items, int cur,
                                              const RowRing<S, 3>& ring, int lane, int warp, int nwarps) {
@@ -413,10 +423,12 @@ __device__ __forceinline__ void batch2_sweep(const BatchInst* __restrict__ insts
     uint32_t xwall = 0;
     if (d_wall == kWallBox && !d_px) {
       if (t == 0) xwall |= swapped ? 2u : 1u;
-      if (t == nq - 1) xwall |= swapped ? 4u : 8u;
+      if (t == I.hi_quad)
+        xwall |= HIA && (I.pad & 1) ? (swapped ? 1u : 2u) : (swapped ? 4u : 8u);
     }
     const bool x_lo_wall = d_wall == kWallBox && !d_px && t == 0 && interior;
-    const bool x_hi_wall = d_wall == kWallBox && !d_px && t == nq - 1 && interior;
+    const bool x_hi_wall = d_wall == kWallBox && !d_px && t == I.hi_quad && interior;
+    const bool hi_a = HIA && (I.pad & 1) != 0;  // the right wall is lane a.y of its quad instead of b.y
     // x-wall lanes: the wall node's fields in the final row stored next (walls
     // keep their values, so the intermediate row's are the input's)
     C wk[K] = {C(0), C(0), C(0)};
@@ -472,7 +484,7 @@ __device__ __forceinline__ void batch2_sweep(const BatchInst* __restrict__ insts
       if (!interior) return;
       if (!d_py && (y == 0 || y == d_ny - 1)) return;
       const int64_t off = (int64_t)y * d_nx + 4 * t;
-      batch_store<S>(out, n, off, d_mask, d_wall, x_lo_wall, x_hi_wall, wk, acc, force);
+      batch_store<S, HIA>(out, n, off, d_mask, d_wall, x_lo_wall, x_hi_wall, hi_a, wk, acc, force);
     };
 
     // sums of the first update for row d in A[(d - y0 + 3) % 3], of the second in B[...]
@@ -487,7 +499,7 @@ __device__ __forceinline__ void batch2_sweep(const BatchInst* __restrict__ insts
     };
     auto keep_wall = [&]() {  // wk <- intermediate row just emitted, the final row stored next
 #pragma unroll
-      for (int f = 0; f < K; ++f) wk[f] = x_lo_wall ? mid[f][0].x : mid[f][1].y;
+      for (int f = 0; f < K; ++f) wk[f] = x_lo_wall ? mid[f][0].x : (hi_a ? mid[f][0].y : mid[f][1].y);
     };
     auto keep = [&]() {  // prev <- st: the input of the row the next emission completes
 #pragma unroll
@@ -556,7 +568,7 @@ __device__ __forceinline__ void batch2_sweep(const BatchInst* __restrict__ insts
 }
 
 // FP32: three blocks per SM; FP64 needs more registers (two blocks)
-template <typename S>
+template <typename S, bool HIA>
 __global__ void __launch_bounds__(128, sizeof(S) == 8 ? 2 : 3) batch_step2_d2q9(const BatchInst* __restrict__ insts,
                                                            const BatchItem* __restrict__ items,
                                                            int n_items, int cur) {
@@ -567,7 +579,7 @@ __global__ void __launch_bounds__(128, sizeof(S) == 8 ? 2 : 3) batch_step2_d2q9(
   const RowRing<S, 3> ring(batch_smem, threadIdx.x >> 5, lane);
   pdl_wait();  // the previous step's writes are visible from here on
   pdl_launch_next();
-  batch2_sweep<S>(insts, items, n_items, cur, ring, lane, warp, nwarps);
+  batch2_sweep<S, HIA>(insts, items, n_items, cur, ring, lane, warp, nwarps);
 }
 
 __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
@@ -591,7 +603,7 @@ __device__ __forceinline__ void st_release_gpu(unsigned* p, unsigned v) {
 // and one that runs out sets bit 1 of *status and ends the block's sweeps (its
 // neighbours' waits then run out in turn).  The state is read through the row ring only
 // (cp.async.cg, from L2), so a block never sees another block's stale values.
-template <typename S>
+template <typename S, bool HIA>
 __global__ void __launch_bounds__(128, sizeof(S) == 8 ? 2 : 3)
     batch_step2_persist(const BatchInst* __restrict__ insts, const BatchItem* __restrict__ items, int n_items,
                         int cur, int sweeps, const int* __restrict__ deps, unsigned* __restrict__ done,
@@ -603,7 +615,7 @@ __global__ void __launch_bounds__(128, sizeof(S) == 8 ? 2 : 3)
   const RowRing<S, 3> ring(batch_smem, threadIdx.x >> 5, lane);
   const int d0 = deps[blockIdx.x], d1 = deps[blockIdx.x + 1];
   for (int k = 0; k < sweeps; ++k) {
-    batch2_sweep<S>(insts, items, n_items, cur ^ (k & 1), ring, lane, warp, nwarps);
+    batch2_sweep<S, HIA>(insts, items, n_items, cur ^ (k & 1), ring, lane, warp, nwarps);
     if (k + 1 == sweeps) break;
     cp_async_wait<0>();  // no row copy of this sweep lands after the next one starts
     __syncthreads();
@@ -631,49 +643,50 @@ __global__ void __launch_bounds__(128, sizeof(S) == 8 ? 2 : 3)
 
 template <typename S>
 static cudaError_t launch_batch2_t(const BatchInst* insts, const BatchItem* items, int n_items,
-                                   int cur, int blocks, cudaStream_t st, int overlap) {
+                                   int cur, int blocks, bool odd, cudaStream_t st, int overlap) {
   constexpr size_t smem = 4 * RowRing<S, 3>::warp_bytes;  // 4 warps
-  return launch_kernel(batch_step2_d2q9<S>, dim3(blocks), dim3(128), smem, st, overlap, insts, items,
+  return launch_kernel(odd ? batch_step2_d2q9<S, true> : batch_step2_d2q9<S, false>, dim3(blocks), dim3(128), smem, st, overlap, insts, items,
                        n_items, cur);
 }
 
 template <typename S>
 static cudaError_t launch_batch_t(const BatchInst* insts, const BatchItem* items, int n_items,
-                                  int cur, int blocks, int segw, cudaStream_t st, int overlap) {
-  return launch_kernel(batch_step_d2q9<S>, dim3(blocks), dim3(256), 0, st, overlap, insts, items, n_items,
+                                  int cur, int blocks, int segw, bool odd, cudaStream_t st, int overlap) {
+  return launch_kernel(odd ? batch_step_d2q9<S, true> : batch_step_d2q9<S, false>, dim3(blocks), dim3(256), 0, st, overlap, insts, items, n_items,
                        cur, segw);
 }
 
 cudaError_t launch_batch_step(int precision, const void* insts, const void* items, int n_items,
-                              int cur, int blocks, int segw, cudaStream_t st, int overlap) {
+                              int cur, int blocks, int segw, bool odd, cudaStream_t st, int overlap) {
   const BatchInst* I = static_cast<const BatchInst*>(insts);
   const BatchItem* T = static_cast<const BatchItem*>(items);
   if (segw < 1 || segw > 30) return cudaErrorInvalidValue;
   switch (precision) {
-    case MACLAB_F64: return launch_batch_t<double>(I, T, n_items, cur, blocks, segw, st, overlap);
-    case MACLAB_F32: return launch_batch_t<float>(I, T, n_items, cur, blocks, segw, st, overlap);
-    case MACLAB_BF16_STORE: return launch_batch_t<__nv_bfloat16>(I, T, n_items, cur, blocks, segw, st, overlap);
-    case MACLAB_F16_STORE: return launch_batch_t<__half>(I, T, n_items, cur, blocks, segw, st, overlap);
+    case MACLAB_F64: return launch_batch_t<double>(I, T, n_items, cur, blocks, segw, odd, st, overlap);
+    case MACLAB_F32: return launch_batch_t<float>(I, T, n_items, cur, blocks, segw, odd, st, overlap);
+    case MACLAB_BF16_STORE: return launch_batch_t<__nv_bfloat16>(I, T, n_items, cur, blocks, segw, odd, st, overlap);
+    case MACLAB_F16_STORE: return launch_batch_t<__half>(I, T, n_items, cur, blocks, segw, odd, st, overlap);
   }
   return cudaErrorInvalidValue;
 }
 
 // Two steps per launch: FP32 and FP64 storage only.
 cudaError_t launch_batch_step2(int precision, const void* insts, const void* items, int n_items,
-                               int cur, int blocks, cudaStream_t st, int overlap) {
+                               int cur, int blocks, bool odd, cudaStream_t st, int overlap) {
   const BatchInst* I = static_cast<const BatchInst*>(insts);
   const BatchItem* T = static_cast<const BatchItem*>(items);
   switch (precision) {
-    case MACLAB_F64: return launch_batch2_t<double>(I, T, n_items, cur, blocks, st, overlap);
-    case MACLAB_F32: return launch_batch2_t<float>(I, T, n_items, cur, blocks, st, overlap);
+    case MACLAB_F64: return launch_batch2_t<double>(I, T, n_items, cur, blocks, odd, st, overlap);
+    case MACLAB_F32: return launch_batch2_t<float>(I, T, n_items, cur, blocks, odd, st, overlap);
   }
   return cudaErrorInvalidValue;
 }
 
+// odd: the instance that takes odd padding (either needs the setting before a launch)
 template <typename S>
-static cudaError_t persist_setup(int* capacity) {
+static cudaError_t persist_setup(int* capacity, bool odd) {
   constexpr size_t smem = 4 * RowRing<S, 3>::warp_bytes;  // 4 warps
-  auto kern = batch_step2_persist<S>;
+  auto kern = odd ? batch_step2_persist<S, true> : batch_step2_persist<S, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0, dev = 0, sms = 0;
@@ -685,11 +698,11 @@ static cudaError_t persist_setup(int* capacity) {
 }
 
 // Blocks of the persistent launch that can be resident at once (its limit).
-cudaError_t batch_persist_capacity(int precision, int* capacity) {
+cudaError_t batch_persist_capacity(int precision, bool odd, int* capacity) {
   *capacity = 0;
   switch (precision) {
-    case MACLAB_F64: return persist_setup<double>(capacity);
-    case MACLAB_F32: return persist_setup<float>(capacity);
+    case MACLAB_F64: return persist_setup<double>(capacity, odd);
+    case MACLAB_F32: return persist_setup<float>(capacity, odd);
   }
   return cudaErrorInvalidValue;
 }
@@ -697,10 +710,10 @@ cudaError_t batch_persist_capacity(int precision, int* capacity) {
 template <typename S>
 static cudaError_t launch_batch2_persist_t(const BatchInst* insts, const BatchItem* items, int n_items, int cur,
                                            int blocks, int sweeps, const int* deps, unsigned* done,
-                                           unsigned* status, unsigned wait_limit, cudaStream_t st) {
+                                           unsigned* status, unsigned wait_limit, bool odd, cudaStream_t st) {
   constexpr size_t smem = 4 * RowRing<S, 3>::warp_bytes;
   int capacity = 0;
-  cudaError_t e = persist_setup<S>(&capacity);
+  cudaError_t e = persist_setup<S>(&capacity, odd);
   if (e != cudaSuccess) return e;
   // a cooperative launch: every block resident at once (the waits need it);
   // the dependency lists were built for exactly this block count
@@ -716,7 +729,7 @@ static cudaError_t launch_batch2_persist_t(const BatchInst* insts, const BatchIt
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, batch_step2_persist<S>, insts, items, n_items, cur, sweeps, deps, done, status,
+  return cudaLaunchKernelEx(&cfg, odd ? batch_step2_persist<S, true> : batch_step2_persist<S, false>, insts, items, n_items, cur, sweeps, deps, done, status,
                             wait_limit);
 }
 
@@ -725,15 +738,15 @@ static cudaError_t launch_batch2_persist_t(const BatchInst* insts, const BatchIt
 // done: `blocks` counters (zeroed here); wait_limit: polls before a wait gives up.
 cudaError_t launch_batch_step2_persist(int precision, const void* insts, const void* items, int n_items, int cur,
                                        int blocks, int sweeps, const int* deps, unsigned* done, unsigned* status,
-                                       unsigned wait_limit, cudaStream_t st) {
+                                       unsigned wait_limit, bool odd, cudaStream_t st) {
   const BatchInst* I = static_cast<const BatchInst*>(insts);
   const BatchItem* T = static_cast<const BatchItem*>(items);
   if (sweeps < 1 || !deps || !done) return cudaErrorInvalidValue;
   switch (precision) {
     case MACLAB_F64:
-      return launch_batch2_persist_t<double>(I, T, n_items, cur, blocks, sweeps, deps, done, status, wait_limit, st);
+      return launch_batch2_persist_t<double>(I, T, n_items, cur, blocks, sweeps, deps, done, status, wait_limit, odd, st);
     case MACLAB_F32:
-      return launch_batch2_persist_t<float>(I, T, n_items, cur, blocks, sweeps, deps, done, status, wait_limit, st);
+      return launch_batch2_persist_t<float>(I, T, n_items, cur, blocks, sweeps, deps, done, status, wait_limit, odd, st);
   }
   return cudaErrorInvalidValue;
 }
@@ -797,6 +810,8 @@ void batch_fill_inst(void* dst, const Geometry& g, void* buf0, void* buf1, const
   b->px = (g.periodic & 1u) ? 1 : 0;
   b->py = (g.periodic & 2u) ? 1 : 0;
   b->wall_mode = g.wall_mode;
+  b->pad = g.pad;
+  b->hi_quad = hi_wall_quad(g.nx, g.pad);
   b->force[0] = (float)force[0];
   b->force[1] = (float)force[1];
   b->force64[0] = force[0];

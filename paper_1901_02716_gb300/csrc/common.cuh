@@ -179,14 +179,30 @@ enum WallMode : int {
 struct Geometry {
   int lattice;        // kD2Q9 / kD3Q19
   int d;              // 2 or 3
-  int nx, ny, nz;     // nz = 1 for D2Q9
+  int nx, ny, nz;     // nz = 1 for D2Q9; nx is the length of a stored row
   int64_t n;          // nx * ny * nz
   uint32_t periodic;  // bit0 x, bit1 y, bit2 z
   int wall_mode;      // WallMode
   const uint8_t* mask;  // device node types in storage order (kWallMask), else unused
   int ilv;            // 1: the two halves of every x row are interleaved in storage
   int hx;             // nx / 2 (used when ilv)
+  // Stored rows may end in pad = 1..3 positions beyond the domain's last node
+  // (x = nx - pad .. nx - 1), which bring a closed x axis of any width to the
+  // interleaved rows of the fast kernels (FP32 step of the 251^3 cavity: 508 us
+  // on the one-thread-per-node kernel, 142 us now; of the 401^2 cavity: 4.3 and
+  // 2.1 us).  The domain's right wall is then at x = nx - 1 -
+  // pad and shields it: whatever a step leaves in the padding reaches only wall
+  // nodes, which keep their values.  In mask mode the padding is marked as wall.
+  int pad;
 };
+
+// Narrower closed domains than this keep their natural rows: at least two
+// quads must lie between the two x-walls, so that no quad holds both.
+constexpr int kMinPadWidth = 17;
+
+// The thread (quad) of a row that holds the right wall, and whether the wall is
+// lane a.y of that quad (pad odd) or lane b.y (pad even).
+__host__ __device__ inline int hi_wall_quad(int nx, int pad) { return (nx >> 2) - 1 - (pad >> 1); }
 
 // Storage position within an x row of logical x, and its inverse.  With ilv
 // (nx % 4 == 0) node x is stored at 2 (x mod H) + [x >= H], H = nx / 2, so that
@@ -240,8 +256,8 @@ int segment_depth(const Geometry& g, int precision, int ty);
 // batch_persist_capacity: the most blocks that can be resident at once.
 cudaError_t launch_batch_step2_persist(int precision, const void* insts, const void* items, int n_items, int cur,
                                        int blocks, int sweeps, const int* deps, unsigned* done, unsigned* status,
-                                       unsigned wait_limit, cudaStream_t st);
-cudaError_t batch_persist_capacity(int precision, int* capacity);
+                                       unsigned wait_limit, bool odd, cudaStream_t st);
+cudaError_t batch_persist_capacity(int precision, bool odd, int* capacity);
 // ny[i], py[i]: rows and y periodicity of domain i of the work list.
 void batch_persist_deps(const std::vector<int>& items4, const std::vector<int>& ny, const std::vector<int>& py,
                         int blocks, std::vector<int>& out);
@@ -257,7 +273,8 @@ cudaError_t launch_tiled(const StepLaunch& s, cudaStream_t stream, int ty, int t
 int tiled_threads(const Geometry& g, int precision, int ty, int tz);
 
 // Defined in step_fold.cu (D3Q19 FP32 without halo-row threads).
-bool fold_supported(const Geometry& g, int precision, int ty);
+// ragged: also where the rows of the tile do not divide ny
+bool fold_supported(const Geometry& g, int precision, int ty, bool ragged = false);
 int fold_threads(const Geometry& g, int precision, int ty);
 cudaError_t launch_fold(const StepLaunch& s, cudaStream_t stream, int ty, int tz);
 // Chunks of the march axis for a grid of ytiles tiles per plane with per_sm
@@ -265,7 +282,7 @@ cudaError_t launch_fold(const StepLaunch& s, cudaStream_t stream, int ty, int tz
 int fold_chunks(int nplanes, int ytiles, int tz_req, int per_sm);
 
 // Defined in step_rows2.cu (D3Q19, two rows per thread; FP32 arithmetic).
-bool rows2_supported(const Geometry& g, int precision, int ty);
+bool rows2_supported(const Geometry& g, int precision, int ty, bool ragged = false);
 int rows2_threads(const Geometry& g, int precision, int ty);
 cudaError_t launch_rows2(const StepLaunch& s, cudaStream_t stream, int ty, int tz);
 // The viscosity term of one reverse step (maclab_adjoint_nu_term) on the two-rows
@@ -313,19 +330,21 @@ cudaError_t launch_adjoint_finish(const Geometry& g, int precision, const void* 
                                   void* gu, int dtype, double* wall, double* dot, cudaStream_t st);
 
 // Defined in batch.cu.
-// segw: quads per segment of the work list (30 when it was cut for one step per launch)
+// segw: quads per segment of the work list (30 when it was cut for one step per launch);
+// odd: a domain of the list has odd padding (Geometry)
 cudaError_t launch_batch_step(int precision, const void* insts, const void* items, int n_items,
-                              int cur, int blocks, int segw, cudaStream_t st, int overlap);
+                              int cur, int blocks, int segw, bool odd, cudaStream_t st, int overlap);
 constexpr int kBatchSegW1 = 30, kBatchSegW2 = 28;
 // two time steps per launch (FP32 / FP64 storage, every nx >= 8), 128-thread blocks
 cudaError_t launch_batch_step2(int precision, const void* insts, const void* items, int n_items,
-                               int cur, int blocks, cudaStream_t st, int overlap);
+                               int cur, int blocks, bool odd, cudaStream_t st, int overlap);
 size_t batch_inst_bytes();
 size_t batch_item_bytes();
 void batch_fill_inst(void* dst, const Geometry& g, void* buf0, void* buf1, const double force[3]);
 void batch_items(int inst, const Geometry& g, int rows, int depth, std::vector<int>& out4);
 
 // Defined in convert.cu.
+// g: the stored rows; nx: the caller's row length (g.nx - g.pad)
 cudaError_t launch_set_physical(const Geometry& g, int precision, const void* rho,
                                 const void* u, int dtype, double rho0, double e,
                                 const uint8_t* node_type, const double* wall_lat,
@@ -336,6 +355,11 @@ cudaError_t launch_get_physical(const Geometry& g, int precision, const void* st
 cudaError_t launch_set_wall_values(const Geometry& g, int precision, const void* rho, const void* u,
                                    int dtype, double rho0, double e, const uint8_t* node_type, void* s0,
                                    void* s1, cudaStream_t stream);
+// Planes [p0, p0 + count) of the march axis between the stored rows of g and the
+// raw layout of a state without padding ([field][plane][row] of g.nx - g.pad
+// nodes in their natural order); to_raw: out of the state, else into it.
+cudaError_t launch_repack(const Geometry& g, int precision, void* state, void* raw, int64_t p0, int64_t count,
+                          bool to_raw, cudaStream_t stream);
 cudaError_t launch_copy_walls(const Geometry& g, int precision, const uint8_t* node_type, const void* src,
                               void* dst, cudaStream_t stream);
 cudaError_t launch_fill_walls(const Geometry& g, int precision, const uint8_t* node_type,
@@ -347,7 +371,8 @@ cudaError_t launch_fill_walls(const Geometry& g, int precision, const uint8_t* n
 // ------------------------------------------------------------------ the handle
 
 struct maclab_ctx {
-  maclab::Geometry g{};
+  maclab::Geometry g{};            // the state buffers' rows
+  maclab::Geometry raw{};          // the raw state's rows (the caller's; = g unless g.pad > 0)
   int precision = MACLAB_F32;
   double dx = 0, nu = 0, rho0 = 1, e = 0, dt = 0, rle = 0;
   double force_phys[3] = {0, 0, 0};
@@ -358,7 +383,8 @@ struct maclab_ctx {
   int64_t n_fluid = 0;
   cudaStream_t stream = nullptr;
   int device = 0;
-  uint8_t* d_node_type = nullptr;  // device copy of the node types (if any walls)
+  uint8_t* d_node_type = nullptr;  // device copy of the node types (if any walls), rows of g
+  uint8_t* d_node_type_raw = nullptr;  // the same in rows of raw (g.pad > 0 only)
   double* d_wall_lat = nullptr;    // device copy of wall_lat
   void* buf[2] = {nullptr, nullptr};
   int cur = 0;                     // buf[cur] holds the current state

@@ -34,10 +34,12 @@ struct UnitMap {
   double rho0, e, inv_rho0, inv_e;
   float f_rho0, f_inv_rho0;      // exact (rho0 a power of two)
   float e_hi, e_lo, ie_hi, ie_lo;  // e and 1 / e as sums of two floats
+  int64_t nu;                      // nodes of the user arrays (their field stride)
 };
 
 // Whether the FP32 forms above apply.
-static bool unit_map(double rho0, double e, UnitMap* m) {
+static bool unit_map(const Geometry& g, double rho0, double e, UnitMap* m) {
+  m->nu = g.n / g.nx * (g.nx - g.pad);
   m->rho0 = rho0;
   m->e = e;
   m->inv_rho0 = 1.0 / rho0;
@@ -97,48 +99,85 @@ struct alignas(4 * sizeof(S) > 16 ? 16 : 4 * sizeof(S)) Four {
 
 // The kernels walk the user arrays in order (a warp touches contiguous runs of
 // each user array, which may be page-locked host memory read or written over
-// the host link).  QUAD (interleaved rows, nx % 4 == 0, user arrays aligned to
-// two values): a thread takes one storage quad, the nodes (2t, 2t + H,
-// 2t + 1, 2t + 1 + H) of a row, i.e. two runs of two user values per field and
-// one wide store, so a warp moves whole sectors on both sides; otherwise a
-// thread takes one node.  I: index type (32 bits wherever the count allows, as
-// the division by the row length is the largest integer cost).
-template <typename I, bool QUAD, typename Fn>
+// the host link).  kQuad2 (interleaved rows without padding, user arrays
+// aligned to two values): a thread takes one storage quad, the nodes (2t,
+// 2t + H, 2t + 1, 2t + 1 + H) of a row, i.e. two runs of two user values per
+// field and one wide store, so a warp moves whole sectors on both sides.
+// kQuad1 (padded rows or unaligned user arrays): the same quad with single user
+// values, of which the one or two beyond the domain's last node do not exist.
+// kNode (natural rows): a thread takes one node, at the same place on both
+// sides.  I: index type (32 bits wherever the count allows, as the division by
+// the row length is the largest integer cost).
+enum Unit { kNode, kQuad1, kQuad2 };
+
+// fn(storage index, user index, x of the unit's first node)
+template <typename I, int U, typename Fn>
 __device__ __forceinline__ void for_units(const Geometry& g, Fn&& fn) {
-  const I per_row = (I)(QUAD ? g.nx / 4 : g.nx);
-  const I units = (I)(QUAD ? g.n / 4 : g.n);
+  const I units = (I)(U != kNode ? g.n / 4 : g.n);
   for (I k = (I)blockIdx.x * blockDim.x + threadIdx.x; k < units; k += (I)gridDim.x * blockDim.x) {
-    const I row = k / per_row;
-    const int t = (int)(k - row * per_row);
-    if constexpr (QUAD) {
-      fn((int64_t)4 * k, (int64_t)row * g.nx + 2 * t);
+    if constexpr (U == kNode) {
+      fn((int64_t)k, (int64_t)k, 0);
     } else {
-      fn((int64_t)row * g.nx + mem_x(g, t), (int64_t)k);
+      const I per_row = (I)(g.nx / 4);
+      const I row = k / per_row;
+      const int x = 2 * (int)(k - row * per_row);
+      fn((int64_t)4 * k, (int64_t)row * (g.nx - g.pad) + x, x);
     }
+  }
+}
+
+// Nodes (x, x + H, x + 1, x + 1 + H) of a user row, j the index of x; those past
+// the end of a padded row read as 0 and are not written.
+template <int U, typename T>
+__device__ __forceinline__ void ld_user(const Geometry& g, const T* p, int64_t j, int x, T (&v)[4]) {
+  if constexpr (U == kQuad2) {
+    const Two<T> a = *reinterpret_cast<const Two<T>*>(p + j);
+    const Two<T> b = *reinterpret_cast<const Two<T>*>(p + j + g.hx);
+    v[0] = a.x;
+    v[1] = b.x;
+    v[2] = a.y;
+    v[3] = b.y;
+  } else {
+    const int last = g.nx - g.pad - 1 - g.hx;
+    v[0] = p[j];
+    v[1] = x <= last ? p[j + g.hx] : T(0);
+    v[2] = p[j + 1];
+    v[3] = x + 1 <= last ? p[j + 1 + g.hx] : T(0);
+  }
+}
+template <int U, typename T>
+__device__ __forceinline__ void st_user(const Geometry& g, T* p, int64_t j, int x, const T (&v)[4]) {
+  if constexpr (U == kQuad2) {
+    *reinterpret_cast<Two<T>*>(p + j) = Two<T>{v[0], v[2]};
+    *reinterpret_cast<Two<T>*>(p + j + g.hx) = Two<T>{v[1], v[3]};
+  } else {
+    const int last = g.nx - g.pad - 1 - g.hx;
+    p[j] = v[0];
+    p[j + 1] = v[2];
+    if (x <= last) p[j + g.hx] = v[1];
+    if (x + 1 <= last) p[j + 1 + g.hx] = v[3];
   }
 }
 
 // Both state buffers are given: wall nodes are written into both (the step
 // kernels never write them), fluid nodes into s0 only, as every step writes
 // all fluid nodes of the buffer it fills.
-template <typename S, typename T, bool FAST, typename I, bool QUAD>
+template <typename S, typename T, bool FAST, typename I, int U>
 __global__ void __launch_bounds__(256) set_physical_k(Geometry g, const T* __restrict__ rho, const T* __restrict__ u,
                                                       UnitMap m, const uint8_t* __restrict__ node_type,
                                                       const double* __restrict__ wall_lat, int n_wall_ids,
                                                       S* __restrict__ s0, S* __restrict__ s1) {
   using MP = Map<S, FAST>;
-  const int64_t N = g.n;
+  const int64_t N = g.n, NU = m.nu;  // field strides: state, user arrays
   const int d = g.d;
-  for_units<I, QUAD>(g, [&](int64_t i, int64_t j) {
-    if constexpr (QUAD) {
+  for_units<I, U>(g, [&](int64_t i, int64_t j, int x) {
+    if constexpr (U != kNode) {
       Four<S> q[4];
 #pragma unroll
       for (int f = 0; f < 4; ++f) {
         if (f > d) continue;
-        const T* src = f == 0 ? rho : u + (f - 1) * N;
-        const Two<T> a = *reinterpret_cast<const Two<T>*>(src + j);
-        const Two<T> b = *reinterpret_cast<const Two<T>*>(src + j + g.hx);
-        const T v[4] = {a.x, b.x, a.y, b.y};
+        T v[4];
+        ld_user<U, T>(g, f == 0 ? rho : u + (f - 1) * NU, j, x, v);
 #pragma unroll
         for (int c = 0; c < 4; ++c) q[f].v[c] = f == 0 ? MP::rho_in(v[c], m) : MP::u_in(v[c], m);
       }
@@ -194,16 +233,29 @@ __global__ void fill_walls_k(int d, int64_t N, const uint8_t* __restrict__ node_
 // physical (rho, u), in both state buffers (the step kernels never write a
 // wall node, so whichever buffer is current reads them); fluid entries of the
 // arrays are not read.
-template <typename S, typename T, bool FAST, typename I>
+template <typename S, typename T, bool FAST, typename I, int U>
 __global__ void __launch_bounds__(256) set_walls_k(Geometry g, const T* __restrict__ rho, const T* __restrict__ u,
                                                    UnitMap m, const uint8_t* __restrict__ node_type,
                                                    S* __restrict__ s0, S* __restrict__ s1) {
   using MP = Map<S, FAST>;
-  const int64_t N = g.n;
-  for_units<I, false>(g, [&](int64_t i, int64_t j) {
-    if (node_type[i] == 0) return;
-    s0[i] = s1[i] = MP::rho_in(rho[j], m);
-    for (int c = 0; c < g.d; ++c) s0[(1 + c) * N + i] = s1[(1 + c) * N + i] = MP::u_in(u[c * N + j], m);
+  const int64_t N = g.n, NU = m.nu;
+  for_units<I, U>(g, [&](int64_t i, int64_t j, int x) {
+    if constexpr (U != kNode) {
+      const uchar4 k4 = *reinterpret_cast<const uchar4*>(node_type + i);
+      const bool wall[4] = {k4.x != 0, k4.y != 0, k4.z != 0, k4.w != 0};
+      if (!(wall[0] | wall[1] | wall[2] | wall[3])) return;
+      for (int f = 0; f <= g.d; ++f) {
+        T v[4];
+        ld_user<U, T>(g, f == 0 ? rho : u + (f - 1) * NU, j, x, v);
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (wall[c]) s0[f * N + i + c] = s1[f * N + i + c] = f == 0 ? MP::rho_in(v[c], m) : MP::u_in(v[c], m);
+      }
+    } else {
+      if (node_type[i] == 0) return;
+      s0[i] = s1[i] = MP::rho_in(rho[j], m);
+      for (int c = 0; c < g.d; ++c) s0[(1 + c) * N + i] = s1[(1 + c) * N + i] = MP::u_in(u[c * NU + j], m);
+    }
   });
 }
 
@@ -216,14 +268,39 @@ __global__ void __launch_bounds__(256) copy_walls_k(int d, int64_t N, const uint
       for (int f = 0; f <= d; ++f) dst[f * N + i] = src[f * N + i];
 }
 
-template <typename S, typename T, bool FAST, typename I, bool QUAD>
+// Rows of planes [p0, p0 + count) between padded storage and the raw layout
+// (kQuad1 units of the rows; `rows` rows a field).
+template <typename S, typename I, bool TO_RAW>
+__global__ void __launch_bounds__(256) repack_k(Geometry g, int64_t row0, int64_t rows, S* __restrict__ state,
+                                                S* __restrict__ raw) {
+  const int64_t N = g.n, NU = rows * (g.nx - g.pad);
+  Geometry part = g;  // the planes' rows only
+  part.n = rows * g.nx;
+  for_units<I, kQuad1>(part, [&](int64_t i, int64_t j, int x) {
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      if (f > g.d) continue;
+      Four<S>* const q = reinterpret_cast<Four<S>*>(state + f * N + row0 * g.nx + i);
+      if constexpr (TO_RAW) {
+        const Four<S> v = *q;
+        st_user<kQuad1, S>(g, raw + f * NU, j, x, v.v);
+      } else {
+        Four<S> v;
+        ld_user<kQuad1, S>(g, raw + f * NU, j, x, v.v);
+        *q = v;
+      }
+    }
+  });
+}
+
+template <typename S, typename T, bool FAST, typename I, int U>
 __global__ void __launch_bounds__(256) get_physical_k(Geometry g, const S* __restrict__ state, UnitMap m,
                                                       T* __restrict__ rho, T* __restrict__ u) {
   using MP = Map<S, FAST>;
-  const int64_t N = g.n;
+  const int64_t N = g.n, NU = m.nu;  // field strides: state, user arrays
   const int d = g.d;
-  for_units<I, QUAD>(g, [&](int64_t i, int64_t j) {
-    if constexpr (QUAD) {
+  for_units<I, U>(g, [&](int64_t i, int64_t j, int x) {
+    if constexpr (U != kNode) {
 #pragma unroll
       for (int f = 0; f < 4; ++f) {
         if (f > d) continue;
@@ -232,9 +309,7 @@ __global__ void __launch_bounds__(256) get_physical_k(Geometry g, const S* __res
 #pragma unroll
         for (int c = 0; c < 4; ++c)
           v[c] = f == 0 ? MP::template rho_out<T>(q.v[c], m) : MP::template u_out<T>(q.v[c], m);
-        T* dst = f == 0 ? rho : u + (f - 1) * N;
-        *reinterpret_cast<Two<T>*>(dst + j) = Two<T>{v[0], v[2]};
-        *reinterpret_cast<Two<T>*>(dst + j + g.hx) = Two<T>{v[1], v[3]};
+        st_user<U, T>(g, f == 0 ? rho : u + (f - 1) * NU, j, x, v);
       }
     } else {
       rho[j] = MP::template rho_out<T>(state[i], m);
@@ -255,34 +330,40 @@ static unsigned grid_for(int64_t n) {
 // 32-bit unit indices where neither the count nor a grid stride past it overflows.
 static bool small_index(int64_t units) { return units < ((int64_t)1 << 31); }
 
-static bool aligned_to(const void* a, const void* b, size_t bytes) {
-  return (reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) % bytes == 0;
+static Unit unit_of(const Geometry& g, const void* a, const void* b, size_t bytes) {
+  if (!g.ilv) return kNode;
+  return !g.pad && (reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) % bytes == 0 ? kQuad2 : kQuad1;
 }
 
-template <typename S, typename T, bool FAST, typename I, bool QUAD>
-static cudaError_t set_launch(const Geometry& g, const void* rho, const void* u, const UnitMap& m, const uint8_t* nt,
-                              const double* wl, int nw, void* s0, void* s1, cudaStream_t st) {
-  set_physical_k<S, T, FAST, I, QUAD><<<grid_for(QUAD ? g.n / 4 : g.n), 256, 0, st>>>(
-      g, (const T*)rho, (const T*)u, m, nt, wl, nw, (S*)s0, (S*)s1);
-  return cudaGetLastError();
+// launch(index type, std::integral_constant<int, unit>) for the unit and node count
+template <typename Fn>
+static cudaError_t by_unit(const Geometry& g, Unit unit, Fn&& launch) {
+  const unsigned grid = grid_for(unit == kNode ? g.n : g.n / 4);
+  auto with_index = [&](auto index) {
+    switch (unit) {
+      case kNode: return launch(grid, index, std::integral_constant<int, kNode>{});
+      case kQuad1: return launch(grid, index, std::integral_constant<int, kQuad1>{});
+      default: return launch(grid, index, std::integral_constant<int, kQuad2>{});
+    }
+  };
+  return small_index(g.n) ? with_index(uint32_t{}) : with_index(int64_t{});
 }
 
 template <typename S, typename T, bool FAST>
 static cudaError_t set_t(const Geometry& g, const void* rho, const void* u, const UnitMap& m, const uint8_t* nt,
                          const double* wl, int nw, void* s0, void* s1, cudaStream_t st) {
-  const bool small = small_index(g.n);
-  if (g.ilv && aligned_to(rho, u, 2 * sizeof(T)))
-    return small ? set_launch<S, T, FAST, uint32_t, true>(g, rho, u, m, nt, wl, nw, s0, s1, st)
-                 : set_launch<S, T, FAST, int64_t, true>(g, rho, u, m, nt, wl, nw, s0, s1, st);
-  return small ? set_launch<S, T, FAST, uint32_t, false>(g, rho, u, m, nt, wl, nw, s0, s1, st)
-               : set_launch<S, T, FAST, int64_t, false>(g, rho, u, m, nt, wl, nw, s0, s1, st);
+  return by_unit(g, unit_of(g, rho, u, 2 * sizeof(T)), [&](unsigned grid, auto index, auto unit) {
+    set_physical_k<S, T, FAST, decltype(index), decltype(unit)::value>
+        <<<grid, 256, 0, st>>>(g, (const T*)rho, (const T*)u, m, nt, wl, nw, (S*)s0, (S*)s1);
+    return cudaGetLastError();
+  });
 }
 
 template <typename S>
 static cudaError_t set_s(const Geometry& g, const void* rho, const void* u, int dtype, double rho0, double e,
                          const uint8_t* nt, const double* wl, int nw, void* s0, void* s1, cudaStream_t st) {
   UnitMap m;
-  const bool fast = unit_map(rho0, e, &m);
+  const bool fast = unit_map(g, rho0, e, &m);
   if (dtype == MACLAB_DTYPE_F64) return set_t<S, double, false>(g, rho, u, m, nt, wl, nw, s0, s1, st);
   if constexpr (!std::is_same<S, double>::value)
     if (fast) return set_t<S, float, true>(g, rho, u, m, nt, wl, nw, s0, s1, st);
@@ -301,29 +382,20 @@ cudaError_t launch_set_physical(const Geometry& g, int precision, const void* rh
   return cudaErrorInvalidValue;
 }
 
-template <typename S, typename T, bool FAST, typename I, bool QUAD>
-static cudaError_t get_launch(const Geometry& g, const void* state, const UnitMap& m, void* rho, void* u,
-                              cudaStream_t st) {
-  get_physical_k<S, T, FAST, I, QUAD><<<grid_for(QUAD ? g.n / 4 : g.n), 256, 0, st>>>(g, (const S*)state, m, (T*)rho,
-                                                                                     (T*)u);
-  return cudaGetLastError();
-}
-
 template <typename S, typename T, bool FAST>
 static cudaError_t get_t(const Geometry& g, const void* state, const UnitMap& m, void* rho, void* u, cudaStream_t st) {
-  const bool small = small_index(g.n);
-  if (g.ilv && aligned_to(rho, u, 2 * sizeof(T)))
-    return small ? get_launch<S, T, FAST, uint32_t, true>(g, state, m, rho, u, st)
-                 : get_launch<S, T, FAST, int64_t, true>(g, state, m, rho, u, st);
-  return small ? get_launch<S, T, FAST, uint32_t, false>(g, state, m, rho, u, st)
-               : get_launch<S, T, FAST, int64_t, false>(g, state, m, rho, u, st);
+  return by_unit(g, unit_of(g, rho, u, 2 * sizeof(T)), [&](unsigned grid, auto index, auto unit) {
+    get_physical_k<S, T, FAST, decltype(index), decltype(unit)::value>
+        <<<grid, 256, 0, st>>>(g, (const S*)state, m, (T*)rho, (T*)u);
+    return cudaGetLastError();
+  });
 }
 
 template <typename S>
 static cudaError_t get_s(const Geometry& g, const void* state, void* rho, void* u, int dtype, double rho0, double e,
                          cudaStream_t st) {
   UnitMap m;
-  const bool fast = unit_map(rho0, e, &m);
+  const bool fast = unit_map(g, rho0, e, &m);
   if (dtype == MACLAB_DTYPE_F64) return get_t<S, double, false>(g, state, m, rho, u, st);
   if constexpr (!std::is_same<S, double>::value)
     if (fast) return get_t<S, float, true>(g, state, m, rho, u, st);
@@ -344,20 +416,18 @@ cudaError_t launch_get_physical(const Geometry& g, int precision, const void* st
 template <typename S, typename T, bool FAST>
 static cudaError_t walls_t(const Geometry& g, const void* rho, const void* u, const UnitMap& m, const uint8_t* nt,
                            void* s0, void* s1, cudaStream_t st) {
-  if (small_index(g.n))
-    set_walls_k<S, T, FAST, uint32_t><<<grid_for(g.n), 256, 0, st>>>(g, (const T*)rho, (const T*)u, m, nt, (S*)s0,
-                                                                    (S*)s1);
-  else
-    set_walls_k<S, T, FAST, int64_t><<<grid_for(g.n), 256, 0, st>>>(g, (const T*)rho, (const T*)u, m, nt, (S*)s0,
-                                                                   (S*)s1);
-  return cudaGetLastError();
+  return by_unit(g, unit_of(g, rho, u, 2 * sizeof(T)), [&](unsigned grid, auto index, auto unit) {
+    set_walls_k<S, T, FAST, decltype(index), decltype(unit)::value>
+        <<<grid, 256, 0, st>>>(g, (const T*)rho, (const T*)u, m, nt, (S*)s0, (S*)s1);
+    return cudaGetLastError();
+  });
 }
 
 template <typename S>
 static cudaError_t walls_s(const Geometry& g, const void* rho, const void* u, int dtype, double rho0, double e,
                            const uint8_t* nt, void* s0, void* s1, cudaStream_t st) {
   UnitMap m;
-  const bool fast = unit_map(rho0, e, &m);
+  const bool fast = unit_map(g, rho0, e, &m);
   if (dtype == MACLAB_DTYPE_F64) return walls_t<S, double, false>(g, rho, u, m, nt, s0, s1, st);
   if constexpr (!std::is_same<S, double>::value)
     if (fast) return walls_t<S, float, true>(g, rho, u, m, nt, s0, s1, st);
@@ -373,6 +443,33 @@ cudaError_t launch_set_wall_values(const Geometry& g, int precision, const void*
     case MACLAB_F32: return walls_s<float>(g, rho, u, dtype, rho0, e, nt, s0, s1, st);
     case MACLAB_BF16_STORE: return walls_s<__nv_bfloat16>(g, rho, u, dtype, rho0, e, nt, s0, s1, st);
     case MACLAB_F16_STORE: return walls_s<__half>(g, rho, u, dtype, rho0, e, nt, s0, s1, st);
+  }
+  return cudaErrorInvalidValue;
+}
+
+template <typename S>
+static cudaError_t repack_t(const Geometry& g, void* state, void* raw, int64_t row0, int64_t rows, bool to_raw,
+                            cudaStream_t st) {
+  const unsigned grid = grid_for(rows * g.nx / 4);
+  S* const s = (S*)state;
+  S* const r = (S*)raw;
+  if (small_index(g.n)) {
+    if (to_raw) repack_k<S, uint32_t, true><<<grid, 256, 0, st>>>(g, row0, rows, s, r);
+    else repack_k<S, uint32_t, false><<<grid, 256, 0, st>>>(g, row0, rows, s, r);
+  } else {
+    if (to_raw) repack_k<S, int64_t, true><<<grid, 256, 0, st>>>(g, row0, rows, s, r);
+    else repack_k<S, int64_t, false><<<grid, 256, 0, st>>>(g, row0, rows, s, r);
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_repack(const Geometry& g, int precision, void* state, void* raw, int64_t p0, int64_t count,
+                          bool to_raw, cudaStream_t st) {
+  const int64_t plane_rows = g.d == 3 ? g.ny : 1;
+  switch (storage_bytes(precision)) {
+    case 8: return repack_t<double>(g, state, raw, p0 * plane_rows, count * plane_rows, to_raw, st);
+    case 4: return repack_t<float>(g, state, raw, p0 * plane_rows, count * plane_rows, to_raw, st);
+    case 2: return repack_t<uint16_t>(g, state, raw, p0 * plane_rows, count * plane_rows, to_raw, st);
   }
   return cudaErrorInvalidValue;
 }

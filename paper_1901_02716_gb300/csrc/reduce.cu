@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(256) diag_partial(Geometry g, const S* __restr
       wall = g.mask[m] != 0;
     } else if (g.wall_mode == kWallBox) {
       const int x = log_x(g, mx);
-      if (!(g.periodic & 1u)) wall |= (x == 0) | (x == g.nx - 1);
+      if (!(g.periodic & 1u)) wall |= (x == 0) | (x >= g.nx - 1 - g.pad);
       if (!(g.periodic & 2u)) wall |= (y == 0) | (y == g.ny - 1);
       if (g.d == 3 && !(g.periodic & 4u)) wall |= (z == 0) | (z == g.nz - 1);
     }
@@ -283,8 +283,8 @@ __global__ void __launch_bounds__(256) diag_partial(Geometry g, const S* __restr
 // Rows of x (nx % 4 == 0): a warp takes whole rows, each lane 16-byte quads of
 // the four stored values of a node quad (vector loads, many in flight); rows on
 // a closed y or z boundary are wall rows and skipped as a whole, and in box
-// mode only the storage positions 0 and nx - 1 of a row (x = 0, nx - 1) are
-// x-walls.  The stored density deviations are exact inputs and enter the
+// mode only the nodes x = 0 and nx - 1 of a row are x-walls (with the padding,
+// if any, beyond).  The stored density deviations are exact inputs and enter the
 // float-float sum node by node, as in diag_partial.  The per-node products
 // (rho |u|^2, rho u_i, |u - u_prev|^2, |u|^2) are formed on the quad's two node
 // pairs with paired arithmetic, each rounded to the arithmetic type; a quad's
@@ -313,6 +313,7 @@ __global__ void __launch_bounds__(256, sizeof(S) == 8 ? 1 : 2) diag_rows(Geometr
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int64_t rows = N / g.nx;
   const int quads = g.nx >> 2;
+  const int x_last = g.nx - 1 - g.pad - g.hx;  // pair of the domain's last node
   const bool xw = g.wall_mode == kWallBox && !(g.periodic & 1u);
   const bool yw = g.wall_mode == kWallBox && !(g.periodic & 2u);
   const bool zw = g.wall_mode == kWallBox && g.d == 3 && !(g.periodic & 4u);
@@ -337,8 +338,10 @@ __global__ void __launch_bounds__(256, sizeof(S) == 8 ? 1 : 2) diag_rows(Geometr
         const uchar4 mk = *reinterpret_cast<const uchar4*>(g.mask + m);
         wall[0] = mk.x != 0; wall[1] = mk.y != 0; wall[2] = mk.z != 0; wall[3] = mk.w != 0;
       } else if (xw) {
+        // the second-half nodes of the last quads: the right wall and the padding beyond it
         wall[0] = q == 0;
-        wall[3] = q == quads - 1;
+        wall[1] = 2 * q >= x_last;
+        wall[3] = 2 * q + 1 >= x_last;
       }
       P r[2], u[3][2], v[3][2];
       Quad<S>::ld(cur + m, r[0], r[1]);

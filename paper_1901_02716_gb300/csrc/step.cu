@@ -34,7 +34,7 @@ __device__ __forceinline__ bool is_wall_node(const Geometry& g, int x, int y, in
   if (g.wall_mode == kWallNone) return false;
   if (g.wall_mode == kWallMask) return g.mask[node] != 0;
   bool w = false;
-  if (!(g.periodic & 1u)) w |= (x == 0) | (x == g.nx - 1);
+  if (!(g.periodic & 1u)) w |= (x == 0) | (x >= g.nx - 1 - g.pad);
   if (!(g.periodic & 2u)) w |= (y == 0) | (y == g.ny - 1);
   if (Lattice<LAT>::D == 3 && !(g.periodic & 4u)) w |= (z == 0) | (z == g.nz - 1);
   return w;
@@ -164,9 +164,8 @@ bool step_kernel_supported(const Geometry& g, int precision, int kernel) {
 // defaults, and than the block kernel above 512^2); else the tiled one, else
 // the reference kernel.
 int pick_step_kernel(const Geometry& g, int precision) {
-  if (precision == MACLAB_F32 && step_kernel_supported(g, precision, MACLAB_KERNEL_ROWS2))
-    return MACLAB_KERNEL_ROWS2;
-  if (step_kernel_supported(g, precision, MACLAB_KERNEL_FOLDED)) return MACLAB_KERNEL_FOLDED;
+  if (precision == MACLAB_F32 && rows2_supported(g, precision, 0, true)) return MACLAB_KERNEL_ROWS2;
+  if (fold_supported(g, precision, 0, true)) return MACLAB_KERNEL_FOLDED;
   if ((int64_t)(g.nx / 2) * g.ny <= 131072 && step_kernel_supported(g, precision, MACLAB_KERNEL_BLOCK))
     return MACLAB_KERNEL_BLOCK;
   if (step_kernel_supported(g, precision, MACLAB_KERNEL_SEGMENT)) return MACLAB_KERNEL_SEGMENT;
@@ -244,9 +243,9 @@ cudaError_t launch_step(const StepLaunch& s, cudaStream_t stream, int kernel) {
       if (!s.seg_inst || !s.seg_items) return cudaErrorInvalidValue;
       if (s.seg_steps == 2)
         return launch_batch_step2(s.precision, s.seg_inst, s.seg_items, s.seg_n_items, s.cur, s.seg_blocks,
-                                  stream, s.overlap);
+                                  (s.g.pad & 1) != 0, stream, s.overlap);
       return launch_batch_step(s.precision, s.seg_inst, s.seg_items, s.seg_n_items, s.cur, s.seg_blocks,
-                               s.seg_depth == 2 ? kBatchSegW2 : kBatchSegW1, stream, s.overlap);
+                               s.seg_depth == 2 ? kBatchSegW2 : kBatchSegW1, (s.g.pad & 1) != 0, stream, s.overlap);
     default:
       return cudaErrorInvalidValue;
   }

@@ -53,6 +53,7 @@ struct BlockArgs {
   const uint8_t* mask;  // node types in storage order (kWallMask)
   int64_t n;            // nodes (field stride)
   int nx, ny, hx;       // hx = nx / 2
+  int x_last;           // the domain's last node of a row (nx - 1 less the padding)
   int px, py;           // periodic flags
   int wall_mode;
   double force[2];      // lattice-unit force increment
@@ -147,8 +148,8 @@ __global__ void __launch_bounds__(kBlockBX * BY, 1) step_block_d2q9(BlockArgs a)
     } else if (a.wall_mode == kWallBox) {
       const int x0 = swapped ? p + H : p, x1 = swapped ? p : p + H;
       const bool yw = !a.py && (ym == 0 || ym == a.ny - 1);
-      const bool w0 = yw || (!a.px && (x0 == 0 || x0 == a.nx - 1));
-      const bool w1 = yw || (!a.px && (x1 == 0 || x1 == a.nx - 1));
+      const bool w0 = yw || (!a.px && (x0 == 0 || x0 >= a.x_last));
+      const bool w1 = yw || (!a.px && (x1 == 0 || x1 >= a.x_last));
       keep = (w0 ? 1u : 0u) | (w1 ? 2u : 0u);
     } else {
       keep = 0u;
@@ -365,8 +366,8 @@ __global__ void __launch_bounds__(256, 2) step_block2_d2q9(BlockArgs a) {  // FP
         } else if (a.wall_mode == kWallBox) {
           const int x0 = swapped ? p + H : p, x1 = swapped ? p : p + H;
           const bool yw = !a.py && (ym == 0 || ym == a.ny - 1);
-          const bool w0 = yw || (!a.px && (x0 == 0 || x0 == a.nx - 1));
-          const bool w1 = yw || (!a.px && (x1 == 0 || x1 == a.nx - 1));
+          const bool w0 = yw || (!a.px && (x0 == 0 || x0 >= a.x_last));
+          const bool w1 = yw || (!a.px && (x1 == 0 || x1 >= a.x_last));
           kp = (w0 ? 1u : 0u) | (w1 ? 2u : 0u);
         } else {
           kp = 0u;
@@ -491,6 +492,7 @@ cudaError_t launch_block_t(const StepLaunch& s, cudaStream_t stream) {
   a.nx = s.g.nx;
   a.ny = s.g.ny;
   a.hx = s.g.nx / 2;
+  a.x_last = s.g.nx - 1 - s.g.pad;
   a.px = (s.g.periodic & 1u) ? 1 : 0;
   a.py = (s.g.periodic & 2u) ? 1 : 0;
   a.wall_mode = s.g.wall_mode;
@@ -516,6 +518,7 @@ cudaError_t launch_block2_t(const StepLaunch& s, cudaStream_t stream) {
   a.nx = s.g.nx;
   a.ny = s.g.ny;
   a.hx = s.g.nx / 2;
+  a.x_last = s.g.nx - 1 - s.g.pad;
   a.px = (s.g.periodic & 1u) ? 1 : 0;
   a.py = (s.g.periodic & 2u) ? 1 : 0;
   a.wall_mode = s.g.wall_mode;

@@ -5,6 +5,16 @@
 
 namespace maclab {
 
+MACLAB_FOLD_DISPATCH(extern, float, kRowsPlain)
+MACLAB_FOLD_DISPATCH(extern, float, kRowsEven)
+MACLAB_FOLD_DISPATCH(extern, float, kRowsOdd)
+MACLAB_FOLD_DISPATCH(extern, __nv_bfloat16, kRowsPlain)
+MACLAB_FOLD_DISPATCH(extern, __nv_bfloat16, kRowsEven)
+MACLAB_FOLD_DISPATCH(extern, __nv_bfloat16, kRowsOdd)
+MACLAB_FOLD_DISPATCH(extern, __half, kRowsPlain)
+MACLAB_FOLD_DISPATCH(extern, __half, kRowsEven)
+MACLAB_FOLD_DISPATCH(extern, __half, kRowsOdd)
+
 namespace {
 
 // Instantiated (BXC, TY) in order of preference for each width (the first whose
@@ -19,34 +29,27 @@ bool fold_shape_built(const FoldShape& s, int precision) {
   return false;
 }
 
-bool fold_shape(const Geometry& g, int precision, int ty_req, FoldShape* out) {
+// ragged: where no TY divides ny, the first that does not exceed it (the last
+// tile recomputes at most TY - 1 rows; the tiled kernel, which otherwise serves
+// these, forms two halo rows for every tile: 15 steps of a 256 x 327 x 377
+// cavity in BF16 storage take 6.0 ms on it and 3.5 ms here).
+bool fold_shape(const Geometry& g, int precision, int ty_req, FoldShape* out, bool ragged) {
   if (g.d != 3 || g.lattice != kD3Q19 || !g.ilv || precision == MACLAB_F64) return false;
   const int bx = g.nx / 4;
   int bxc = 0;
   for (int c : {16, 32, 64, 128})
     if (bx <= c) { bxc = c; break; }
   if (!bxc) return false;
-  for (const FoldShape& s : kFoldShapes) {
-    if (s.bxc != bxc || (ty_req > 0 && s.ty != ty_req) || !fold_shape_built(s, precision)) continue;
-    if (g.ny % s.ty != 0) continue;  // every row of a tile exists
-    *out = s;
-    return true;
+  for (const bool divides : {true, false}) {
+    if (!divides && !ragged) break;
+    for (const FoldShape& s : kFoldShapes) {
+      if (s.bxc != bxc || (ty_req > 0 && s.ty != ty_req) || !fold_shape_built(s, precision)) continue;
+      if (divides ? g.ny % s.ty != 0 : g.ny < s.ty) continue;
+      *out = s;
+      return true;
+    }
   }
   return false;
-}
-
-template <typename S>
-cudaError_t fold_dispatch(const FoldShape& s, const TiledArgs& ta, const void* in, void* out,
-                          cudaStream_t st, dim3 grid, int* resident) {
-  switch (s.bxc * 100 + s.ty) {
-    case 1608: return launch_fold_shape<S, 16, 8>(ta, in, out, st, grid, resident);
-    case 3204: return launch_fold_shape<S, 32, 4>(ta, in, out, st, grid, resident);
-    case 3208: return launch_fold_shape<S, 32, 8>(ta, in, out, st, grid, resident);
-    case 6404: return launch_fold_shape<S, 64, 4>(ta, in, out, st, grid, resident);
-    case 6408: return launch_fold_shape<S, 64, 8>(ta, in, out, st, grid, resident);
-    case 12804: return launch_fold_shape<S, 128, 4>(ta, in, out, st, grid, resident);
-  }
-  return cudaErrorInvalidValue;
 }
 
 }  // namespace
@@ -81,20 +84,20 @@ int fold_chunks(int nplanes, int ytiles, int tz_req, int per_sm) {
 }
 
 
-bool fold_supported(const Geometry& g, int precision, int ty) {
+bool fold_supported(const Geometry& g, int precision, int ty, bool ragged) {
   FoldShape s;
-  return fold_shape(g, precision, ty, &s);
+  return fold_shape(g, precision, ty, &s, ragged);
 }
 
 int fold_threads(const Geometry& g, int precision, int ty) {
   FoldShape s;
-  return fold_shape(g, precision, ty, &s) ? s.bxc * s.ty : 0;
+  return fold_shape(g, precision, ty, &s, true) ? s.bxc * s.ty : 0;
 }
 
 cudaError_t launch_fold(const StepLaunch& sl, cudaStream_t stream, int ty, int tz) {
   const Geometry& g = sl.g;
   FoldShape s;
-  if (!fold_shape(g, sl.precision, ty, &s)) return cudaErrorInvalidValue;
+  if (!fold_shape(g, sl.precision, ty, &s, true)) return cudaErrorInvalidValue;
   TiledArgs ta{};
   ta.nx = g.nx;
   ta.ny = g.ny;
@@ -102,10 +105,23 @@ cudaError_t launch_fold(const StepLaunch& sl, cudaStream_t stream, int ty, int t
   ta.n = g.n;
   ta.plane_stride = (int64_t)g.nx * g.ny;
   ta.ty = s.ty;
-  const int ytiles = g.ny / s.ty;
+  const int ytiles = (g.ny + s.ty - 1) / s.ty;
+  const RowMode rows = (g.pad & 1) ? kRowsOdd : (g.pad || g.ny % s.ty != 0) ? kRowsEven : kRowsPlain;
   auto dispatch = [&](const void* in, void* out, dim3 grid, int* resident) {
-    return sl.precision == MACLAB_F32 ? fold_dispatch<float>(s, ta, in, out, stream, grid, resident)
-                                      : fold_dispatch_s16(sl.precision, s, ta, in, out, stream, grid, resident);
+    auto typed = [&](auto zero) {
+      using S = decltype(zero);
+      switch (rows) {
+        case kRowsPlain: return fold_dispatch<S, kRowsPlain>(s, ta, in, out, stream, grid, resident);
+        case kRowsEven: return fold_dispatch<S, kRowsEven>(s, ta, in, out, stream, grid, resident);
+        default: return fold_dispatch<S, kRowsOdd>(s, ta, in, out, stream, grid, resident);
+      }
+    };
+    switch (sl.precision) {
+      case MACLAB_F32: return typed(float{});
+      case MACLAB_BF16_STORE: return typed(__nv_bfloat16{});
+      case MACLAB_F16_STORE: return typed(__half{});
+    }
+    return cudaErrorInvalidValue;
   };
   int resident = 0;
   cudaError_t e = dispatch(nullptr, nullptr, dim3(), &resident);
@@ -117,7 +133,7 @@ cudaError_t launch_fold(const StepLaunch& sl, cudaStream_t stream, int ty, int t
   ta.wall_mode = g.wall_mode;
   ta.mask = g.mask;
   for (int i = 0; i < 3; ++i) ta.force[i] = sl.force[i];
-  ta.overlap = sl.overlap;
+  ta.set_overlap_pad(sl.overlap, g.pad);
   return dispatch(sl.in, sl.out, dim3(ta.nzc, ytiles), nullptr);
 }
 

@@ -14,7 +14,9 @@
 // then does the full update and a block needs two fewer warps for the same
 // rows, so more blocks fit on an SM.
 //
-// Requires ny % TY == 0 and TY >= 2 (the first and last rows are distinct).
+// Requires ny >= TY and TY >= 2 (the first and last rows are distinct).  Where
+// TY does not divide ny, the last tile is moved up to end at the last row; the
+// rows it shares with the tile before are stored by that one only.
 #pragma once
 #include "step_tiled.cuh"
 
@@ -24,11 +26,6 @@ namespace maclab {
 struct FoldShape {
   int bxc, ty;
 };
-
-// Launch dispatch for 16-bit storage (step_fold_s16.cu): shapes (32, 8),
-// (32, 4), (64, 4) and (128, 4); with resident set, only the blocks one SM holds.
-cudaError_t fold_dispatch_s16(int precision, const FoldShape& s, const TiledArgs& ta, const void* in,
-                              void* out, cudaStream_t st, dim3 grid, int* resident);
 
 template <typename S, int BXC, int TY>
 struct FoldLayout {
@@ -418,7 +415,7 @@ __device__ __forceinline__ void fold_update_xs(const typename Pair<C>::P (&st)[4
 // value, wv (its four fields, kept when the plane was taken), in place of the
 // computed one and stores the whole quad.  Masks, and a quad holding both
 // x-walls (nx = 4), take store_plane's per-node path.
-template <typename S>
+template <typename S, int RM>
 __device__ __forceinline__ void fold_store(S* const (&fp)[4], const uint8_t* mrow, const TiledArgs& ta,
                                            int64_t off, bool x_lo_wall, bool x_hi_wall, const float4& wv,
                                            bool skip, typename Quad<S>::P (&acc)[2][4],
@@ -427,7 +424,7 @@ __device__ __forceinline__ void fold_store(S* const (&fp)[4], const uint8_t* mro
   using O = Pair<C>;
   using P = typename O::P;
   if (ta.wall_mode == kWallMask || (x_lo_wall && x_hi_wall)) {
-    store_plane<kD3Q19, S>(fp, mrow, ta, off, x_lo_wall, x_hi_wall, skip, acc, force);
+    store_plane<kD3Q19, S, RM>(fp, mrow, ta, off, x_lo_wall, x_hi_wall, skip, acc, force);
     return;
   }
   if (skip) return;
@@ -443,12 +440,16 @@ __device__ __forceinline__ void fold_store(S* const (&fp)[4], const uint8_t* mro
 #pragma unroll
   for (int f = 0; f < 4; ++f) {
     if (x_lo_wall) v[f][0].x = C(w[f]);
-    if (x_hi_wall) v[f][1].y = C(w[f]);
+    if (x_hi_wall) {
+      if constexpr (RM == kRowsOdd) v[f][0].y = C(w[f]);
+      else v[f][1].y = C(w[f]);
+    }
     Quad<S>::st(fp[f] + off, v[f][0], v[f][1]);
   }
 }
 
-template <typename S, int BXC, int TY>
+// RM: the rows it serves (RowMode).
+template <typename S, int BXC, int TY, int RM = kRowsPlain>
 __global__ void __launch_bounds__(BXC * TY, FoldLayout<S, BXC, TY>::MIN_BLOCKS)
     step_fold(TiledArgs ta, const S* __restrict__ in, S* __restrict__ out) {
   using Lay = FoldLayout<S, BXC, TY>;
@@ -494,21 +495,24 @@ __global__ void __launch_bounds__(BXC * TY, FoldLayout<S, BXC, TY>::MIN_BLOCKS)
   xs.wr = tx == 0;
   int ybuf = 0;
 
-  // own row (every row of the tile exists: ny % TY == 0) and the halo row of
-  // the first (+1: row - 1) and last (-1: row + 1) rows
-  const int row = blockIdx.y * TY + r;
+  // own row and the halo row of the first (+1: row - 1) and last (-1: row + 1)
+  // rows; the last tile of a ragged ny ends at the last row
+  const int first_row = blockIdx.y * TY;  // rows before it are the previous tile's
+  const int row = (RM == kRowsPlain ? first_row : min(first_row, ta.ny - TY)) + r;
   int halo = r == 0 ? 1 : (r == TY - 1 ? -1 : 0);
   int hrow = row - halo;
   if (halo != 0 && (hrow < 0 || hrow >= ta.ny)) {
     if (ta.py) hrow = (hrow + ta.ny) % ta.ny;
     else halo = 0;  // no row beyond a closed y boundary: nothing to fold in
   }
-  const bool row_wall = !ta.py && (row == 0 || row == ta.ny - 1);
+  const bool row_wall = (!ta.py && (row == 0 || row == ta.ny - 1)) ||
+                        (RM != kRowsPlain && row < first_row);  // not stored
   const int64_t row_off = (int64_t)row * ta.nx + 4 * tx;
   const int64_t halo_delta = (int64_t)(hrow - row) * ta.nx;  // halo quad - own quad
-  // box walls at x = 0 (lane a.x of thread 0) and x = nx - 1 (lane b.y of the last)
+  // box walls at x = 0 (lane a.x of thread 0) and the domain's last node (lane
+  // b.y of the last thread; a.y or the thread before it with padding)
   const bool x_lo_wall = ta.wall_mode == kWallBox && !ta.px && tx == 0;
-  const bool x_hi_wall = ta.wall_mode == kWallBox && !ta.px && tx == bxr - 1;
+  const bool x_hi_wall = ta.wall_mode == kWallBox && !ta.px && tx == (RM == kRowsPlain ? bxr - 1 : hi_wall_quad(ta.nx, ta.pad()));
 
   const S* ip[4];
   S* op[4];
@@ -575,9 +579,11 @@ __global__ void __launch_bounds__(BXC * TY, FoldLayout<S, BXC, TY>::MIN_BLOCKS)
         st[f][0] = st[f][1] = O::splat(C(0));
       }
     }
-    if (xwall1 && ok)
+    if (xwall1 && ok) {
       wring[i & (kStages - 1)] = x_lo_wall ? make_float4(st[0][0].x, st[1][0].x, st[2][0].x, st[3][0].x)
+                                 : RM == kRowsOdd ? make_float4(st[0][0].y, st[1][0].y, st[2][0].y, st[3][0].y)
                                            : make_float4(st[0][1].y, st[1][1].y, st[2][1].y, st[3][1].y);
+    }
   };
 
   // one source plane into the sums of destination planes p - 1, p, p + 1
@@ -609,7 +615,7 @@ __global__ void __launch_bounds__(BXC * TY, FoldLayout<S, BXC, TY>::MIN_BLOCKS)
   auto store = [&](int q, P(&acc)[2][K]) {
     float4 wv = make_float4(0.f, 0.f, 0.f, 0.f);
     if (xwall1) wv = wring[(q - z0 + 1) & (kStages - 1)];  // kept when plane q was taken
-    fold_store<S>(op, mrow, ta, (int64_t)q * ps, x_lo_wall, x_hi_wall, wv, store_skip(q), acc, force);
+    fold_store<S, RM>(op, mrow, ta, (int64_t)q * ps, x_lo_wall, x_hi_wall, wv, store_skip(q), acc, force);
   };
 
   // full plane p: contributions to the sums A (dest p - 1), B (dest p), N (dest
@@ -647,10 +653,10 @@ __global__ void __launch_bounds__(BXC * TY, FoldLayout<S, BXC, TY>::MIN_BLOCKS)
 
 // Launch one instance (the instances are in step_fold.cu).  With resident_out
 // set, only report the blocks of this shape one SM holds.
-template <typename S, int BXC, int TY>
+template <typename S, int BXC, int TY, int RM = kRowsPlain>
 cudaError_t launch_fold_shape(const TiledArgs& ta, const void* in, void* out, cudaStream_t stream, dim3 grid,
                               int* resident_out) {
-  auto kern = step_fold<S, BXC, TY>;
+  auto kern = step_fold<S, BXC, TY, RM>;
   constexpr size_t smem = FoldLayout<S, BXC, TY>::smem;
   static int resident_dev[64] = {};  // per device
   int dev = 0;
@@ -671,8 +677,33 @@ cudaError_t launch_fold_shape(const TiledArgs& ta, const void* in, void* out, cu
     *resident_out = resident;
     return cudaSuccess;
   }
-  return launch_kernel(kern, grid, dim3(BXC, TY), smem, stream, ta.overlap, ta, static_cast<const S*>(in),
+  return launch_kernel(kern, grid, dim3(BXC, TY), smem, stream, ta.overlap(), ta, static_cast<const S*>(in),
                        static_cast<S*>(out));
 }
+
+// Launch of the instance of shape s for storage type S and row mode RM
+// (instances in step_fold_f32*.cu and step_fold_s16*.cu, which compile in
+// parallel): FP32 every shape, 16-bit storage (32, 8), (32, 4), (64, 4) and
+// (128, 4).  With resident set, only the blocks one SM holds.
+template <typename S, int RM>
+cudaError_t fold_dispatch(const FoldShape& s, const TiledArgs& ta, const void* in, void* out, cudaStream_t st,
+                          dim3 grid, int* resident) {
+  if constexpr (sizeof(S) == 4) {
+    switch (s.bxc * 100 + s.ty) {
+      case 1608: return launch_fold_shape<S, 16, 8, RM>(ta, in, out, st, grid, resident);
+      case 6408: return launch_fold_shape<S, 64, 8, RM>(ta, in, out, st, grid, resident);
+    }
+  }
+  switch (s.bxc * 100 + s.ty) {
+    case 3204: return launch_fold_shape<S, 32, 4, RM>(ta, in, out, st, grid, resident);
+    case 3208: return launch_fold_shape<S, 32, 8, RM>(ta, in, out, st, grid, resident);
+    case 6404: return launch_fold_shape<S, 64, 4, RM>(ta, in, out, st, grid, resident);
+    case 12804: return launch_fold_shape<S, 128, 4, RM>(ta, in, out, st, grid, resident);
+  }
+  return cudaErrorInvalidValue;
+}
+#define MACLAB_FOLD_DISPATCH(EXTERN, S, RM)                                                                        \
+  EXTERN template cudaError_t fold_dispatch<S, RM>(const FoldShape&, const TiledArgs&, const void*, void*,         \
+                                                    cudaStream_t, dim3, int*);
 
 }  // namespace maclab

@@ -7,6 +7,16 @@
 
 namespace maclab {
 
+MACLAB_ROWS2_DISPATCH(extern, float, kRowsPlain)
+MACLAB_ROWS2_DISPATCH(extern, float, kRowsEven)
+MACLAB_ROWS2_DISPATCH(extern, float, kRowsOdd)
+MACLAB_ROWS2_DISPATCH(extern, __nv_bfloat16, kRowsPlain)
+MACLAB_ROWS2_DISPATCH(extern, __nv_bfloat16, kRowsEven)
+MACLAB_ROWS2_DISPATCH(extern, __nv_bfloat16, kRowsOdd)
+MACLAB_ROWS2_DISPATCH(extern, __half, kRowsPlain)
+MACLAB_ROWS2_DISPATCH(extern, __half, kRowsEven)
+MACLAB_ROWS2_DISPATCH(extern, __half, kRowsOdd)
+
 namespace {
 
 // (BXC, TYT) in order of preference for each row width (the first whose tile
@@ -21,21 +31,25 @@ bool rows2_precision(int precision) {
 }
 
 // ty: rows per tile asked (0 = default), i.e. 2 TYT
-bool rows2_shape(const Geometry& g, int precision, int ty, Rows2Shape* out) {
+// ragged: where no tile's rows divide ny, the first that do not exceed it
+bool rows2_shape(const Geometry& g, int precision, int ty, Rows2Shape* out, bool ragged) {
   if (g.d != 3 || g.lattice != kD3Q19 || !g.ilv || !rows2_precision(precision)) return false;
   const int bx = g.nx / 4;
   int bxc = 0;
   for (int c : {16, 32})
     if (bx <= c) { bxc = c; break; }
   if (!bxc) return false;
-  for (const Rows2Shape& s : kRows2Shapes) {
-    if (s.bxc != bxc || (ty > 0 && 2 * s.tyt != ty)) continue;
-    if (precision != MACLAB_F32 && s.tyt != 4) continue;
-    // a tile copy's row is nx stored values: a multiple of 16 bytes
-    if (precision != MACLAB_F32 && g.nx % 8 != 0) continue;
-    if (g.ny % (2 * s.tyt) != 0) continue;
-    *out = s;
-    return true;
+  for (const bool divides : {true, false}) {
+    if (!divides && !ragged) break;
+    for (const Rows2Shape& s : kRows2Shapes) {
+      if (s.bxc != bxc || (ty > 0 && 2 * s.tyt != ty)) continue;
+      if (precision != MACLAB_F32 && s.tyt != 4) continue;
+      // a tile copy's row is nx stored values: a multiple of 16 bytes
+      if (precision != MACLAB_F32 && g.nx % 8 != 0) continue;
+      if (divides ? g.ny % (2 * s.tyt) != 0 : g.ny < 2 * s.tyt) continue;
+      *out = s;
+      return true;
+    }
   }
   return false;
 }
@@ -85,34 +99,20 @@ cudaError_t rows2_maps(const Geometry& g, int precision, int ty, const void* bas
 
 }  // namespace
 
-template <typename S>
-cudaError_t rows2_dispatch(int bxc, int tyt, const TiledArgs& ta, const void* in, void* out,
-                           const CUtensorMap& tm_own, const CUtensorMap& tm_halo, cudaStream_t st, dim3 grid,
-                           int* resident) {
-  switch (bxc * 100 + tyt) {
-    case 1604: return launch_rows2_shape<S, 16, 4>(ta, in, out, tm_own, tm_halo, st, grid, resident);
-    case 3202: return launch_rows2_shape<S, 32, 2>(ta, in, out, tm_own, tm_halo, st, grid, resident);
-    case 3204: return launch_rows2_shape<S, 32, 4>(ta, in, out, tm_own, tm_halo, st, grid, resident);
-  }
-  return cudaErrorInvalidValue;
-}
-template cudaError_t rows2_dispatch<float>(int, int, const TiledArgs&, const void*, void*, const CUtensorMap&,
-                                          const CUtensorMap&, cudaStream_t, dim3, int*);
-
-bool rows2_supported(const Geometry& g, int precision, int ty) {
+bool rows2_supported(const Geometry& g, int precision, int ty, bool ragged) {
   Rows2Shape s;
-  return rows2_shape(g, precision, ty, &s);
+  return rows2_shape(g, precision, ty, &s, ragged);
 }
 
 int rows2_threads(const Geometry& g, int precision, int ty) {
   Rows2Shape s;
-  return rows2_shape(g, precision, ty, &s) ? s.bxc * s.tyt : 0;
+  return rows2_shape(g, precision, ty, &s, true) ? s.bxc * s.tyt : 0;
 }
 
 cudaError_t launch_rows2(const StepLaunch& sl, cudaStream_t stream, int ty, int tz) {
   const Geometry& g = sl.g;
   Rows2Shape s;
-  if (!rows2_shape(g, sl.precision, ty, &s)) return cudaErrorInvalidValue;
+  if (!rows2_shape(g, sl.precision, ty, &s, true)) return cudaErrorInvalidValue;
   TiledArgs ta{};
   ta.nx = g.nx;
   ta.ny = g.ny;
@@ -120,16 +120,25 @@ cudaError_t launch_rows2(const StepLaunch& sl, cudaStream_t stream, int ty, int 
   ta.n = g.n;
   ta.plane_stride = (int64_t)g.nx * g.ny;
   ta.ty = 2 * s.tyt;
-  const int ytiles = g.ny / ta.ty;
+  const int ytiles = (g.ny + ta.ty - 1) / ta.ty;
   CUtensorMap tm_own{}, tm_halo{};
+  const RowMode rows = (g.pad & 1) ? kRowsOdd : (g.pad || g.ny % ta.ty != 0) ? kRowsEven : kRowsPlain;
+  auto typed = [&](auto zero, const void* in, void* out, dim3 grid, int* resident) {
+    using S = decltype(zero);
+    switch (rows) {
+      case kRowsPlain:
+        return rows2_dispatch<S, kRowsPlain>(s.bxc, s.tyt, ta, in, out, tm_own, tm_halo, stream, grid, resident);
+      case kRowsEven:
+        return rows2_dispatch<S, kRowsEven>(s.bxc, s.tyt, ta, in, out, tm_own, tm_halo, stream, grid, resident);
+      default:
+        return rows2_dispatch<S, kRowsOdd>(s.bxc, s.tyt, ta, in, out, tm_own, tm_halo, stream, grid, resident);
+    }
+  };
   auto dispatch = [&](const void* in, void* out, dim3 grid, int* resident) {
     switch (sl.precision) {
-      case MACLAB_F32:
-        return rows2_dispatch<float>(s.bxc, s.tyt, ta, in, out, tm_own, tm_halo, stream, grid, resident);
-      case MACLAB_BF16_STORE:
-        return rows2_dispatch<__nv_bfloat16>(s.bxc, s.tyt, ta, in, out, tm_own, tm_halo, stream, grid, resident);
-      case MACLAB_F16_STORE:
-        return rows2_dispatch<__half>(s.bxc, s.tyt, ta, in, out, tm_own, tm_halo, stream, grid, resident);
+      case MACLAB_F32: return typed(float{}, in, out, grid, resident);
+      case MACLAB_BF16_STORE: return typed(__nv_bfloat16{}, in, out, grid, resident);
+      case MACLAB_F16_STORE: return typed(__half{}, in, out, grid, resident);
     }
     return cudaErrorInvalidValue;
   };
@@ -145,7 +154,7 @@ cudaError_t launch_rows2(const StepLaunch& sl, cudaStream_t stream, int ty, int 
   ta.wall_mode = g.wall_mode;
   ta.mask = g.mask;
   for (int i = 0; i < 3; ++i) ta.force[i] = sl.force[i];
-  ta.overlap = sl.overlap;
+  ta.set_overlap_pad(sl.overlap, g.pad);
   ta.bounds = bounds_log();
   ta.status = step_status();
   return dispatch(sl.in, sl.out, dim3(ta.nzc, ytiles), nullptr);
@@ -153,13 +162,13 @@ cudaError_t launch_rows2(const StepLaunch& sl, cudaStream_t stream, int ty, int 
 
 bool rows2_nu_supported(const Geometry& g, int precision) {
   Rows2Shape s;
-  return precision == MACLAB_F32 && rows2_shape(g, precision, 0, &s);
+  return precision == MACLAB_F32 && rows2_shape(g, precision, 0, &s, true);
 }
 
 cudaError_t launch_rows2_nu(const Geometry& g, const void* state_n, const void* state_np1, const float* lam,
                             const double force[3], double* acc, int overlap, cudaStream_t stream) {
   Rows2Shape s;
-  if (!rows2_nu_supported(g, MACLAB_F32) || !rows2_shape(g, MACLAB_F32, 0, &s)) return cudaErrorInvalidValue;
+  if (!rows2_nu_supported(g, MACLAB_F32) || !rows2_shape(g, MACLAB_F32, 0, &s, true)) return cudaErrorInvalidValue;
   TiledArgs ta{};
   ta.nx = g.nx;
   ta.ny = g.ny;
@@ -167,7 +176,7 @@ cudaError_t launch_rows2_nu(const Geometry& g, const void* state_n, const void* 
   ta.n = g.n;
   ta.plane_stride = (int64_t)g.nx * g.ny;
   ta.ty = 2 * s.tyt;
-  const int ytiles = g.ny / ta.ty;
+  const int ytiles = (g.ny + ta.ty - 1) / ta.ty;
   CUtensorMap tm_own{}, tm_halo{};
   int resident = 0;
   cudaError_t e = rows2_nu_dispatch(s.bxc, s.tyt, ta, nullptr, nullptr, tm_own, tm_halo, stream, dim3(), &resident);
@@ -181,7 +190,7 @@ cudaError_t launch_rows2_nu(const Geometry& g, const void* state_n, const void* 
   ta.wall_mode = g.wall_mode;
   ta.mask = g.mask;
   for (int i = 0; i < 3; ++i) ta.force[i] = force[i];
-  ta.overlap = overlap;  // waits for the previous kernel before reading (pdl_wait)
+  ta.set_overlap_pad(overlap, g.pad);  // waits for the previous kernel before reading (pdl_wait)
   ta.bounds = bounds_log();
   ta.lam = lam;
   ta.nu_acc = acc;

@@ -41,7 +41,9 @@
 //    held across a plane's update do not fit.)
 //
 // Requires: D3Q19, FP32 arithmetic (FP32, BF16 or FP16 storage), nx % 4 == 0,
-// nx / 4 <= BXC, ny % TY == 0, TYT >= 2.
+// nx / 4 <= BXC, ny >= TY, TYT >= 2.  Where TY does not divide ny, the last tile
+// is moved up to end at the last row; the rows it shares with the tile before
+// are stored by that one only.
 //
 // Viscosity-term mode (NU, FP32 storage): the same march and exchanges gather
 // the moments of g_a = w_a (drho + rho (3/2 u.u - 9/2 (c.u)^2)) (the
@@ -263,7 +265,8 @@ struct Rows2Sum {
 // Tile copies: tm_own maps the state as [4 fields][nz][ny][nx] with a box of the
 // tile's TY own rows of every field; tm_halo the same tensor with a box of one
 // row of every field.
-template <typename S, int BXC, int TYT, bool NU = false>
+// RM: the rows it serves (RowMode).
+template <typename S, int BXC, int TYT, bool NU = false, int RM = kRowsPlain>
 __global__ void __launch_bounds__(BXC * TYT, Rows2Layout<S, BXC, TYT>::MIN_BLOCKS)
     step_rows2(TiledArgs ta, const S* __restrict__ in, S* __restrict__ out,
                const __grid_constant__ CUtensorMap tm_own, const __grid_constant__ CUtensorMap tm_halo) {
@@ -312,19 +315,21 @@ __global__ void __launch_bounds__(BXC * TYT, Rows2Layout<S, BXC, TYT>::MIN_BLOCK
   // rows: own rows 2 tr, 2 tr + 1 of the tile; the first thread-row also
   // forms the equilibria of the row below the tile, the last one those of the
   // row above (staged with the tile)
-  const int row0 = blockIdx.y * TY + 2 * tr;
+  const int first_row = blockIdx.y * TY;  // rows before it are the previous tile's
+  const int tile_row0 = RM == kRowsPlain ? first_row : min(first_row, ta.ny - TY);
+  const int row0 = tile_row0 + 2 * tr;
   int halo = tr == 0 ? 1 : (tr == TYT - 1 ? -1 : 0);
   {
     const int hrow = halo == 1 ? row0 - 1 : row0 + 2;
     if (halo != 0 && (hrow < 0 || hrow >= ta.ny) && !ta.py)
       halo = 0;  // beyond a closed y boundary: the row next to it is a wall row
   }
-  bool row_wall[2];
-  row_wall[0] = !ta.py && row0 == 0;
-  row_wall[1] = !ta.py && row0 + 1 == ta.ny - 1;
+  bool row_wall[2];  // not stored: a wall row, or the previous tile's
+  row_wall[0] = (!ta.py && row0 == 0) || (RM != kRowsPlain && row0 < first_row);
+  row_wall[1] = (!ta.py && row0 + 1 == ta.ny - 1) || (RM != kRowsPlain && row0 + 1 < first_row);
   const int64_t row_off = (int64_t)row0 * ta.nx + 4 * tx;
   const bool x_lo_wall = ta.wall_mode == kWallBox && !ta.px && tx == 0;
-  const bool x_hi_wall = ta.wall_mode == kWallBox && !ta.px && tx == bxr - 1;
+  const bool x_hi_wall = ta.wall_mode == kWallBox && !ta.px && tx == (RM == kRowsPlain ? bxr - 1 : hi_wall_quad(ta.nx, ta.pad()));
   const bool box_x = ta.wall_mode == kWallBox && !ta.px;
   const bool per_node_store = ta.wall_mode == kWallMask || (x_lo_wall && x_hi_wall);
   // box x-walls: the lanes holding x = 0 or nx - 1 keep the wall node's values
@@ -367,7 +372,6 @@ __global__ void __launch_bounds__(BXC * TYT, Rows2Layout<S, BXC, TYT>::MIN_BLOCK
   const uint32_t stage_sh = smem_u32(smem_raw);
   const int np = z1 - z0 + 2;  // planes z0 - 1 .. z1
   // halo rows of the tile (wrapped on a periodic y axis; none beyond a closed one)
-  const int tile_row0 = blockIdx.y * TY;
   int lo_row = tile_row0 - 1, hi_row = tile_row0 + TY;
   bool lo_ok = true, hi_ok = true;
   if (lo_row < 0) {
@@ -429,7 +433,7 @@ __global__ void __launch_bounds__(BXC * TYT, Rows2Layout<S, BXC, TYT>::MIN_BLOCK
 #pragma unroll
         for (int f = 0; f < 4; ++f)
           if (bounds_ok(ta.bounds, w + 4 * j + f, (int64_t)(Lay::wall_bytes / sizeof(float))))
-            WV[w + 4 * j + f] = x_lo_wall ? st[j][f][0].x : st[j][f][1].y;
+            WV[w + 4 * j + f] = x_lo_wall ? st[j][f][0].x : (RM == kRowsOdd ? st[j][f][0].y : st[j][f][1].y);
     }
   };
 
@@ -671,7 +675,7 @@ __global__ void __launch_bounds__(BXC * TYT, Rows2Layout<S, BXC, TYT>::MIN_BLOCK
       const int64_t off = (int64_t)q * ps + j * nx64;
       if (per_node_store) {
         S* const fp[4] = {op[0], op[1], op[2], op[3]};
-        store_plane<kD3Q19, S>(fp, mrow, ta, off, x_lo_wall, x_hi_wall, skip, acc[j], force);
+        store_plane<kD3Q19, S, RM>(fp, mrow, ta, off, x_lo_wall, x_hi_wall, skip, acc[j], force);
         continue;
       }
       if (skip) continue;
@@ -694,7 +698,8 @@ __global__ void __launch_bounds__(BXC * TYT, Rows2Layout<S, BXC, TYT>::MIN_BLOCK
 #pragma unroll
       for (int f = 0; f < 4; ++f) {
         v[f][0].x = x_lo_wall ? wv[f] : v[f][0].x;
-        v[f][1].y = x_hi_wall ? wv[f] : v[f][1].y;
+        if constexpr (RM == kRowsOdd) v[f][0].y = x_hi_wall ? wv[f] : v[f][0].y;
+        else v[f][1].y = x_hi_wall ? wv[f] : v[f][1].y;
         if (bounds_ok(ta.bounds, f * ta.n + in_off + off, n4 - 3)) Quad<S>::st(op[f] + off, v[f][0], v[f][1]);
       }
     }
@@ -773,23 +778,18 @@ __global__ void __launch_bounds__(BXC * TYT, Rows2Layout<S, BXC, TYT>::MIN_BLOCK
   }
 }
 
-// Launch of the instance (bxc, tyt) for storage type S (FP32 instances in
-// step_rows2.cu, 16-bit storage in step_rows2_s16.cu).
-template <typename S>
-cudaError_t rows2_dispatch(int bxc, int tyt, const TiledArgs& ta, const void* in, void* out,
-                           const CUtensorMap& tm_own, const CUtensorMap& tm_halo, cudaStream_t st, dim3 grid,
-                           int* resident);
-// The viscosity-term mode, FP32 storage (instances in step_rows2_nu.cu).
+// The viscosity-term mode, FP32 storage (instances in step_rows2_nu.cu): rows
+// without padding, any ny of at least a tile.
 cudaError_t rows2_nu_dispatch(int bxc, int tyt, const TiledArgs& ta, const void* in, const void* out,
                               const CUtensorMap& tm_own, const CUtensorMap& tm_halo, cudaStream_t st, dim3 grid,
                               int* resident);
 
 // Launch one instance.  With resident_out set,
 // only report the blocks of this shape one SM holds.
-template <typename S, int BXC, int TYT, bool NU = false>
+template <typename S, int BXC, int TYT, bool NU = false, int RM = kRowsPlain>
 cudaError_t launch_rows2_shape(const TiledArgs& ta, const void* in, void* out, const CUtensorMap& tm_own,
                                const CUtensorMap& tm_halo, cudaStream_t stream, dim3 grid, int* resident_out) {
-  auto kern = step_rows2<S, BXC, TYT, NU>;
+  auto kern = step_rows2<S, BXC, TYT, NU, RM>;
   constexpr size_t smem = Rows2Layout<S, BXC, TYT>::smem;
   static int resident_dev[64] = {};
   int dev = 0;
@@ -810,8 +810,30 @@ cudaError_t launch_rows2_shape(const TiledArgs& ta, const void* in, void* out, c
     *resident_out = resident;
     return cudaSuccess;
   }
-  return launch_kernel(kern, grid, dim3(BXC, TYT), smem, stream, ta.overlap, ta, static_cast<const S*>(in),
+  return launch_kernel(kern, grid, dim3(BXC, TYT), smem, stream, ta.overlap(), ta, static_cast<const S*>(in),
                        static_cast<S*>(out), tm_own, tm_halo);
 }
+
+// Launch of the instance (bxc, tyt) for storage type S and row mode RM
+// (instances in step_rows2_f32*.cu and step_rows2_s16*.cu, which compile in
+// parallel).
+template <typename S, int RM>
+cudaError_t rows2_dispatch(int bxc, int tyt, const TiledArgs& ta, const void* in, void* out,
+                           const CUtensorMap& tm_own, const CUtensorMap& tm_halo, cudaStream_t st, dim3 grid,
+                           int* resident) {
+  switch (bxc * 100 + tyt) {
+    case 1604: return launch_rows2_shape<S, 16, 4, false, RM>(ta, in, out, tm_own, tm_halo, st, grid, resident);
+    case 3202:
+      if constexpr (sizeof(S) == 4)
+        return launch_rows2_shape<S, 32, 2, false, RM>(ta, in, out, tm_own, tm_halo, st, grid, resident);
+      break;
+    case 3204: return launch_rows2_shape<S, 32, 4, false, RM>(ta, in, out, tm_own, tm_halo, st, grid, resident);
+  }
+  return cudaErrorInvalidValue;
+}
+#define MACLAB_ROWS2_DISPATCH(EXTERN, S, RM)                                                                    \
+  EXTERN template cudaError_t rows2_dispatch<S, RM>(int, int, const TiledArgs&, const void*, void*,             \
+                                                     const CUtensorMap&, const CUtensorMap&, cudaStream_t, dim3, \
+                                                     int*);
 
 }  // namespace maclab

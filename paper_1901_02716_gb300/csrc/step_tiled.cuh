@@ -74,12 +74,25 @@ struct TiledArgs {
   int wall_mode;
   const uint8_t* mask;     // node types in storage order (kWallMask)
   double force[3];
-  int overlap;             // host side: launch with programmatic dependent launch
+  // bit 0: launch with programmatic dependent launch (host side); above it the
+  // storage positions of a row beyond the domain (Geometry::pad).  One word, as
+  // the kernels compile to two registers more and 2 % slower with another field
+  int overlap_pad;
   BoundsLog* bounds;       // debug builds: where bad indices are recorded (bounds_ok)
   const float* lam;        // viscosity-term launches: the adjoint of the state after the step
   double* nu_acc;          // viscosity-term launches: the sum's accumulator (one double)
   unsigned* status;        // bit 0 set when a bounded wait on a copy ran out (step_status())
+
+  __host__ __device__ int overlap() const { return overlap_pad & 1; }
+  __host__ __device__ int pad() const { return overlap_pad >> 1; }
+  void set_overlap_pad(int overlap, int pad) { overlap_pad = (overlap ? 1 : 0) | (pad << 1); }
 };
+
+// What rows an instance of the 3D kernels serves: whole tiles of rows without
+// padding; any ny, with even padding (0 or 2); any ny, with odd padding (the
+// right wall is then lane a.y of its quad instead of b.y).  Instances of their
+// own: as run-time choices the last two cost the first 4 to 8 % at 128^3.
+enum RowMode { kRowsPlain, kRowsEven, kRowsOdd };
 
 // ------------------------------------------------------------------ lane pairs
 
@@ -599,7 +612,8 @@ __device__ __forceinline__ void plane_update(
 // fp: per-field pointers at the thread's quad of plane 0; mrow: the node-type
 // mask at the same quad; off: offset of the destination plane.  Lane order of
 // the quad: (a.x, a.y, b.x, b.y) = nodes (x0, x0 + H, x0 + 1, x0 + 1 + H).
-template <int LAT, typename S>
+// RM: the rows served (-1: known at run time only).
+template <int LAT, typename S, int RM = -1>
 __device__ __forceinline__ void store_plane(S* const (&fp)[4], const uint8_t* mrow,
                                             const TiledArgs& ta, int64_t off, bool x_lo_wall,
                                             bool x_hi_wall, bool skip,
@@ -610,7 +624,8 @@ __device__ __forceinline__ void store_plane(S* const (&fp)[4], const uint8_t* mr
   using P = typename O::P;
   constexpr int D = Lattice<LAT>::D;
   if (skip) return;
-  bool wall[4] = {x_lo_wall, false, false, x_hi_wall};
+  const bool hi_a = RM < 0 ? (ta.pad() & 1) != 0 : RM == kRowsOdd;  // the right wall is lane a.y instead of b.y
+  bool wall[4] = {x_lo_wall, x_hi_wall && hi_a, false, x_hi_wall && !hi_a};
   bool any = x_lo_wall || x_hi_wall;
   if (ta.wall_mode == kWallMask) {
     const uchar4 m = *reinterpret_cast<const uchar4*>(mrow + off);
@@ -713,9 +728,9 @@ __global__ void __launch_bounds__(BXC * RY, TiledMinBlocks<BXC, RY>::value)
   const bool row_wall = D == 3 && !ta.py && (row == 0 || row == ta.ny - 1);
   const int64_t row_off = (int64_t)row_mem * ta.nx + 4 * tx;
   const bool loads = active && row_exists && role != 3;
-  // box walls at x = 0 (lane a.x of thread 0) and x = nx - 1 (lane b.y of the last)
+  // box walls at x = 0 (lane a.x of thread 0) and the domain's last node (lane b.y of the last thread, see pad)
   const bool x_lo_wall = ta.wall_mode == kWallBox && !ta.px && tx == 0;
-  const bool x_hi_wall = ta.wall_mode == kWallBox && !ta.px && tx == bxr - 1;
+  const bool x_hi_wall = ta.wall_mode == kWallBox && !ta.px && tx == hi_wall_quad(ta.nx, ta.pad());
 
   const S* ip[4];
   S* op[4];
@@ -872,7 +887,7 @@ cudaError_t launch_shape(const TiledArgs& ta, const TiledShape& s, const void* i
           cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
       if (e != cudaSuccess) return e;                                                         \
     }                                                                                         \
-    return launch_kernel(kern, grid, dim3(BXC, RY), smem, stream, ta.overlap, ta,            \
+    return launch_kernel(kern, grid, dim3(BXC, RY), smem, stream, ta.overlap(), ta,            \
                          static_cast<const S*>(in), static_cast<S*>(out));                    \
   }
 
