@@ -163,11 +163,10 @@ maclab_status maclab_step(maclab_handle h, int64_t n);
  * rows); MACLAB_KERNEL_SEGMENT is the batched D2Q9 kernel run on one domain
  * (a warp per 30-quad row segment, x exchange by warp shuffles; with two
  * steps per launch the rows are staged four ahead in the warp's own shared
- * memory; nx % 4 == 0; the tile's tz is its rows per work item, default 2
- * up to 65,536 quads, 4 above and 32 with two steps above 524,288 quads, and
- * ty the time steps per launch, 1 or 2, default 2 below 200,000 quads and,
- * with FP32 storage, above 524,288 quads, where two steps are supported, see
- * maclab_batch_set_depth), the default for D2Q9 grids with nx % 4 == 0 that the
+ * memory; nx % 4 == 0; the tile's tz is its rows per work item, by default as
+ * few as make one wave of resident warps, and ty the time steps per launch, 1
+ * or 2, default 2 with FP32 storage and, with FP64 storage, below 200,000 quads,
+ * see maclab_batch_set_depth), the default for D2Q9 grids with nx % 4 == 0 that the
  * block kernel does not take (below).  All compute Eqs.
  * (4)-(5) with the same terms per node (the folded kernel sums them in
  * another order; the segment and tiled kernels give identical bits).
@@ -180,20 +179,22 @@ maclab_status maclab_step(maclab_handle h, int64_t n);
  * summed in yet another order, so it agrees with the others to rounding.
  * MACLAB_KERNEL_BLOCK is the block-resident D2Q9 kernel (FP32 or FP64
  * storage, nx % 4 == 0): a launch takes ty steps (1, 2, 4 or, with FP32, 8;
- * default 8 up to 65,536 node pairs and 4 above; FP64 4 up to 16,384 pairs
- * and 2 above) on tiles of 32 x 32 node pairs (pair j of a row holds x = j
- * and x = j + nx / 2; FP32: 2 x 2 pairs per thread, FP64: 32 x 16 pairs, one
- * per thread) held in registers, exchanging equilibria through warp shuffles
+ * default 8 up to 65,536 node pairs and 4 above; FP64 1 below 8,192 pairs, 4 up
+ * to 16,384 and 2 above) on tiles of 32 pair columns (pair j of a row holds x = j
+ * and x = j + nx / 2; FP32: 32 rows, 2 x 1 or 2 x 2 pairs per thread, FP64: up to
+ * 20 rows, one pair per thread) held in registers, exchanging what crosses
+ * between threads through warp shuffles
  * and shared memory, each tile with a halo of ty pairs and rows, so the state
  * passes through global memory once per ty steps; a run of n steps ends with
  * a one-step launch (the previous state is step n - 1).  Its sums run in the
- * tiled kernel's order: identical bits.  The default for FP32 and FP64 D2Q9
- * grids of up to 131,072 node pairs (512^2).
+ * tiled kernel's order: identical bits.  The default for FP32 D2Q9 grids of
+ * fewer than 524,288 node pairs and FP64 ones of up to 131,072 (512^2).
  * The default also takes these kernels where a choice by hand is refused: a
  * closed x axis of at least 17 nodes whose width is not a multiple of 4 is
- * stored in rows padded to one (the raw state keeps its (d + 1) * N values),
- * and the two-rows and folded kernels run on row counts that their tiles do not
- * divide (at least one tile of rows). */
+ * stored in rows padded to one (the raw state keeps its (d + 1) * N values), the
+ * block kernel takes a periodic x axis of any width of at least 32 nodes, and the
+ * two-rows and folded kernels run on row counts that their tiles do not divide
+ * (at least one tile of rows). */
 #define MACLAB_KERNEL_AUTO 0
 #define MACLAB_KERNEL_REFERENCE 1
 #define MACLAB_KERNEL_TILED 2
@@ -317,7 +318,8 @@ maclab_status maclab_batch_member(maclab_batch b, int32_t i, maclab_handle *out)
  * every member's other buffer holds step n - 1 as after single steps. */
 maclab_status maclab_batch_step(maclab_batch b, int64_t n);
 
-/* Rows of a domain per work item (the tuning knob of the single launch);
+/* Rows of a domain per work item, at most (the tuning knob of the single
+ * launch; an item takes fewer where that fills the last wave of the launch);
  * 0 = library default.  Rebuilds the work list. */
 maclab_status maclab_batch_set_rows(maclab_batch b, int32_t rows);
 

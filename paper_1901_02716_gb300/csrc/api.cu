@@ -11,6 +11,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <new>
@@ -778,6 +779,16 @@ maclab_status maclab_step(maclab_handle h, int64_t n) {
     CUDA_TRY(launch_step(step_launch(h, h->cur), h->stream, h->kernel), "step launch");
     h->cur ^= 1;
   }
+  // the block kernel takes what remains of the bulk in launches of 4, 2 and 1
+  // steps (7 steps: 3 launches)
+  for (int part = k / 2; h->kernel == MACLAB_KERNEL_BLOCK && part > 1; part /= 2)
+    if (bulk - done >= part) {
+      StepLaunch sl = step_launch(h, h->cur);
+      sl.seg_steps = part;
+      CUDA_TRY(launch_step(sl, h->stream, h->kernel), "step launch");
+      h->cur ^= 1;
+      done += part;
+    }
   for (; done < n; ++done) {
     StepLaunch sl = step_launch(h, h->cur);
     sl.seg_steps = 1;
@@ -1144,7 +1155,8 @@ maclab_status maclab_get_launch_overlap(maclab_handle h, int32_t* on) {
 maclab_status maclab_set_tile(maclab_handle h, int32_t ty, int32_t tz) {
   if (!h) return fail(MACLAB_ERR_INVALID, "NULL handle");
   if (ty < 0 || tz < 0 || tz > (1 << 20)) return fail(MACLAB_ERR_INVALID, "bad tile shape");
-  if (h->g.pad) return fail(MACLAB_ERR_UNSUPPORTED, "no built tiled instance has this shape");
+  if (h->g.pad || (!h->g.ilv && h->kernel == MACLAB_KERNEL_BLOCK))
+    return fail(MACLAB_ERR_UNSUPPORTED, "no built tiled instance has this shape");
   bool ok = h->kernel == MACLAB_KERNEL_FOLDED          ? fold_supported(h->g, h->precision, ty, true)
                   : h->kernel == MACLAB_KERNEL_ROWS2   ? rows2_supported(h->g, h->precision, ty, true)
                   : h->kernel == MACLAB_KERNEL_BLOCK   ? block_supported(h->g, h->precision, ty)  // ty: steps
@@ -1261,7 +1273,7 @@ struct maclab_batch_ctx {
   void* d_insts = nullptr;
   void* d_items = nullptr;
   int n_items = 0;
-  int rows = 0;                // rows per work item
+  int rows = 0;                // rows per work item, at most
   int depth = 1;               // time steps per launch (1 or 2)
   int blocks = 0;
   // the persistent form (depth 3 in maclab_batch_set_depth): the two-step
@@ -1330,8 +1342,19 @@ maclab_status batch_build_items(maclab_batch_ctx* b, int rows, int depth) {
     b->depth = 1;
     return MACLAB_OK;
   }
-  std::vector<int> items;
-  for (size_t i = 0; i < b->members.size(); ++i) batch_items((int)i, b->members[i]->g, rows, depth, items);
+  // of at most `rows` rows an item, as few as make no more waves of resident warps
+  // (a wave that is nearly empty costs as much as a full one: 64 cavities at two
+  // steps per launch, 21.2 us a step in 16 rows, the best of the powers of two;
+  // one full wave 18.0)
+  std::vector<int> items, quads, heights;
+  for (maclab_ctx* m : b->members) {
+    quads.push_back(m->g.nx / 4);
+    heights.push_back(m->g.ny);
+  }
+  const int64_t slots = batch_warp_slots(b->precision, depth);
+  const int64_t waves = (batch_item_count(quads, heights, depth, rows) + slots - 1) / slots;
+  const int cut = std::min(rows, batch_fit_rows(quads, heights, depth, waves * slots));
+  for (size_t i = 0; i < b->members.size(); ++i) batch_items((int)i, b->members[i]->g, cut, depth, items);
   void* d = nullptr;
   if (cudaMalloc(&d, items.size() * sizeof(int)) != cudaSuccess) {
     cudaGetLastError();
@@ -1496,7 +1519,7 @@ maclab_status maclab_batch_create(const maclab_config* cfgs, int32_t count, macl
   // built, and the block kernel would take one step per launch
   if (!b->one_launch)
     for (maclab_ctx* m : b->members)
-      if (m->kernel == MACLAB_KERNEL_SEGMENT || m->kernel == MACLAB_KERNEL_BLOCK)
+      if (m->g.ilv && (m->kernel == MACLAB_KERNEL_SEGMENT || m->kernel == MACLAB_KERNEL_BLOCK))
         m->kernel = tiled_supported(m->g, m->precision, 0, 0) ? MACLAB_KERNEL_TILED : MACLAB_KERNEL_REFERENCE;
   if (b->one_launch) {
     std::vector<unsigned char> insts(batch_inst_bytes() * b->members.size());
@@ -1669,7 +1692,7 @@ bool shape_supported(const maclab_ctx* h, int kernel, int ty, int tz) {
     return step_kernel_supported(h->g, h->precision, MACLAB_KERNEL_SEGMENT) &&
            (ty <= 1 || segment_depth(h->g, h->precision, ty) == 2);
   if (kernel == MACLAB_KERNEL_ROWS2) return rows2_supported(h->g, h->precision, ty, true);
-  if (kernel == MACLAB_KERNEL_BLOCK) return block_supported(h->g, h->precision, ty);
+  if (kernel == MACLAB_KERNEL_BLOCK) return block_supported(h->g, h->precision, ty, true);
   return kernel == MACLAB_KERNEL_FOLDED ? fold_supported(h->g, h->precision, ty, true)
                                         : tiled_supported(h->g, h->precision, ty, tz);
 }
@@ -1841,7 +1864,7 @@ maclab_status maclab_tune(maclab_handle h, int32_t out[2]) {
     return ms;
   };
   // candidates (kernel, ty, tz): tiled and folded shapes; the segment kernel
-  // with one or two steps per launch (ty) and 2, 4 or 8 rows per work item (tz)
+  // with one or two steps per launch (ty) and several rows per work item (tz)
   struct Cand {
     int kernel, ty, tz;
   };
@@ -1850,12 +1873,16 @@ maclab_status maclab_tune(maclab_handle h, int32_t out[2]) {
     for (int a = 0; a < n_ty; ++a)
       for (int tz : tzs) cands.push_back(Cand{kernel, h->g.d == 3 ? tys3[a] : 0, tz});
   for (int ty : {1, 2, 3})  // 3: two steps per sweep, runs in one persistent launch
-    for (int tz : {2, 4, 8, 16, 32}) cands.push_back(Cand{MACLAB_KERNEL_SEGMENT, ty, tz});
-  // the block kernel up to 131,072 node pairs (512^2), where it was measured
-  // to win; above it the segment kernel is faster in sustained runs (1024^2:
-  // 5.5 against 5.6-5.7 us/step), though a short timing can rank them the
-  // other way
-  if ((int64_t)(h->g.nx / 2) * h->g.ny <= 131072)
+    for (int waves : {0, 1, 2, 4}) {  // rows that make so many waves of resident warps (0: four rows)
+      const int depth = segment_depth(h->g, h->precision, ty);
+      const int tz = waves ? batch_fit_rows({h->g.nx / 4}, {h->g.ny}, depth,
+                                            (int64_t)waves * batch_warp_slots(h->precision, depth))
+                           : 4;
+      cands.push_back(Cand{MACLAB_KERNEL_SEGMENT, ty, tz});
+    }
+  // the block kernel where it was measured to win; above that the segment kernel
+  // is faster in sustained runs, though a short timing can rank them the other way
+  if (block_grid(h->g, h->precision) || !h->g.ilv)
     for (int ty : {1, 2, 4, 8}) cands.push_back(Cand{MACLAB_KERNEL_BLOCK, ty, 0});  // ty: steps per launch
   if (h->g.d == 3)
     for (int ty : {4, 8})

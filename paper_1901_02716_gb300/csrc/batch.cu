@@ -1,8 +1,7 @@
 // batch.cu -- many independent D2Q9 domains advanced by one persistent launch.
 //
 // Same update as step_naive / step_tiled (Eqs. (2), (4), (5) in the drho form
-// of step.cu, the factored equilibrium and exact integer weights of
-// step_tiled.cuh), organised for a batch of domains of different sizes:
+// of step.cu, factored by rows as in d2q9.cuh), organised for a batch of domains of different sizes:
 //
 //  * Work item = (domain, x segment, chunk of rows).  A warp takes items from
 //    a work list (item = warp id + k * warps in the grid); items of all
@@ -14,18 +13,18 @@
 //    a = (2t, 2t + H) and b = (2t + 1, 2t + 1 + H); a halo quad that wraps
 //    around the row end is lane-swapped on load, which is what the seam
 //    between the half rows needs.
-//  * Equilibria moving +x leave pair b for the next lane's pair a, those moving
-//    -x leave pair a for the previous lane's pair b: warp shuffles, no block
-//    barrier.  The halo lanes' own sums are discarded.
+//  * What moves +x leaves pair b for the next lane's pair a, what moves -x
+//    leaves pair a for the previous lane's pair b: three values each way by warp
+//    shuffles, no block barrier.  The halo lanes' own sums are discarded.
 //  * Input rows are prefetched one row ahead in registers (the two-step
 //    kernel below stages them four rows ahead through shared memory).
-//  * The three destination rows of momentum sums live in registers, as in
-//    step_tiled.
+//  * Two values sent on to the next row and the three sums of the row being
+//    completed live in registers.
 
 #include <algorithm>
 #include <vector>
 
-#include "step_tiled.cuh"
+#include "d2q9.cuh"
 
 namespace maclab {
 
@@ -61,64 +60,47 @@ __device__ __forceinline__ P shfl_down_pair(P v, int d) {
   return r;
 }
 
-// index of direction a among the directions with the same x component
-template <int LAT>
-__host__ __device__ constexpr int same_fx_index(int a) {
-  int s = 0;
-  for (int b = 0; b < a; ++b) s += Frame<LAT>::fx(b) == Frame<LAT>::fx(a) ? 1 : 0;
-  return s;
+// What one source row (state st of this lane's two pairs) adds to the rows
+// around it (d2q9.cuh): the values crossing to the neighbouring lanes move by
+// shuffles, three each way.
+template <typename C>
+__device__ __forceinline__ void batch_row(const typename Pair<C>::P (&st)[3][2], D9Row<C> (&w)[2]) {
+  using P = typename Pair<C>::P;
+  d9_quad<C>(st, w, [](P v, int) { return shfl_up_pair(v, 1); }, [](P v, int) { return shfl_down_pair(v, 1); });
 }
 
-// Contributions of one source row (state st of this lane's two pairs) to the
-// sums of destination rows y - 1 (ap), y (ac), y + 1 (an); MODE as in step_tiled.
-template <typename C, int MODE>
-__device__ __forceinline__ void batch_row_update(const typename Pair<C>::P (&st)[3][2],
-                                                 typename Pair<C>::P (&ap)[2][3],
-                                                 typename Pair<C>::P (&ac)[2][3],
-                                                 typename Pair<C>::P (&an)[2][3]) {
-  using O = Pair<C>;
-  using P = typename O::P;
-  using L = Lattice<kD2Q9>;
-  using F = Frame<kD2Q9>;
-  P out_b[3], out_a[3];  // equilibria leaving pair b (+x) / pair a (-x)
+// The sums a march carries: `next` what the last source row sent to the row
+// after it (gp, hp), `cur` the sums of that source row itself, which the next
+// source row completes.
+template <typename C>
+struct BatchSums {
+  using P = typename Pair<C>::P;
+  P next[2][2], cur[2][3];
+
+  // the row before the first: only what it sends on
+  __device__ __forceinline__ void first(const D9Row<C> (&w)[2]) {
 #pragma unroll
-  for (int k = 0; k < 3; ++k) out_b[k] = out_a[k] = O::splat(C(0));
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    Terms<2, C> tm;
-    const P u[3] = {st[1][q], st[2][q], O::splat(C(0))};
-    make_terms<2, C>(st[0][q], u, tm);
-    static_for<0, L::Q>([&](auto Ia) {
-      constexpr int a = decltype(Ia)::value;
-      if constexpr (mode_allows<kD2Q9, MODE>(a)) {
-        constexpr int fx = F::fx(a), fz = F::fz(a);
-        const P T = term<kD2Q9, C, a>(tm);
-        const int qd = q + fx;
-        if (qd >= 0 && qd < 2) {
-          accum<kD2Q9, C, a>(pick<fz>(ap, ac, an)[qd], T);
-        } else {
-          if constexpr (fx == 1) out_b[same_fx_index<kD2Q9>(a)] = T;
-          else if constexpr (fx == -1) out_a[same_fx_index<kD2Q9>(a)] = T;
-        }
-      }
-    });
-  }
-  // +x: lane l - 1's pair b feeds lane l's pair a; -x: lane l + 1's pair a feeds pair b
-  static_for<0, L::Q>([&](auto Ia) {
-    constexpr int a = decltype(Ia)::value;
-    if constexpr (mode_allows<kD2Q9, MODE>(a) && F::fx(a) != 0) {
-      constexpr int fx = F::fx(a), fz = F::fz(a);
-      if constexpr (fx == 1) {
-        const P v = shfl_up_pair(out_b[same_fx_index<kD2Q9>(a)], 1);
-        accum<kD2Q9, C, a>(pick<fz>(ap, ac, an)[0], v);
-      } else {
-        const P v = shfl_down_pair(out_a[same_fx_index<kD2Q9>(a)], 1);
-        accum<kD2Q9, C, a>(pick<fz>(ap, ac, an)[1], v);
-      }
+    for (int q = 0; q < 2; ++q) {
+      next[q][0] = w[q].gp;
+      next[q][1] = w[q].hp;
     }
-  });
-}
-
+  }
+  __device__ __forceinline__ void none() {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) next[q][0] = next[q][1] = Pair<C>::splat(C(0));
+  }
+  // completes the previous row's sums in cur
+  __device__ __forceinline__ void finish(const D9Row<C> (&w)[2]) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) d9_above<C>(cur[q], w[q].gm, w[q].hm);
+  }
+  // starts this row's sums (after the previous ones were used)
+  __device__ __forceinline__ void start(const D9Row<C> (&w)[2]) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) d9_own<C>(cur[q], next[q][0], next[q][1], w[q]);
+    first(w);
+  }
+};
 
 // Store of one final row (Eq. (5): u' = M / (36 + R) + F).  In box mode every
 // lane stores its whole quad: a lane whose quad holds one x-wall node (a.x at
@@ -138,10 +120,10 @@ __device__ __forceinline__ void batch_store(S* out, int64_t n, int64_t off, cons
   P v[K][2];
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
-    const P inv = O::rcp(O::add(O::splat(C(36)), acc[q][0]));
-    v[0][q] = O::mul(acc[q][0], O::splat(C(1.0 / 36.0)));
-    v[1][q] = O::fma(acc[q][1], inv, force[0]);
-    v[2][q] = O::fma(acc[q][2], inv, force[1]);
+    P x[3];
+    d9_state<C>(acc[q], force, x);
+#pragma unroll
+    for (int f = 0; f < K; ++f) v[f][q] = x[f];
   }
   if (wall_mode == kWallMask || (x_lo_wall && x_hi_wall)) {
     bool wall[4] = {x_lo_wall, x_hi_wall && hi_a, false, x_hi_wall && !hi_a};
@@ -181,14 +163,12 @@ __device__ __forceinline__ void batch_store(S* out, int64_t n, int64_t off, cons
 // right wall is lane a.y of its quad instead of b.y; an instance of its own, as
 // the run-time choice costs 6 % at 1024^2).
 template <typename S, bool HIA>
-__global__ void __launch_bounds__(256) batch_step_d2q9(const BatchInst* __restrict__ insts,
+__global__ void __launch_bounds__(256, sizeof(S) == 8 ? 1 : 2) batch_step_d2q9(const BatchInst* __restrict__ insts,
                                                        const BatchItem* __restrict__ items,
                                                        int n_items, int cur, int segw) {
   using C = typename Store<S>::C;
   using O = Pair<C>;
   using P = typename O::P;
-  using L = Lattice<kD2Q9>;
-  using F = Frame<kD2Q9>;
   constexpr int K = 3;
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -252,56 +232,44 @@ __global__ void __launch_bounds__(256) batch_step_d2q9(const BatchInst* __restri
       batch_store<S, HIA>(out, n, off, d_mask, d_wall, x_lo_wall, x_hi_wall, hi_a, wk, acc, force);
     };
 
-    P R0[2][K], R1[2][K], R2[2][K];
-#pragma unroll
-    for (int q = 0; q < 2; ++q)
-#pragma unroll
-      for (int k = 0; k < K; ++k) R0[q][k] = R1[q][k] = R2[q][k] = O::splat(C(0));
+    BatchSums<C> sums;
+    D9Row<C> w[2];
     P st[K][2], nxt[K][2];
     const int y0 = item.y0, y1 = item.y1;
     load(y0 - 1, st);
     load(y0, nxt);
-    if (row_exists(y0 - 1))
-      batch_row_update<C, kFirst>(st, R0, R2, R1);
-    // source row y: sums A, B, N of destination rows y - 1, y, y + 1; then row
-    // y - 1 is complete
-    auto row = [&](int y, P(&A)[2][K], P(&B)[2][K], P(&N)[2][K]) {
+    sums.none();
+    if (row_exists(y0 - 1)) {
+      batch_row<C>(st, w);
+      sums.first(w);
+    }
+    // source row y completes row y - 1 (unrolled by two: the row in flight and the
+    // sums sent on change registers instead of being moved; three spend more on
+    // instruction fetch)
+#pragma unroll 2
+    for (int y = y0; y < y1; ++y) {
 #pragma unroll
       for (int f = 0; f < K; ++f) {
         st[f][0] = nxt[f][0];
         st[f][1] = nxt[f][1];
       }
       load(y + 1, nxt);
-      batch_row_update<C, kMid>(st, A, B, N);
-      if (y - 1 >= y0) store(y - 1, A);
-#pragma unroll
-      for (int f = 0; f < K; ++f) wk[f] = x_lo_wall ? st[f][0].x : (hi_a ? st[f][0].y : st[f][1].y);  // row y, stored next
-#pragma unroll
-      for (int q = 0; q < 2; ++q)
-#pragma unroll
-        for (int k = 0; k < K; ++k) A[q][k] = O::splat(C(0));
-    };
-    // source row y1 (beyond the chunk): its contributions to row y1 - 1 (= B)
-    auto last = [&](P(&B)[2][K]) {
-      if (row_exists(y1)) {
-#pragma unroll
-        for (int f = 0; f < K; ++f) {
-          st[f][0] = nxt[f][0];
-          st[f][1] = nxt[f][1];
-        }
-        batch_row_update<C, kLast>(st, B, R0, R0);
+      batch_row<C>(st, w);
+      if (y > y0) {
+        sums.finish(w);
+        store(y - 1, sums.cur);
       }
-      store(y1 - 1, B);
-    };
-    // the three row sums rotate with period 3
-    for (int y = y0;;) {
-      if (y >= y1) { last(R0); break; }
-      row(y++, R0, R1, R2);
-      if (y >= y1) { last(R1); break; }
-      row(y++, R1, R2, R0);
-      if (y >= y1) { last(R2); break; }
-      row(y++, R2, R0, R1);
+      sums.start(w);
+#pragma unroll
+      for (int f = 0; f < K; ++f)  // row y, stored next
+        wk[f] = x_lo_wall ? st[f][0].x : (hi_a ? st[f][0].y : st[f][1].y);
     }
+    // source row y1 (beyond the chunk)
+    if (row_exists(y1)) {
+      batch_row<C>(nxt, w);
+      sums.finish(w);
+    }
+    store(y1 - 1, sums.cur);
   }
 }
 
@@ -361,10 +329,10 @@ __device__ __forceinline__ void batch_emit(const typename Pair<C>::P (&acc)[2][3
   }
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
-    const P inv = O::rcp(O::add(O::splat(C(36)), acc[q][0]));
-    out[0][q] = O::mul(acc[q][0], O::splat(C(1.0 / 36.0)));
-    out[1][q] = O::fma(acc[q][1], inv, force[0]);
-    out[2][q] = O::fma(acc[q][2], inv, force[1]);
+    P x[3];
+    d9_state<C>(acc[q], force, x);
+#pragma unroll
+    for (int f = 0; f < 3; ++f) out[f][q] = x[f];
   }
 #pragma unroll
   for (int f = 0; f < 3; ++f) {
@@ -373,14 +341,6 @@ __device__ __forceinline__ void batch_emit(const typename Pair<C>::P (&acc)[2][3
     if (wall & 4u) out[f][1].x = in[f][1].x;
     if (wall & 8u) out[f][1].y = in[f][1].y;
   }
-}
-
-template <typename P>
-__device__ __forceinline__ void zero_sums(P (&a)[2][3]) {
-#pragma unroll
-  for (int q = 0; q < 2; ++q)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) a[q][k] = P{0, 0};
 }
 
 // Two updates of every work item, reading buffer cur and writing cur ^ 1:
@@ -487,10 +447,8 @@ __device__ __forceinline__ void batch2_sweep(const BatchInst* __restrict__ insts
       batch_store<S, HIA>(out, n, off, d_mask, d_wall, x_lo_wall, x_hi_wall, hi_a, wk, acc, force);
     };
 
-    // sums of the first update for row d in A[(d - y0 + 3) % 3], of the second in B[...]
-    P A0[2][K], A1[2][K], A2[2][K], B0[2][K], B1[2][K], B2[2][K];
-    zero_sums(A0); zero_sums(A1); zero_sums(A2);
-    zero_sums(B0); zero_sums(B1); zero_sums(B2);
+    BatchSums<C> A, B;  // of the first and the second update
+    D9Row<C> w[2];
     P st[K][2], prev[K][2], mid[K][2];
     uint32_t w_st = 0, w_prev = 0;
     auto advance = [&](int y) {  // st <- input row y; start copying row y + kRowRing
@@ -513,57 +471,60 @@ __device__ __forceinline__ void batch2_sweep(const BatchInst* __restrict__ insts
     // input row y0 - 2: only its sums into row y0 - 1
 #pragma unroll
     for (int i = 0; i < kRowRing; ++i) issue(i);
+    A.none();
     advance(y0 - 2);
-    if (row_exists(y0 - 2)) batch_row_update<C, kFirst>(st, A0, A1, A2);
+    if (row_exists(y0 - 2)) {
+      batch_row<C>(st, w);
+      A.first(w);
+    }
     // input row y0 - 1 (row y0 - 2 of the first update is not needed)
     advance(y0 - 1);
-    batch_row_update<C, kMid>(st, A1, A2, A0);
-    zero_sums(A1);
+    batch_row<C>(st, w);
+    A.start(w);
     keep();
     // input row y0 completes intermediate row y0 - 1, the second update's first source
     advance(y0);
-    batch_row_update<C, kMid>(st, A2, A0, A1);
-    batch_emit<C>(A2, prev, w_prev, row_exists(y0 - 1), force, mid);
-    zero_sums(A2);
+    batch_row<C>(st, w);
+    A.finish(w);
+    batch_emit<C>(A.cur, prev, w_prev, row_exists(y0 - 1), force, mid);
+    A.start(w);
     keep();
     keep_wall();
-    if (row_exists(y0 - 1)) batch_row_update<C, kFirst>(mid, B1, B2, B0);
-
-    // input row ys: intermediate row ys - 1 complete, fed to the second update,
-    // which completes final row ys - 2.  Ap/Ac/An: first-update sums of rows
-    // ys - 1, ys, ys + 1; Bp/Bc/Bn: second-update sums of rows ys - 2, ys - 1, ys.
-    auto body = [&](int ys, P(&Ap)[2][K], P(&Ac)[2][K], P(&An)[2][K], P(&Bp)[2][K], P(&Bc)[2][K],
-                    P(&Bn)[2][K]) {
-      advance(ys);
-      batch_row_update<C, kMid>(st, Ap, Ac, An);
-      batch_emit<C>(Ap, prev, w_prev, row_exists(ys - 1), force, mid);
-      zero_sums(Ap);
-      keep();
-      batch_row_update<C, kMid>(mid, Bp, Bc, Bn);
-      if (ys - 2 >= y0) store(ys - 2, Bp);
-      keep_wall();
-      zero_sums(Bp);
-    };
-    // input row y1 + 1: completes intermediate row y1 and final row y1 - 1
-    auto last = [&](P(&Ap)[2][K], P(&Ac)[2][K], P(&An)[2][K], P(&Bp)[2][K], P(&Bc)[2][K],
-                    P(&Bn)[2][K]) {
-      if (row_exists(y1 + 1)) {
-        advance(y1 + 1);
-        batch_row_update<C, kLast>(st, Ap, Ac, An);
-      }
-      batch_emit<C>(Ap, prev, w_prev, row_exists(y1), force, mid);
-      if (row_exists(y1)) batch_row_update<C, kLast>(mid, Bp, Bc, Bn);
-      store(y1 - 1, Bp);
-    };
-    // the sums rotate with period 3
-    for (int ys = y0 + 1;;) {
-      if (ys > y1) { last(A0, A1, A2, B2, B0, B1); break; }
-      body(ys++, A0, A1, A2, B2, B0, B1);
-      if (ys > y1) { last(A1, A2, A0, B0, B1, B2); break; }
-      body(ys++, A1, A2, A0, B0, B1, B2);
-      if (ys > y1) { last(A2, A0, A1, B1, B2, B0); break; }
-      body(ys++, A2, A0, A1, B1, B2, B0);
+    B.none();
+    if (row_exists(y0 - 1)) {
+      batch_row<C>(mid, w);
+      B.first(w);
     }
+    // input row ys: intermediate row ys - 1 complete, fed to the second update,
+    // which completes final row ys - 2
+#pragma unroll 2
+    for (int ys = y0 + 1; ys <= y1; ++ys) {
+      advance(ys);
+      batch_row<C>(st, w);
+      A.finish(w);
+      batch_emit<C>(A.cur, prev, w_prev, row_exists(ys - 1), force, mid);
+      A.start(w);
+      keep();
+      batch_row<C>(mid, w);
+      if (ys - 2 >= y0) {
+        B.finish(w);
+        store(ys - 2, B.cur);
+      }
+      B.start(w);
+      keep_wall();
+    }
+    // input row y1 + 1: completes intermediate row y1 and final row y1 - 1
+    if (row_exists(y1 + 1)) {
+      advance(y1 + 1);
+      batch_row<C>(st, w);
+      A.finish(w);
+    }
+    batch_emit<C>(A.cur, prev, w_prev, row_exists(y1), force, mid);
+    if (row_exists(y1)) {
+      batch_row<C>(mid, w);
+      B.finish(w);
+    }
+    store(y1 - 1, B.cur);
   }
 }
 
@@ -793,6 +754,38 @@ void batch_persist_deps(const std::vector<int>& items4, const std::vector<int>& 
     out.insert(out.end(), dep[b].begin(), dep[b].end());
   }
   out[blocks] = (int)out.size();
+}
+
+// One step per launch: 256-thread blocks, two per SM (FP64 one); two steps:
+// 128-thread blocks, three per SM (FP64 two).
+int batch_warp_slots(int precision, int depth) {
+  static int sms = 0;
+  if (!sms) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 148;
+  }
+  const bool f64 = precision == MACLAB_F64;
+  return sms * (depth == 2 ? (f64 ? 8 : 12) : (f64 ? 8 : 16));
+}
+
+int64_t batch_item_count(const std::vector<int>& nq, const std::vector<int>& ny, int depth, int rows) {
+  const int segw = depth == 2 ? kBatchSegW2 : kBatchSegW1;
+  int64_t n = 0;
+  for (size_t i = 0; i < nq.size(); ++i)
+    n += (int64_t)((nq[i] + segw - 1) / segw) * (((int64_t)ny[i] + rows - 1) / rows);
+  return n;
+}
+
+int batch_fit_rows(const std::vector<int>& nq, const std::vector<int>& ny, int depth, int64_t slots) {
+  int lo = 2, hi = 2;
+  for (int y : ny) hi = std::max(hi, y);
+  while (lo < hi) {  // the count falls as rows grow
+    const int mid = lo + (hi - lo) / 2;
+    if (batch_item_count(nq, ny, depth, mid) <= slots) hi = mid;
+    else lo = mid + 1;
+  }
+  return lo;
 }
 
 size_t batch_inst_bytes() { return sizeof(BatchInst); }

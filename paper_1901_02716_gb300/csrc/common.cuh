@@ -245,10 +245,22 @@ bool step_kernel_supported(const Geometry& g, int precision, int kernel);
 // Defined in step_block.cu: the block-resident D2Q9 kernel (ty = steps per
 // launch: 1, 2, 4 or, with FP32 storage, 8; 0 = by size; FP32 / FP64 storage, nx % 4 == 0).
 int block_steps(const Geometry& g, int precision, int ty);
-bool block_supported(const Geometry& g, int precision, int ty);
-int block_threads(int precision);
+// natural: also a periodic x axis of any width of at least 32 nodes.
+bool block_supported(const Geometry& g, int precision, int ty, bool natural = false);
+int block_threads(const Geometry& g, int precision, int steps);
 cudaError_t launch_block(const StepLaunch& s, cudaStream_t stream, int steps);
+// Grids where the block kernel is faster than the segment kernel (step.cu).
+inline bool block_grid(const Geometry& g, int precision) {
+  const int64_t pairs = (int64_t)(g.nx / 2) * g.ny;
+  return precision == MACLAB_F32 ? pairs < 524288 : pairs <= 131072;
+}
 int segment_depth(const Geometry& g, int precision, int ty);
+// Defined in batch.cu: warps of the segment kernels the device holds at once, the
+// work items of domains of nq[i] quads by ny[i] rows cut for `depth` steps per
+// launch, and the fewest rows per item (at least 2) that make at most `slots`.
+int batch_warp_slots(int precision, int depth);
+int64_t batch_item_count(const std::vector<int>& nq, const std::vector<int>& ny, int depth, int rows);
+int batch_fit_rows(const std::vector<int>& nq, const std::vector<int>& ny, int depth, int64_t slots);
 // Defined in batch.cu: `sweeps` two-step launches of the segment kernel in one
 // persistent cooperative launch of `blocks` blocks, each waiting between sweeps
 // (at most wait_limit polls; status bit 1 on a timeout) for the blocks on its

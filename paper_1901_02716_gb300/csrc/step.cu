@@ -120,28 +120,25 @@ static cudaError_t launch_naive_lat(const StepLaunch& s, cudaStream_t stream) {
 
 // Time steps per launch of the segment kernel for the tile setting ty (2 asks
 // for two steps per launch: FP32 or FP64 storage and nx >= 8; otherwise 1).
-// Segment kernel defaults (measured on a GB300, FP32 cavities of 64^2 to
-// 8192^2): two steps per launch below 200,000 quads (small grids are bound by
-// the launches) and, with FP32 storage, above 524,288 quads (large grids are
-// bound by memory traffic, which two steps halve: 1.57x at 2048^2, 1.8x at
-// 8192^2; FP64 is bound by its arithmetic, which the halo rows only add to),
-// one step in between (1024^2); rows per work item 2 up to 65,536 quads, 4
-// above, and 32 for two steps above 524,288 quads (the two halo rows each
-// side of an item then cost an eighth of its rows).
-static bool segment_large(const Geometry& g) { return (int64_t)(g.nx / 4) * g.ny > 524288; }
-
+// Default: two with FP32 storage, which halves the state's traffic and the
+// launches (1024^2: 4.71 us a step, 5.58 with one); FP64 is bound by its
+// arithmetic, which the second step's halo rows add to, and takes two only on
+// small grids, where the launches count.
 int segment_depth(const Geometry& g, int precision, int ty) {
   const bool two_ok = (precision == MACLAB_F32 || precision == MACLAB_F64) && g.nx >= 8;
-  if (ty == 0)
-    return two_ok && ((int64_t)(g.nx / 4) * g.ny < 200000 || (segment_large(g) && precision == MACLAB_F32)) ? 2
-                                                                                                             : 1;
+  if (ty == 0) return two_ok && (precision == MACLAB_F32 || (int64_t)(g.nx / 4) * g.ny < 200000) ? 2 : 1;
   return (ty == 2 || ty == 3) && two_ok ? 2 : 1;  // 3: two steps, runs in one persistent launch
 }
 
+// Rows per work item: asked for, or as few as make one wave of resident warps.
+// Every item repeats the sums of the halo rows at its ends, and a second wave
+// that is nearly empty costs as much as a full one (FP32 cavities, us a step,
+// with the fixed rows before -> one wave: 1024^2 5.6 -> 4.7, 2048^2 14.2 -> 12.0,
+// 4096^2 53.9 -> 40.1, 8192^2 173 -> 165).
 int segment_rows(const Geometry& g, int precision, int ty, int tz) {
   if (tz > 0) return tz;
-  if (segment_large(g) && segment_depth(g, precision, ty) == 2) return 32;
-  return (int64_t)(g.nx / 4) * g.ny <= 65536 ? 2 : 4;
+  const int depth = segment_depth(g, precision, ty);
+  return batch_fit_rows({g.nx / 4}, {g.ny}, depth, batch_warp_slots(precision, depth));
 }
 
 bool step_kernel_supported(const Geometry& g, int precision, int kernel) {
@@ -157,17 +154,16 @@ bool step_kernel_supported(const Geometry& g, int precision, int kernel) {
 // D3Q19 with FP32 storage: the two-rows-per-thread kernel where it applies
 // (rows of up to 128 nodes), else the folded one where it is built (ny a
 // multiple of its tile rows); for D2Q9 grids with nx % 4 == 0 the block kernel
-// with FP32 or FP64 storage up to 131,072 node pairs (512^2; measured on a
-// GB300, FP32: 1.9x the segment kernel at 128^2 and 256^2, 1.16x at 512^2;
-// FP64: 1.9x to 2.4x), else the segment
-// kernel (faster than the tiled one from 64^2 to 1024^2 with its size
-// defaults, and than the block kernel above 512^2); else the tiled one, else
-// the reference kernel.
+// with FP32 storage below 524,288 node pairs (us a step, block and segment
+// kernel: 256^2 0.84 and 2.1, 560^2 1.77 and 2.91, 800^2 3.05 and 3.81, 1000^2
+// 4.08 and 4.26, 1200^2 5.76 and 5.63, 2048^2 15.3 and 12.0) and with FP64
+// storage up to 131,072 (1.9x to 2.4x), else the segment kernel; else the tiled
+// one, else the reference kernel.
 int pick_step_kernel(const Geometry& g, int precision) {
   if (precision == MACLAB_F32 && rows2_supported(g, precision, 0, true)) return MACLAB_KERNEL_ROWS2;
   if (fold_supported(g, precision, 0, true)) return MACLAB_KERNEL_FOLDED;
-  if ((int64_t)(g.nx / 2) * g.ny <= 131072 && step_kernel_supported(g, precision, MACLAB_KERNEL_BLOCK))
-    return MACLAB_KERNEL_BLOCK;
+  if ((block_grid(g, precision) || !g.ilv) && block_supported(g, precision, 0, true))
+    return MACLAB_KERNEL_BLOCK;  // natural rows have no other fast kernel
   if (step_kernel_supported(g, precision, MACLAB_KERNEL_SEGMENT)) return MACLAB_KERNEL_SEGMENT;
   return step_kernel_supported(g, precision, MACLAB_KERNEL_TILED) ? MACLAB_KERNEL_TILED
                                                                  : MACLAB_KERNEL_REFERENCE;
@@ -216,7 +212,8 @@ KernelInfo describe_step_kernel(const Geometry& g, int precision, int kernel, in
   if (kernel == MACLAB_KERNEL_ROWS2)
     return KernelInfo{MACLAB_KERNEL_ROWS2, 1, 1, rows2_threads(g, precision, ty), kernel_name(g, precision, kernel)};
   if (kernel == MACLAB_KERNEL_BLOCK)
-    return KernelInfo{MACLAB_KERNEL_BLOCK, block_steps(g, precision, ty), 1, block_threads(precision),
+    return KernelInfo{MACLAB_KERNEL_BLOCK, block_steps(g, precision, ty), 1,
+                      block_threads(g, precision, block_steps(g, precision, ty)),
                       kernel_name(g, precision, kernel)};
 
   if (kernel == MACLAB_KERNEL_SEGMENT) {

@@ -150,7 +150,19 @@ struct Pair<double> {
   __device__ __forceinline__ static P fma(P a, P b, P c) {
     return make_double2(__fma_rn(a.x, b.x, c.x), __fma_rn(a.y, b.y, c.y));
   }
-  __device__ __forceinline__ static P rcp(P a) { return make_double2(1.0 / a.x, 1.0 / a.y); }
+  // 1/a: the hardware approximation r0 (rcp.approx.ftz.f64: about 20 bits) and
+  // one third-order step of the Newton family, r1 = r0 (1 + e + e^2) with e =
+  // 1 - a r0 (exact from the FMA), which leaves e^3 = 2^-60: three FP64
+  // operations where the division takes about ten, on a pipe of two lanes per
+  // SM.  Within an ulp of 1/a for arguments away from zero and infinity, as
+  // 36 + R and 1 + drho' are.
+  __device__ __forceinline__ static double rcp1(double a) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
+    const double e = __fma_rn(-a, r, 1.0);
+    return __fma_rn(r, __fma_rn(e, e, e), r);
+  }
+  __device__ __forceinline__ static P rcp(P a) { return make_double2(rcp1(a.x), rcp1(a.y)); }
   __device__ __forceinline__ static P swap(P a) { return make_double2(a.y, a.x); }
 };
 
@@ -509,6 +521,14 @@ __device__ __forceinline__ void halo_publish(const typename Pair<C>::P (&st)[Lat
   }
 }
 
+// One source row of the 2D lattice, factored (d2q9.cuh): the values leaving the
+// thread's quad in x go through the six x slots, (ap, bp, e) of pair b to the
+// right and (am, bm, e) of pair a to the left.  Defined there.
+template <typename C, int MODE, int BXC>
+__device__ __forceinline__ void row_update_2d(const typename Pair<C>::P (&st)[3][2], typename Pair<C>::P (&ap)[2][3],
+                                              typename Pair<C>::P (&ac)[2][3], typename Pair<C>::P (&an)[2][3],
+                                              const SmemBase<typename Pair<C>::P>& sb, bool active);
+
 // One source plane: publish outgoing equilibria, gather incoming ones.
 // st: the plane's state (field, pair); ap/ac/an: sums (pair, component) of
 // destination planes p - 1, p, p + 1.
@@ -528,6 +548,10 @@ __device__ __forceinline__ void plane_update(
   constexpr int XS = RY * W;      // stride between x slots
   constexpr int YR = 2 * W;       // stride between rows of a y slot
   constexpr int YS = RY * YR;     // stride between y slots
+  if constexpr (LAT == kD2Q9) {
+    row_update_2d<C, MODE, BXC>(st, ap, ac, an, sb0, active);
+    return;
+  }
   const SmemBase<P> sb = sb0.template buffer<kDoubleBuffer ? BUF : 0,
                                              Frame<LAT>::count_x() * RY * W +
                                                  Frame<LAT>::count_y() * RY * 2 * W>();

@@ -1,5 +1,5 @@
 // Instances of the tiled step kernel: D2Q9, every storage type.
-#include "step_tiled.cuh"
+#include "d2q9.cuh"
 
 namespace maclab {
 MACLAB_TILED_LAUNCH_DEF
