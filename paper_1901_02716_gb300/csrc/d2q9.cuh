@@ -36,11 +36,12 @@ __device__ __forceinline__ D9Node<C> d9_node(typename Pair<C>::P r, typename Pai
   using P = typename O::P;
   D9Node<C> n;
   const P g = O::fma(r, O::splat(C(3)), O::splat(C(3)));  // 3 rho
-  const P bx = O::mul(g, u);
-  n.by = O::mul(g, v);
+  // products that enter sums: never contracted, so that every kernel rounds alike
+  const P bx = O::mul_exact(g, u);
+  n.by = O::mul_exact(g, v);
   const P qx = O::mul(bx, u), qy = O::mul(n.by, v);  // 3 rho u_i^2
-  n.A = O::fma(O::add(qx, qy), O::splat(C(-0.5)), r);
-  n.e = O::mul(qy, O::splat(C(1.5)));
+  n.A = O::fma(O::fma(n.by, v, qx), O::splat(C(-0.5)), r);
+  n.e = O::mul_exact(qy, O::splat(C(1.5)));
   const P S = O::fma(qx, O::splat(C(1.5)), n.A);
   const P c = O::mul(bx, v);  // 3 rho u_x u_y
   n.ap = O::add(S, bx);

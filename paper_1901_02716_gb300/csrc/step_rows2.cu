@@ -24,6 +24,7 @@ namespace {
 struct Rows2Shape {
   int bxc, tyt;
 };
+constexpr ChunkCost kRows2Cost = {3.0, 1.0, 0.45};  // see fold_chunks
 constexpr Rows2Shape kRows2Shapes[] = {{16, 4}, {32, 4}, {32, 2}};
 
 bool rows2_precision(int precision) {
@@ -71,8 +72,8 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 }
 
 // Tile copies of the state at `base` (layout [4 fields][nz][ny][nx], storage
-// type of `precision`): a box of ty rows of every field, and one of a single row.
-cudaError_t rows2_maps(const Geometry& g, int precision, int ty, const void* base, CUtensorMap* own,
+// type of `precision`): a box of ty rows of bxc quads of every field, and one of a single row.
+cudaError_t rows2_maps(const Geometry& g, int precision, int bxc, int ty, const void* base, CUtensorMap* own,
                        CUtensorMap* halo) {
   const PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
   if (!encode) return cudaErrorNotSupported;
@@ -83,8 +84,9 @@ cudaError_t rows2_maps(const Geometry& g, int precision, int ty, const void* bas
   const cuuint64_t es = precision == MACLAB_F32 ? 4 : 2;
   const cuuint64_t dims[4] = {(cuuint64_t)g.nx, (cuuint64_t)g.ny, (cuuint64_t)g.nz, 4};
   const cuuint64_t strides[3] = {(cuuint64_t)g.nx * es, (cuuint64_t)g.nx * g.ny * es, (cuuint64_t)g.n * es};
-  const cuuint32_t box_own[4] = {(cuuint32_t)g.nx, (cuuint32_t)ty, 1, 4};
-  const cuuint32_t box_row[4] = {(cuuint32_t)g.nx, 1, 1, 4};
+  const cuuint32_t width = (cuuint32_t)(4 * bxc);
+  const cuuint32_t box_own[4] = {width, (cuuint32_t)ty, 1, 4};
+  const cuuint32_t box_row[4] = {width, 1, 1, 4};
   const cuuint32_t estr[4] = {1, 1, 1, 1};
   void* gp = const_cast<void*>(base);
   if (encode(own, dt, 4, gp, dims, strides, box_own, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -145,9 +147,9 @@ cudaError_t launch_rows2(const StepLaunch& sl, cudaStream_t stream, int ty, int 
   int resident = 0;
   cudaError_t e = dispatch(nullptr, nullptr, dim3(), &resident);
   if (e != cudaSuccess) return e;
-  e = rows2_maps(g, sl.precision, ta.ty, sl.in, &tm_own, &tm_halo);
+  e = rows2_maps(g, sl.precision, s.bxc, ta.ty, sl.in, &tm_own, &tm_halo);
   if (e != cudaSuccess) return e;
-  ta.nzc = fold_chunks(ta.nplanes, ytiles, tz, resident);
+  ta.nzc = fold_chunks(ta.nplanes, ytiles, tz, resident, s.bxc * s.tyt, kRows2Cost);
   ta.px = (g.periodic & 1u) ? 1 : 0;
   ta.py = (g.periodic & 2u) ? 1 : 0;
   ta.pz = (g.periodic & 4u) ? 1 : 0;
@@ -181,9 +183,9 @@ cudaError_t launch_rows2_nu(const Geometry& g, const void* state_n, const void* 
   int resident = 0;
   cudaError_t e = rows2_nu_dispatch(s.bxc, s.tyt, ta, nullptr, nullptr, tm_own, tm_halo, stream, dim3(), &resident);
   if (e != cudaSuccess) return e;
-  e = rows2_maps(g, MACLAB_F32, ta.ty, state_n, &tm_own, &tm_halo);
+  e = rows2_maps(g, MACLAB_F32, s.bxc, ta.ty, state_n, &tm_own, &tm_halo);
   if (e != cudaSuccess) return e;
-  ta.nzc = fold_chunks(ta.nplanes, ytiles, 0, resident);
+  ta.nzc = fold_chunks(ta.nplanes, ytiles, 0, resident, s.bxc * s.tyt, kRows2Cost);
   ta.px = (g.periodic & 1u) ? 1 : 0;
   ta.py = (g.periodic & 2u) ? 1 : 0;
   ta.pz = (g.periodic & 4u) ? 1 : 0;

@@ -7,30 +7,25 @@
 // the destination planes p - 1, p, p + 1 in registers.  What differs:
 //
 //  * Each thread owns the quads of two adjacent rows (r0 = 2 tr, r1 = r0 + 1)
-//    of a tile of TY = 2 TYT rows.  Equilibria moving between its two rows
-//    stay in registers (or go to a neighbouring lane by a warp shuffle when
-//    they also move in x); only those leaving the thread's row pair in y go
-//    through shared memory: half the exchange of one row per thread.  The
-//    terms of one node pair are formed at a time, and each row's x-crossing
-//    values go by shuffle as soon as its two pairs are done, which keeps the
-//    register footprint near what two blocks per SM allow without spilling.
-//  * The y exchange is laid out for the receiver: for each direction and each
-//    receiving thread-row there is one 16-byte unit per column holding the two
-//    values its pairs a and b gather, so a receiver reads a direction with one
-//    16-byte load.  Senders of the diagonal directions write their pair-b (+x)
-//    or pair-a (-x) value into the neighbouring column; at the seam between
-//    the row's halves the lane-swapped value is written, chosen per lane with
-//    selects (no divergent stores).
+//    of a tile of TY = 2 TYT rows, and the update is factored by rows and planes
+//    (d3q19.cuh): what a node sends along x moves to the neighbouring lanes by
+//    shuffles (five values each way and row), what the thread's rows send each
+//    other stays in registers, and only the four values leaving the row pair
+//    upwards and the four leaving it downwards go through shared memory, one
+//    16-byte unit per column and value, at the sender's own column.
+//  * Between planes a thread keeps four sums of the plane about to be completed
+//    and three of what the last plane sent on.
 //  * The halo rows next to the tile are loaded by the first and last
-//    thread-rows, which publish the halo's inward equilibria into the same
-//    exchange units a neighbouring thread-row would have filled: every thread
-//    then gathers the same way, with no branch on its position.
-//  * Terms of Eq. (2) per node: B_i = 3 rho u_i, P_ii = 3/2 B_i u_i,
-//    A = drho - (P_xx + P_yy + P_zz) / 3, S_i = A + P_ii, and for each axis
-//    pair (i, j) the sums S_i + P_jj +- 3 B_i u_j and B_i +- B_j.  A direction
-//    along an axis has T = S_i +- B_i and is added with its integer weight 2 by
-//    a fused multiply-add; the rest direction adds 12 A; the diagonals add 1 T.
-//    The sums are R = 36 drho' and M = 36 m', u' = M / (36 + R) + F.
+//    thread-rows, which publish what they send into the tile in the units a
+//    neighbouring thread-row would have filled: every thread then gathers the
+//    same way, with no branch on its position.
+//  * Measured at 128^3 (FP32 cavity): 14.3 us a step, 7.1 M warp instructions,
+//    213 registers, where forming the nineteen terms took 15.2 us, 7.8 M and 253.
+//    With the whole update replaced by a copy of the staged quads it takes 7.8
+//    us: neither memory nor issue (42 %) bounds it but the plane's chain of
+//    dependent operations, at two 128-thread blocks per SM; a lone block takes
+//    1.0 us a plane, two together 1.45.  A fifth warp for the halo rows leaves
+//    168 registers per thread (three warps on one scheduler) and spills: 19.5 us.
 //  * Box x-walls: the lanes holding x = 0 or x = nx - 1 store the wall node's
 //    unchanged values in place of the computed ones, with selects, so every
 //    lane stores whole quads.  The values come from the staged plane: when a
@@ -56,160 +51,10 @@
 // maclab_adjoint_nu_term, per node as in adj_nu_term).
 
 #pragma once
+#include "d3q19.cuh"
 #include "step_fold.cuh"
 
 namespace maclab {
-
-// ------------------------------------------------------------------ terms
-
-template <typename C>
-struct Terms3 {
-  using P = typename Pair<C>::P;
-  P A;      // drho - 3/2 rho u.u
-  P B[3];   // 3 rho u_i
-  P S[3];   // A + 9/2 rho u_i^2
-  P Ep[3], Em[3];  // pair k = (i, j): S_i + 9/2 rho u_j^2 +- 9 rho u_i u_j
-  P Op[3], Om[3];  // B_i +- B_j
-};
-
-template <typename C>
-__device__ __forceinline__ void make_terms3(typename Pair<C>::P r, const typename Pair<C>::P (&u)[3],
-                                            Terms3<C>& t) {
-  using O = Pair<C>;
-  using P = typename O::P;
-  const P g = O::fma(r, O::splat(C(3)), O::splat(C(3)));  // 3 (1 + drho)
-  P Pd[3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    t.B[i] = O::mul(g, u[i]);
-    Pd[i] = O::mul(O::mul(t.B[i], u[i]), O::splat(C(1.5)));
-  }
-  const P psum = O::add(O::add(Pd[0], Pd[1]), Pd[2]);
-  t.A = O::fma(psum, O::splat(C(-1.0 / 3.0)), r);
-#pragma unroll
-  for (int i = 0; i < 3; ++i) t.S[i] = O::add(t.A, Pd[i]);
-  // 9 rho u_i u_j = (3 B_i) u_j, formed inside the fused multiply-adds
-  const P B30 = O::mul(t.B[0], O::splat(C(3)));
-  const P B31 = O::mul(t.B[1], O::splat(C(3)));
-  const P nu1 = O::sub(O::splat(C(0)), u[1]);
-  const P nu2 = O::sub(O::splat(C(0)), u[2]);
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = i + 1; j < 3; ++j) {
-      const int k = pair_index(i, j);
-      const P base = O::add(t.S[i], Pd[j]);
-      const P b3 = i == 0 ? B30 : B31;
-      t.Ep[k] = O::fma(b3, u[j], base);
-      t.Em[k] = O::fma(b3, j == 1 ? nu1 : nu2, base);
-      t.Op[k] = O::add(t.B[i], t.B[j]);
-      t.Om[k] = O::sub(t.B[i], t.B[j]);
-    }
-}
-
-// Terms of g_a / w_a = drho + rho (3/2 u.u - 9/2 (c.u)^2) in the same slots:
-// A = drho + 3/2 rho u.u, S_i = A - 9/2 rho u_i^2, and for the pair (i, j)
-// Ep = S_i - 9/2 rho u_j^2 - 9 rho u_i u_j, Em = ... + 9 rho u_i u_j; no B, O.
-template <typename C>
-__device__ __forceinline__ void make_terms3_nu(typename Pair<C>::P r, const typename Pair<C>::P (&u)[3],
-                                               Terms3<C>& t) {
-  using O = Pair<C>;
-  using P = typename O::P;
-  const P g = O::fma(r, O::splat(C(3)), O::splat(C(3)));  // 3 (1 + drho)
-  P B[3], Pd[3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    B[i] = O::mul(g, u[i]);
-    Pd[i] = O::mul(O::mul(B[i], u[i]), O::splat(C(1.5)));  // 9/2 rho u_i^2
-  }
-  const P psum = O::add(O::add(Pd[0], Pd[1]), Pd[2]);
-  t.A = O::fma(psum, O::splat(C(1.0 / 3.0)), r);
-#pragma unroll
-  for (int i = 0; i < 3; ++i) t.S[i] = O::sub(t.A, Pd[i]);
-  const P B30 = O::mul(B[0], O::splat(C(3)));
-  const P B31 = O::mul(B[1], O::splat(C(3)));
-  const P nu1 = O::sub(O::splat(C(0)), u[1]);
-  const P nu2 = O::sub(O::splat(C(0)), u[2]);
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = i + 1; j < 3; ++j) {
-      const int k = pair_index(i, j);
-      const P base = O::sub(t.S[i], Pd[j]);
-      const P b3 = i == 0 ? B30 : B31;
-      t.Ep[k] = O::fma(b3, j == 1 ? nu1 : nu2, base);
-      t.Em[k] = O::fma(b3, u[j], base);
-    }
-}
-
-// T_a of both lanes (axis directions undoubled: they carry the weight 2)
-template <typename C, int A, bool NU = false>
-__device__ __forceinline__ typename Pair<C>::P term3(const Terms3<C>& t) {
-  using L = Lattice<kD3Q19>;
-  using O = Pair<C>;
-  constexpr int nzc = Dir<kD3Q19>::nz(A);
-  constexpr int i0 = Dir<kD3Q19>::first(A), i1 = Dir<kD3Q19>::second(A);
-  if constexpr (nzc == 0) {
-    return t.A;
-  } else if constexpr (nzc == 1) {
-    if constexpr (NU) return t.S[i0];
-    else if constexpr (L::c(A, i0) > 0) return O::add(t.S[i0], t.B[i0]);
-    else return O::sub(t.S[i0], t.B[i0]);
-  } else {
-    constexpr int k = pair_index(i0, i1);
-    constexpr int s0 = L::c(A, i0), s1 = L::c(A, i1);
-    if constexpr (NU) {
-      return s0 == s1 ? t.Ep[k] : t.Em[k];
-    } else if constexpr (s0 == s1) {
-      if constexpr (s0 > 0) return O::add(t.Ep[k], t.Op[k]);
-      else return O::sub(t.Ep[k], t.Op[k]);
-    } else {
-      if constexpr (s0 > 0) return O::add(t.Em[k], t.Om[k]);
-      else return O::sub(t.Em[k], t.Om[k]);
-    }
-  }
-}
-
-// Constants of the weighted sums, held in registers once.
-template <typename C>
-struct Weights3 {
-  using P = typename Pair<C>::P;
-  P w12, w2, wm2;
-};
-
-// acc[0] += w36 T; acc[1 + i] += c_i w36 T
-template <typename C, int A>
-__device__ __forceinline__ void accum3(typename Pair<C>::P (&acc)[4], typename Pair<C>::P T,
-                                       const Weights3<C>& w) {
-  using L = Lattice<kD3Q19>;
-  using O = Pair<C>;
-  constexpr int wt = L::w36(A);
-  if constexpr (wt == 1) {
-    acc[0] = O::add(acc[0], T);
-    static_for<0, 3>([&](auto I) {
-      constexpr int i = decltype(I)::value;
-      if constexpr (L::c(A, i) == 1) acc[1 + i] = O::add(acc[1 + i], T);
-      else if constexpr (L::c(A, i) == -1) acc[1 + i] = O::sub(acc[1 + i], T);
-    });
-  } else if constexpr (wt == 2) {
-    acc[0] = O::fma(w.w2, T, acc[0]);
-    static_for<0, 3>([&](auto I) {
-      constexpr int i = decltype(I)::value;
-      if constexpr (L::c(A, i) == 1) acc[1 + i] = O::fma(w.w2, T, acc[1 + i]);
-      else if constexpr (L::c(A, i) == -1) acc[1 + i] = O::fma(w.wm2, T, acc[1 + i]);
-    });
-  } else {
-    acc[0] = O::fma(w.w12, T, acc[0]);
-  }
-}
-
-// index of direction a among the five with the same c_y (c_y != 0)
-__host__ __device__ constexpr int rows2_ykey(int a) {
-  using F = Frame<kD3Q19>;
-  int k = 0;
-  for (int b = 0; b < a; ++b) k += F::fy(b) == F::fy(a) ? 1 : 0;
-  return k;
-}
 
 // ------------------------------------------------------------------ layout
 
@@ -217,15 +62,14 @@ template <typename S, int BXC, int TYT>
 struct Rows2Layout {
   static constexpr int TY = 2 * TYT;
   static constexpr int RS = TY + 2;       // staged rows: lower halo, TY own, upper halo
-  static constexpr int YC = BXC + 1;      // units per slot row (+1: the idle lanes' column)
   static constexpr int NSLOT = TYT + 1;   // receiving rows per sign (see step_rows2)
-  static constexpr int DIR_UNITS = NSLOT * YC;
-  static constexpr int SIGN_UNITS = 5 * DIR_UNITS;
+  static constexpr int VAL_UNITS = NSLOT * BXC;
+  static constexpr int SIGN_UNITS = 4 * VAL_UNITS;  // G, H, T of c_z = +1 and -1
   static constexpr int BUF_UNITS = 2 * SIGN_UNITS;
   static constexpr size_t y_bytes = (size_t)2 * BUF_UNITS * 16;  // two buffers of 16-byte units
   // a stage slot: the TY own rows [4 fields][TY][row], then the halo rows
   // below and above, [4 fields][row] each, as the tile copies lay them out
-  // (a row is nx stored values); offsets are multiples of 128 bytes
+  // (BXC quads a row); offsets are multiples of 128 bytes
   static constexpr size_t QB = (size_t)BXC * Quad<S>::BYTES;  // the widest row
   static constexpr size_t slot_bytes = 4 * RS * QB;
   static constexpr size_t halo_lo = 4 * TY * QB;
@@ -260,6 +104,12 @@ struct Rows2Sum {
   }
 };
 
+// Whether value k (G, H, T of c_z = +1, T of c_z = -1) crosses rows in this mode.
+template <int MODE>
+__host__ __device__ constexpr bool rows2_sends(int k) {
+  return k < 2 ? MODE == kMid : k == 2 ? MODE != kLast : MODE != kFirst;
+}
+
 // NU: viscosity-term mode (see the top of this file); `out` is then the state
 // after the step, read only.
 // Tile copies: tm_own maps the state as [4 fields][nz][ny][nx] with a box of the
@@ -274,11 +124,7 @@ __global__ void __launch_bounds__(BXC * TYT, Rows2Layout<S, BXC, TYT>::MIN_BLOCK
   using C = float;
   using O = Pair<C>;
   using P = typename O::P;
-  using L = Lattice<kD3Q19>;
-  using F = Frame<kD3Q19>;
   constexpr int TY = Lay::TY;
-  constexpr int RS = Lay::RS;
-  constexpr int YC = Lay::YC;
   extern __shared__ __align__(128) unsigned char smem_dyn[];
   // stage slots at a 128-byte boundary (tile copies land on it), then the
   // mbarriers, then the y exchange
@@ -301,13 +147,8 @@ __global__ void __launch_bounds__(BXC * TYT, Rows2Layout<S, BXC, TYT>::MIN_BLOCK
   const bool active = tx < bxr;
   float4* const Y = reinterpret_cast<float4*>(smem_raw + Lay::y_off);
 
-  // columns: own, the right neighbour's (the unit a +x diagonal value goes to)
-  // and the left one's (-x); idle lanes write into the spare column BXC
-  const int col = tx;
-  const int col_r = !active ? BXC : (tx + 1 == bxr ? 0 : tx + 1);
-  const int col_l = !active ? BXC : (tx == 0 ? bxr - 1 : tx - 1);
-  const bool seam_r = tx == bxr - 1;  // +x across the seam: send lane-swapped
-  const bool seam_l = tx == 0;        // -x across the seam
+  const bool seam_r = tx == bxr - 1;  // right neighbour across the seam: its lanes swapped
+  const bool seam_l = tx == 0;        // left neighbour across the seam
   // shuffle sources and lane swaps of the x exchange (width BXC)
   const int src_l = tx == 0 ? bxr - 1 : tx - 1;
   const int src_r = tx == bxr - 1 ? 0 : tx + 1;
@@ -318,12 +159,11 @@ __global__ void __launch_bounds__(BXC * TYT, Rows2Layout<S, BXC, TYT>::MIN_BLOCK
   const int first_row = blockIdx.y * TY;  // rows before it are the previous tile's
   const int tile_row0 = RM == kRowsPlain ? first_row : min(first_row, ta.ny - TY);
   const int row0 = tile_row0 + 2 * tr;
-  int halo = tr == 0 ? 1 : (tr == TYT - 1 ? -1 : 0);
-  {
-    const int hrow = halo == 1 ? row0 - 1 : row0 + 2;
-    if (halo != 0 && (hrow < 0 || hrow >= ta.ny) && !ta.py)
-      halo = 0;  // beyond a closed y boundary: the row next to it is a wall row
-  }
+  const int halo = tr == 0 ? 1 : (tr == TYT - 1 ? -1 : 0);
+  // whether some thread of the warp has a halo row: its shuffles take the whole
+  // warp.  (Beyond a closed y boundary the values are of no row; the row next to
+  // it is a wall row and keeps its values.)
+  const bool warp_halo = BXC >= 32 ? halo != 0 : true;
   bool row_wall[2];  // not stored: a wall row, or the previous tile's
   row_wall[0] = (!ta.py && row0 == 0) || (RM != kRowsPlain && row0 < first_row);
   row_wall[1] = (!ta.py && row0 + 1 == ta.ny - 1) || (RM != kRowsPlain && row0 + 1 < first_row);
@@ -340,18 +180,12 @@ __global__ void __launch_bounds__(BXC * TYT, Rows2Layout<S, BXC, TYT>::MIN_BLOCK
   float* const WV = reinterpret_cast<float*>(smem_raw + Lay::wall_off);
   auto wall_slot = [&](int parity) { return ((parity * TYT + tr) * 2 + (x_hi_wall ? 1 : 0)) * 8; };
 
-  S* op[4];
-#pragma unroll
-  for (int f = 0; f < 4; ++f) op[f] = out + (int64_t)f * ta.n + row_off;
+  // field f of this thread's quad in row j of plane 0: out + f * n + row_off + j * nx
+  S* const op0 = out + row_off;
   const uint8_t* mrow = ta.wall_mode == kWallMask ? ta.mask + row_off : nullptr;
   P force[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) force[i] = O::splat(C(ta.force[i]));
-  Weights3<C> wts;
-  wts.w12 = O::splat(C(12));
-  wts.w2 = O::splat(C(2));
-  wts.wm2 = O::splat(C(-2));
-
   const int z0 = (int)(((int64_t)blockIdx.x * ta.nplanes) / ta.nzc);
   const int z1 = (int)(((int64_t)(blockIdx.x + 1) * ta.nplanes) / ta.nzc);
   const int64_t ps = ta.plane_stride;
@@ -361,12 +195,13 @@ __global__ void __launch_bounds__(BXC * TYT, Rows2Layout<S, BXC, TYT>::MIN_BLOCK
   const bool zwall = !ta.pz;
 
   // stage slots (Lay): own row j of this thread at row 2 tr + j of the own
-  // block, the halo row below or above in its block; rows are nx values
-  // (rowB bytes) as the tile copies write them
+  // block, the halo row below or above in its block; the tile copies write rows
+  // of BXC quads (what lies beyond the end of a row is filled with zeros), so
+  // every offset in a slot is a constant
   constexpr int QW = Quad<S>::BYTES;
   static_assert(kStages == 2, "two stage slots, two mbarriers");
-  const uint32_t rowB = (uint32_t)bxr * QW;
-  const uint32_t fieldB = (uint32_t)TY * rowB;  // own block: [4 fields][TY rows]
+  constexpr uint32_t rowB = (uint32_t)Lay::QB;
+  constexpr uint32_t fieldB = (uint32_t)TY * rowB;  // own block: [4 fields][TY rows]
   const uint32_t own_off = (uint32_t)(2 * tr) * rowB + (uint32_t)tx * QW;
   const uint32_t halo_off = (uint32_t)(halo == 1 ? Lay::halo_lo : Lay::halo_hi) + (uint32_t)tx * QW;
   const uint32_t stage_sh = smem_u32(smem_raw);
@@ -407,203 +242,216 @@ __global__ void __launch_bounds__(BXC * TYT, Rows2Layout<S, BXC, TYT>::MIN_BLOCK
       mbar_arrive(bar);
     }
   };
-  P st[2][4][2];
   const unsigned char* slot_base = smem_raw;
-  auto take = [&](int i) {
-    const int p = z0 - 1 + i;
+  int slot_parity = 0;
+  auto take = [&](int i) {  // wait for plane z0 - 1 + i
     const uint32_t s = (uint32_t)(i & 1);
     if (!mbar_wait(mbar0 + 8 * s, (uint32_t)(i >> 1) & 1u) && ta.status) atomicOr(ta.status, 1u);
-    const bool ok = active && plane_exists(p);
     slot_base = smem_raw + (size_t)s * Lay::slot_bytes;
+    slot_parity = i & 1;
+  };
+  // a quad of the plane taken, at byte `off` of its field 0 and fields `stride` apart
+  auto quad = [&](P(&v)[4][2], uint32_t off, uint32_t stride) {
 #pragma unroll
-    for (int j = 0; j < 2; ++j)
-#pragma unroll
-      for (int f = 0; f < 4; ++f) {
-        const int64_t b = (int64_t)s * Lay::slot_bytes + own_off + j * rowB + f * fieldB;
-        if (ok && bounds_ok(ta.bounds, b, (int64_t)Lay::stage_bytes - QW + 1)) {
-          Quad<S>::lds(reinterpret_cast<const S*>(smem_raw + b), st[j][f][0], st[j][f][1]);
-        } else {
-          st[j][f][0] = st[j][f][1] = O::splat(C(0));
-        }
+    for (int f = 0; f < 4; ++f) {
+      const int64_t b = (int64_t)(slot_base - smem_raw) + off + f * stride;
+      if (bounds_ok(ta.bounds, b, (int64_t)Lay::stage_bytes - QW + 1)) {
+        Quad<S>::lds(reinterpret_cast<const S*>(smem_raw + b), v[f][0], v[f][1]);
+      } else {
+        v[f][0] = v[f][1] = O::splat(C(0));
       }
-    if (keep_walls) {
-      const int w = wall_slot(i & 1);
-#pragma unroll
-      for (int j = 0; j < 2; ++j)
-#pragma unroll
-        for (int f = 0; f < 4; ++f)
-          if (bounds_ok(ta.bounds, w + 4 * j + f, (int64_t)(Lay::wall_bytes / sizeof(float))))
-            WV[w + 4 * j + f] = x_lo_wall ? st[j][f][0].x : (RM == kRowsOdd ? st[j][f][0].y : st[j][f][1].y);
     }
   };
 
   // ---------------------------------------------------------------- one plane
+  // a value of the lane holding the node pair at x - 1 / x + 1
+  auto from_left = [&](P v) {
+    v = fold_shfl<BXC>(v, src_l);
+    return seam_l ? O::swap(v) : v;
+  };
+  auto from_right = [&](P v) {
+    v = fold_shfl<BXC>(v, src_r);
+    return seam_r ? O::swap(v) : v;
+  };
+  // Sums of plane p - 1 (cur: R, M_x, M_y, M_z) and what plane p - 1 sent on to
+  // plane p (next: R = M_z, M_x, M_y), of [row][pair].
+  P cur[2][2][4] = {}, next[2][2][3] = {};
   int ybuf = 0;
-  // publish the equilibria of pair values (Ta, Tb) of direction A into the
-  // units of slot row `slot` of sign FY (receivers: the thread-row that owns
-  // that slot)
-  auto publish = [&](float4* ybase, auto dir, int slot, P Ta, P Tb) {
-    constexpr int A = decltype(dir)::value;
-    constexpr int FY = F::fy(A), FX = F::fx(A);
-    float4* const u = ybase + (FY == 1 ? 0 : Lay::SIGN_UNITS) + rows2_ykey(A) * Lay::DIR_UNITS + slot * YC;
-    auto unit_ok = [&](int c) { return bounds_ok(ta.bounds, (u + c) - Y, 2 * Lay::BUF_UNITS); };
-    if constexpr (FX == 0) {
-      if (unit_ok(col)) u[col] = make_float4(Ta.x, Ta.y, Tb.x, Tb.y);
-    } else if constexpr (FX == 1) {
-      // receiver column c gathers (left neighbour's b, own a)
-      if (unit_ok(col)) reinterpret_cast<float2*>(u + col)[1] = Ta;
-      const P b = seam_r ? O::swap(Tb) : Tb;
-      if (unit_ok(col_r)) reinterpret_cast<float2*>(u + col_r)[0] = b;
-    } else {
-      // receiver column c gathers (own b, right neighbour's a)
-      if (unit_ok(col)) reinterpret_cast<float2*>(u + col)[0] = Tb;
-      const P a = seam_l ? O::swap(Ta) : Ta;
-      if (unit_ok(col_l)) reinterpret_cast<float2*>(u + col_l)[1] = a;
-    }
+  auto unit = [&](float4* ybase, int sign, int val, int slot) {
+    float4* const u = ybase + sign * Lay::SIGN_UNITS + val * Lay::VAL_UNITS + slot * BXC + tx;
+    return bounds_ok(ta.bounds, u - Y, 2 * Lay::BUF_UNITS) ? u : nullptr;
+  };
+  auto publish = [&](float4* ybase, int sign, int val, int slot, P a, P b) {
+    if (float4* const u = unit(ybase, sign, val, slot)) *u = make_float4(a.x, a.y, b.x, b.y);
+  };
+  auto receive = [&](float4* ybase, int sign, int val, int slot, P(&v)[2]) {
+    float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (const float4* const u = unit(ybase, sign, val, slot)) t = *u;
+    v[0] = O::make(t.x, t.y);
+    v[1] = O::make(t.z, t.w);
   };
 
-  // the value of one pair (q) of direction A into its half of the receiver's unit
-  auto publish_half = [&](float4* ybase, auto dir, auto qc, int slot, P T) {
-    constexpr int A = decltype(dir)::value;
-    constexpr int q = decltype(qc)::value;
-    constexpr int FY = F::fy(A), FX = F::fx(A);
-    float4* const u = ybase + (FY == 1 ? 0 : Lay::SIGN_UNITS) + rows2_ykey(A) * Lay::DIR_UNITS + slot * YC;
-    auto unit_ok = [&](int c) { return bounds_ok(ta.bounds, (u + c) - Y, 2 * Lay::BUF_UNITS); };
-    if constexpr (FX == 0) {
-      if (unit_ok(col)) reinterpret_cast<float2*>(u + col)[q] = T;
-    } else if constexpr (FX == 1) {
-      if constexpr (q == 0) {
-        if (unit_ok(col)) reinterpret_cast<float2*>(u + col)[1] = T;
-      } else {
-        const P b = seam_r ? O::swap(T) : T;
-        if (unit_ok(col_r)) reinterpret_cast<float2*>(u + col_r)[0] = b;
-      }
-    } else {
-      if constexpr (q == 1) {
-        if (unit_ok(col)) reinterpret_cast<float2*>(u + col)[0] = T;
-      } else {
-        const P a = seam_l ? O::swap(T) : T;
-        if (unit_ok(col_l)) reinterpret_cast<float2*>(u + col_l)[1] = a;
-      }
-    }
-  };
-  auto update = [&](auto mode, P(&ap)[2][2][4], P(&ac)[2][2][4], P(&an)[2][2][4]) {
+  // Source plane p: completes cur (plane p - 1), which stays for the store, and
+  // leaves plane p's own sums in `own` and what it sends on in `next`.
+  auto update = [&](auto mode, P(&own)[2][2][4]) {
     constexpr int MODE = decltype(mode)::value;
-    const int ybuf_units = ybuf * Lay::BUF_UNITS;
-    float4* const ybase = Y + ybuf_units;
+    constexpr bool kUp = MODE != kLast, kDown = MODE != kFirst, kOwn = MODE == kMid;
+    float4* const ybase = Y + ybuf * Lay::BUF_UNITS;
     ybuf ^= 1;
-    // one pair at a time (terms of one pair live at once); each row's x-crossing
-    // values go by shuffle as soon as the row is done
-    auto shuffle_in = [&](auto dir, auto jdc, P vb_or_va) {
-      constexpr int a = decltype(dir)::value;
-      constexpr int jd = decltype(jdc)::value;
-      constexpr int fx = F::fx(a), fz = F::fz(a);
-      auto& dst = pick<fz>(ap, ac, an)[jd];
-      if constexpr (fx == 1) {
-        P v = fold_shfl<BXC>(vb_or_va, src_l);
-        if (seam_l) v = O::swap(v);
-        accum3<C, a>(dst[0], v, wts);
-      } else {
-        P v = fold_shfl<BXC>(vb_or_va, src_r);
-        if (seam_r) v = O::swap(v);
-        accum3<C, a>(dst[1], v, wts);
+    P down[2][2] = {};  // R of what goes to plane p - 1 (its M_z: the negative)
+    P link[4][2] = {};  // what the lower row gets from the upper one
+    // the row below (SIGN 1) or above (-1) adds (g, h, t of c_z = +1, t of c_z = -1)
+    auto add_row = [&](auto signc, int j, int q, P g, P h, P tp, P tm) {
+      constexpr int SIGN = decltype(signc)::value;
+      auto signed_add = [](P x, P y) { return SIGN > 0 ? O::add(x, y) : O::sub(x, y); };
+      if constexpr (kOwn) {
+        own[j][q][0] = O::add(own[j][q][0], g);
+        own[j][q][1] = O::add(own[j][q][1], h);
+        own[j][q][2] = signed_add(own[j][q][2], g);
+      }
+      if constexpr (kDown) {
+        down[j][q] = O::add(down[j][q], tm);
+        cur[j][q][2] = signed_add(cur[j][q][2], tm);
+      }
+      if constexpr (kUp) {
+        next[j][q][0] = O::add(next[j][q][0], tp);
+        next[j][q][2] = SIGN > 0 ? tp : O::sub(next[j][q][2], tp);
       }
     };
+    using Below = std::integral_constant<int, 1>;
+    using Above = std::integral_constant<int, -1>;
+    P up0[4][2] = {};   // what the upper row gets from the lower one
     static_for<0, 2>([&](auto jc) {
       constexpr int j = decltype(jc)::value;
-      constexpr int jd = 1 - j;
-      P xb[4], xa[4];  // [k]: k < 3 own c_y = 0 directions, 3: the diagonal into row jd
+      P st[4][2];
+      quad(st, own_off + j * rowB, fieldB);
+      if (keep_walls) {
+        const int w = wall_slot(slot_parity) + 4 * j;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) xb[k] = xa[k] = O::splat(C(0));
+        for (int f = 0; f < 4; ++f)
+          if (bounds_ok(ta.bounds, w + f, (int64_t)(Lay::wall_bytes / sizeof(float))))
+            WV[w + f] = x_lo_wall ? st[f][0].x : (RM == kRowsOdd ? st[f][0].y : st[f][1].y);
+      }
+      const D3Node<C> a = d3_node<C, NU>(st[0][0], st[1][0], st[2][0], st[3][0]);
+      const D3Node<C> b = d3_node<C, NU>(st[0][1], st[1][1], st[2][1], st[3][1]);
+      D3Node<C> l, r;  // the neighbouring lanes' pair b and pair a
+      l.ap = from_left(b.ap);
+      l.bp = from_left(b.bp);
+      l.dp = from_left(b.dp);
+      l.e = from_left(b.e);
+      l.f = from_left(b.f);
+      r.am = from_right(a.am);
+      r.bm = from_right(a.bm);
+      r.dm = from_right(a.dm);
+      r.e = from_right(a.e);
+      r.f = from_right(a.f);
+      P send[2][4][2];  // [below, above] of the values for the row above / below
       static_for<0, 2>([&](auto qc) {
         constexpr int q = decltype(qc)::value;
-        Terms3<C> t;
-        {
-          const P u[3] = {st[j][1][q], st[j][2][q], st[j][3][q]};
-          if constexpr (NU) make_terms3_nu<C>(st[j][0][q], u, t);
-          else make_terms3<C>(st[j][0][q], u, t);
+        const D3Node<C>& n = q == 0 ? a : b;
+        const D3Row<C> w = q == 0 ? d3_row<C, NU>(a, l, b) : d3_row<C, NU>(b, a, r);
+        if constexpr (kDown) {
+          down[j][q] = w.km;
+          cur[j][q][1] = O::add(cur[j][q][1], w.xm);
         }
-        static_for<0, L::Q>([&](auto I) {
-          constexpr int a = decltype(I)::value;
-          if constexpr (mode_allows<kD3Q19, MODE>(a)) {
-            constexpr int fx = F::fx(a), fy = F::fy(a), fz = F::fz(a);
-            const P T = term3<C, a, NU>(t);
-            if constexpr (fy == 0) {
-              auto& dst = pick<fz>(ap, ac, an)[j];
-              constexpr int qd = q + fx;
-              if constexpr (qd >= 0 && qd < 2) accum3<C, a>(dst[qd], T, wts);
-              else if constexpr (fx == 1) xb[fold_xidx(a)] = T;
-              else xa[fold_xidx(a)] = T;
-            } else if constexpr ((j == 0 && fy == 1) || (j == 1 && fy == -1)) {
-              auto& dst = pick<fz>(ap, ac, an)[jd];
-              constexpr int qd = q + fx;
-              if constexpr (qd >= 0 && qd < 2) accum3<C, a>(dst[qd], T, wts);
-              else if constexpr (fx == 1) xb[3] = T;
-              else xa[3] = T;
-            } else {
-              publish_half(ybase, I, qc, j == 1 ? tr + 1 : tr, T);
-            }
+        if constexpr (kOwn) {
+          own[j][q][0] = O::fma(n.A, O::splat(C(12)), O::fma(w.sA, O::splat(C(2)), next[j][q][0]));
+          own[j][q][1] = O::fma(w.dA, O::splat(C(2)), next[j][q][1]);
+          own[j][q][2] = next[j][q][2];
+          own[j][q][3] = next[j][q][0];
+        }
+        if constexpr (kUp) {
+          next[j][q][0] = w.kp;
+          next[j][q][1] = w.xp;
+        }
+        send[0][0][q] = w.gp;
+        send[0][1][q] = w.hp;
+        send[0][2][q] = n.tpp;
+        send[0][3][q] = n.tpm;
+        send[1][0][q] = w.gm;
+        send[1][1][q] = w.hm;
+        send[1][2][q] = n.tmp;
+        send[1][3][q] = n.tmm;
+      });
+      static_for<0, 4>([&](auto kc) {
+        constexpr int k = decltype(kc)::value;
+        if constexpr (rows2_sends<MODE>(k)) {
+          if constexpr (j == 0) {
+            publish(ybase, 1, k, tr, send[1][k][0], send[1][k][1]);  // to the thread-row below
+            up0[k][0] = send[0][k][0];
+            up0[k][1] = send[0][k][1];
+          } else {
+            publish(ybase, 0, k, tr + 1, send[0][k][0], send[0][k][1]);  // to the thread-row above
+            link[k][0] = send[1][k][0];
+            link[k][1] = send[1][k][1];
           }
-        });
+        }
       });
-      static_for<0, L::Q>([&](auto I) {
-        constexpr int a = decltype(I)::value;
-        constexpr int fx = F::fx(a), fy = F::fy(a), fz = F::fz(a);
-        if constexpr (mode_allows<kD3Q19, MODE>(a) && fy == 0 && fx != 0)
-          shuffle_in(I, jc, fx == 1 ? xb[fold_xidx(a)] : xa[fold_xidx(a)]);
-        if constexpr (mode_allows<kD3Q19, MODE>(a) && fz == 0 && fx != 0 &&
-                      ((j == 0 && fy == 1) || (j == 1 && fy == -1)))
-          shuffle_in(I, std::integral_constant<int, jd>{}, fx == 1 ? xb[3] : xa[3]);
-      });
+      if constexpr (j == 1) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) add_row(Below{}, 1, q, up0[0][q], up0[1][q], up0[2][q], up0[3][q]);
+      }
     });
-    // ---- halo row: its inward equilibria into the slot its neighbour reads
-    if (halo != 0) {  // idle lanes publish into their own or the spare column
-      P hs[4][2];
-      const int64_t hb = (int64_t)(slot_base - smem_raw) + halo_off;
-#pragma unroll
-      for (int f = 0; f < 4; ++f) {
-        if (bounds_ok(ta.bounds, hb + f * rowB, (int64_t)Lay::stage_bytes - QW + 1))
-          Quad<S>::lds(reinterpret_cast<const S*>(smem_raw + hb + f * rowB), hs[f][0], hs[f][1]);
-        else
-          hs[f][0] = hs[f][1] = O::splat(C(0));
+    // ---- halo row: what it sends into the tile.  The row above the tile is the
+    // mirror image in y of the row below it: with u_y negated it sends upwards
+    // what it sends downwards.
+    if (warp_halo) {
+      P st[4][2];
+      quad(st, halo_off, rowB);
+      if (halo == -1) {
+        st[2][0] = O::sub(O::splat(C(0)), st[2][0]);
+        st[2][1] = O::sub(O::splat(C(0)), st[2][1]);
       }
-      Terms3<C> t[2];
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const P u[3] = {hs[1][q], hs[2][q], hs[3][q]};
-        if constexpr (NU) make_terms3_nu<C>(hs[0][q], u, t[q]);
-        else make_terms3<C>(hs[0][q], u, t[q]);
+      const D3Node<C> a = d3_node<C, NU>(st[0][0], st[1][0], st[2][0], st[3][0]);
+      const D3Node<C> b = d3_node<C, NU>(st[0][1], st[1][1], st[2][1], st[3][1]);
+      const int sign = halo == 1 ? 0 : 1, slot = halo == 1 ? 0 : TYT;
+      if constexpr (kOwn) {
+        D3Node<C> l = a, r = b;
+        l.ap = from_left(b.ap);
+        l.bp = from_left(b.bp);
+        l.e = from_left(b.e);
+        r.am = from_right(a.am);
+        r.bm = from_right(a.bm);
+        r.e = from_right(a.e);
+        const D3Row<C> wa = d3_row<C, NU>(a, l, b), wb = d3_row<C, NU>(b, a, r);
+        if (halo != 0) {
+          publish(ybase, sign, 0, slot, wa.gp, wb.gp);
+          publish(ybase, sign, 1, slot, wa.hp, wb.hp);
+        }
       }
-      if (halo == 1) {
-        static_for<0, L::Q>([&](auto I) {
-          constexpr int a = decltype(I)::value;
-          if constexpr (mode_allows<kD3Q19, MODE>(a) && F::fy(a) == 1)
-            publish(ybase, I, 0, term3<C, a, NU>(t[0]), term3<C, a, NU>(t[1]));
-        });
-      } else {
-        static_for<0, L::Q>([&](auto I) {
-          constexpr int a = decltype(I)::value;
-          if constexpr (mode_allows<kD3Q19, MODE>(a) && F::fy(a) == -1)
-            publish(ybase, I, TYT, term3<C, a, NU>(t[0]), term3<C, a, NU>(t[1]));
-        });
+      if (halo != 0) {
+        if constexpr (kUp) publish(ybase, sign, 2, slot, a.tpp, b.tpp);
+        if constexpr (kDown) publish(ybase, sign, 3, slot, a.tpm, b.tpm);
       }
     }
     __syncthreads();
-    // ---- gather: row 0 the +y units of slot tr, row 1 the -y units of slot tr + 1
-    static_for<0, L::Q>([&](auto I) {
-      constexpr int a = decltype(I)::value;
-      constexpr int fy = F::fy(a), fz = F::fz(a);
-      if constexpr (mode_allows<kD3Q19, MODE>(a) && fy != 0) {
-        constexpr int j = fy == 1 ? 0 : 1;
-        const int slot = fy == 1 ? tr : tr + 1;
-        const int64_t unit = (int64_t)ybuf_units + (fy == 1 ? 0 : Lay::SIGN_UNITS) + rows2_ykey(a) * Lay::DIR_UNITS +
-                             slot * YC + col;
-        const float4 v = bounds_ok(ta.bounds, unit, 2 * Lay::BUF_UNITS) ? Y[unit] : make_float4(0.f, 0.f, 0.f, 0.f);
-        auto& dst = pick<fz>(ap, ac, an)[j];
-        accum3<C, a>(dst[0], O::make(v.x, v.y), wts);
-        accum3<C, a>(dst[1], O::make(v.z, v.w), wts);
-      }
+    P v[4][2];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k][0] = v[k][1] = O::splat(C(0));
+    static_for<0, 4>([&](auto kc) {
+      constexpr int k = decltype(kc)::value;
+      if constexpr (rows2_sends<MODE>(k)) receive(ybase, 0, k, tr, v[k]);
     });
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      add_row(Below{}, 0, q, v[0][q], v[1][q], v[2][q], v[3][q]);
+      add_row(Above{}, 0, q, link[0][q], link[1][q], link[2][q], link[3][q]);
+    }
+    static_for<0, 4>([&](auto kc) {
+      constexpr int k = decltype(kc)::value;
+      if constexpr (rows2_sends<MODE>(k)) receive(ybase, 1, k, tr + 1, v[k]);
+    });
+#pragma unroll
+    for (int q = 0; q < 2; ++q) add_row(Above{}, 1, q, v[0][q], v[1][q], v[2][q], v[3][q]);
+    if constexpr (kDown) {
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          cur[j][q][0] = O::add(cur[j][q][0], down[j][q]);
+          cur[j][q][3] = O::sub(cur[j][q][3], down[j][q]);
+        }
+    }
   };
 
   // ---------------------------------------------------------------- store
@@ -674,7 +522,7 @@ __global__ void __launch_bounds__(BXC * TYT, Rows2Layout<S, BXC, TYT>::MIN_BLOCK
       const bool skip = !active || row_wall[j] || zskip;
       const int64_t off = (int64_t)q * ps + j * nx64;
       if (per_node_store) {
-        S* const fp[4] = {op[0], op[1], op[2], op[3]};
+        S* const fp[4] = {op0, op0 + ta.n, op0 + 2 * ta.n, op0 + 3 * ta.n};
         store_plane<kD3Q19, S, RM>(fp, mrow, ta, off, x_lo_wall, x_hi_wall, skip, acc[j], force);
         continue;
       }
@@ -700,66 +548,49 @@ __global__ void __launch_bounds__(BXC * TYT, Rows2Layout<S, BXC, TYT>::MIN_BLOCK
         v[f][0].x = x_lo_wall ? wv[f] : v[f][0].x;
         if constexpr (RM == kRowsOdd) v[f][0].y = x_hi_wall ? wv[f] : v[f][0].y;
         else v[f][1].y = x_hi_wall ? wv[f] : v[f][1].y;
-        if (bounds_ok(ta.bounds, f * ta.n + in_off + off, n4 - 3)) Quad<S>::st(op[f] + off, v[f][0], v[f][1]);
+        if (bounds_ok(ta.bounds, f * ta.n + in_off + off, n4 - 3)) Quad<S>::st(op0 + f * ta.n + off, v[f][0], v[f][1]);
       }
     }
   };
 
-  P R0[2][2][4], R1[2][2][4], R2[2][2][4];
-  auto zero = [&](P(&A)[2][2][4]) {
-#pragma unroll
-    for (int j = 0; j < 2; ++j)
-#pragma unroll
-      for (int q = 0; q < 2; ++q)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) A[j][q][k] = O::splat(C(0));
-  };
-  zero(R0);
-  zero(R1);
-  zero(R2);
+  P own[2][2][4] = {};
 
 #pragma unroll
   for (int i = 0; i < kStages - 1; ++i) fetch(i);
-  // first (halo) plane z0 - 1: only the equilibria moving up the march axis
+  // first (halo) plane z0 - 1: only what it sends up the march axis
   fetch(kStages - 1);
   take(0);
   // (the barrier inside update, or this one, keeps slot 0's next copy behind
   // every thread's wait for its current one)
-  if (plane_exists(z0 - 1)) update(std::integral_constant<int, kFirst>{}, R0, R2, R1);
+  if (plane_exists(z0 - 1)) update(std::integral_constant<int, kFirst>{}, own);
   else __syncthreads();
 
-  // full planes: R0, R1, R2 hold the sums of planes p - 1, p, p + 1; after
-  // plane p, p - 1 is complete and the sums move down by one plane.  The
-  // loop body is not unrolled: one copy of the two-row update keeps the code
-  // within the instruction cache (the moves cost less than the misses of a
-  // three-way unrolled body, whose copies would rename the sums instead).
+  // full planes: after plane p, plane p - 1 is complete.  The loop body is not
+  // unrolled: one copy of the two-row update keeps the code within the
+  // instruction cache.
 #pragma unroll 1
   for (int p = z0; p < z1; ++p) {
     const int i = p - z0 + 1;
     fetch(i + kStages - 1);
     nu_prefetch(p - 1);
     take(i);
-    update(std::integral_constant<int, kMid>{}, R0, R1, R2);
-    if (p - 1 >= z0) store(p - 1, R0);
+    update(std::integral_constant<int, kMid>{}, own);
+    if (p - 1 >= z0) store(p - 1, cur);
 #pragma unroll
     for (int j = 0; j < 2; ++j)
 #pragma unroll
       for (int q = 0; q < 2; ++q)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          R0[j][q][k] = R1[j][q][k];
-          R1[j][q][k] = R2[j][q][k];
-          R2[j][q][k] = O::splat(C(0));
-        }
+        for (int k = 0; k < 4; ++k) cur[j][q][k] = own[j][q][k];
   }
-  // last (halo) plane z1: only the equilibria moving down, into plane z1 - 1 (R0)
+  // last (halo) plane z1: only what it sends down, to plane z1 - 1
   {
     const int i = np - 1;
     fetch(i + kStages - 1);
     nu_prefetch(z1 - 1);
     take(i);
-    if (plane_exists(z1)) update(std::integral_constant<int, kLast>{}, R0, R1, R1);
-    store(z1 - 1, R0);
+    if (plane_exists(z1)) update(std::integral_constant<int, kLast>{}, own);
+    store(z1 - 1, cur);
   }
   if constexpr (NU) {
     // block sum: warp shuffles, one value per warp, one FP64 atomic per block

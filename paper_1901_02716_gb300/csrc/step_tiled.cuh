@@ -122,6 +122,14 @@ struct Pair<float> {
   }
   __device__ __forceinline__ static P mul(P a, P b) { return __fmul2_rn(a, b); }
   __device__ __forceinline__ static P fma(P a, P b, P c) { return __ffma2_rn(a, b, c); }
+  // a product that is never contracted with a sum it enters (the compiler may
+  // fuse __fmul2_rn with __fadd2_rn, and does so in one instance of a loop body
+  // and not in another)
+  __device__ __forceinline__ static P mul_exact(P a, P b) {
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pk(a)), "l"(pk(b)));
+    return upk(d);
+  }
   // 1/a on both lanes: the hardware approximation r0 (rcp.approx, relative
   // error below 2^-22) refined by one Newton-Raphson step for f(r) = 1/r - a,
   // r1 = r0 + r0 (1 - a r0), on the paired FMA datapath.  The residual
@@ -147,6 +155,9 @@ struct Pair<double> {
   __device__ __forceinline__ static P add(P a, P b) { return make_double2(a.x + b.x, a.y + b.y); }
   __device__ __forceinline__ static P sub(P a, P b) { return make_double2(a.x - b.x, a.y - b.y); }
   __device__ __forceinline__ static P mul(P a, P b) { return make_double2(a.x * b.x, a.y * b.y); }
+  __device__ __forceinline__ static P mul_exact(P a, P b) {
+    return make_double2(__dmul_rn(a.x, b.x), __dmul_rn(a.y, b.y));
+  }
   __device__ __forceinline__ static P fma(P a, P b, P c) {
     return make_double2(__fma_rn(a.x, b.x, c.x), __fma_rn(a.y, b.y, c.y));
   }
