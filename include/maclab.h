@@ -189,12 +189,13 @@ maclab_status maclab_step(maclab_handle h, int64_t n);
  * a one-step launch (the previous state is step n - 1).  Its sums run in the
  * tiled kernel's order: identical bits.  The default for FP32 D2Q9 grids of
  * fewer than 524,288 node pairs and FP64 ones of up to 131,072 (512^2).
- * The default also takes these kernels where a choice by hand is refused: a
- * closed x axis of at least 17 nodes whose width is not a multiple of 4 is
- * stored in rows padded to one (the raw state keeps its (d + 1) * N values), the
- * block kernel takes a periodic x axis of any width of at least 32 nodes, and the
- * two-rows and folded kernels run on row counts that their tiles do not divide
- * (at least one tile of rows). */
+ * The default also takes these kernels where a choice by hand is refused: an x
+ * axis of at least 17 nodes whose width is not a multiple of 4 is stored in rows
+ * padded to one (D2Q9: closed axes; D3Q19 with FP32 or 16-bit storage: closed from
+ * 50,000 nodes on, periodic from 150,000; the raw state keeps its (d + 1) * N
+ * values); with D2Q9 the block kernel takes a periodic x axis of any width of at
+ * least 32 nodes; and the two-rows and folded kernels run on row counts that their
+ * tiles do not divide (at least one tile of rows). */
 #define MACLAB_KERNEL_AUTO 0
 #define MACLAB_KERNEL_REFERENCE 1
 #define MACLAB_KERNEL_TILED 2

@@ -122,6 +122,13 @@ size_t buffer_bytes(const maclab_ctx* h) { return (size_t)(h->g.d + 1) * (size_t
 // Put the current buffer's wall values into the other one as well (wall nodes
 // are never written by the step kernels; every fluid node of a buffer is
 // written by the step that fills it, so nothing else needs to be copied).
+// And the periodic images of padded rows, wherever nodes were written from outside.
+maclab_status refresh_images(maclab_ctx* h, int buffer) {
+  if (wrap_columns(h->g))
+    CUDA_TRY(launch_wrap_columns(h->g, h->precision, h->buf[buffer], h->stream, 0), "periodic images");
+  return MACLAB_OK;
+}
+
 maclab_status mirror_walls(maclab_ctx* h) {
   CUDA_TRY(launch_copy_walls(h->g, h->precision, h->d_node_type, h->buf[h->cur], h->buf[h->cur ^ 1], h->stream),
            "mirror wall values");
@@ -306,8 +313,9 @@ maclab_status maclab_create(const maclab_config* cfg, maclab_handle* out) {
   h->n_fluid = N - n_wall;
   g.wall_mode = n_wall == 0 ? kWallNone : (box ? kWallBox : kWallMask);
   h->raw = g;
-  if (!(g.periodic & 1u) && nx % 4 != 0 && nx >= kMinPadWidth) {  // interleaved rows with padding (Geometry)
-    g.pad = (int)(4 - nx % 4);
+  const bool px = (g.periodic & 1u) != 0;
+  if (pad_rows(g, h->precision)) {  // interleaved rows with padding
+    g.pad = (int)((nx + (px ? 2 : 0) + 3) / 4 * 4 - nx);
     g.nx += g.pad;
     g.n = (int64_t)g.nx * ny * nz;
     g.ilv = 1;
@@ -367,6 +375,7 @@ maclab_status maclab_create(const maclab_config* cfg, maclab_handle* out) {
   if (e == cudaSuccess)
     e = launch_fill_walls(g, h->precision, h->d_node_type, h->d_wall_lat, h->n_wall_ids, h->buf[0],
                           h->stream);
+  if (e == cudaSuccess && wrap_columns(g)) e = launch_wrap_columns(g, h->precision, h->buf[0], h->stream, 0);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h->buf[1], h->buf[0], sb, cudaMemcpyDeviceToDevice, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
@@ -450,6 +459,7 @@ maclab_status maclab_set_state(maclab_handle h, const void* rho, const void* u, 
   CUDA_TRY(launch_set_physical(h->g, h->precision, r, v, dtype, h->rho0, h->e, h->d_node_type,
                                h->d_wall_lat, h->n_wall_ids, h->buf[h->cur], h->buf[h->cur ^ 1], h->stream),
            "set_state kernel");
+  if (maclab_status s = refresh_images(h, h->cur)) return s;
   h->steps = 0;
   h->prev_valid = false;
   if (where == MACLAB_HOST) CUDA_TRY(cudaStreamSynchronize(h->stream), "set_state sync");
@@ -487,6 +497,8 @@ maclab_status maclab_set_wall_state(maclab_handle h, const void* rho, const void
   CUDA_TRY(launch_set_wall_values(h->g, h->precision, r, v, dtype, h->rho0, h->e, h->d_node_type,
                                   h->buf[0], h->buf[1], h->stream),
            "set_wall_state kernel");
+  for (int b = 0; b < 2; ++b)
+    if (maclab_status s = refresh_images(h, b)) return s;
   if (where == MACLAB_HOST) CUDA_TRY(cudaStreamSynchronize(h->stream), "set_wall_state sync");
   return MACLAB_OK;
 }
@@ -573,6 +585,7 @@ maclab_status maclab_set_lattice_state(maclab_handle h, const void* state, int32
     CUDA_TRY(launch_repack(h->g, h->precision, h->buf[h->cur], const_cast<void*>(raw), 0, march_planes(h), false,
                            h->stream),
              "set_lattice_state repack");
+    if (maclab_status s = refresh_images(h, h->cur)) return s;
   } else {
     CUDA_TRY(cudaMemcpyAsync(h->buf[h->cur], state, state_bytes(h),
                              where == MACLAB_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice,
@@ -1041,6 +1054,7 @@ maclab_status maclab_set_planes(maclab_handle h, int64_t p0, int64_t count, cons
     CUDA_TRY(cudaMemcpyAsync(h->d_staging, src, bytes, cudaMemcpyDefault, h->stream), "set_planes copy");
     CUDA_TRY(launch_repack(h->g, h->precision, h->buf[h->cur], h->d_staging, p0, count, false, h->stream),
              "set_planes repack");
+    if ((s = refresh_images(h, h->cur)) != MACLAB_OK) return s;
     if (where == MACLAB_HOST) CUDA_TRY(cudaStreamSynchronize(h->stream), "set_planes sync");
     return MACLAB_OK;
   }

@@ -193,12 +193,30 @@ struct Geometry {
   // 2.1 us).  The domain's right wall is then at x = nx - 1 -
   // pad and shields it: whatever a step leaves in the padding reaches only wall
   // nodes, which keep their values.  In mask mode the padding is marked as wall.
+  // On a periodic x axis (D3Q19) the padding is 2 to 5 positions: the first holds a
+  // copy of node 0 and the last, the seam's neighbour of node 0, one of the
+  // domain's last node; they are copied after every step (launch_wrap_columns; FP32
+  // step of a periodic 251^3 grid: 498 us on the one-thread-per-node kernel, 148
+  // now; 95^3: 26.4 and 15.7).
   int pad;
 };
 
-// Narrower closed domains than this keep their natural rows: at least two
-// quads must lie between the two x-walls, so that no quad holds both.
-constexpr int kMinPadWidth = 17;
+// Whether a domain of natural rows (g as the caller gave it) is stored in padded
+// ones.  At least 17 nodes wide, so that two quads lie between the two x-walls and
+// no quad holds both.  D3Q19: not with FP64 storage, whose tiled kernel's halo rows
+// cost what the one-thread-per-node kernel's repeated terms do on a pipe that
+// bounds both (45^3 closed: 66 us a step on the latter, 148 padded); and only where
+// the fast kernels' longer start pays (us a step, natural and padded rows, FP32:
+// closed 33^3 3.7 and 4.0, 37^3 4.2 and 3.8, 63^3 9.5 and 5.1; periodic, with the
+// images' extra launch, 51^3 6.3 and 6.7, 55^3 7.8 and 6.8, 79^3 16.2 and 10.5).
+inline bool pad_rows(const Geometry& g, int precision) {
+  if (g.nx % 4 == 0 || g.nx < 17) return false;
+  const bool px = (g.periodic & 1u) != 0;
+  if (g.d == 2) return !px;  // periodic: the block kernel takes natural rows
+  return precision != MACLAB_F64 && g.n >= (px ? 150000 : 50000);
+}
+
+__host__ __device__ inline bool wrap_columns(const Geometry& g) { return g.pad > 0 && (g.periodic & 1u); }
 
 // The thread (quad) of a row that holds the right wall, and whether the wall is
 // lane a.y of that quad (pad odd) or lane b.y (pad even).
@@ -375,6 +393,8 @@ cudaError_t launch_set_wall_values(const Geometry& g, int precision, const void*
 // nodes in their natural order); to_raw: out of the state, else into it.
 cudaError_t launch_repack(const Geometry& g, int precision, void* state, void* raw, int64_t p0, int64_t count,
                           bool to_raw, cudaStream_t stream);
+// The periodic images of a state in padded rows (wrap_columns).
+cudaError_t launch_wrap_columns(const Geometry& g, int precision, void* state, cudaStream_t stream, int overlap);
 cudaError_t launch_copy_walls(const Geometry& g, int precision, const uint8_t* node_type, const void* src,
                               void* dst, cudaStream_t stream);
 cudaError_t launch_fill_walls(const Geometry& g, int precision, const uint8_t* node_type,

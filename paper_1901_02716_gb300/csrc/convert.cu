@@ -127,7 +127,8 @@ __device__ __forceinline__ void for_units(const Geometry& g, Fn&& fn) {
 }
 
 // Nodes (x, x + H, x + 1, x + 1 + H) of a user row, j the index of x; those past
-// the end of a padded row read as 0 and are not written.
+// the end of a padded row read as its first node (launch_wrap_columns then puts
+// the periodic images in place) and are not written.
 template <int U, typename T>
 __device__ __forceinline__ void ld_user(const Geometry& g, const T* p, int64_t j, int x, T (&v)[4]) {
   if constexpr (U == kQuad2) {
@@ -140,9 +141,9 @@ __device__ __forceinline__ void ld_user(const Geometry& g, const T* p, int64_t j
   } else {
     const int last = g.nx - g.pad - 1 - g.hx;
     v[0] = p[j];
-    v[1] = x <= last ? p[j + g.hx] : T(0);
+    v[1] = p[x <= last ? j + g.hx : j - x];
     v[2] = p[j + 1];
-    v[3] = x + 1 <= last ? p[j + 1 + g.hx] : T(0);
+    v[3] = p[x + 1 <= last ? j + 1 + g.hx : j - x];
   }
 }
 template <int U, typename T>
@@ -470,6 +471,36 @@ cudaError_t launch_repack(const Geometry& g, int precision, void* state, void* r
     case 8: return repack_t<double>(g, state, raw, p0 * plane_rows, count * plane_rows, to_raw, st);
     case 4: return repack_t<float>(g, state, raw, p0 * plane_rows, count * plane_rows, to_raw, st);
     case 2: return repack_t<uint16_t>(g, state, raw, p0 * plane_rows, count * plane_rows, to_raw, st);
+  }
+  return cudaErrorInvalidValue;
+}
+
+// One thread copies a row's two images in one field.
+template <typename S>
+__global__ void __launch_bounds__(256) wrap_columns_k(int64_t count, int nx, int first, int last, int image0,
+                                                      S* __restrict__ state) {
+  pdl_wait();  // the step before this kernel has completed and its writes are visible
+  pdl_launch_next();
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= count) return;
+  S* const row = state + k * nx;  // fields follow one another: row k of the whole state
+  row[image0] = row[first];
+  row[nx - 1] = row[last];
+}
+
+template <typename S>
+static cudaError_t wrap_t(const Geometry& g, void* state, cudaStream_t st, int overlap) {
+  const int64_t count = g.n / g.nx * (g.d + 1);
+  const int nx = g.nx - g.pad;
+  return launch_kernel(wrap_columns_k<S>, dim3((unsigned)((count + 255) / 256)), dim3(256), 0, st, overlap, count, g.nx,
+                       mem_x(g, 0), mem_x(g, nx - 1), mem_x(g, nx), (S*)state);
+}
+
+cudaError_t launch_wrap_columns(const Geometry& g, int precision, void* state, cudaStream_t st, int overlap) {
+  switch (storage_bytes(precision)) {
+    case 8: return wrap_t<double>(g, state, st, overlap);
+    case 4: return wrap_t<float>(g, state, st, overlap);
+    case 2: return wrap_t<uint16_t>(g, state, st, overlap);
   }
   return cudaErrorInvalidValue;
 }

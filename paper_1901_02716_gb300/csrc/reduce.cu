@@ -313,7 +313,10 @@ __global__ void __launch_bounds__(256, sizeof(S) == 8 ? 1 : 2) diag_rows(Geometr
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int64_t rows = N / g.nx;
   const int quads = g.nx >> 2;
-  const int x_last = g.nx - 1 - g.pad - g.hx;  // pair of the domain's last node
+  const bool images = g.pad > 0 && (g.periodic & 1u);
+  // second-half nodes from this pair on do not count: the right wall and what lies
+  // beyond it, or the padding of a periodic row
+  const int x_last = g.nx - g.pad - g.hx - (images ? 0 : 1);
   const bool xw = g.wall_mode == kWallBox && !(g.periodic & 1u);
   const bool yw = g.wall_mode == kWallBox && !(g.periodic & 2u);
   const bool zw = g.wall_mode == kWallBox && g.d == 3 && !(g.periodic & 4u);
@@ -337,9 +340,8 @@ __global__ void __launch_bounds__(256, sizeof(S) == 8 ? 1 : 2) diag_rows(Geometr
       if (g.wall_mode == kWallMask) {
         const uchar4 mk = *reinterpret_cast<const uchar4*>(g.mask + m);
         wall[0] = mk.x != 0; wall[1] = mk.y != 0; wall[2] = mk.z != 0; wall[3] = mk.w != 0;
-      } else if (xw) {
-        // the second-half nodes of the last quads: the right wall and the padding beyond it
-        wall[0] = q == 0;
+      } else if (xw || images) {
+        wall[0] = xw && q == 0;
         wall[1] = 2 * q >= x_last;
         wall[3] = 2 * q + 1 >= x_last;
       }

@@ -202,7 +202,7 @@ static const char* kernel_name(const Geometry& g, int precision, int kernel) {
   return names[kernel == MACLAB_KERNEL_TILED ? 1 : 0][g.lattice == kD2Q9 ? 0 : 1][precision & 3];
 }
 
-KernelInfo describe_step_kernel(const Geometry& g, int precision, int kernel, int ty, int tz) {
+static KernelInfo describe_kernel(const Geometry& g, int precision, int kernel, int ty, int tz) {
   if (kernel == MACLAB_KERNEL_TILED)
     return KernelInfo{MACLAB_KERNEL_TILED, 1, 1, tiled_threads(g, precision, ty, tz),
                       kernel_name(g, precision, kernel)};
@@ -223,7 +223,7 @@ KernelInfo describe_step_kernel(const Geometry& g, int precision, int kernel, in
   return KernelInfo{MACLAB_KERNEL_REFERENCE, 1, 1, 256, kernel_name(g, precision, kernel)};
 }
 
-cudaError_t launch_step(const StepLaunch& s, cudaStream_t stream, int kernel) {
+static cudaError_t launch_step_kernel(const StepLaunch& s, cudaStream_t stream, int kernel) {
   switch (kernel) {
     case MACLAB_KERNEL_REFERENCE:
       return s.g.lattice == kD2Q9 ? launch_naive_lat<kD2Q9>(s, stream)
@@ -246,6 +246,18 @@ cudaError_t launch_step(const StepLaunch& s, cudaStream_t stream, int kernel) {
     default:
       return cudaErrorInvalidValue;
   }
+}
+
+KernelInfo describe_step_kernel(const Geometry& g, int precision, int kernel, int ty, int tz) {
+  KernelInfo k = describe_kernel(g, precision, kernel, ty, tz);
+  if (wrap_columns(g)) ++k.launches;  // the periodic images
+  return k;
+}
+
+cudaError_t launch_step(const StepLaunch& s, cudaStream_t stream, int kernel) {
+  const cudaError_t e = launch_step_kernel(s, stream, kernel);
+  if (e != cudaSuccess || !wrap_columns(s.g)) return e;
+  return launch_wrap_columns(s.g, s.precision, s.out, stream, s.overlap);
 }
 
 }  // namespace maclab

@@ -118,7 +118,8 @@ cudaError_t launch_fold(const StepLaunch& sl, cudaStream_t stream, int ty, int t
   ta.plane_stride = (int64_t)g.nx * g.ny;
   ta.ty = s.ty;
   const int ytiles = (g.ny + s.ty - 1) / s.ty;
-  const RowMode rows = (g.pad & 1) ? kRowsOdd : (g.pad || g.ny % s.ty != 0) ? kRowsEven : kRowsPlain;
+  const int wall_pad = (g.periodic & 1u) ? 0 : g.pad;  // what moves the right wall
+  const RowMode rows = (wall_pad & 1) ? kRowsOdd : (wall_pad || g.ny % s.ty != 0) ? kRowsEven : kRowsPlain;
   auto dispatch = [&](const void* in, void* out, dim3 grid, int* resident) {
     auto typed = [&](auto zero) {
       using S = decltype(zero);

@@ -124,7 +124,8 @@ cudaError_t launch_rows2(const StepLaunch& sl, cudaStream_t stream, int ty, int 
   ta.ty = 2 * s.tyt;
   const int ytiles = (g.ny + ta.ty - 1) / ta.ty;
   CUtensorMap tm_own{}, tm_halo{};
-  const RowMode rows = (g.pad & 1) ? kRowsOdd : (g.pad || g.ny % ta.ty != 0) ? kRowsEven : kRowsPlain;
+  const int wall_pad = (g.periodic & 1u) ? 0 : g.pad;  // what moves the right wall
+  const RowMode rows = (wall_pad & 1) ? kRowsOdd : (wall_pad || g.ny % ta.ty != 0) ? kRowsEven : kRowsPlain;
   auto typed = [&](auto zero, const void* in, void* out, dim3 grid, int* resident) {
     using S = decltype(zero);
     switch (rows) {

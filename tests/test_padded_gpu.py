@@ -1,6 +1,6 @@
-"""Closed x axes whose width is not a multiple of 4 (stored in padded rows) and
-row counts that no tile divides (a last tile moved up), against the oracle, and
-the calls that show the raw state: its layout has no padding.
+"""X axes whose width is not a multiple of 4 (stored in padded rows) and row
+counts that no tile divides (a last tile moved up), against the oracle, and the
+calls that show the raw state: its layout has no padding.
 
 The bars are those of test_parity_gpu (the same arithmetic on other rows).
 """
@@ -24,14 +24,22 @@ def _built():
 
 
 # widths with one, two and three padding positions, the narrowest padded one,
-# box and mask walls, every kernel the library picks for the widths and types
+# box and mask walls, every kernel the library picks for the widths and types (3D:
+# from the node counts on where rows are padded)
 PADDED = [
     (D2, (17, 13), 0b00, "box"), (D2, (18, 9), 0b10, "box"), (D2, (23, 40), 0b00, "mixed"),
     (D2, (401, 37), 0b00, "box"), (D2, (1026, 1030), 0b10, "box"),
-    (D3, (17, 9, 6), 0b110, "box"), (D3, (30, 16, 9), 0b000, "mixed"), (D3, (63, 8, 7), 0b100, "box"),
-    (D3, (65, 13, 6), 0b000, "box"), (D3, (126, 12, 5), 0b010, "box"), (D3, (127, 11, 6), 0b000, "mixed"),
-    (D3, (133, 10, 5), 0b010, "box"), (D3, (251, 9, 6), 0b000, "box"), (D3, (257, 7, 5), 0b100, "mixed"),
-    (D3, (511, 6, 5), 0b000, "box"),
+    (D3, (17, 49, 61), 0b110, "box"), (D3, (30, 40, 42), 0b000, "mixed"), (D3, (63, 16, 50), 0b100, "box"),
+    (D3, (65, 29, 27), 0b000, "box"), (D3, (126, 20, 20), 0b010, "box"), (D3, (127, 21, 19), 0b000, "mixed"),
+    (D3, (133, 18, 21), 0b010, "box"), (D3, (251, 17, 12), 0b000, "box"), (D3, (257, 14, 14), 0b100, "mixed"),
+    (D3, (511, 10, 10), 0b000, "box"),
+]
+# periodic x: two to five padding positions, which hold the periodic images
+WRAPPED = [
+    (D3, (17, 96, 92), 0b111, "none"), (D3, (18, 92, 91), 0b001, "box"), (D3, (19, 88, 90), 0b101, "mixed"),
+    (D3, (33, 69, 66), 0b111, "none"), (D3, (62, 48, 51), 0b011, "box"), (D3, (95, 42, 38), 0b111, "mixed"),
+    (D3, (126, 40, 30), 0b111, "none"), (D3, (127, 33, 36), 0b011, "box"), (D3, (251, 25, 24), 0b111, "none"),
+    (D3, (258, 24, 25), 0b001, "mixed"), (D3, (511, 18, 17), 0b111, "none"),
 ]
 RAGGED = [
     (D3, (32, 13, 6), 0b111, "none"), (D3, (64, 11, 5), 0b000, "box"), (D3, (128, 10, 7), 0b010, "box"),
@@ -40,7 +48,7 @@ RAGGED = [
 ]
 
 
-@pytest.mark.parametrize("lat,dims,periodic,walls", PADDED + RAGGED)
+@pytest.mark.parametrize("lat,dims,periodic,walls", PADDED + WRAPPED + RAGGED)
 @pytest.mark.parametrize("precision", [M.F64, M.F32, M.BF16_STORE])
 def test_matches_oracle(lat, dims, periodic, walls, precision):
     case = inputs.random_case(lat, dims, periodic, seed=131, u_amp=0.08, rho_amp=0.02, walls=walls,
@@ -48,7 +56,7 @@ def test_matches_oracle(lat, dims, periodic, walls, precision):
     assert_parity(*run_both(case, precision, 3 if dims[0] > 1000 else 11), precision)
 
 
-@pytest.mark.parametrize("lat,dims,periodic,walls", [PADDED[2], PADDED[3], PADDED[6], PADDED[12]])
+@pytest.mark.parametrize("lat,dims,periodic,walls", [PADDED[2], PADDED[3], PADDED[6], PADDED[12], WRAPPED[1], WRAPPED[5], WRAPPED[8]])
 @pytest.mark.parametrize("precision", [M.F64, M.F32, M.F16_STORE])
 def test_raw_state_has_no_padding(lat, dims, periodic, walls, precision):
     """The raw state is (d + 1) * N values in natural order; a run resumed from it, on the host or the
@@ -66,7 +74,8 @@ def test_raw_state_has_no_padding(lat, dims, periodic, walls, precision):
     assert np.array_equal(fields[0].astype(np.float64) + 1.0, r)
     assert np.array_equal(fields[1:].astype(np.float64), u)
     wall = case.wall_mask
-    assert np.array_equal(fields[1:, wall], case.u[:, wall].astype(np_t))
+    if wall is not None:
+        assert np.array_equal(fields[1:, wall], case.u[:, wall].astype(np_t))
     dev = torch.empty(s.state_bytes() + 1, dtype=torch.uint8, device="cuda")
     for t in (dev[:-1], dev[1:]):  # aligned, and a byte off
         s.get_lattice_state(t)
@@ -90,7 +99,7 @@ def test_raw_state_has_no_padding(lat, dims, periodic, walls, precision):
     s.close()
 
 
-@pytest.mark.parametrize("lat,dims,periodic,walls", [PADDED[1], PADDED[2], PADDED[12], RAGGED[3]])
+@pytest.mark.parametrize("lat,dims,periodic,walls", [PADDED[1], PADDED[2], PADDED[12], RAGGED[3], WRAPPED[2], WRAPPED[4]])
 def test_diagnostics_and_wall_values(lat, dims, periodic, walls):
     """Diagnostics skip the padding; per-node wall values reach every wall node."""
     case = inputs.random_case(lat, dims, periodic, seed=133, u_amp=0.06, rho_amp=0.02, walls=walls)
@@ -133,7 +142,7 @@ def test_batch_of_odd_widths(depth, precision):
 
 
 def test_tuned_padded_domain_keeps_the_result():
-    case = inputs.random_case(D3, (70, 13, 9), 0b000, seed=136, u_amp=0.06, rho_amp=0.02, walls="box")
+    case = inputs.random_case(D3, (70, 27, 29), 0b000, seed=136, u_amp=0.06, rho_amp=0.02, walls="box")
     s = M.Solver.from_case(case, M.F32)
     s.tune()
     s.step(9)
