@@ -25,6 +25,7 @@
 
 #include "common.cuh"
 #include "lattice.cuh"
+#include "units.cuh"
 
 namespace maclab {
 
@@ -453,34 +454,130 @@ cudaError_t launch_adjoint_nu_term(const Geometry& g, int precision, const void*
 //
 // Physical output gradients (logical order) -> adjoint of the stored state
 // (storage order): rho = rho0 (1 + drho) and u = e ut, so dL/ddrho = rho0 dL/drho
-// and dL/dut = e dL/du.  Also sums lam_ut . ut over all nodes (the output's
-// dependence on e, for dL/de).
-template <typename S, typename T>
-__global__ void adj_seed(Geometry g, const T* __restrict__ grho, const T* __restrict__ gu,
-                         const S* __restrict__ state, double rho0, double e,
-                         typename Store<S>::C* __restrict__ lam, double* __restrict__ dot) {
+// and dL/dut = e dL/du; and back at the start of the rollout.  Both ends also
+// sum lam_ut . ut over all nodes (the dependence of output and input on e).
+//
+// With 32-bit arrays and arithmetic the maps take the FP32 forms of UnitMap,
+// and the sums products and additions whose rounding errors are kept (an fma
+// gives a product's, two-sum an addition's), one storage quad at a time: about
+// 47 bits of a quad's sum, which is then added in FP64.  A quad whose sum could
+// have left the range of these forms (large, or so small that an error term
+// could be subnormal) is summed in FP64.  Done in FP64 throughout, seven
+// conversions and multiply-adds per value on a pipe of two lanes per SM (and
+// the divisions by e) bounded both kernels.  96^3 FP32, whole calls with their
+// read-back: seed 60 -> 36 us, finish 119 -> 41 us.
+
+// Sum of a[i] b[i].
+template <int N>
+__device__ __forceinline__ double dot_unit(const float (&a)[N], const float (&b)[N]) {
+  float hi = 0.f, lo = 0.f;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const float p = __fmul_rn(a[i], b[i]);
+    const float s = __fadd_rn(hi, p), bb = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(p, bb)), __fmaf_rn(a[i], b[i], -p)));
+    hi = s;
+  }
+  if (fabsf(hi) > 0x1p-76f && fabsf(hi) < 0x1p100f) return (double)hi + (double)lo;
+  double v = 0.0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) v += (double)a[i] * (double)b[i];
+  return v;
+}
+template <int N>
+__device__ __forceinline__ double dot_unit(const double (&a)[N], const double (&b)[N]) {
+  double v = 0.0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) v += a[i] * b[i];
+  return v;
+}
+
+// Adds the block's sum of v to *out: one FP64 atomic per block of 256 threads.
+__device__ __forceinline__ void add_block_sum(double v, double* out) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  __shared__ double red[8];
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) v += red[w];
+    atomicAdd(out, v);
+  }
+}
+
+// The ends of a unit of W nodes at storage index i, user index j (units.cuh);
+// kNode also takes interleaved rows whose arrays are not aligned to quads.
+template <int U>
+__device__ __forceinline__ int64_t user_index(const Geometry& g, int64_t i, int64_t j) {
+  if (U != kNode || !g.ilv) return j;
+  const int64_t row = i / g.nx;
+  return row * g.nx + log_x(g, (int)(i - row * g.nx));
+}
+template <int U, typename T, int W>
+__device__ __forceinline__ void ld_unit(const Geometry& g, const T* p, int64_t j, int x, T (&v)[W]) {
+  if constexpr (W == 4) ld_user<U, T>(g, p, j, x, v);
+  else v[0] = p[j];
+}
+template <int U, typename T, int W>
+__device__ __forceinline__ void st_unit(const Geometry& g, T* p, int64_t j, int x, const T (&v)[W]) {
+  if constexpr (W == 4) st_user<U, T>(g, p, j, x, v);
+  else p[j] = v[0];
+}
+template <int W, typename S>
+__device__ __forceinline__ void ld_stored(const S* p, S (&v)[W]) {
+  if constexpr (W == 4) {
+    const Four<S> q = *reinterpret_cast<const Four<S>*>(p);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) v[c] = q.v[c];
+  } else {
+    v[0] = p[0];
+  }
+}
+
+// FAST: 32-bit arrays and the FP32 forms (then the sums are of gu . ut, times e at the end).
+template <int D, typename S, typename T, bool FAST, typename I, int U>
+__global__ void __launch_bounds__(256) adj_seed(Geometry g, const T* __restrict__ grho, const T* __restrict__ gu,
+                                                const S* __restrict__ state, UnitMap m,
+                                                typename Store<S>::C* __restrict__ lam, double* __restrict__ dot) {
   using C = typename Store<S>::C;
+  using A = typename std::conditional<FAST, float, double>::type;  // of the products
+  constexpr int W = U == kNode ? 1 : 4;
   const int64_t N = g.n;
   double acc = 0.0;
-  for (int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; m < N;
-       m += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t row = m / g.nx;
-    const int64_t j = row * g.nx + log_x(g, (int)(m - row * g.nx));
-    lam[m] = grho ? C(rho0 * (double)grho[j]) : C(0);
-    for (int i = 0; i < g.d; ++i) {
-      const double l = gu ? e * (double)gu[i * N + j] : 0.0;
-      lam[(1 + i) * N + m] = C(l);
-      acc += l * (double)Store<S>::from(state[(1 + i) * N + m]);
+  for_units<I, U>(g, [&](int64_t i, int64_t j0, int x) {
+    const int64_t j = user_index<U>(g, i, j0);
+    T v[1 + D][W];
+    S ut[D][W];
+#pragma unroll
+    for (int f = 0; f <= D; ++f) {
+      const T* const p = f == 0 ? grho : gu ? gu + (f - 1) * N : nullptr;
+#pragma unroll
+      for (int c = 0; c < W; ++c) v[f][c] = T(0);
+      if (p) ld_unit<U, T, W>(g, p, j, x, v[f]);
+      if (f > 0) ld_stored<W, S>(state + f * N + i, ut[f - 1]);
     }
-  }
-  __shared__ double red[256];
-  red[threadIdx.x] = acc;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) atomicAdd(dot, red[0]);
+    A a[D * W], b[D * W];
+#pragma unroll
+    for (int f = 0; f <= D; ++f) {
+      C out[W];
+#pragma unroll
+      for (int c = 0; c < W; ++c) {
+        if constexpr (FAST) {
+          out[c] = f == 0 ? __fmul_rn(v[f][c], m.f_rho0) : mul_pair(v[f][c], m.e_hi, m.e_lo);
+          if (f > 0) a[(f - 1) * W + c] = v[f][c];
+        } else {
+          const double l = (f == 0 ? m.rho0 : m.e) * (double)v[f][c];
+          out[c] = C(l);
+          if (f > 0) a[(f - 1) * W + c] = l;
+        }
+        if (f > 0) b[(f - 1) * W + c] = (A)Store<S>::from(ut[f - 1][c]);
+      }
+      if constexpr (W == 4) *reinterpret_cast<Four<C>*>(lam + f * N + i) = Four<C>{{out[0], out[1], out[2], out[3]}};
+      else lam[f * N + i] = out[0];
+    }
+    acc += dot_unit(a, b);
+  });
+  add_block_sum(FAST ? m.e * acc : acc, dot);
 }
 
 // Adjoint of the initial stored state -> gradients of the physical inputs.
@@ -488,97 +585,132 @@ __global__ void adj_seed(Geometry g, const T* __restrict__ grho, const T* __rest
 // wall nodes get 0 there (their initial values come from the wall tables) and
 // their adjoint is summed per wall id into wall[k * 4 + (0: rho, 1..3: u)].
 // dot += sum over all nodes of lam_ut . ut (the inputs' dependence on e).
-template <typename S, typename T>
-__global__ void adj_finish(Geometry g, const typename Store<S>::C* __restrict__ lam,
-                           const S* __restrict__ state, const uint8_t* __restrict__ node_type,
-                           int n_wall_ids, double rho0, double e, T* __restrict__ grho,
-                           T* __restrict__ gu, double* __restrict__ wall, double* __restrict__ dot) {
+template <int D, typename S, typename T, bool FAST, typename I, int U>
+__global__ void __launch_bounds__(256) adj_finish(Geometry g, const typename Store<S>::C* __restrict__ lam,
+                                                  const S* __restrict__ state, const uint8_t* __restrict__ node_type,
+                                                  int n_wall_ids, UnitMap m, T* __restrict__ grho, T* __restrict__ gu,
+                                                  double* __restrict__ wall, double* __restrict__ dot) {
+  using C = typename Store<S>::C;
+  using A = typename std::conditional<FAST, float, double>::type;
+  constexpr int W = U == kNode ? 1 : 4;
   const int64_t N = g.n;
   double acc = 0.0;
-  for (int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; m < N;
-       m += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t row = m / g.nx;
-    const int64_t j = row * g.nx + log_x(g, (int)(m - row * g.nx));
-    const int k = node_type ? (int)node_type[m] : 0;
-    const double lr = (double)lam[m];
-    for (int i = 0; i < g.d; ++i)
-      acc += (double)lam[(1 + i) * N + m] * (double)Store<S>::from(state[(1 + i) * N + m]);
-    if (k > 0 && k <= n_wall_ids) {
-      if (grho) grho[j] = T(0);
-      if (wall) atomicAdd(wall + 4 * (k - 1), lr / rho0);
-      for (int i = 0; i < g.d; ++i) {
-        if (gu) gu[i * N + j] = T(0);
-        if (wall) atomicAdd(wall + 4 * (k - 1) + 1 + i, (double)lam[(1 + i) * N + m] / e);
-      }
-    } else {
-      if (grho) grho[j] = T(lr / rho0);
-      for (int i = 0; i < g.d; ++i)
-        if (gu) gu[i * N + j] = T((double)lam[(1 + i) * N + m] / e);
+  for_units<I, U>(g, [&](int64_t i, int64_t j0, int x) {
+    const int64_t j = user_index<U>(g, i, j0);
+    C l[1 + D][W];
+    S ut[D][W];
+    uint8_t kind[W];
+#pragma unroll
+    for (int f = 0; f <= D; ++f) {
+      ld_stored<W, C>(lam + f * N + i, l[f]);
+      if (f > 0) ld_stored<W, S>(state + f * N + i, ut[f - 1]);
     }
-  }
-  __shared__ double red[256];
-  red[threadIdx.x] = acc;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) atomicAdd(dot, red[0]);
+#pragma unroll
+    for (int c = 0; c < W; ++c) kind[c] = 0;
+    if (node_type) ld_stored<W, uint8_t>(node_type + i, kind);
+    A a[D * W], b[D * W];
+#pragma unroll
+    for (int f = 1; f <= D; ++f)
+#pragma unroll
+      for (int c = 0; c < W; ++c) {
+        a[(f - 1) * W + c] = (A)l[f][c];
+        b[(f - 1) * W + c] = (A)Store<S>::from(ut[f - 1][c]);
+      }
+    acc += dot_unit(a, b);
+#pragma unroll
+    for (int f = 0; f <= D; ++f) {
+      T* const p = f == 0 ? grho : gu ? gu + (f - 1) * N : nullptr;
+      T out[W];
+#pragma unroll
+      for (int c = 0; c < W; ++c) {
+        if (kind[c] > 0 && kind[c] <= n_wall_ids) {
+          out[c] = T(0);
+          if (wall) atomicAdd(wall + 4 * (kind[c] - 1) + f, (double)l[f][c] / (f == 0 ? m.rho0 : m.e));
+        } else if constexpr (FAST) {
+          out[c] = f == 0 ? __fmul_rn(l[f][c], m.f_inv_rho0) : mul_pair(l[f][c], m.ie_hi, m.ie_lo);
+        } else {
+          out[c] = T((double)l[f][c] / (f == 0 ? m.rho0 : m.e));
+        }
+      }
+      if (p) st_unit<U, T, W>(g, p, j, x, out);
+    }
+  });
+  add_block_sum(acc, dot);
 }
 
-template <typename S>
-static cudaError_t seed_t(const Geometry& g, const void* grho, const void* gu, int dtype,
-                          const void* state, double rho0, double e, void* lam, double* dot,
-                          cudaStream_t st) {
-  if (dtype == MACLAB_DTYPE_F64)
-    adj_seed<S, double><<<grid256(g.n), 256, 0, st>>>(g, (const double*)grho, (const double*)gu,
-                                                      (const S*)state, rho0, e,
-                                                      (typename Store<S>::C*)lam, dot);
-  else
-    adj_seed<S, float><<<grid256(g.n), 256, 0, st>>>(g, (const float*)grho, (const float*)gu,
-                                                     (const S*)state, rho0, e,
-                                                     (typename Store<S>::C*)lam, dot);
-  return cudaGetLastError();
+// launch(grid, index type, unit): quads where the state, lam (and the node
+// types, the library's own) are aligned to them.
+template <typename S, typename T, typename Fn>
+static cudaError_t by_adjoint_unit(const Geometry& g, const void* a, const void* b, const void* state, const void* lam,
+                                   Fn&& launch) {
+  Unit unit = unit_of(g, a, b, 2 * sizeof(T));
+  if ((reinterpret_cast<uintptr_t>(state) | reinterpret_cast<uintptr_t>(lam)) % 16 != 0) unit = kNode;
+  return by_unit(g, unit, [&](unsigned, auto index, auto u) {
+    return launch(grid256(unit == kNode ? g.n : g.n / 4), index, u);
+  });
 }
 
-template <typename S>
-static cudaError_t finish_t(const Geometry& g, const void* lam, const void* state, const uint8_t* nt,
-                            int nw, double rho0, double e, void* grho, void* gu, int dtype,
-                            double* wall, double* dot, cudaStream_t st) {
-  using C = typename Store<S>::C;
-  if (dtype == MACLAB_DTYPE_F64)
-    adj_finish<S, double><<<grid256(g.n), 256, 0, st>>>(g, (const C*)lam, (const S*)state, nt, nw,
-                                                        rho0, e, (double*)grho, (double*)gu, wall, dot);
-  else
-    adj_finish<S, float><<<grid256(g.n), 256, 0, st>>>(g, (const C*)lam, (const S*)state, nt, nw,
-                                                       rho0, e, (float*)grho, (float*)gu, wall, dot);
-  return cudaGetLastError();
+template <int D, typename S, typename T, bool FAST>
+static cudaError_t seed_t(const Geometry& g, const void* grho, const void* gu, const void* state, const UnitMap& m,
+                          void* lam, double* dot, cudaStream_t st) {
+  return by_adjoint_unit<S, T>(g, grho, gu, state, lam, [&](unsigned grid, auto index, auto unit) {
+    adj_seed<D, S, T, FAST, decltype(index), decltype(unit)::value><<<grid, 256, 0, st>>>(
+        g, (const T*)grho, (const T*)gu, (const S*)state, m, (typename Store<S>::C*)lam, dot);
+    return cudaGetLastError();
+  });
+}
+
+template <int D, typename S, typename T, bool FAST>
+static cudaError_t finish_t(const Geometry& g, const void* lam, const void* state, const uint8_t* nt, int nw,
+                            const UnitMap& m, void* grho, void* gu, double* wall, double* dot, cudaStream_t st) {
+  return by_adjoint_unit<S, T>(g, grho, gu, state, lam, [&](unsigned grid, auto index, auto unit) {
+    adj_finish<D, S, T, FAST, decltype(index), decltype(unit)::value><<<grid, 256, 0, st>>>(
+        g, (const typename Store<S>::C*)lam, (const S*)state, nt, nw, m, (T*)grho, (T*)gu, wall, dot);
+    return cudaGetLastError();
+  });
+}
+
+// fn(dimension, storage type, array type, FAST)
+template <typename S, typename Fn>
+static cudaError_t by_map(const Geometry& g, int dtype, bool fast, Fn&& fn) {
+  auto with_d = [&](auto d) {
+    if (dtype == MACLAB_DTYPE_F64) return fn(d, S{}, double{}, std::false_type{});
+    if constexpr (!std::is_same<S, double>::value)
+      if (fast) return fn(d, S{}, float{}, std::true_type{});
+    return fn(d, S{}, float{}, std::false_type{});
+  };
+  return g.d == 3 ? with_d(std::integral_constant<int, 3>{}) : with_d(std::integral_constant<int, 2>{});
+}
+template <typename Fn>
+static cudaError_t by_storage(const Geometry& g, int precision, int dtype, bool fast, Fn&& fn) {
+  switch (precision) {
+    case MACLAB_F64: return by_map<double>(g, dtype, fast, fn);
+    case MACLAB_F32: return by_map<float>(g, dtype, fast, fn);
+    case MACLAB_BF16_STORE: return by_map<__nv_bfloat16>(g, dtype, fast, fn);
+    case MACLAB_F16_STORE: return by_map<__half>(g, dtype, fast, fn);
+  }
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_adjoint_seed(const Geometry& g, int precision, const void* grho, const void* gu,
                                 int dtype, const void* state, double rho0, double e, void* lam,
                                 double* dot, cudaStream_t st) {
-  switch (precision) {
-    case MACLAB_F64: return seed_t<double>(g, grho, gu, dtype, state, rho0, e, lam, dot, st);
-    case MACLAB_F32: return seed_t<float>(g, grho, gu, dtype, state, rho0, e, lam, dot, st);
-    case MACLAB_BF16_STORE: return seed_t<__nv_bfloat16>(g, grho, gu, dtype, state, rho0, e, lam, dot, st);
-    case MACLAB_F16_STORE: return seed_t<__half>(g, grho, gu, dtype, state, rho0, e, lam, dot, st);
-  }
-  return cudaErrorInvalidValue;
+  UnitMap m;
+  const bool fast = unit_map(g, rho0, e, &m);
+  return by_storage(g, precision, dtype, fast, [&](auto d, auto s, auto t, auto f) {
+    return seed_t<decltype(d)::value, decltype(s), decltype(t), decltype(f)::value>(g, grho, gu, state, m, lam, dot, st);
+  });
 }
 
 cudaError_t launch_adjoint_finish(const Geometry& g, int precision, const void* lam, const void* state,
                                   const uint8_t* nt, int nw, double rho0, double e, void* grho,
                                   void* gu, int dtype, double* wall, double* dot, cudaStream_t st) {
-  switch (precision) {
-    case MACLAB_F64: return finish_t<double>(g, lam, state, nt, nw, rho0, e, grho, gu, dtype, wall, dot, st);
-    case MACLAB_F32: return finish_t<float>(g, lam, state, nt, nw, rho0, e, grho, gu, dtype, wall, dot, st);
-    case MACLAB_BF16_STORE:
-      return finish_t<__nv_bfloat16>(g, lam, state, nt, nw, rho0, e, grho, gu, dtype, wall, dot, st);
-    case MACLAB_F16_STORE:
-      return finish_t<__half>(g, lam, state, nt, nw, rho0, e, grho, gu, dtype, wall, dot, st);
-  }
-  return cudaErrorInvalidValue;
+  UnitMap m;
+  const bool fast = unit_map(g, rho0, e, &m);
+  return by_storage(g, precision, dtype, fast, [&](auto d, auto s, auto t, auto f) {
+    return finish_t<decltype(d)::value, decltype(s), decltype(t), decltype(f)::value>(g, lam, state, nt, nw, m, grho, gu,
+                                                                                     wall, dot, st);
+  });
 }
 
 }  // namespace maclab
