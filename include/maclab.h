@@ -155,6 +155,17 @@ maclab_status maclab_set_lattice_state(maclab_handle h, const void *state, int32
  * asynchronously on the handle's stream. */
 maclab_status maclab_step(maclab_handle h, int64_t n);
 
+/* One step from the raw state `in` to `out` (device pointers to
+ * maclab_state_bytes each, not overlapping), asynchronously on the handle's
+ * stream, without a copy: the walls are taken from `in`.  NULL `in`: the
+ * handle's state; NULL `out`: the handle's state becomes the result (and
+ * counts a step).  With `out` given the handle's state stays as it is.
+ * Errors: MACLAB_ERR_INVALID (NULL handle, out == in), MACLAB_ERR_UNSUPPORTED
+ * (domains whose rows are stored padded, 2D domains on the segment kernel
+ * that the tiled kernel does not take, pointers not aligned to 16 bytes: copy
+ * with the calls above instead). */
+maclab_status maclab_step_raw(maclab_handle h, const void *in, void *out);
+
 /* Step kernels.  MACLAB_KERNEL_AUTO lets the library choose (the default);
  * MACLAB_KERNEL_REFERENCE is the simple one-thread-per-node gather, kept as the
  * GPU-side yardstick; MACLAB_KERNEL_TILED is the staged, vectorised kernel;

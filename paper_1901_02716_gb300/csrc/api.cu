@@ -813,6 +813,39 @@ maclab_status maclab_step(maclab_handle h, int64_t n) {
   return MACLAB_OK;
 }
 
+maclab_status maclab_step_raw(maclab_handle h, const void* in, void* out) {
+  NvtxRange nvtx_range("maclab_step_raw");
+  if (!h) return fail(MACLAB_ERR_INVALID, "NULL handle");
+  if (in && in == out) return fail(MACLAB_ERR_INVALID, "out must not alias in");
+  // the segment kernel's descriptor names the handle's buffers: the tiled
+  // kernel takes its place (the same bits)
+  int kernel = h->kernel, ty = h->ty, tz = h->tz;
+  if (kernel == MACLAB_KERNEL_SEGMENT) kernel = MACLAB_KERNEL_TILED, ty = tz = 0;
+  if (h->g.pad || (kernel == MACLAB_KERNEL_TILED && !tiled_supported(h->g, h->precision, ty, tz)))
+    return fail(MACLAB_ERR_UNSUPPORTED, "the domain's rows are padded or its kernel takes no other buffers");
+  if ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) % 16 != 0)
+    return fail(MACLAB_ERR_UNSUPPORTED, "raw states must be aligned to 16 bytes");
+  DeviceGuard dg(h->device);
+  StepLaunch sl = step_launch(h, h->cur);
+  sl.ty = ty;
+  sl.tz = tz;
+  sl.seg_steps = 1;
+  if (in) sl.in = in;
+  if (out) sl.out = out;
+  // walls are not written by the step: into the output, and after an outside
+  // input into both own buffers
+  auto walls_to = [&](void* dst) { return launch_copy_walls(h->g, h->precision, h->d_node_type, sl.in, dst, h->stream); };
+  if (in || out) CUDA_TRY(walls_to(sl.out), "wall values");
+  if (in && !out) CUDA_TRY(walls_to(h->buf[h->cur]), "wall values");
+  CUDA_TRY(launch_step(sl, h->stream, kernel), "step launch");
+  if (!out) {
+    h->cur ^= 1;
+    h->steps += 1;
+    h->prev_valid = !in;
+  }
+  return MACLAB_OK;
+}
+
 maclab_status maclab_set_graph(maclab_handle h, int32_t steps) {
   if (!h) return fail(MACLAB_ERR_INVALID, "NULL handle");
   if (steps < 0 || steps > (1 << 20)) return fail(MACLAB_ERR_INVALID, "bad graph length");

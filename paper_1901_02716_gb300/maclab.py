@@ -75,6 +75,7 @@ SIGNATURES = {
     "maclab_get_lattice_state": (_S, [_H, _VP, ctypes.c_int32]),
     "maclab_set_lattice_state": (_S, [_H, _VP, ctypes.c_int32]),
     "maclab_step": (_S, [_H, ctypes.c_int64]),
+    "maclab_step_raw": (_S, [_H, _VP, _VP]),
     "maclab_sync": (_S, [_H]),
     "maclab_set_wait_limit": (_S, [_H, ctypes.c_int64]),
     "maclab_debug_segment_waits": (_S, [ctypes.c_int32, ctypes.c_int32, ctypes.c_int32, ctypes.c_int32,
@@ -263,6 +264,16 @@ def maclab_set_lattice_state(h, state):
 
 def maclab_step(h, n):
     return _check(lib().maclab_step(h, int(n)), "maclab_step")
+
+
+def maclab_step_raw(h, state_in=None, state_out=None):
+    """One step between raw states (device pointers or tensors; None: the
+    handle's own).  False where the domain does not serve it (see maclab.h)."""
+    s = lib().maclab_step_raw(h, _dev(state_in), _dev(state_out))
+    if s == ERR_UNSUPPORTED:
+        return False
+    _check(s, "maclab_step_raw")
+    return True
 
 
 def maclab_sync(h):
