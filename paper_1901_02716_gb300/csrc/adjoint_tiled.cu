@@ -1,28 +1,50 @@
-// adjoint_tiled.cu -- host side of the tiled reverse step (adjoint_tiled.cuh):
+// adjoint_tiled.cu -- host side of the tiled reverse steps (adjoint_tiled.cuh, adjoint_rows.cuh):
 // block shapes, instantiations and the launch.
 
-#include "adjoint_tiled.cuh"
+#include "adjoint_rows.cuh"
 
 namespace maclab {
 
 namespace {
 
 struct AdjShape {
-  int bxc, ry, ty;
+  int bxc, ry, ty;  // threads along x, rows with halo, rows
+  bool rows;        // adjoint_rows.cuh
 };
 
-// Widths built: D2Q9 (BXC, 1); D3Q19 (BXC, TY + 2).  FP64 up to 64 quads per row in 3D,
-// 128 in 2D.
+// Tiled reverse steps built (us a step, periodic):
+//  * adj_step_rows for natural rows in FP32 and interleaved rows in FP64, of 3
+//    to 128 nodes in 3D and to 512 in 2D.  FP32 97x96x95: 35.4 (reference kernels
+//    62.8), 33x40x50 10.5 (16.6), 255x256 5.7 (12.4); FP64 96^3: 325
+//    (adj_step_tiled 479), 256^2 18.5 (32.1).
+//  * adj_step_tiled for interleaved FP32 rows, whose threads keep twice the bytes
+//    in flight: 96^3 19.6 (adj_step_rows 27.3), 128^3 38.8 (72.5); up to 512
+//    nodes in 3D, 1024 in 2D.
+// The rest takes the reference kernels, natural FP64 rows because they are
+// faster there (97x64x64: 160, adj_step_rows 190).
+// Blocks of adj_step_rows: FP32 8 rows with the halo, 53x61x47 12.2 (10 rows, one
+// block an SM: 16.4) and 127x80x80 25.9 (6 rows: 32.7); FP64 is bound by its
+// arithmetic, not by the blocks an SM holds: 32^3 34 (10 rows: 45), but with 64
+// columns its registers spill (96^3: 356 with 64 x 8 threads).
 bool adj_shape(const Geometry& g, int precision, AdjShape* s) {
-  if (!g.ilv || precision == MACLAB_BF16_STORE || precision == MACLAB_F16_STORE) return false;
+  if (precision == MACLAB_BF16_STORE || precision == MACLAB_F16_STORE || g.nx < 3) return false;
+  const bool f64 = precision == MACLAB_F64;
+  if (f64 == (g.ilv != 0)) {  // FP32 natural, FP64 interleaved: AdjRows::NAT
+    const int pairs = (g.nx + 1) / 2;
+    if (g.d == 2) *s = pairs <= 64 ? AdjShape{64, 1, 1, true} : AdjShape{256, 1, 1, true};
+    else if (pairs <= 32) *s = AdjShape{32, 8, 6, true};
+    else if (f64) *s = pairs <= 48 ? AdjShape{48, 6, 4, true} : AdjShape{64, 6, 4, true};
+    else *s = AdjShape{64, 8, 6, true};
+    return pairs <= s->bxc;
+  }
+  if (f64) return false;
   const int bx = g.nx / 4;
   int bxc = 0;
   for (int c : {16, 32, 64, 128, 256})
     if (bx <= c) { bxc = c; break; }
   if (!bxc) return false;
   if (g.d == 2) {
-    if (precision == MACLAB_F64 && bxc > 128) return false;
-    *s = AdjShape{bxc, 1, 1};
+    *s = AdjShape{bxc, 1, 1, false};
     return true;
   }
   int ty = 0;
@@ -33,9 +55,7 @@ bool adj_shape(const Geometry& g, int precision, AdjShape* s) {
     case 128: ty = 2; break;
     default: return false;
   }
-  if (precision == MACLAB_F64 && bxc > 64) return false;
-  if ((g.periodic & 2u) && g.ny % ty != 0) return false;  // a periodic y needs whole tiles
-  *s = AdjShape{bxc, ty + 2, ty};
+  *s = AdjShape{bxc, ty + 2, ty, false};
   return true;
 }
 
@@ -53,29 +73,38 @@ template <int LAT, typename S>
 cudaError_t tiled_dispatch(const AdjShape& s, const AdjArgs& A, const void* sn, const void* sn1,
                            const void* lam1, void* lam0, double* gf, cudaStream_t st, int ytiles,
                            int* resident) {
-#define MACLAB_ADJ_LAUNCH(BXC, RY) \
-  launch_adj_tiled<LAT, S, BXC, RY>(A, sn, sn1, lam1, lam0, gf, st, ytiles, resident)
-  if (LAT == kD2Q9) {
-    switch (s.bxc) {
-      case 16: return MACLAB_ADJ_LAUNCH(16, 1);
-      case 32: return MACLAB_ADJ_LAUNCH(32, 1);
-      case 64: return MACLAB_ADJ_LAUNCH(64, 1);
-      case 128: return MACLAB_ADJ_LAUNCH(128, 1);
-      case 256:
-        if constexpr (sizeof(S) == 4) return MACLAB_ADJ_LAUNCH(256, 1);
-        break;
+#define MACLAB_ADJ_ROWS(BXC, RY)         \
+  if (s.rows && s.bxc == BXC && s.ry == RY) \
+    return launch_adj_rows<LAT, S, BXC, RY>(A, sn, sn1, lam1, lam0, gf, st, ytiles, resident);
+#define MACLAB_ADJ_TILED(BXC, RY) \
+  if (!s.rows && s.bxc == BXC)    \
+    return launch_adj_tiled<LAT, S, BXC, RY>(A, sn, sn1, lam1, lam0, gf, st, ytiles, resident);
+  constexpr bool f64 = sizeof(S) == 8;
+  if constexpr (LAT == kD2Q9) {
+    MACLAB_ADJ_ROWS(64, 1)
+    MACLAB_ADJ_ROWS(256, 1)
+    if constexpr (!f64) {
+      MACLAB_ADJ_TILED(16, 1)
+      MACLAB_ADJ_TILED(32, 1)
+      MACLAB_ADJ_TILED(64, 1)
+      MACLAB_ADJ_TILED(128, 1)
+      MACLAB_ADJ_TILED(256, 1)
     }
-    return cudaErrorInvalidValue;
+  } else {
+    MACLAB_ADJ_ROWS(32, 8)
+    if constexpr (f64) {
+      MACLAB_ADJ_ROWS(48, 6)
+      MACLAB_ADJ_ROWS(64, 6)
+    } else {
+      MACLAB_ADJ_ROWS(64, 8)
+      MACLAB_ADJ_TILED(16, 10)
+      MACLAB_ADJ_TILED(32, 6)
+      MACLAB_ADJ_TILED(64, 6)
+      MACLAB_ADJ_TILED(128, 4)
+    }
   }
-  switch (s.bxc * 100 + s.ry) {
-    case 1610: return MACLAB_ADJ_LAUNCH(16, 10);
-    case 3206: return MACLAB_ADJ_LAUNCH(32, 6);
-    case 6406: return MACLAB_ADJ_LAUNCH(64, 6);
-    case 12804:
-      if constexpr (sizeof(S) == 4) return MACLAB_ADJ_LAUNCH(128, 4);
-      break;
-  }
-#undef MACLAB_ADJ_LAUNCH
+#undef MACLAB_ADJ_ROWS
+#undef MACLAB_ADJ_TILED
   return cudaErrorInvalidValue;
 }
 

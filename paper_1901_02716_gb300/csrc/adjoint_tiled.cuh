@@ -1,4 +1,4 @@
-// adjoint_tiled.cuh -- tiled reverse step for domains stored with interleaved
+// adjoint_tiled.cuh -- tiled FP32 reverse step for domains stored with interleaved
 // row halves (nx % 4 == 0).  Same arithmetic as adjoint.cu:
 //   L_r(x) = lam_rho'(x) - lam_u'(x) . (u'(x) - force) / rho'(x),  L_m(x) = lam_u'(x) / rho'(x),
 //   g_a(x) = L_r(x) + c_a . L_m(x),

@@ -893,7 +893,7 @@ maclab_status maclab_adjoint_step(maclab_handle h, const void* state_n, const vo
   if (lam_n == lam_np1) return fail(MACLAB_ERR_INVALID, "lam_n must not alias lam_np1");
   DeviceGuard dg(h->device);
   // the tiled reverse step where it is built (unless the reference kernel was chosen)
-  const bool tiled = h->kernel != MACLAB_KERNEL_REFERENCE && tiled_adjoint_supported(h->raw, h->precision);
+  const bool tiled = !h->reference_asked && tiled_adjoint_supported(h->raw, h->precision);
   maclab_status s = ensure_adjoint(h, !tiled);
   if (s != MACLAB_OK) return s;
   if (tiled) {
@@ -1166,6 +1166,7 @@ maclab_status maclab_set_kernel(maclab_handle h, int32_t kernel) {
   if (!h) return fail(MACLAB_ERR_INVALID, "NULL handle");
   drop_graphs(h);
   if (kernel == MACLAB_KERNEL_AUTO) {
+    h->reference_asked = false;
     h->kernel = pick_step_kernel(h->g, h->precision);
     return MACLAB_OK;
   }
@@ -1177,6 +1178,7 @@ maclab_status maclab_set_kernel(maclab_handle h, int32_t kernel) {
   if (!step_kernel_supported(h->raw, h->precision, kernel))
     return fail(MACLAB_ERR_UNSUPPORTED, "kernel does not support this domain");
   h->kernel = kernel;
+  h->reference_asked = kernel == MACLAB_KERNEL_REFERENCE;
   // a tile shape the new kernel lacks falls back to its default
   if (kernel == MACLAB_KERNEL_FOLDED && !fold_supported(h->g, h->precision, h->ty)) h->ty = 0;
   if (kernel == MACLAB_KERNEL_ROWS2 && !rows2_supported(h->g, h->precision, h->ty)) h->ty = 0;
