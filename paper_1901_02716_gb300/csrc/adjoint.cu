@@ -212,26 +212,6 @@ __global__ void __launch_bounds__(256) adj_gather(Geometry g, const S* __restric
 // the end-point products lam_T . ut_T and lam_0 . ut_0, which nearly cancel.
 // Sums use the integer weights 36 w_a and drop their constant parts exactly
 // (sum 36 w_a = 36, sum 36 w_a c_a = 0).
-// Running sum of one thread: FP64 for FP64 storage; float-float (Knuth's
-// two-sum, the error of every FP32 addition kept in lo) otherwise, so the
-// per-node terms, formed in FP32, are added without FP64 arithmetic.
-template <typename C>
-struct NuAcc {
-  double v = 0.0;
-  __device__ __forceinline__ void add(double x) { v += x; }
-  __device__ __forceinline__ double value() const { return v; }
-};
-template <>
-struct NuAcc<float> {
-  float hi = 0.f, lo = 0.f;
-  __device__ __forceinline__ void add(float x) {
-    const float s = __fadd_rn(hi, x);
-    const float bb = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(x, bb)));
-    hi = s;
-  }
-  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
 
 // One thread per node along the grid stride; the node's storage coordinates
 // advance with the stride (no division per node), and the storage offsets of

@@ -17,6 +17,7 @@
 // in FP64 by the arithmetic pipe (96^3: 325 us, the direct sums 478).
 #pragma once
 #include "adjoint_tiled.cuh"
+#include "units.cuh"
 
 namespace maclab {
 
@@ -74,7 +75,7 @@ __global__ void __launch_bounds__(BXC * RY, (AdjRows<LAT, S, BXC, RY>::MIN_BLOCK
   pdl_wait();  // the previous kernel's writes are visible from here on
   pdl_launch_next();
   const int tx = threadIdx.x, r = threadIdx.y;
-    const int H = (A.nx + 1) >> 1;
+  const int H = (A.nx + 1) >> 1;
   const int bxr = H;
   const bool active = tx < bxr;
 
@@ -100,11 +101,10 @@ __global__ void __launch_bounds__(BXC * RY, (AdjRows<LAT, S, BXC, RY>::MIN_BLOCK
   auto plane_exists = [&](int p) { return (p >= 0 && p < A.nplanes) || A.pz; };
   auto plane_mem = [&](int p) { return p < 0 ? p + A.nplanes : (p >= A.nplanes ? p - A.nplanes : p); };
 
-  // wall lanes (a.x, a.y, b.x, b.y) as bits 0..3; box walls off the march axis are fixed per thread
+  // wall lanes as bits 0 and 1; box walls off the march axis are fixed per thread
   uint32_t box_bits = 0;
   if (A.wall_mode == kWallBox) {
-    if (!A.px) box_bits |= (tx == 0 ? 1u : 0u) | (tx == A.nx - 1 - H ? 2u : 0u) |
-                           (two ? 0u : 2u);
+    if (!A.px) box_bits |= (tx == 0 ? 1u : 0u) | (tx == A.nx - 1 - H || !two ? 2u : 0u);
     if (D == 3 && !A.py && (row_mem == 0 || row_mem == A.ny - 1)) box_bits = 3u;
   }
 
@@ -399,40 +399,242 @@ __global__ void __launch_bounds__(BXC * RY, (AdjRows<LAT, S, BXC, RY>::MIN_BLOCK
   }
 }
 
-// Launch helper (instantiated in adjoint_tiled.cu).  Returns the number of
-// blocks of this shape one SM holds through *resident.
-template <int LAT, typename S, int BXC, int RY>
-cudaError_t launch_adj_rows(const AdjArgs& A, const void* in_state, const void* out_state,
-                             const void* lam1, void* lam0, double* grad_force, cudaStream_t st,
-                             int ytiles, int* resident_out) {
-  using T = AdjRows<LAT, S, BXC, RY>;
-  using C = typename T::C;
-  auto kern = adj_step_rows<LAT, S, BXC, RY>;
+// The viscosity term of adjoint.cu (its definition and sums) on natural FP32
+// rows of D3Q19, given the state after the step (m' / rho' = u' - F there), with
+// the same staging of the state alone.  Of a source (drho, u) with
+// e = 3/2 rho u.u, r = rho c.u and h = 9/2 rho (c.u)^2, direction c carries
+//   w (drho + e - h)         to sum c w rho (1 - 9/2 (c.u)^2 + 3/2 u.u) and
+//   w (3 r + 2 (h - e))      to sum dF;
+// h is shared by c and -c, so by the planes above and below.  97x96x95: 32.6 us,
+// the per-node kernel of adjoint.cu (19 gathers of four values) 47.2; 127x80x80
+// 23.8 and 43.1, 25^3 6.6 and 8.2.  Bound by latency, one block an SM.
+template <int BXC, int RY>
+__global__ void __launch_bounds__(BXC * RY, (AdjRows<kD3Q19, float, BXC, RY>::MIN_BLOCKS))
+    adj_nu_rows(AdjArgs A, const float* __restrict__ state, const float* __restrict__ next,
+                const float* __restrict__ lam, double* __restrict__ acc) {
+  using T = AdjRows<kD3Q19, float, BXC, RY>;
+  using O = Pair<float>;
+  using P = float2;
+  using U = AdjUnit<P>;
+  extern __shared__ __align__(16) uint4 units[];
+  pdl_wait();  // the previous kernel's writes are visible from here on
+  pdl_launch_next();
+  const int tx = threadIdx.x, r = threadIdx.y;
+  const int H = (A.nx + 1) >> 1;
+  const int row = blockIdx.y * A.ty + r - 1;
+  const bool active = tx < H;
+  const bool interior = active && r >= 1 && r <= RY - 2 && row < A.ny;
+  const bool inside = row >= 0 && row < A.ny;
+  const int row_mem = inside ? row : (row + A.ny) % A.ny;
+  const bool stages_own = active && (inside || A.py);
+  const int64_t row_off = (int64_t)row_mem * A.nx + tx;
+  const bool two = tx + H < A.nx;  // lane y of the last pair of an odd row is the image of node 0
+  const int hi = two ? H : -tx;
+  const int z0 = (int)(((int64_t)blockIdx.x * A.nplanes) / A.nzc);
+  const int z1 = (int)(((int64_t)(blockIdx.x + 1) * A.nplanes) / A.nzc);
+  auto ld = [&](const float* p) { return make_float2(p[0], p[hi]); };
+
+  struct Raw {
+    P st[4];
+  };
+  auto load_raw = [&](int p, Raw& R) {
+    const bool have = stages_own && ((p >= 0 && p < A.nplanes) || A.pz);
+    const int pm = p < 0 ? p + A.nplanes : (p >= A.nplanes ? p - A.nplanes : p);
+#pragma unroll
+    for (int f = 0; f < 4; ++f)
+      R.st[f] = have ? ld(state + f * A.n + (int64_t)pm * A.plane_stride + row_off) : make_float2(0.f, 0.f);
+  };
+  auto stage = [&](int p, const Raw& R) {
+    if (!active) return;
+    const int k = p & (T::STAGES - 1);
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      U::st(&units[T::unit(k, r, u, tx)], &R.st[2 * u]);
+      // the left neighbours (nx - 1, H - 1) of the first pair
+      float* const seam = reinterpret_cast<float*>(&units[T::unit(k, r, u, T::SEAM_L)]);
+      if (tx == A.nx - 1 - H) seam[0] = R.st[2 * u].y, seam[2] = R.st[2 * u + 1].y;
+      if (tx == H - 1) seam[1] = R.st[2 * u].x, seam[3] = R.st[2 * u + 1].x;
+      if (tx == 0) U::st_swapped(&units[T::unit(k, r, u, T::SEAM_R)], &R.st[2 * u]);
+    }
+  };
+  const int col_l = tx == 0 ? T::SEAM_L : tx - 1;
+  const int col_r = tx == H - 1 ? T::SEAM_R : tx + 1;
+  // a source and what its directions share
+  struct Src {
+    P a, e, rho, u[3];
+  };
+  auto src = [&](int cx, int cy, int p) {  // the source of direction (cx, cy)
+    P v[4];
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+      U::ld(&units[T::unit(p & (T::STAGES - 1), r - cy, u, cx == 0 ? tx : cx == 1 ? col_l : col_r)], &v[2 * u]);
+    Src s;
+    s.rho = O::add(O::splat(1.f), v[0]);
+    const P uu = O::fma(v[1], v[1], O::fma(v[2], v[2], O::mul(v[3], v[3])));
+    s.e = O::mul(O::mul(uu, O::splat(1.5f)), s.rho);
+    s.a = O::add(v[0], s.e);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) s.u[i] = v[1 + i];
+    return s;
+  };
+  // weights of one: g to the momentum sums, the return value to sum dF
+  auto dir = [&](const Src& s, P t, P& g) {
+    const P rt = O::mul(s.rho, t), h = O::mul(O::mul(t, O::splat(4.5f)), rt);
+    g = adj_sub<float>(s.a, h);
+    const P d = adj_sub<float>(h, s.e);
+    return O::fma(rt, O::splat(3.f), O::add(d, d));
+  };
+  struct Sums {
+    P d, m[3];
+  };
+  Sums pend{}, below{};  // of plane p - 1: without the plane above; what plane p - 1 sends up
+  NuAcc<float> total;
+  Raw R;
+  load_raw(z0 - 1, R);
+  stage(z0 - 1, R);
+  load_raw(z0, R);
+  for (int p = z0 - 1; p <= z1; ++p) {
+    const int q = p - 1;  // the plane this one completes
+    __syncthreads();      // plane p is staged, the reads of plane p - 1 are done
+    if (p < z1) {
+      stage(p + 1, R);
+      if (p + 1 < z1) load_raw(p + 2, R);
+    }
+    if (!interior) continue;
+    P nx4[4], lm[4];
+    if (q >= z0) {
+      const int64_t off = (int64_t)q * A.plane_stride + row_off;
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        nx4[f] = ld(next + f * A.n + off);
+        lm[f] = ld(lam + f * A.n + off);
+      }
+    }
+    Sums own, up, dn;  // destinations in this plane, above (c_z = 1), below (c_z = -1)
+    P g;
+    {
+      const Src s = src(0, 0, p);
+      own.d = O::mul(s.e, O::splat(-24.f));
+      own.m[0] = own.m[1] = own.m[2] = O::splat(0.f);
+      const P d = dir(s, s.u[2], g), r3 = O::mul(O::mul(s.rho, s.u[2]), O::splat(6.f));
+      up.d = O::add(d, d);
+      dn.d = adj_sub<float>(adj_sub<float>(up.d, r3), r3);
+      up.m[2] = O::add(g, g);
+      dn.m[2] = O::mul(g, O::splat(-2.f));
+      up.m[0] = up.m[1] = dn.m[0] = dn.m[1] = O::splat(0.f);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int i = k >> 1, sg = 1 - 2 * (k & 1);  // the axis and its sign
+      const Src s = src(i == 0 ? sg : 0, i == 1 ? sg : 0, p);
+      const P t = O::mul(s.u[i], O::splat(float(sg)));
+      P d = dir(s, t, g);
+      own.d = O::fma(d, O::splat(2.f), own.d);
+      own.m[i] = O::fma(g, O::splat(2.f * sg), own.m[i]);
+      d = dir(s, O::add(t, s.u[2]), g);
+      up.d = O::add(up.d, d);
+      up.m[i] = O::fma(g, O::splat(float(sg)), up.m[i]);
+      up.m[2] = O::add(up.m[2], g);
+      d = dir(s, adj_sub<float>(t, s.u[2]), g);
+      dn.d = O::add(dn.d, d);
+      dn.m[i] = O::fma(g, O::splat(float(sg)), dn.m[i]);
+      dn.m[2] = adj_sub<float>(dn.m[2], g);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int cx = 1 - 2 * (k & 1), cy = 1 - (k & 2);
+      const Src s = src(cx, cy, p);
+      const P t = O::fma(s.u[0], O::splat(float(cx)), O::mul(s.u[1], O::splat(float(cy))));
+      own.d = O::add(own.d, dir(s, t, g));
+      own.m[0] = O::fma(g, O::splat(float(cx)), own.m[0]);
+      own.m[1] = O::fma(g, O::splat(float(cy)), own.m[1]);
+    }
+    if (q >= z0) {
+      const P k36 = O::splat(1.f / 36.f);
+      const P inv = O::rcp(O::add(O::splat(1.f), nx4[0]));
+      const P dR = O::mul(O::add(pend.d, dn.d), k36);
+      P t = adj_sub<float>(O::splat(0.f), O::mul(lm[0], dR));
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const P f = O::splat(float(A.force[i]));
+        const P unf = adj_sub<float>(nx4[1 + i], f);  // m' / rho'
+        const P md = O::mul(O::add(pend.m[i], dn.m[i]), k36);
+        t = O::fma(lm[1 + i], adj_sub<float>(O::mul(O::fma(unf, dR, md), inv), f), t);
+      }
+      bool w0 = false, w1 = !two;
+      if (A.wall_mode == kWallMask) {
+        const uint8_t* const mk = A.mask + (int64_t)q * A.plane_stride + row_off;
+        w0 = mk[0];
+        w1 = w1 || mk[hi];
+      } else if (A.wall_mode == kWallBox) {
+        const bool all = (!A.pz && (q == 0 || q == A.nplanes - 1)) || (!A.py && (row == 0 || row == A.ny - 1));
+        w0 = all || (!A.px && tx == 0);
+        w1 = w1 || all || (!A.px && tx == A.nx - 1 - H);
+      }
+      if (!w0) total.add(t.x);
+      if (!w1) total.add(t.y);
+    }
+    pend.d = O::add(own.d, below.d);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) pend.m[i] = O::add(own.m[i], below.m[i]);
+    below = up;
+  }
+  // block sum: warp shuffles, one value per warp, one FP64 atomic per block
+  double v = total.value();
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  __shared__ double red[32];
+  const int id = threadIdx.y * blockDim.x + threadIdx.x;
+  if ((id & 31) == 0) red[id >> 5] = v;
+  __syncthreads();
+  if (id == 0) {
+    for (int w = 1; w < (int)(blockDim.x * blockDim.y) >> 5; ++w) v += red[w];
+    atomicAdd(acc, v);
+  }
+}
+
+// Launch helper of both kernels (instantiated in adjoint_tiled.cu): the arguments
+// after A go to the kernel.  Returns the number of blocks of this shape one SM
+// holds through *resident.
+template <typename T, int BXC, int RY, typename Kern, typename... Args>
+cudaError_t launch_rows(Kern kern, const AdjArgs& A, cudaStream_t st, int ytiles, int* resident, Args... args) {
   constexpr size_t smem = T::smem_bytes();
   static int resident_dev[64] = {};  // per instantiation and device
   int dev = 0;
   cudaError_t e0 = cudaGetDevice(&dev);
   if (e0 != cudaSuccess) return e0;
-  int& resident = resident_dev[dev & 63];
-  if (!resident) {
+  if (resident && (*resident = resident_dev[dev & 63])) return cudaSuccess;
+  if (resident) {  // sizing query only
     if (smem > 48 * 1024) {
       cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
     }
     int nb = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, T::THREADS, smem);
-    if (e != cudaSuccess) return e;
-    resident = nb < 1 ? 1 : nb;
-  }
-  if (resident_out) {  // sizing query only
-    *resident_out = resident;
-    return cudaSuccess;
+    if (e == cudaSuccess) *resident = resident_dev[dev & 63] = nb < 1 ? 1 : nb;
+    return e;
   }
   const int unit = RY % 4 == 0 ? 8 : RY % 2 == 0 ? 16 : 32;  // whole warps a block
   const int width = ((A.nx + 1) / 2 + unit - 1) / unit * unit;
-  return launch_kernel(kern, dim3(A.nzc, ytiles), dim3(width, RY), smem, st, A.overlap, A,
-                       static_cast<const S*>(in_state), static_cast<const S*>(out_state),
-                       static_cast<const C*>(lam1), static_cast<C*>(lam0), grad_force);
+  return launch_kernel(kern, dim3(A.nzc, ytiles), dim3(width, RY), smem, st, A.overlap, A, args...);
+}
+
+template <int LAT, typename S, int BXC, int RY>
+cudaError_t launch_adj_rows(const AdjArgs& A, const void* in_state, const void* out_state, const void* lam1, void* lam0,
+                            double* grad_force, cudaStream_t st, int ytiles, int* resident) {
+  using T = AdjRows<LAT, S, BXC, RY>;
+  using C = typename T::C;
+  return launch_rows<T, BXC, RY>(adj_step_rows<LAT, S, BXC, RY>, A, st, ytiles, resident,
+                                 static_cast<const S*>(in_state), static_cast<const S*>(out_state),
+                                 static_cast<const C*>(lam1), static_cast<C*>(lam0), grad_force);
+}
+
+template <int BXC, int RY>
+cudaError_t launch_nu_rows(const AdjArgs& A, const void* state, const void* next, const void* lam, double* acc,
+                           cudaStream_t st, int ytiles, int* resident) {
+  return launch_rows<AdjRows<kD3Q19, float, BXC, RY>, BXC, RY>(
+      adj_nu_rows<BXC, RY>, A, st, ytiles, resident, static_cast<const float*>(state), static_cast<const float*>(next),
+      static_cast<const float*>(lam), acc);
 }
 
 }  // namespace maclab

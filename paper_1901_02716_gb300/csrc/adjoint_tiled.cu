@@ -69,6 +69,37 @@ int sms() {
   return n;
 }
 
+AdjArgs adj_args(const Geometry& g, int ty, const double* force, int overlap) {
+  AdjArgs A{};
+  A.overlap = overlap;
+  A.nx = g.nx;
+  A.ny = g.d == 3 ? g.ny : 1;
+  A.nplanes = g.d == 3 ? g.nz : g.ny;
+  A.n = g.n;
+  A.plane_stride = (int64_t)g.nx * A.ny;
+  A.ty = ty;
+  A.px = (g.periodic & 1u) ? 1 : 0;
+  A.py = g.d == 3 ? ((g.periodic & 2u) ? 1 : 0) : 0;
+  A.pz = g.d == 3 ? ((g.periodic & 4u) ? 1 : 0) : ((g.periodic & 2u) ? 1 : 0);
+  A.wall_mode = g.wall_mode;
+  A.mask = g.mask;
+  for (int i = 0; i < 3; ++i) A.force[i] = force[i];
+  return A;
+}
+
+// Blocks along the march axis.
+int adj_chunks(int nplanes, int ytiles, int resident) {
+  // about 8 planes per block, rounded up to whole waves of resident blocks
+  int nzc = (nplanes + 7) / 8;
+  const long slots = (long)resident * sms();
+  const long blocks = (long)nzc * ytiles;
+  const long waves = (blocks + slots - 1) / slots;
+  nzc = (int)((waves * slots) / ytiles);
+  if (nzc > nplanes / 2) nzc = nplanes / 2 > 0 ? nplanes / 2 : 1;
+  if (nzc < 1) nzc = 1;
+  return nzc;
+}
+
 template <int LAT, typename S>
 cudaError_t tiled_dispatch(const AdjShape& s, const AdjArgs& A, const void* sn, const void* sn1,
                            const void* lam1, void* lam0, double* gf, cudaStream_t st, int ytiles,
@@ -112,33 +143,12 @@ template <int LAT, typename S>
 cudaError_t tiled_adjoint_t(const Geometry& g, const AdjShape& s, const void* sn, const void* sn1,
                             const void* lam1, void* lam0, const double* force, double* gf,
                             int overlap, cudaStream_t st) {
-  AdjArgs A{};
-  A.overlap = overlap;
-  A.nx = g.nx;
-  A.ny = g.d == 3 ? g.ny : 1;
-  A.nplanes = g.d == 3 ? g.nz : g.ny;
-  A.n = g.n;
-  A.plane_stride = (int64_t)g.nx * A.ny;
-  A.ty = s.ty;
-  A.px = (g.periodic & 1u) ? 1 : 0;
-  A.py = g.d == 3 ? ((g.periodic & 2u) ? 1 : 0) : 0;
-  A.pz = g.d == 3 ? ((g.periodic & 4u) ? 1 : 0) : ((g.periodic & 2u) ? 1 : 0);
-  A.wall_mode = g.wall_mode;
-  A.mask = g.mask;
-  for (int i = 0; i < 3; ++i) A.force[i] = force[i];
+  AdjArgs A = adj_args(g, s.ty, force, overlap);
   const int ytiles = g.d == 3 ? (A.ny + s.ty - 1) / s.ty : 1;
   int resident = 0;
   cudaError_t e = tiled_dispatch<LAT, S>(s, A, sn, sn1, lam1, lam0, gf, st, ytiles, &resident);
   if (e != cudaSuccess) return e;
-  // about 8 planes per block, rounded up to whole waves of resident blocks
-  int nzc = (A.nplanes + 7) / 8;
-  const long slots = (long)resident * sms();
-  const long blocks = (long)nzc * ytiles;
-  const long waves = (blocks + slots - 1) / slots;
-  nzc = (int)((waves * slots) / ytiles);
-  if (nzc > A.nplanes / 2) nzc = A.nplanes / 2 > 0 ? A.nplanes / 2 : 1;
-  if (nzc < 1) nzc = 1;
-  A.nzc = nzc;
+  A.nzc = adj_chunks(A.nplanes, ytiles, resident);
   return tiled_dispatch<LAT, S>(s, A, sn, sn1, lam1, lam0, gf, st, ytiles, nullptr);
 }
 
@@ -162,6 +172,28 @@ cudaError_t launch_tiled_adjoint(const Geometry& g, int precision, const void* s
   if (precision == MACLAB_F64)
     return tiled_adjoint_t<kD3Q19, double>(g, s, state_n, state_np1, lam_np1, lam_n, force_lat, grad_force, overlap, st);
   return tiled_adjoint_t<kD3Q19, float>(g, s, state_n, state_np1, lam_np1, lam_n, force_lat, grad_force, overlap, st);
+}
+
+bool rows_nu_supported(const Geometry& g, int precision) {
+  AdjShape s;
+  return precision == MACLAB_F32 && g.d == 3 && adj_shape(g, precision, &s) && s.rows;
+}
+
+cudaError_t launch_rows_nu(const Geometry& g, const void* state_n, const void* state_np1, const void* lam_np1,
+                           const double force_lat[3], double* acc, int overlap, cudaStream_t st) {
+  AdjShape s;
+  if (!rows_nu_supported(g, MACLAB_F32) || !adj_shape(g, MACLAB_F32, &s)) return cudaErrorInvalidValue;
+  AdjArgs A = adj_args(g, s.ty, force_lat, overlap);
+  const int ytiles = (A.ny + s.ty - 1) / s.ty;
+  auto launch = [&](int* resident) {
+    return s.bxc == 32 ? launch_nu_rows<32, 8>(A, state_n, state_np1, lam_np1, acc, st, ytiles, resident)
+                       : launch_nu_rows<64, 8>(A, state_n, state_np1, lam_np1, acc, st, ytiles, resident);
+  };
+  int resident = 0;
+  const cudaError_t e = launch(&resident);
+  if (e != cudaSuccess) return e;
+  A.nzc = adj_chunks(A.nplanes, ytiles, resident);
+  return launch(nullptr);
 }
 
 }  // namespace maclab

@@ -921,6 +921,11 @@ maclab_status maclab_adjoint_nu_term(maclab_handle h, const void* state_n, const
              "adjoint nu term (two-rows kernel)");
     return MACLAB_OK;
   }
+  if (state_np1 && !h->reference_asked && rows_nu_supported(h->raw, h->precision)) {
+    CUDA_TRY(launch_rows_nu(h->raw, state_n, state_np1, lam_np1, h->force_lat, acc, h->overlap, h->stream),
+             "adjoint nu term (natural rows)");
+    return MACLAB_OK;
+  }
   CUDA_TRY(launch_adjoint_nu_term(h->raw, h->precision, state_n, lam_np1, h->force_lat, acc, h->stream),
            "adjoint nu term");
   return MACLAB_OK;

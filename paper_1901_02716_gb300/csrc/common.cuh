@@ -321,6 +321,9 @@ cudaError_t launch_rows2(const StepLaunch& s, cudaStream_t stream, int ty, int t
 // The viscosity term of one reverse step (maclab_adjoint_nu_term) on the two-rows
 // kernel: FP32 storage where the step kernel is built; acc += the sum.
 bool rows2_nu_supported(const Geometry& g, int precision);
+bool rows_nu_supported(const Geometry& g, int precision);  // natural rows
+cudaError_t launch_rows_nu(const Geometry& g, const void* state_n, const void* state_np1, const void* lam_np1,
+                           const double force_lat[3], double* acc, int overlap, cudaStream_t st);
 cudaError_t launch_rows2_nu(const Geometry& g, const void* state_n, const void* state_np1, const float* lam,
                             const double force[3], double* acc, int overlap, cudaStream_t stream);
 

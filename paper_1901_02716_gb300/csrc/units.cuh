@@ -172,4 +172,25 @@ static cudaError_t by_unit(const Geometry& g, Unit unit, Fn&& launch) {
   return small_index(g.n) ? with_index(uint32_t{}) : with_index(int64_t{});
 }
 
+// Running sum of one thread: FP64 for FP64 storage; float-float (Knuth's
+// two-sum, the error of every FP32 addition kept in lo) otherwise, so the
+// per-node terms, formed in FP32, are added without FP64 arithmetic.
+template <typename C>
+struct NuAcc {
+  double v = 0.0;
+  __device__ __forceinline__ void add(double x) { v += x; }
+  __device__ __forceinline__ double value() const { return v; }
+};
+template <>
+struct NuAcc<float> {
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float s = __fadd_rn(hi, x);
+    const float bb = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(x, bb)));
+    hi = s;
+  }
+  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+
 }  // namespace maclab

@@ -52,3 +52,27 @@ def test_reverse_step_on_any_rows(lat, dims, periodic, walls, precision):
     assert np.abs(u1 - u2).max() <= tol * np.abs(u1).max()
     assert np.allclose(w1, w2, rtol=tol * 10, atol=tol * max(np.abs(r1).max(), np.abs(u1).max()))
     assert np.allclose(f1, f2, rtol=1e-6 if precision == M.F32 else 1e-12, atol=tol * np.abs(u1).max())
+
+
+@pytest.mark.parametrize("dims,periodic,walls", [
+    ((3, 3, 3), 0b111, "none"), ((5, 6, 4), 0b111, "none"), ((7, 13, 5), 0b000, "box"), ((63, 9, 8), 0b101, "mixed"),
+    ((65, 10, 9), 0b111, "none"), ((97, 11, 6), 0b011, "box"), ((127, 5, 7), 0b110, "mixed"), ((30, 7, 33), 0b100, "box")])
+def test_viscosity_term_on_natural_rows(dims, periodic, walls):
+    """The pass over natural rows (the state after the step given) against the
+    per-node kernel.  A node's term is a sum of about 40 products of lam with
+    values below 0.1 (second order in u = 0.08, first in drho = 0.02), so both
+    differ by at most 40 * 0.1 * 2^-24 < 2^-21 of the sum of |lam|."""
+    torch = pytest.importorskip("torch")
+    case = inputs.random_case(D3, dims, periodic, seed=80, u_amp=0.08, rho_amp=0.02, walls=walls, force=(3e-4,) * 3)
+    with M.Solver.from_case(case, M.F32) as s:
+        s0, s1 = (torch.empty(s.state_bytes(), dtype=torch.uint8, device="cuda") for _ in range(2))
+        s.get_lattice_state(s0)
+        s.step(1)
+        s.get_lattice_state(s1)
+        g = inputs.rng(81)
+        lam = torch.tensor(g.standard_normal(s.adjoint_bytes() // 4), dtype=torch.float32, device="cuda")
+        node, rows = (torch.zeros(1, dtype=torch.float64, device="cuda") for _ in range(2))
+        M.maclab_adjoint_nu_term(s.handle, s0, lam, node)
+        M.maclab_adjoint_nu_term(s.handle, s0, lam, rows, s1)
+    assert abs(float(node) - float(rows)) <= 2.0 ** -21 * float(lam.abs().double().sum())
+    assert float(node) != 0.0
