@@ -145,7 +145,8 @@ def traffic_from_profiles(kernel_tag, source_hash):
 def step_source_hash():
     h = hashlib.sha256()
     for f in ("step.cu", "step_tiled.cuh", "step_tiled.cu", "step_fold.cuh", "step_fold.cu", "lattice.cuh",
-              "common.cuh", "step_rows2.cuh", "step_rows2.cu"):
+              "common.cuh", "step_rows2.cuh", "step_rows2.cu", "d2q9.cuh", "d3q19.cuh", "step_rows2_f32.cu",
+              "step_rows2_f32_any.cu", "step_fold_f32.cu", "step_fold_f32_any.cu"):
         with open(os.path.join(ROOT, "paper_1901_02716_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

@@ -203,6 +203,11 @@ __global__ void __launch_bounds__(BXC * RY, (AdjRows<LAT, S, BXC, RY>::MIN_BLOCK
   const int col_l = tx == 0 ? T::SEAM_L : tx - 1;
   const int col_r = tx == bxr - 1 ? T::SEAM_R : tx + 1;
   constexpr int iy = D == 3 ? 1 : 0, iz = D - 1;  // components along y (3D) and the march axis
+  // The rounded weights are those of the reference kernels: 1 / 36 scales all
+  // (axes: twice that), and a rest weight rounded by itself differs from wc / 36
+  // by a little more.  In sum lam grows by 1.5e-8 a step, as there; dL/dnu keeps
+  // the offset against the forward steps' rounding that it had with them.
+  constexpr C rest = C((double)(C(D == 3 ? 12 : 16) / C(36)) / (double)C(1.0 / 36.0) - (D == 3 ? 12.0 : 16.0));
   constexpr int wc = D == 3 ? 12 : 16, wa = D == 3 ? 2 : 4;  // 36 w: rest, axes (diagonals 1)
 
   AdjPend<P> pend{};    // of plane p - 1: its own plane's sums and those from below
@@ -255,7 +260,7 @@ __global__ void __launch_bounds__(BXC * RY, (AdjRows<LAT, S, BXC, RY>::MIN_BLOCK
     AdjPend<P> own{};
     own.x = O::mul(de, O::splat(C(wa)));
     own.xx = O::mul(se, O::splat(C(wa)));
-    own.g0 = O::fma(vc[0], O::splat(C(wc)), own.xx);
+    own.g0 = O::fma(vc[0], O::splat(C(wc)), O::fma(vc[0], O::splat(rest), own.xx));
     if constexpr (D == 3) {
       P vn[NU * G], vs[NU * G];
       rec(0, 1, vn);
@@ -405,9 +410,9 @@ __global__ void __launch_bounds__(BXC * RY, (AdjRows<LAT, S, BXC, RY>::MIN_BLOCK
 // e = 3/2 rho u.u, r = rho c.u and h = 9/2 rho (c.u)^2, direction c carries
 //   w (drho + e - h)         to sum c w rho (1 - 9/2 (c.u)^2 + 3/2 u.u) and
 //   w (3 r + 2 (h - e))      to sum dF;
-// h is shared by c and -c, so by the planes above and below.  97x96x95: 32.6 us,
+// h is shared by c and -c, so by the planes above and below.  97x96x95: 34.0 us,
 // the per-node kernel of adjoint.cu (19 gathers of four values) 47.2; 127x80x80
-// 23.8 and 43.1, 25^3 6.6 and 8.2.  Bound by latency, one block an SM.
+// 24.6 and 43.1, 25^3 7.2 and 8.2.  Bound by latency, one block an SM.
 template <int BXC, int RY>
 __global__ void __launch_bounds__(BXC * RY, (AdjRows<kD3Q19, float, BXC, RY>::MIN_BLOCKS))
     adj_nu_rows(AdjArgs A, const float* __restrict__ state, const float* __restrict__ next,
@@ -550,16 +555,16 @@ __global__ void __launch_bounds__(BXC * RY, (AdjRows<kD3Q19, float, BXC, RY>::MI
       own.m[1] = O::fma(g, O::splat(float(cy)), own.m[1]);
     }
     if (q >= z0) {
-      const P k36 = O::splat(1.f / 36.f);
       const P inv = O::rcp(O::add(O::splat(1.f), nx4[0]));
-      const P dR = O::mul(O::add(pend.d, dn.d), k36);
+      const P dR = O::add(pend.d, dn.d);  // x 36, as all below
       P t = adj_sub<float>(O::splat(0.f), O::mul(lm[0], dR));
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
         const P f = O::splat(float(A.force[i]));
         const P unf = adj_sub<float>(nx4[1 + i], f);  // m' / rho'
-        const P md = O::mul(O::add(pend.m[i], dn.m[i]), k36);
-        t = O::fma(lm[1 + i], adj_sub<float>(O::mul(O::fma(unf, dR, md), inv), f), t);
+        const P md = O::add(pend.m[i], dn.m[i]);
+        const P du = O::mul(O::fma(unf, dR, md), inv);
+        t = O::fma(lm[1 + i], O::fma(f, O::splat(-36.f), du), t);
       }
       bool w0 = false, w1 = !two;
       if (A.wall_mode == kWallMask) {
@@ -589,7 +594,7 @@ __global__ void __launch_bounds__(BXC * RY, (AdjRows<kD3Q19, float, BXC, RY>::MI
   __syncthreads();
   if (id == 0) {
     for (int w = 1; w < (int)(blockDim.x * blockDim.y) >> 5; ++w) v += red[w];
-    atomicAdd(acc, v);
+    atomicAdd(acc, v / 36.0);
   }
 }
 

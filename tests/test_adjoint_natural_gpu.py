@@ -1,6 +1,5 @@
 """The tiled reverse step on rows of any width (natural rows, odd and even, with
-the image of node 0 in the last pair's second lane) and on ragged tiles of a
-periodic y axis, against the reference two-kernel reverse step on the same
+the image of node 0 in the last pair's second lane; ragged tiles), against the reference two-kernel reverse step on the same
 states: gradients, wall sums and the force gradient.  Both sum the same terms in
 another order: bounds as for the interleaved rows (FP64 1e-12, FP32 2e-6 of the
 largest value)."""
