@@ -151,15 +151,22 @@ bool step_kernel_supported(const Geometry& g, int precision, int kernel) {
   return false;
 }
 
-// D3Q19 with FP32 or 16-bit storage: the two-rows-per-thread kernel where it
-// applies (rows of up to 128 nodes; BF16 128^3: 14.1 us a step, folded 17.0),
-// else the folded one where it is built (at least a tile of rows); for D2Q9 grids with nx % 4 == 0 the block kernel
+// D3Q19 with 16-bit storage: the folded kernel wherever its tiles are whole rows
+// of the caller's width.  The two-rows kernel is faster there (BF16 128^3: 14.1 us
+// a step, folded 17.0), but it sums in another order, and every step's rounding to
+// 16 bits shows that in the state (BF16 128^3, 20 steps: 1.2e-3 of the largest
+// value): such runs and their checkpoints keep the values they have.  Else, and
+// with FP32 storage, the two-rows-per-thread kernel where it applies (rows of up to
+// 128 nodes), else the folded one where it is built (at least a tile of rows).
+// D2Q9 grids with nx % 4 == 0: the block kernel
 // with FP32 storage below 524,288 node pairs (us a step, block and segment
 // kernel: 256^2 0.84 and 2.1, 560^2 1.77 and 2.91, 800^2 3.05 and 3.81, 1000^2
 // 4.08 and 4.26, 1200^2 5.76 and 5.63, 2048^2 15.3 and 12.0) and with FP64
 // storage up to 131,072 (1.9x to 2.4x), else the segment kernel; else the tiled
 // one, else the reference kernel.
 int pick_step_kernel(const Geometry& g, int precision) {
+  const bool s16 = precision == MACLAB_BF16_STORE || precision == MACLAB_F16_STORE;
+  if (s16 && g.pad == 0 && fold_supported(g, precision, 0)) return MACLAB_KERNEL_FOLDED;
   if (rows2_supported(g, precision, 0, true)) return MACLAB_KERNEL_ROWS2;
   if (fold_supported(g, precision, 0, true)) return MACLAB_KERNEL_FOLDED;
   if ((block_grid(g, precision) || !g.ilv) && block_supported(g, precision, 0, true))
