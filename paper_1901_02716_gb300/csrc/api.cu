@@ -12,6 +12,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <algorithm>
+#include <initializer_list>
 #include <map>
 #include <mutex>
 #include <new>
@@ -859,6 +860,15 @@ static size_t adjoint_bytes(const maclab_ctx* h) {
   return (size_t)(h->raw.d + 1) * (size_t)h->raw.n * (h->precision == MACLAB_F64 ? 8 : 4);
 }
 
+// Raw states and adjoints that the kernels for interleaved rows can read a quad or
+// a pair at a time; the kernels for natural rows and the reference kernels read
+// single values.
+static bool quads_aligned(std::initializer_list<const void*> arrays) {
+  for (const void* p : arrays)
+    if (reinterpret_cast<uintptr_t>(p) % 16 != 0) return false;
+  return true;
+}
+
 // records: the per-node (L_r, L_m) buffer that only the reference kernels use
 static maclab_status ensure_adjoint(maclab_ctx* h, bool records = false) {
   if (records && !h->d_adj_scratch) {
@@ -893,7 +903,8 @@ maclab_status maclab_adjoint_step(maclab_handle h, const void* state_n, const vo
   if (lam_n == lam_np1) return fail(MACLAB_ERR_INVALID, "lam_n must not alias lam_np1");
   DeviceGuard dg(h->device);
   // the tiled reverse step where it is built (unless the reference kernel was chosen)
-  const bool tiled = !h->reference_asked && tiled_adjoint_supported(h->raw, h->precision);
+  const bool tiled = !h->reference_asked && tiled_adjoint_supported(h->raw, h->precision) &&
+                     (!h->raw.ilv || quads_aligned({state_n, state_np1, lam_np1, lam_n}));
   maclab_status s = ensure_adjoint(h, !tiled);
   if (s != MACLAB_OK) return s;
   if (tiled) {
@@ -913,9 +924,8 @@ maclab_status maclab_adjoint_nu_term(maclab_handle h, const void* state_n, const
   NvtxRange nvtx_range("maclab_adjoint_nu_term");
   if (!h || !state_n || !lam_np1 || !acc) return fail(MACLAB_ERR_INVALID, "NULL argument");
   DeviceGuard dg(h->device);
-  auto aligned = [](const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; };
   if (state_np1 && h->kernel != MACLAB_KERNEL_REFERENCE && rows2_nu_supported(h->raw, h->precision) &&
-      aligned(state_n) && aligned(state_np1) && aligned(lam_np1)) {
+      quads_aligned({state_n, state_np1, lam_np1})) {
     CUDA_TRY(launch_rows2_nu(h->raw, state_n, state_np1, static_cast<const float*>(lam_np1), h->force_lat, acc,
                              h->overlap, h->stream),
              "adjoint nu term (two-rows kernel)");
