@@ -17,7 +17,6 @@
 // in FP64 by the arithmetic pipe (96^3: 325 us, the direct sums 478).
 #pragma once
 #include "adjoint_tiled.cuh"
-#include "units.cuh"
 
 namespace maclab {
 
@@ -111,8 +110,7 @@ __global__ void __launch_bounds__(BXC * RY, (AdjRows<LAT, S, BXC, RY>::MIN_BLOCK
   P force[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) force[i] = O::splat(C(A.force[i]));
-  C gfp[3] = {C(0), C(0), C(0)};
-  double gfd[3] = {0.0, 0.0, 0.0};
+  NuAcc<C> gf[3];  // sums of lam' over the fluid nodes
 
   auto ld = [&](const C* p) {
     P v;
@@ -173,13 +171,10 @@ __global__ void __launch_bounds__(BXC * RY, (AdjRows<LAT, S, BXC, RY>::MIN_BLOCK
       }
       if (counted) {
 #pragma unroll
-        for (int i = 0; i < D; ++i) gfp[i] += (w0 ? C(0) : R.lm[1 + i].x) + (w1 || !two ? C(0) : R.lm[1 + i].y);
-        if (((p - z0) & 7) == 7)
-#pragma unroll
-          for (int i = 0; i < D; ++i) {
-            gfd[i] += (double)gfp[i];
-            gfp[i] = C(0);
-          }
+        for (int i = 0; i < D; ++i) {
+          gf[i].add(w0 ? C(0) : R.lm[1 + i].x);
+          gf[i].add(w1 || !two ? C(0) : R.lm[1 + i].y);
+        }
       }
     }
 #pragma unroll
@@ -389,7 +384,7 @@ __global__ void __launch_bounds__(BXC * RY, (AdjRows<LAT, S, BXC, RY>::MIN_BLOCK
     const int nwarps = (blockDim.x * blockDim.y + 31) >> 5;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      double v = gfd[i] + (double)gfp[i];
+      double v = gf[i].value();
 #pragma unroll
       for (int s = 16; s > 0; s >>= 1) v += __shfl_down_sync(0xffffffffu, v, s);
       if (lane == 0) red[i][warp] = v;

@@ -24,6 +24,7 @@
 // lane-swapped copy of their edge pair into two extra columns.
 #pragma once
 #include "step_tiled.cuh"
+#include "units.cuh"
 
 namespace maclab {
 
@@ -144,8 +145,7 @@ __global__ void __launch_bounds__(BXC * RY, (AdjTile<LAT, S, BXC, RY>::MIN_BLOCK
   P force[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) force[i] = O::splat(C(A.force[i]));
-  C gfp[3] = {C(0), C(0), C(0)};
-  double gfd[3] = {0.0, 0.0, 0.0};
+  NuAcc<C> gf[3];  // sums of lam' over the fluid nodes
 
   // post-step state and lam' of this thread's quad in one plane
   struct Raw {
@@ -205,15 +205,11 @@ __global__ void __launch_bounds__(BXC * RY, (AdjTile<LAT, S, BXC, RY>::MIN_BLOCK
         }
         if (counted)
 #pragma unroll
-          for (int i = 0; i < D; ++i)
-            gfp[i] += (w0 ? C(0) : R.lm[1 + i][q].x) + (w1 ? C(0) : R.lm[1 + i][q].y);
+          for (int i = 0; i < D; ++i) {
+            gf[i].add(w0 ? C(0) : R.lm[1 + i][q].x);
+            gf[i].add(w1 ? C(0) : R.lm[1 + i][q].y);
+          }
       }
-      if (counted && ((p - z0) & 7) == 7)
-#pragma unroll
-        for (int i = 0; i < D; ++i) {
-          gfd[i] += (double)gfp[i];
-          gfp[i] = C(0);
-        }
     }
 #pragma unroll
     for (int q = 0; q < 2; ++q)
@@ -358,7 +354,7 @@ __global__ void __launch_bounds__(BXC * RY, (AdjTile<LAT, S, BXC, RY>::MIN_BLOCK
     const int nwarps = (blockDim.x * blockDim.y + 31) >> 5;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      double v = gfd[i] + (double)gfp[i];
+      double v = gf[i].value();
 #pragma unroll
       for (int s = 16; s > 0; s >>= 1) v += __shfl_down_sync(0xffffffffu, v, s);
       if (lane == 0) red[i][warp] = v;
