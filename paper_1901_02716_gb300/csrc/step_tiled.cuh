@@ -161,19 +161,8 @@ struct Pair<double> {
   __device__ __forceinline__ static P fma(P a, P b, P c) {
     return make_double2(__fma_rn(a.x, b.x, c.x), __fma_rn(a.y, b.y, c.y));
   }
-  // 1/a: the hardware approximation r0 (rcp.approx.ftz.f64: about 20 bits) and
-  // one third-order step of the Newton family, r1 = r0 (1 + e + e^2) with e =
-  // 1 - a r0 (exact from the FMA), which leaves e^3 = 2^-60: three FP64
-  // operations where the division takes about ten, on a pipe of two lanes per
-  // SM.  Within an ulp of 1/a for arguments away from zero and infinity, as
-  // 36 + R and 1 + drho' are.
-  __device__ __forceinline__ static double rcp1(double a) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-    const double e = __fma_rn(-a, r, 1.0);
-    return __fma_rn(r, __fma_rn(e, e, e), r);
-  }
-  __device__ __forceinline__ static P rcp(P a) { return make_double2(rcp1(a.x), rcp1(a.y)); }
+  // the division itself: correctly rounded, and 0 and infinity give what they should
+  __device__ __forceinline__ static P rcp(P a) { return make_double2(1.0 / a.x, 1.0 / a.y); }
   __device__ __forceinline__ static P swap(P a) { return make_double2(a.y, a.x); }
 };
 
