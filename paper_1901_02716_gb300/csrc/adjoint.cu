@@ -437,28 +437,38 @@ cudaError_t launch_adjoint_nu_term(const Geometry& g, int precision, const void*
 // and dL/dut = e dL/du; and back at the start of the rollout.  Both ends also
 // sum lam_ut . ut over all nodes (the dependence of output and input on e).
 //
-// With 32-bit arrays and arithmetic the maps take the FP32 forms of UnitMap,
-// and the sums products and additions whose rounding errors are kept (an fma
-// gives a product's, two-sum an addition's), one storage quad at a time: about
-// 47 bits of a quad's sum, which is then added in FP64.  A quad whose sum could
-// have left the range of these forms (large, or so small that an error term
-// could be subnormal) is summed in FP64.  Done in FP64 throughout, seven
-// conversions and multiply-adds per value on a pipe of two lanes per SM (and
-// the divisions by e) bounded both kernels.  96^3 FP32, whole calls with their
-// read-back: seed 60 -> 36 us, finish 119 -> 41 us.
+// With 32-bit arrays and arithmetic the maps take the FP32 forms of UnitMap, and
+// the sums are formed one storage quad at a time with products and additions
+// whose rounding errors are kept (an fma gives a product's, two-sum an
+// addition's) and added with theirs kept in turn: the quad's sum to more than
+// 53 bits, rounded once to FP64, where FP64 additions of the exact products
+// rounded at every one.  A quad whose sum could have left the range of these forms
+// (large, or so small that an error term could be subnormal) is summed in FP64.
+// Done in FP64 throughout, seven conversions and multiply-adds per value on a
+// pipe of two lanes per SM (and the divisions by e) bounded both kernels.  96^3
+// FP32, whole calls with their read-back: seed 60 -> 36 us, finish 119 -> 41 us.
+
+// a + b; *err is what the rounding of the sum left out.
+__device__ __forceinline__ float two_sum(float a, float b, float* err) {
+  const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+  *err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+  return s;
+}
 
 // Sum of a[i] b[i].
 template <int N>
 __device__ __forceinline__ double dot_unit(const float (&a)[N], const float (&b)[N]) {
-  float hi = 0.f, lo = 0.f;
+  float hi = 0.f, mid = 0.f, lo = 0.f;
 #pragma unroll
   for (int i = 0; i < N; ++i) {
+    float e, e1, e2;
     const float p = __fmul_rn(a[i], b[i]);
-    const float s = __fadd_rn(hi, p), bb = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(p, bb)), __fmaf_rn(a[i], b[i], -p)));
-    hi = s;
+    hi = two_sum(hi, p, &e);
+    mid = two_sum(mid, e, &e1);
+    mid = two_sum(mid, __fmaf_rn(a[i], b[i], -p), &e2);
+    lo = __fadd_rn(lo, __fadd_rn(e1, e2));
   }
-  if (fabsf(hi) > 0x1p-76f && fabsf(hi) < 0x1p100f) return (double)hi + (double)lo;
+  if (fabsf(hi) > 0x1p-76f && fabsf(hi) < 0x1p100f) return (double)hi + ((double)mid + (double)lo);
   double v = 0.0;
 #pragma unroll
   for (int i = 0; i < N; ++i) v += (double)a[i] * (double)b[i];
