@@ -869,6 +869,13 @@ static bool quads_aligned(std::initializer_list<const void*> arrays) {
   return true;
 }
 
+// The reverse step follows the kernel chosen for the forward one where that is the
+// reference kernel by choice (set_kernel, or a stored tuning result), not where the
+// library takes it because no other serves the domain.
+static bool reference_by_hand(const maclab_ctx* h) {
+  return h->kernel_by_hand && h->kernel == MACLAB_KERNEL_REFERENCE;
+}
+
 // records: the per-node (L_r, L_m) buffer that only the reference kernels use
 static maclab_status ensure_adjoint(maclab_ctx* h, bool records = false) {
   if (records && !h->d_adj_scratch) {
@@ -903,7 +910,7 @@ maclab_status maclab_adjoint_step(maclab_handle h, const void* state_n, const vo
   if (lam_n == lam_np1) return fail(MACLAB_ERR_INVALID, "lam_n must not alias lam_np1");
   DeviceGuard dg(h->device);
   // the tiled reverse step where it is built (unless the reference kernel was chosen)
-  const bool tiled = !h->reference_asked && tiled_adjoint_supported(h->raw, h->precision) &&
+  const bool tiled = !reference_by_hand(h) && tiled_adjoint_supported(h->raw, h->precision) &&
                      (!h->raw.ilv || quads_aligned({state_n, state_np1, lam_np1, lam_n}));
   maclab_status s = ensure_adjoint(h, !tiled);
   if (s != MACLAB_OK) return s;
@@ -924,14 +931,14 @@ maclab_status maclab_adjoint_nu_term(maclab_handle h, const void* state_n, const
   NvtxRange nvtx_range("maclab_adjoint_nu_term");
   if (!h || !state_n || !lam_np1 || !acc) return fail(MACLAB_ERR_INVALID, "NULL argument");
   DeviceGuard dg(h->device);
-  if (state_np1 && h->kernel != MACLAB_KERNEL_REFERENCE && rows2_nu_supported(h->raw, h->precision) &&
+  if (state_np1 && !reference_by_hand(h) && rows2_nu_supported(h->raw, h->precision) &&
       quads_aligned({state_n, state_np1, lam_np1})) {
     CUDA_TRY(launch_rows2_nu(h->raw, state_n, state_np1, static_cast<const float*>(lam_np1), h->force_lat, acc,
                              h->overlap, h->stream),
              "adjoint nu term (two-rows kernel)");
     return MACLAB_OK;
   }
-  if (state_np1 && !h->reference_asked && rows_nu_supported(h->raw, h->precision)) {
+  if (state_np1 && !reference_by_hand(h) && rows_nu_supported(h->raw, h->precision)) {
     CUDA_TRY(launch_rows_nu(h->raw, state_n, state_np1, lam_np1, h->force_lat, acc, h->overlap, h->stream),
              "adjoint nu term (natural rows)");
     return MACLAB_OK;
@@ -1181,7 +1188,7 @@ maclab_status maclab_set_kernel(maclab_handle h, int32_t kernel) {
   if (!h) return fail(MACLAB_ERR_INVALID, "NULL handle");
   drop_graphs(h);
   if (kernel == MACLAB_KERNEL_AUTO) {
-    h->reference_asked = false;
+    h->kernel_by_hand = false;
     h->kernel = pick_step_kernel(h->g, h->precision);
     return MACLAB_OK;
   }
@@ -1193,7 +1200,7 @@ maclab_status maclab_set_kernel(maclab_handle h, int32_t kernel) {
   if (!step_kernel_supported(h->raw, h->precision, kernel))
     return fail(MACLAB_ERR_UNSUPPORTED, "kernel does not support this domain");
   h->kernel = kernel;
-  h->reference_asked = kernel == MACLAB_KERNEL_REFERENCE;
+  h->kernel_by_hand = true;
   // a tile shape the new kernel lacks falls back to its default
   if (kernel == MACLAB_KERNEL_FOLDED && !fold_supported(h->g, h->precision, h->ty)) h->ty = 0;
   if (kernel == MACLAB_KERNEL_ROWS2 && !rows2_supported(h->g, h->precision, h->ty)) h->ty = 0;
@@ -1232,7 +1239,10 @@ maclab_status maclab_set_tile(maclab_handle h, int32_t ty, int32_t tz) {
                         tiled_supported(h->g, h->precision, ty, tz);
   if (!ok && !to_tiled) return fail(MACLAB_ERR_UNSUPPORTED, "no built tiled instance has this shape");
   drop_graphs(h);
-  if (to_tiled) h->kernel = MACLAB_KERNEL_TILED;
+  if (to_tiled) {
+    h->kernel = MACLAB_KERNEL_TILED;
+    h->kernel_by_hand = false;
+  }
   h->ty = ty;
   h->tz = tz;
   return MACLAB_OK;
@@ -1868,6 +1878,7 @@ maclab_status maclab_tune(maclab_handle h, int32_t out[2]) {
       if (shape_supported(h, it->second.kernel, it->second.ty, it->second.tz)) {
         drop_graphs(h);
         h->kernel = it->second.kernel;
+        h->kernel_by_hand = h->kernel == MACLAB_KERNEL_REFERENCE;
         h->ty = it->second.ty;
         h->tz = it->second.tz;
         h->overlap = it->second.overlap;
@@ -2018,6 +2029,7 @@ maclab_status maclab_tune(maclab_handle h, int32_t out[2]) {
   }
   drop_graphs(h);
   h->kernel = bkernel;
+  h->kernel_by_hand = false;
   h->ty = bty;
   h->tz = btz;
   {

@@ -429,7 +429,7 @@ struct maclab_ctx {
   size_t elem = 4;                 // bytes per stored value
   int64_t steps = 0;
   int kernel = MACLAB_KERNEL_REFERENCE;
-  bool reference_asked = false;  // chosen by hand: the reverse step then takes its reference kernels too
+  bool kernel_by_hand = false;     // kernel was chosen by maclab_set_kernel and not replaced since
   int ty = 0, tz = 0;              // tiled-kernel shape (0 = default)
   int overlap = 1;                 // programmatic dependent launch of the step kernels
   void* d_staging = nullptr;       // device staging for host set/get
