@@ -1237,8 +1237,18 @@ maclab_status maclab_set_tile(maclab_handle h, int32_t ty, int32_t tz) {
   // a ragged ny that the library serves with another kernel: the tiled kernel's shapes stay available
   const bool to_tiled = !ok && !step_kernel_supported(h->g, h->precision, h->kernel) &&
                         tiled_supported(h->g, h->precision, ty, tz);
-  if (!ok && !to_tiled) return fail(MACLAB_ERR_UNSUPPORTED, "no built tiled instance has this shape");
+  // so do the segment kernel's (rows per item, the persistent form) on the grids that the block
+  // kernel serves by default above the sizes where its own shapes were the only ones
+  const bool to_segment = h->kernel == MACLAB_KERNEL_BLOCK && !h->kernel_by_hand && (!ok || tz > 0) &&
+                          (int64_t)(h->g.nx / 2) * h->g.ny > kBlockOnlyPairs &&
+                          step_kernel_supported(h->g, h->precision, MACLAB_KERNEL_SEGMENT) &&
+                          (ty <= 1 || segment_depth(h->g, h->precision, ty) == 2);
+  if (!ok && !to_tiled && !to_segment) return fail(MACLAB_ERR_UNSUPPORTED, "no built tiled instance has this shape");
   drop_graphs(h);
+  if (to_segment) {
+    h->kernel = MACLAB_KERNEL_SEGMENT;
+    h->kernel_by_hand = false;
+  }
   if (to_tiled) {
     h->kernel = MACLAB_KERNEL_TILED;
     h->kernel_by_hand = false;

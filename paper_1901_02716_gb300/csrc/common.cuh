@@ -267,10 +267,13 @@ int block_steps(const Geometry& g, int precision, int ty);
 bool block_supported(const Geometry& g, int precision, int ty, bool natural = false);
 int block_threads(const Geometry& g, int precision, int steps);
 cudaError_t launch_block(const StepLaunch& s, cudaStream_t stream, int steps);
-// Grids where the block kernel is faster than the segment kernel (step.cu).
+// Grids where the block kernel is faster than the segment kernel (step.cu).  Up to
+// kBlockOnlyPairs it is at any number of steps; above (FP32) in runs, while a
+// single step is the segment kernel's.
+constexpr int64_t kBlockOnlyPairs = 131072;
 inline bool block_grid(const Geometry& g, int precision) {
   const int64_t pairs = (int64_t)(g.nx / 2) * g.ny;
-  return precision == MACLAB_F32 ? pairs < 524288 : pairs <= 131072;
+  return precision == MACLAB_F32 ? pairs < 524288 : pairs <= kBlockOnlyPairs;
 }
 int segment_depth(const Geometry& g, int precision, int ty);
 // Defined in batch.cu: warps of the segment kernels the device holds at once, the

@@ -37,3 +37,31 @@ def test_reverse_step_follows_a_kernel_that_tuning_replaced(lat, dims, monkeypat
     assert not torch.equal(got["library"][0], got["reference"][0])
     scale = float(got["library"][1].abs())
     assert float((got["library"][1] - got["reference, then tuned"][1]).abs()) <= 1e-12 * scale
+
+
+@pytest.mark.parametrize("tile", [(3, 0), (0, 16), (2, 8), (1, 4)])
+def test_segment_tiles_of_a_grid_the_block_kernel_serves(tile):
+    """A tile that only the segment kernel has (rows per item, the persistent form) selects it on
+    the larger grids of the block kernel's default; the bits are those of the default."""
+    case = inputs.random_case(D2, (600, 520), 0, seed=191, u_amp=0.08, rho_amp=0.02, walls="box")
+    out = []
+    for t in (None, tile):
+        with M.Solver.from_case(case, M.F32) as s:
+            if t:
+                s.set_tile(*t)
+                assert s.kernel_info()["kernel"] == M.KERNEL_SEGMENT
+            s.step(11)
+            out.append(s.get_lattice_state())
+    assert (out[0] == out[1]).all()
+
+
+def test_tiles_that_stay_refused():
+    case = inputs.random_case(D2, (64, 40), 0, seed=192, walls="box")
+    with M.Solver.from_case(case, M.F32) as s:  # the block kernel's own range
+        with pytest.raises(M.MacLABError):
+            s.set_tile(3, 0)
+    case = inputs.random_case(D2, (600, 520), 0, seed=193, walls="box")
+    with M.Solver.from_case(case, M.F32) as s:
+        s.set_kernel(M.KERNEL_BLOCK)
+        with pytest.raises(M.MacLABError):
+            s.set_tile(3, 0)
