@@ -627,6 +627,34 @@ static StepLaunch step_launch(const maclab_ctx* h, int from) {
   return s;
 }
 
+// Whether the handle's single steps run on the segment kernel's one-step form: of the
+// segment kernel itself, and of the block kernel taken by default on the larger
+// grids, whose one-step launch loads as many halo rows for one step as for four (us
+// a step, FP32, the block kernel's one-step launch and the segment kernel's: 600^2
+// 5.1 and 4.4, 1000^2 8.9 and 5.7; runs of many steps 2.0 and 4.3, 4.1 and 4.3).
+// The kernels give the same bits.
+static bool segment_single(const maclab_ctx* h) {
+  if (h->kernel == MACLAB_KERNEL_SEGMENT) return true;
+  return h->kernel == MACLAB_KERNEL_BLOCK && !h->kernel_by_hand &&
+         (int64_t)(h->g.nx / 2) * h->g.ny > kBlockOnlyPairs &&
+         step_kernel_supported(h->g, h->precision, MACLAB_KERNEL_SEGMENT);
+}
+
+// The launch of one step from buffer `from`, and its kernel.
+static StepLaunch single_step(const maclab_ctx* h, int from, int* kernel) {
+  StepLaunch s = step_launch(h, from);
+  s.seg_steps = 1;
+  *kernel = h->kernel;
+  if (segment_single(h) && h->d_seg_items) {
+    *kernel = MACLAB_KERNEL_SEGMENT;
+    if (h->seg_depth == 2) s.seg_items = static_cast<const int*>(h->d_seg_items) + 4 * (int64_t)h->seg_n_items;
+    s.seg_n_items = h->seg_n_items1;
+    s.seg_blocks = h->seg_blocks1;
+    s.seg_depth = 1;
+  }
+  return s;
+}
+
 // Time steps one launch of the handle's kernel advances.
 static int launch_depth(const maclab_ctx* h) {
   if (h->kernel == MACLAB_KERNEL_BLOCK) return block_steps(h->g, h->precision, h->ty);
@@ -643,11 +671,6 @@ static int device_sms() {
   return sms;
 }
 
-// The segment kernel's descriptor of this domain and its work list for the
-// current rows per item (tz, default 4) and steps per launch (ty: 2 for two,
-// else one), built on first use and after a change of either; graphs captured
-// with the old list are dropped.  Synchronises the handle's stream when it
-// uploads.
 // The persistent form's wait lists (segment kernel, ty 3): as many blocks as
 // fit at once, each with the list of blocks it waits for between sweeps.
 // Built on first use for the current work list.
@@ -677,14 +700,19 @@ static maclab_status segment_persist_prepare(maclab_ctx* h) {
   return MACLAB_OK;
 }
 
-// The segment kernel's descriptor and work list for the current tile setting
-// (rows per item and steps per launch), rebuilt when they change, and for the
-// persistent form (ty 3) its wait lists.
+// The segment kernel's descriptor and work lists for the current tile setting (rows
+// per item and steps per launch), rebuilt when it changes, and for the persistent
+// form (ty 3) its wait lists.  With two steps per launch a list of its own serves
+// single steps: cut for one step, it has wider segments and rows that fill one
+// wave of the one-step kernel's warps (1024^2: 5.6 us a single step, 7.1 on the
+// two-step list).
 static maclab_status segment_prepare(maclab_ctx* h) {
-  if (h->kernel != MACLAB_KERNEL_SEGMENT) return MACLAB_OK;
-  const int rows = segment_rows(h->g, h->precision, h->ty, h->tz);
-  const int depth = segment_depth(h->g, h->precision, h->ty);
-  if (!(h->d_seg_inst && h->d_seg_items && h->seg_rows == rows && h->seg_depth == depth)) {
+  if (!segment_single(h)) return MACLAB_OK;
+  const int runs = h->kernel == MACLAB_KERNEL_SEGMENT;
+  if (!h->d_seg_items || h->seg_runs != runs || h->seg_ty != h->ty || h->seg_tz != h->tz) {
+    const int depth = runs ? segment_depth(h->g, h->precision, h->ty) : 1;
+    int rows1 = segment_rows(h->g, h->precision, 1, 0);
+    if (runs && h->tz > 0) rows1 = depth == 1 ? h->tz : std::min(h->tz, rows1);
     if (!h->d_seg_inst) {
       if (cudaMalloc(&h->d_seg_inst, batch_inst_bytes()) != cudaSuccess) {
         cudaGetLastError();
@@ -694,8 +722,11 @@ static maclab_status segment_prepare(maclab_ctx* h) {
     }
     std::vector<unsigned char> inst(batch_inst_bytes());
     batch_fill_inst(inst.data(), h->g, h->buf[0], h->buf[1], h->force_lat);
-    std::vector<int> items;
-    batch_items(0, h->g, rows, depth, items);
+    std::vector<int> items, single;
+    batch_items(0, h->g, rows1, 1, single);
+    if (depth == 2) batch_items(0, h->g, segment_rows(h->g, h->precision, h->ty, h->tz), 2, items);
+    const size_t n2 = items.size() / 4, n1 = single.size() / 4;
+    items.insert(items.end(), single.begin(), single.end());
     void* d = nullptr;
     if (cudaMalloc(&d, items.size() * sizeof(int)) != cudaSuccess) {
       cudaGetLastError();
@@ -706,16 +737,24 @@ static maclab_status segment_prepare(maclab_ctx* h) {
     CUDA_TRY(cudaMemcpyAsync(d, items.data(), items.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream),
              "segment work list upload");
     CUDA_TRY(cudaStreamSynchronize(h->stream), "segment upload sync");
+    // one step per launch: 256-thread blocks, two per SM; two: 128-thread blocks, three per SM
+    auto blocks = [&](size_t n, int steps) {
+      const int warps = steps == 2 ? 4 : 8, per_sm = steps == 2 ? 3 : 2;
+      const int want = ((int)n + warps - 1) / warps;
+      return want < per_sm * device_sms() ? (want > 0 ? want : 1) : per_sm * device_sms();
+    };
     cudaFree(h->d_seg_items);
     h->d_seg_items = d;
-    h->seg_n_items = (int)(items.size() / 4);
+    h->seg_n_items1 = (int)n1;
+    h->seg_blocks1 = blocks(n1, 1);
+    h->seg_n_items = depth == 2 ? (int)n2 : (int)n1;
+    h->seg_blocks = depth == 2 ? blocks(n2, 2) : h->seg_blocks1;
+    items.resize(4 * (size_t)h->seg_n_items);
     h->seg_items_host.swap(items);
-    h->seg_rows = rows;
     h->seg_depth = depth;
-    // one step per launch: 256-thread blocks, two per SM; two: 128-thread blocks, three per SM
-    const int warps = depth == 2 ? 4 : 8, per_sm = depth == 2 ? 3 : 2;
-    const int want = (h->seg_n_items + warps - 1) / warps;
-    h->seg_blocks = want < per_sm * device_sms() ? (want > 0 ? want : 1) : per_sm * device_sms();
+    h->seg_runs = runs;
+    h->seg_ty = h->ty;
+    h->seg_tz = h->tz;
     drop_graphs(h);
     cudaFree(h->d_seg_deps);
     cudaFree(h->d_seg_done);
@@ -723,7 +762,7 @@ static maclab_status segment_prepare(maclab_ctx* h) {
     h->d_seg_done = nullptr;
     h->seg_persist_blocks = 0;
   }
-  return h->ty == 3 ? segment_persist_prepare(h) : MACLAB_OK;
+  return runs && h->ty == 3 ? segment_persist_prepare(h) : MACLAB_OK;
 }
 
 // Capture graph_steps / depth launches (graph_steps steps) starting from
@@ -804,9 +843,9 @@ maclab_status maclab_step(maclab_handle h, int64_t n) {
       done += part;
     }
   for (; done < n; ++done) {
-    StepLaunch sl = step_launch(h, h->cur);
-    sl.seg_steps = 1;
-    CUDA_TRY(launch_step(sl, h->stream, h->kernel), "step launch");
+    int kernel;
+    const StepLaunch sl = single_step(h, h->cur, &kernel);
+    CUDA_TRY(launch_step(sl, h->stream, kernel), "step launch");
     h->cur ^= 1;
   }
   h->steps += n;
@@ -1357,9 +1396,10 @@ struct maclab_batch_ctx {
   void* d_insts = nullptr;
   void* d_items = nullptr;
   int n_items = 0;
+  int n_items1 = 0;            // single steps with depth 2: their list follows the other in d_items
   int rows = 0;                // rows per work item, at most
   int depth = 1;               // time steps per launch (1 or 2)
-  int blocks = 0;
+  int blocks = 0, blocks1 = 0;
   // the persistent form (depth 3 in maclab_batch_set_depth): the two-step
   // work list, and every step pair of a call in one cooperative launch whose
   // blocks wait only for the blocks owning rows next to theirs
@@ -1379,6 +1419,8 @@ struct maclab_batch_ctx {
 };
 
 namespace {
+
+constexpr int kBatchRows = 16;  // rows per work item unless asked for
 
 void batch_drop_graphs(maclab_batch_ctx* b) {
   for (int c = 0; c < 2; ++c)
@@ -1435,10 +1477,18 @@ maclab_status batch_build_items(maclab_batch_ctx* b, int rows, int depth) {
     quads.push_back(m->g.nx / 4);
     heights.push_back(m->g.ny);
   }
-  const int64_t slots = batch_warp_slots(b->precision, depth);
-  const int64_t waves = (batch_item_count(quads, heights, depth, rows) + slots - 1) / slots;
-  const int cut = std::min(rows, batch_fit_rows(quads, heights, depth, waves * slots));
-  for (size_t i = 0; i < b->members.size(); ++i) batch_items((int)i, b->members[i]->g, cut, depth, items);
+  auto add_items = [&](int at_most, int steps) {
+    const int64_t slots = batch_warp_slots(b->precision, steps);
+    const int64_t waves = (batch_item_count(quads, heights, steps, at_most) + slots - 1) / slots;
+    const int cut = std::min(at_most, batch_fit_rows(quads, heights, steps, waves * slots));
+    for (size_t i = 0; i < b->members.size(); ++i) batch_items((int)i, b->members[i]->g, cut, steps, items);
+  };
+  add_items(rows, depth);
+  // single steps between launches of two have a list of their own behind the other
+  // (64 cavities: 36 us, 45 on the tuned two-step list)
+  const size_t n_items = items.size() / 4;
+  if (depth == 2) add_items(std::min(rows, kBatchRows), 1);
+  const size_t n_items1 = depth == 2 ? items.size() / 4 - n_items : n_items;
   void* d = nullptr;
   if (cudaMalloc(&d, items.size() * sizeof(int)) != cudaSuccess) {
     cudaGetLastError();
@@ -1451,7 +1501,9 @@ maclab_status batch_build_items(maclab_batch_ctx* b, int rows, int depth) {
   }
   cudaFree(b->d_items);
   b->d_items = d;
-  b->n_items = (int)(items.size() / 4);
+  b->n_items = (int)n_items;
+  b->n_items1 = (int)n_items1;
+  items.resize(4 * n_items);
   b->items_host.swap(items);
   b->rows = rows;
   b->depth = depth;
@@ -1462,9 +1514,13 @@ maclab_status batch_build_items(maclab_batch_ctx* b, int rows, int depth) {
   b->persist_blocks = 0;
   // resident warps: two 256-thread blocks per SM (one step per launch) or
   // three 128-thread blocks (two steps)
-  const int warps_per_block = depth == 2 ? 4 : 8, per_sm = depth == 2 ? 3 : 2;
-  const int want = (b->n_items + warps_per_block - 1) / warps_per_block;
-  b->blocks = want < per_sm * sm_count() ? (want > 0 ? want : 1) : per_sm * sm_count();
+  auto blocks = [&](int n, int steps) {
+    const int warps_per_block = steps == 2 ? 4 : 8, per_sm = steps == 2 ? 3 : 2;
+    const int want = (n + warps_per_block - 1) / warps_per_block;
+    return want < per_sm * sm_count() ? (want > 0 ? want : 1) : per_sm * sm_count();
+  };
+  b->blocks = blocks(b->n_items, depth);
+  b->blocks1 = blocks(b->n_items1, 1);
   batch_drop_graphs(b);
   return MACLAB_OK;
 }
@@ -1515,9 +1571,10 @@ cudaError_t batch_launch_steps(maclab_batch_ctx* b, int c, int steps, cudaStream
   if (b->one_launch && steps == 2)
     return launch_batch_step2(b->precision, b->d_insts, b->d_items, b->n_items, c, b->blocks, b->odd_pad, st,
                               b->overlap);
-  if (b->one_launch)
-    return launch_batch_step(b->precision, b->d_insts, b->d_items, b->n_items, c, b->blocks,
-                             b->depth == 2 ? kBatchSegW2 : kBatchSegW1, b->odd_pad, st, b->overlap);
+  if (b->one_launch) {
+    const int* const items = static_cast<const int*>(b->d_items) + (b->depth == 2 ? 4 * (int64_t)b->n_items : 0);
+    return launch_batch_step(b->precision, b->d_insts, items, b->n_items1, c, b->blocks1, b->odd_pad, st, b->overlap);
+  }
   for (maclab_ctx* m : b->members) {
     StepLaunch sl = step_launch(m, c);
     sl.seg_steps = 1;  // one step per member launch (the block kernel's one-step form)
@@ -1622,7 +1679,7 @@ maclab_status maclab_batch_create(const maclab_config* cfgs, int32_t count, macl
       return cuda_fail(e, "batch descriptor upload");
     }
   }
-  maclab_status s = batch_build_items(b, 16, 1);
+  maclab_status s = batch_build_items(b, kBatchRows, 1);
   if (s != MACLAB_OK) {
     batch_free(b);
     return s;
@@ -1698,7 +1755,7 @@ maclab_status maclab_batch_set_rows(maclab_batch b, int32_t rows) {
   if (!b) return fail(MACLAB_ERR_INVALID, "NULL batch");
   if (rows < 0 || rows > (1 << 20)) return fail(MACLAB_ERR_INVALID, "bad row count");
   DeviceGuard dg(b->device);
-  maclab_status s = batch_build_items(b, rows ? rows : 16, b->depth);
+  maclab_status s = batch_build_items(b, rows ? rows : kBatchRows, b->depth);
   return s == MACLAB_OK && b->persist ? batch_persist_prepare(b) : s;
 }
 
@@ -1711,7 +1768,7 @@ maclab_status maclab_batch_set_depth(maclab_batch b, int32_t depth) {
                 "two steps per launch need one launch per step, FP32 or FP64 storage and nx >= 8");
   DeviceGuard dg(b->device);
   const bool persist = depth == 3;
-  maclab_status s = batch_build_items(b, b->rows ? b->rows : 16, persist ? 2 : depth);
+  maclab_status s = batch_build_items(b, b->rows ? b->rows : kBatchRows, persist ? 2 : depth);
   if (s != MACLAB_OK) return s;
   b->persist = false;
   if (persist) {

@@ -158,14 +158,13 @@ __device__ __forceinline__ void batch_store(S* out, int64_t n, int64_t off, cons
   }
 }
 
-// segw: quads per work item's segment (30, or fewer when the work list was cut
-// for two steps per launch).  HIA: some domain's rows have odd padding (its
+// HIA: some domain's rows have odd padding (its
 // right wall is lane a.y of its quad instead of b.y; an instance of its own, as
 // the run-time choice costs 6 % at 1024^2).
 template <typename S, bool HIA>
 __global__ void __launch_bounds__(256, sizeof(S) == 8 ? 1 : 2) batch_step_d2q9(const BatchInst* __restrict__ insts,
                                                        const BatchItem* __restrict__ items,
-                                                       int n_items, int cur, int segw) {
+                                                       int n_items, int cur) {
   using C = typename Store<S>::C;
   using O = Pair<C>;
   using P = typename O::P;
@@ -185,6 +184,7 @@ __global__ void __launch_bounds__(256, sizeof(S) == 8 ? 1 : 2) batch_step_d2q9(c
     const int d_nx = I.nx, d_ny = I.ny, d_px = I.px, d_py = I.py, d_wall = I.wall_mode;
     const uint8_t* const d_mask = I.mask;
     const int nq = d_nx >> 2;
+    constexpr int segw = kBatchSegW1;
     const int n_int = min(segw, nq - segw * item.seg);
     int t = segw * item.seg - 1 + lane;            // quad of this lane
     const bool interior = lane >= 1 && lane <= n_int;
@@ -612,21 +612,20 @@ static cudaError_t launch_batch2_t(const BatchInst* insts, const BatchItem* item
 
 template <typename S>
 static cudaError_t launch_batch_t(const BatchInst* insts, const BatchItem* items, int n_items,
-                                  int cur, int blocks, int segw, bool odd, cudaStream_t st, int overlap) {
+                                  int cur, int blocks, bool odd, cudaStream_t st, int overlap) {
   return launch_kernel(odd ? batch_step_d2q9<S, true> : batch_step_d2q9<S, false>, dim3(blocks), dim3(256), 0, st, overlap, insts, items, n_items,
-                       cur, segw);
+                       cur);
 }
 
 cudaError_t launch_batch_step(int precision, const void* insts, const void* items, int n_items,
-                              int cur, int blocks, int segw, bool odd, cudaStream_t st, int overlap) {
+                              int cur, int blocks, bool odd, cudaStream_t st, int overlap) {
   const BatchInst* I = static_cast<const BatchInst*>(insts);
   const BatchItem* T = static_cast<const BatchItem*>(items);
-  if (segw < 1 || segw > 30) return cudaErrorInvalidValue;
   switch (precision) {
-    case MACLAB_F64: return launch_batch_t<double>(I, T, n_items, cur, blocks, segw, odd, st, overlap);
-    case MACLAB_F32: return launch_batch_t<float>(I, T, n_items, cur, blocks, segw, odd, st, overlap);
-    case MACLAB_BF16_STORE: return launch_batch_t<__nv_bfloat16>(I, T, n_items, cur, blocks, segw, odd, st, overlap);
-    case MACLAB_F16_STORE: return launch_batch_t<__half>(I, T, n_items, cur, blocks, segw, odd, st, overlap);
+    case MACLAB_F64: return launch_batch_t<double>(I, T, n_items, cur, blocks, odd, st, overlap);
+    case MACLAB_F32: return launch_batch_t<float>(I, T, n_items, cur, blocks, odd, st, overlap);
+    case MACLAB_BF16_STORE: return launch_batch_t<__nv_bfloat16>(I, T, n_items, cur, blocks, odd, st, overlap);
+    case MACLAB_F16_STORE: return launch_batch_t<__half>(I, T, n_items, cur, blocks, odd, st, overlap);
   }
   return cudaErrorInvalidValue;
 }

@@ -369,10 +369,9 @@ cudaError_t launch_adjoint_finish(const Geometry& g, int precision, const void* 
                                   void* gu, int dtype, double* wall, double* dot, cudaStream_t st);
 
 // Defined in batch.cu.
-// segw: quads per segment of the work list (30 when it was cut for one step per launch);
-// odd: a domain of the list has odd padding (Geometry)
+// items cut for one step per launch; odd: a domain of the list has odd padding (Geometry)
 cudaError_t launch_batch_step(int precision, const void* insts, const void* items, int n_items,
-                              int cur, int blocks, int segw, bool odd, cudaStream_t st, int overlap);
+                              int cur, int blocks, bool odd, cudaStream_t st, int overlap);
 constexpr int kBatchSegW1 = 30, kBatchSegW2 = 28;
 // two time steps per launch (FP32 / FP64 storage, every nx >= 8), 128-thread blocks
 cudaError_t launch_batch_step2(int precision, const void* insts, const void* items, int n_items,
@@ -451,7 +450,9 @@ struct maclab_ctx {
   void* d_seg_items = nullptr;
   int* d_seg_deps = nullptr;       // persistent segment launches: each block's wait list
   unsigned* d_seg_done = nullptr;  // and the blocks' finished-sweep counters
-  int seg_n_items = 0, seg_blocks = 0, seg_rows = 0, seg_depth = 1, seg_persist_blocks = 0;
+  int seg_n_items = 0, seg_blocks = 0, seg_depth = 1, seg_persist_blocks = 0;
+  int seg_n_items1 = 0, seg_blocks1 = 0;  // the one-step work list, which follows the other in d_seg_items
+  int seg_runs = 0, seg_ty = -1, seg_tz = -1;  // what the lists were built for (segment_prepare)
   std::vector<int> seg_items_host;  // the work list (4 ints per item) the wait lists are built from
   unsigned wait_limit = maclab::kWaitLimit;  // polls before a wait between blocks gives up
   void* d_adj_scratch = nullptr;   // reference adjoint: (L_r, L_m) at every node

@@ -248,8 +248,9 @@ static cudaError_t launch_step_kernel(const StepLaunch& s, cudaStream_t stream, 
       if (s.seg_steps == 2)
         return launch_batch_step2(s.precision, s.seg_inst, s.seg_items, s.seg_n_items, s.cur, s.seg_blocks,
                                   (s.g.pad & 1) != 0, stream, s.overlap);
+      if (s.seg_depth != 1) return cudaErrorInvalidValue;  // cut for another segment width
       return launch_batch_step(s.precision, s.seg_inst, s.seg_items, s.seg_n_items, s.cur, s.seg_blocks,
-                               s.seg_depth == 2 ? kBatchSegW2 : kBatchSegW1, (s.g.pad & 1) != 0, stream, s.overlap);
+                               (s.g.pad & 1) != 0, stream, s.overlap);
     default:
       return cudaErrorInvalidValue;
   }
