@@ -311,11 +311,8 @@ bool fold_supported(const Geometry& g, int precision, int ty, bool ragged = fals
 int fold_threads(const Geometry& g, int precision, int ty);
 cudaError_t launch_fold(const StepLaunch& s, cudaStream_t stream, int ty, int tz);
 // Chunks of the march axis for a grid of ytiles tiles per plane with per_sm
-// resident blocks of `threads` threads per SM (tz_req > 0: planes per chunk as asked).
-struct ChunkCost {
-  double start, free, share;
-};
-int fold_chunks(int nplanes, int ytiles, int tz_req, int per_sm, int threads, const ChunkCost& cost);
+// resident blocks per SM (tz_req > 0: planes per chunk as asked).
+int fold_chunks(int nplanes, int ytiles, int tz_req, int per_sm);
 
 // Defined in step_rows2.cu (D3Q19, two rows per thread; FP32 arithmetic).
 bool rows2_supported(const Geometry& g, int precision, int ty, bool ragged = false);

@@ -24,7 +24,6 @@ namespace {
 struct Rows2Shape {
   int bxc, tyt;
 };
-constexpr ChunkCost kRows2Cost = {3.0, 1.0, 0.45};  // see fold_chunks
 constexpr Rows2Shape kRows2Shapes[] = {{16, 4}, {32, 4}, {32, 2}};
 
 bool rows2_precision(int precision) {
@@ -150,7 +149,7 @@ cudaError_t launch_rows2(const StepLaunch& sl, cudaStream_t stream, int ty, int 
   if (e != cudaSuccess) return e;
   e = rows2_maps(g, sl.precision, s.bxc, ta.ty, sl.in, &tm_own, &tm_halo);
   if (e != cudaSuccess) return e;
-  ta.nzc = fold_chunks(ta.nplanes, ytiles, tz, resident, s.bxc * s.tyt, kRows2Cost);
+  ta.nzc = fold_chunks(ta.nplanes, ytiles, tz, resident);
   ta.px = (g.periodic & 1u) ? 1 : 0;
   ta.py = (g.periodic & 2u) ? 1 : 0;
   ta.pz = (g.periodic & 4u) ? 1 : 0;
@@ -186,7 +185,7 @@ cudaError_t launch_rows2_nu(const Geometry& g, const void* state_n, const void* 
   if (e != cudaSuccess) return e;
   e = rows2_maps(g, MACLAB_F32, s.bxc, ta.ty, state_n, &tm_own, &tm_halo);
   if (e != cudaSuccess) return e;
-  ta.nzc = fold_chunks(ta.nplanes, ytiles, 0, resident, s.bxc * s.tyt, kRows2Cost);
+  ta.nzc = fold_chunks(ta.nplanes, ytiles, 0, resident);
   ta.px = (g.periodic & 1u) ? 1 : 0;
   ta.py = (g.periodic & 2u) ? 1 : 0;
   ta.pz = (g.periodic & 4u) ? 1 : 0;
