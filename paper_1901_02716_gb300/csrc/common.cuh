@@ -311,8 +311,9 @@ bool fold_supported(const Geometry& g, int precision, int ty, bool ragged = fals
 int fold_threads(const Geometry& g, int precision, int ty);
 cudaError_t launch_fold(const StepLaunch& s, cudaStream_t stream, int ty, int tz);
 // Chunks of the march axis for a grid of ytiles tiles per plane with per_sm
-// resident blocks per SM (tz_req > 0: planes per chunk as asked).
-int fold_chunks(int nplanes, int ytiles, int tz_req, int per_sm);
+// resident blocks per SM (tz_req > 0: planes per chunk as asked; images: the step is followed
+// by the kernel of the periodic images).
+int fold_chunks(int nplanes, int ytiles, int tz_req, int per_sm, bool images);
 
 // Defined in step_rows2.cu (D3Q19, two rows per thread; FP32 arithmetic).
 bool rows2_supported(const Geometry& g, int precision, int ty, bool ragged = false);

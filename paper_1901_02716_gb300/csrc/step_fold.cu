@@ -77,20 +77,30 @@ static int sm_count() {
 // (at least four planes; a cost that grew with the warps of an SM) left some 5 to 15 %
 // behind: 160 x 40 x 100 folded 12.7 -> 11.3, 64 x 64 x 64 two rows 5.5 -> 5.25, 32 x
 // 64 x 256 11.1 -> 9.6.
-int fold_chunks(int nplanes, int ytiles, int tz_req, int per_sm) {
+//
+// images: every step is followed by the kernel that renews the periodic images
+// (launch_wrap_columns).  Its blocks find no place beside a last wave that takes up
+// all there is, and the next step's then come late: 67^3 10.2 us a step with a
+// seventh of the places left free, 13.1 without; 255 x 30 x 30 9.6 and 17.9.  A last
+// wave that leaves less counts 2.4 plane times more, which long steps do not mind.
+int fold_chunks(int nplanes, int ytiles, int tz_req, int per_sm, bool images) {
   if (tz_req > 0) return (nplanes + tz_req - 1) / tz_req;
-  const int64_t slots = (int64_t)sm_count() * (per_sm < 1 ? 1 : per_sm);
-  const int64_t first = (ytiles + slots - 1) / slots;  // waves of one chunk
+  const int64_t all = (int64_t)sm_count() * (per_sm < 1 ? 1 : per_sm), left = images ? all / 7 : 0;
   int best = 1;
   int64_t least = INT64_MAX;
-  for (int64_t w = first; w <= first + 64; ++w) {
-    const int chunks = (int)std::min<int64_t>(nplanes, w * slots / ytiles);
-    const int64_t cost = w * (5 * (int64_t)((nplanes + chunks - 1) / chunks) + 6);
-    if (cost < least) {
-      least = cost;
-      best = chunks;
+  for (const int64_t slots : {all, all - left}) {
+    const int64_t first = (ytiles + slots - 1) / slots;  // waves of one chunk
+    for (int64_t w = first; w <= first + 64; ++w) {
+      const int chunks = (int)std::min<int64_t>(nplanes, w * slots / ytiles);
+      const bool full = w * slots - (int64_t)chunks * ytiles + (all - slots) < left;
+      const int64_t cost = w * (5 * (int64_t)((nplanes + chunks - 1) / chunks) + 6) + (full ? 12 : 0);
+      if (cost < least) {
+        least = cost;
+        best = chunks;
+      }
+      if (chunks == nplanes) break;
     }
-    if (chunks == nplanes) break;
+    if (!images) break;
   }
   return best;
 }
@@ -139,7 +149,7 @@ cudaError_t launch_fold(const StepLaunch& sl, cudaStream_t stream, int ty, int t
   int resident = 0;
   cudaError_t e = dispatch(nullptr, nullptr, dim3(), &resident);
   if (e != cudaSuccess) return e;
-  ta.nzc = fold_chunks(ta.nplanes, ytiles, tz, resident);
+  ta.nzc = fold_chunks(ta.nplanes, ytiles, tz, resident, wrap_columns(g));
   ta.px = (g.periodic & 1u) ? 1 : 0;
   ta.py = (g.periodic & 2u) ? 1 : 0;
   ta.pz = (g.periodic & 4u) ? 1 : 0;

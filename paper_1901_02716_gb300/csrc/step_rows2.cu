@@ -149,7 +149,7 @@ cudaError_t launch_rows2(const StepLaunch& sl, cudaStream_t stream, int ty, int 
   if (e != cudaSuccess) return e;
   e = rows2_maps(g, sl.precision, s.bxc, ta.ty, sl.in, &tm_own, &tm_halo);
   if (e != cudaSuccess) return e;
-  ta.nzc = fold_chunks(ta.nplanes, ytiles, tz, resident);
+  ta.nzc = fold_chunks(ta.nplanes, ytiles, tz, resident, wrap_columns(g));
   ta.px = (g.periodic & 1u) ? 1 : 0;
   ta.py = (g.periodic & 2u) ? 1 : 0;
   ta.pz = (g.periodic & 4u) ? 1 : 0;
@@ -185,7 +185,7 @@ cudaError_t launch_rows2_nu(const Geometry& g, const void* state_n, const void* 
   if (e != cudaSuccess) return e;
   e = rows2_maps(g, MACLAB_F32, s.bxc, ta.ty, state_n, &tm_own, &tm_halo);
   if (e != cudaSuccess) return e;
-  ta.nzc = fold_chunks(ta.nplanes, ytiles, 0, resident);
+  ta.nzc = fold_chunks(ta.nplanes, ytiles, 0, resident, false);
   ta.px = (g.periodic & 1u) ? 1 : 0;
   ta.py = (g.periodic & 2u) ? 1 : 0;
   ta.pz = (g.periodic & 4u) ? 1 : 0;
