@@ -314,14 +314,7 @@ maclab_status maclab_create(const maclab_config* cfg, maclab_handle* out) {
   h->n_fluid = N - n_wall;
   g.wall_mode = n_wall == 0 ? kWallNone : (box ? kWallBox : kWallMask);
   h->raw = g;
-  const bool px = (g.periodic & 1u) != 0;
-  if (pad_rows(g, h->precision)) {  // interleaved rows with padding
-    g.pad = (int)((nx + (px ? 2 : 0) + 3) / 4 * 4 - nx);
-    g.nx += g.pad;
-    g.n = (int64_t)g.nx * ny * nz;
-    g.ilv = 1;
-    g.hx = g.nx / 2;
-  }
+  pad_rows(&g, h->precision);
 
   DeviceGuard dg(h->device);
   const size_t sb = buffer_bytes(h);

@@ -201,20 +201,9 @@ struct Geometry {
   int pad;
 };
 
-// Whether a domain of natural rows (g as the caller gave it) is stored in padded
-// ones.  At least 17 nodes wide, so that two quads lie between the two x-walls and
-// no quad holds both.  D3Q19: not with FP64 storage, whose tiled kernel's halo rows
-// cost what the one-thread-per-node kernel's repeated terms do on a pipe that
-// bounds both (45^3 closed: 66 us a step on the latter, 148 padded); and only where
-// the fast kernels' longer start pays (us a step, natural and padded rows, FP32:
-// closed 33^3 3.7 and 4.0, 37^3 4.2 and 3.8, 63^3 9.5 and 5.1; periodic, with the
-// images' extra launch, 51^3 6.3 and 6.7, 55^3 7.8 and 6.8, 79^3 16.2 and 10.5).
-inline bool pad_rows(const Geometry& g, int precision) {
-  if (g.nx % 4 == 0 || g.nx < 17) return false;
-  const bool px = (g.periodic & 1u) != 0;
-  if (g.d == 2) return !px;  // periodic: the block kernel takes natural rows
-  return precision != MACLAB_F64 && g.n >= (px ? 150000 : 50000);
-}
+// Defined in step.cu: pads the rows of a domain of natural rows (g as the caller gave
+// it) where a faster kernel then serves it.
+void pad_rows(Geometry* g, int precision);
 
 __host__ __device__ inline bool wrap_columns(const Geometry& g) { return g.pad > 0 && (g.periodic & 1u); }
 

@@ -176,6 +176,55 @@ int pick_step_kernel(const Geometry& g, int precision) {
                                                                  : MACLAB_KERNEL_REFERENCE;
 }
 
+// D2Q9, closed x axis (the block kernel takes periodic ones as they are): whether the
+// kernel that would serve the padded rows is faster than the one-thread-per-node
+// kernel on natural ones (us a step, natural and padded).  Narrow rows leave lanes of
+// the block kernel's 32 pairs and of the segment kernel's 28 quads idle, and a
+// tall domain pays for them:
+//   block, FP64:   17 x 1000 11.0 and 9.5, 17 x 2000 12.3 and 13.2, 25 x 3000 20.5 and 19.9
+//   segment, FP32 and 16 bits: 17 x 15882 BF16 8.2 and 7.8, 17 x 17647 8.2 and 8.7,
+//                  25 x 24000 12.3 and 10.1, 17 x 64705 FP32 18.5 and 20.9
+//   segment, FP64: 65 x 4153 64 and 75, 81 x 3333 64.0 and 62.6, 57 x 10526 143 and 134,
+//                  49 x 12244 143 and 158, 33 x 18181 143 and 206
+static bool pad_pays_2d(const Geometry& g, int precision, int kernel) {
+  const int64_t n = (int64_t)(g.nx - g.pad) * g.ny;
+  if (kernel == MACLAB_KERNEL_BLOCK) return precision != MACLAB_F64 || g.nx >= 28 || n < 20000;
+  if (precision != MACLAB_F64) return g.nx >= 28 || n < 270000;
+  const int quads = g.nx / 4, segments = (quads + kBatchSegW2 - 1) / kBatchSegW2;
+  return quads >= 20 * segments || (n >= 500000 && 2 * quads >= 29 * segments);
+}
+
+// D3Q19: where the two-rows or the folded kernel takes the padded rows (or the tiled
+// one in a single tile: 63 x 7 x 400 10.2 and 6.2; elsewhere its halo rows cost more:
+// 131 x 3 x 150 6.2 and 7.6), so not with FP64 storage, rows of more than 512 nodes or
+// 16-bit rows of other than whole 16 bytes, which stay on the one-thread-per-node
+// kernel and only slow it down (513 x 40 x 40 26.8 and 29.4, BF16 51^3 8.2 and 9.5;
+// FP64 45^3 66, 148 on the tiled kernel), and only where the fast kernels' longer
+// start pays (us a step, natural and padded rows, FP32: closed 33^3 3.7 and 4.0,
+// 37^3 4.2 and 3.8, 63^3 9.5 and 5.1; periodic, with the images' extra launch,
+// 51^3 6.3 and 6.7, 55^3 7.8 and 6.8, 79^3 16.2 and 10.5).
+static bool pad_pays_3d(const Geometry& g, int precision, int kernel) {
+  const int64_t n = (int64_t)(g.nx - g.pad) * g.ny * g.nz;
+  if (n < ((g.periodic & 1u) ? 150000 : 50000)) return false;
+  return kernel == MACLAB_KERNEL_ROWS2 || kernel == MACLAB_KERNEL_FOLDED ||
+         (kernel == MACLAB_KERNEL_TILED && precision != MACLAB_F64 && g.nx <= 64);
+}
+
+// At least 17 nodes wide, so that two quads lie between the two x-walls and no
+// quad holds both.
+void pad_rows(Geometry* g, int precision) {
+  const bool px = (g->periodic & 1u) != 0;
+  if (g->nx % 4 == 0 || g->nx < 17 || (g->d == 2 && px)) return;
+  Geometry p = *g;
+  p.pad = (g->nx + (px ? 2 : 0) + 3) / 4 * 4 - g->nx;
+  p.nx += p.pad;
+  p.n = (int64_t)p.nx * p.ny * p.nz;
+  p.ilv = 1;
+  p.hx = p.nx / 2;
+  const int kernel = pick_step_kernel(p, precision);
+  if (g->d == 2 ? pad_pays_2d(p, precision, kernel) : pad_pays_3d(p, precision, kernel)) *g = p;
+}
+
 static const char* kernel_name(const Geometry& g, int precision, int kernel) {
   if (kernel == MACLAB_KERNEL_ROWS2) {
     static const char* rows2[4] = {"step_rows2<D3Q19,f64>", "step_rows2<D3Q19,f32>", "step_rows2<D3Q19,bf16>",
