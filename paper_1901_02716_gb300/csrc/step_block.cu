@@ -439,6 +439,11 @@ cudaError_t launch_block_f64(const StepLaunch& s, cudaStream_t stream) {
   auto kern = step_block_d2q9<double, K, NAT, WRAP>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)((kBlockRowsF64 + 2) * row_bytes));
+  // the same split of L1 and shared memory for every instance and tile height: an SM
+  // changes it only when idle, so a run whose launches take 2, 2, 2, 1 steps waited for
+  // the device to drain at every change (128^2, runs of 3 steps: 12.5 us a step, 6.4 now)
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return e;
   return launch_kernel(kern, dim3((unsigned)xtiles, (unsigned)((a.ny + rows - 1) / rows)), dim3(kBlockBX, by),
                        (by + 2) * row_bytes, stream, s.overlap, a);
