@@ -181,17 +181,18 @@ int pick_step_kernel(const Geometry& g, int precision) {
 // kernel on natural ones (us a step, natural and padded).  Narrow rows leave lanes of
 // the block kernel's 32 pairs and of the segment kernel's 28 quads idle, and a
 // tall domain pays for them:
-//   block, FP64:   17 x 1000 11.0 and 9.5, 17 x 2000 12.3 and 13.2, 25 x 3000 20.5 and 19.9
+//   block, FP64:   17 x 1000 11.0 and 9.5, 17 x 2000 12.3 and 13.7, 25 x 6000 37.2 and
+//                  40.7, 29 x 8000 55.3 and 53.5
 //   segment, FP32 and 16 bits: 17 x 15882 BF16 8.2 and 7.8, 17 x 17647 8.2 and 8.7,
 //                  25 x 24000 12.3 and 10.1, 17 x 64705 FP32 18.5 and 20.9
-//   segment, FP64: 65 x 4153 64 and 75, 81 x 3333 64.0 and 62.6, 57 x 10526 143 and 134,
-//                  49 x 12244 143 and 158, 33 x 18181 143 and 206
+//   segment, FP64: 65 x 4153 64 and 78, 161 x 1863 72 and 79, 257 x 1167 74 and 65;
+//                  57 x 10526 143 and 140, 49 x 12244 143 and 164
 static bool pad_pays_2d(const Geometry& g, int precision, int kernel) {
   const int64_t n = (int64_t)(g.nx - g.pad) * g.ny;
-  if (kernel == MACLAB_KERNEL_BLOCK) return precision != MACLAB_F64 || g.nx >= 28 || n < 20000;
+  if (kernel == MACLAB_KERNEL_BLOCK) return precision != MACLAB_F64 || g.nx >= 32 || n < 20000;
   if (precision != MACLAB_F64) return g.nx >= 28 || n < 270000;
   const int quads = g.nx / 4, segments = (quads + kBatchSegW2 - 1) / kBatchSegW2;
-  return quads >= 20 * segments || (n >= 500000 && 2 * quads >= 29 * segments);
+  return 2 * quads >= (n >= 500000 ? 29 : 43) * segments;
 }
 
 // D3Q19: where the two-rows or the folded kernel takes the padded rows (or the tiled

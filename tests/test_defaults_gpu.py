@@ -41,11 +41,12 @@ def _box(dims, periodic):
     (D3, (513, 40, 40), 0b111, M.F32, "step_naive", 1), (D3, (601, 20, 24), 0b001, M.BF16_STORE, "step_naive", 1),
     (D3, (55, 55, 55), 0b111, M.BF16_STORE, "step_naive", 1), (D3, (131, 3, 150), 0, M.F32, "step_naive", 1),
     (D2, (17, 16000), 0, M.F64, "step_naive", 1), (D2, (65, 4153), 0, M.F64, "step_naive", 1),
+    (D2, (25, 6000), 0, M.F64, "step_naive", 1), (D2, (161, 1863), 0, M.F64, "step_naive", 1),
     (D2, (17, 20000), 0, M.F16_STORE, "step_naive", 1), (D2, (18, 66000), 0, M.F32, "step_naive", 1),
     # and the widths that padding brings to one
     (D3, (509, 40, 40), 0b111, M.F32, "step_fold", 2), (D3, (55, 55, 55), 0b111, M.F32, "step_rows2", 2),
     (D3, (51, 51, 51), 0, M.F32, "step_rows2", 1), (D3, (63, 7, 400), 0, M.F32, "step_tiled", 1),
-    (D2, (17, 900), 0, M.F64, "step_block", 1), (D2, (81, 3333), 0, M.F64, "segment", 1),
+    (D2, (17, 900), 0, M.F64, "step_block", 1), (D2, (257, 1167), 0, M.F64, "segment", 1),
     (D2, (401, 401), 0, M.F32, "step_block", 1), (D2, (25, 24000), 0, M.BF16_STORE, "segment", 1)])
 def test_rows_are_padded_where_a_faster_kernel_takes_them(lat, dims, periodic, precision, name, launches):
     with M.Solver(lat, dims, 1.0, 1.0 / 6.0, precision, periodic, **_box(dims, periodic)) as s:
