@@ -98,6 +98,13 @@ typedef struct {
  * MACLAB_ERR_OOM, MACLAB_ERR_CUDA.  On error *out is NULL. */
 maclab_status maclab_create(const maclab_config *cfg, maclab_handle *out);
 
+/* maclab_create for one slab of a domain that is `planes` planes long along the march
+ * axis (z in 3D, y in 2D; see maclab_get_planes): the library's choices that fix the
+ * order of a node's sums follow the undivided domain's, so the slabs' interiors equal
+ * its run bit for bit whatever their own length.  maclab_create is the same with the
+ * domain's own length.  Errors: as maclab_create, and MACLAB_ERR_INVALID (planes < 1). */
+maclab_status maclab_create_slab(const maclab_config *cfg, int64_t planes, maclab_handle *out);
+
 /* Free the handle and its device memory (synchronises its stream). NULL is OK.
  * No paper counterpart: the end of the procedure after Eq. (6) (step (v):
  * repeat until a solution is reached) leaves the owner to release the state. */

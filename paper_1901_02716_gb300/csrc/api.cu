@@ -216,6 +216,10 @@ maclab_status maclab_measure_fp32_peak(double* tflops) {
 const char* maclab_last_error(void) { return g_last_error.c_str(); }
 
 maclab_status maclab_create(const maclab_config* cfg, maclab_handle* out) {
+  return maclab_create_slab(cfg, cfg ? cfg->dims[cfg->lattice == MACLAB_D2Q9 ? 1 : 2] : 0, out);
+}
+
+maclab_status maclab_create_slab(const maclab_config* cfg, int64_t planes, maclab_handle* out) {
   if (!out) return fail(MACLAB_ERR_INVALID, "out is NULL");
   *out = nullptr;
   if (!cfg) return fail(MACLAB_ERR_INVALID, "cfg is NULL");
@@ -231,6 +235,7 @@ maclab_status maclab_create(const maclab_config* cfg, maclab_handle* out) {
     return fail(MACLAB_ERR_INVALID, "dimension too large");
   const int64_t N = nx * ny * nz;
   if (N > ((int64_t)1 << 40)) return fail(MACLAB_ERR_INVALID, "too many nodes");
+  if (planes < 1 || planes > (1 << 30)) return fail(MACLAB_ERR_INVALID, "planes must be in 1..2^30");
   if (!(cfg->dx > 0) || !(cfg->nu > 0) || !isfinite(cfg->dx) || !isfinite(cfg->nu))
     return fail(MACLAB_ERR_INVALID, "dx and nu must be finite and > 0");
   if (cfg->n_wall_ids < 0 || cfg->n_wall_ids > 255)
@@ -314,7 +319,7 @@ maclab_status maclab_create(const maclab_config* cfg, maclab_handle* out) {
   h->n_fluid = N - n_wall;
   g.wall_mode = n_wall == 0 ? kWallNone : (box ? kWallBox : kWallMask);
   h->raw = g;
-  pad_rows(&g, h->precision);
+  pad_rows(&g, h->precision, planes);
 
   DeviceGuard dg(h->device);
   const size_t sb = buffer_bytes(h);
@@ -1856,7 +1861,10 @@ std::string tune_key(const maclab_ctx* h) {
   char buf[160];
   snprintf(buf, sizeof(buf), "%d/%d/%d/%d/%d/%u/%d/", h->g.lattice, h->precision, h->raw.nx, h->g.ny,
            h->g.nz, h->g.periodic, h->g.wall_mode);
-  return buf + device_tag(h->device);
+  // a slab's rows may be stored another way than those of a domain of its size
+  Geometry alone = h->raw;
+  pad_rows(&alone, h->precision, alone.d == 3 ? alone.nz : alone.ny);
+  return buf + device_tag(h->device) + (alone.pad == h->g.pad ? "" : h->g.pad ? "/padded" : "/natural");
 }
 
 // Tuning results kept across processes: MACLAB_TUNE_CACHE names a text file

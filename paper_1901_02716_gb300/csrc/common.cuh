@@ -202,8 +202,9 @@ struct Geometry {
 };
 
 // Defined in step.cu: pads the rows of a domain of natural rows (g as the caller gave
-// it) where a faster kernel then serves it.
-void pad_rows(Geometry* g, int precision);
+// it) where a faster kernel then serves it; planes: those of the domain along the
+// march axis, or, where it is a slab, of the undivided domain, whose choice it follows.
+void pad_rows(Geometry* g, int precision, int64_t planes);
 
 __host__ __device__ inline bool wrap_columns(const Geometry& g) { return g.pad > 0 && (g.periodic & 1u); }
 

@@ -212,8 +212,9 @@ static bool pad_pays_3d(const Geometry& g, int precision, int kernel) {
 }
 
 // At least 17 nodes wide, so that two quads lie between the two x-walls and no
-// quad holds both.
-void pad_rows(Geometry* g, int precision) {
+// quad holds both.  Padded and natural rows run kernels that sum in different orders,
+// so the slabs of a domain all follow the choice of the whole.
+void pad_rows(Geometry* g, int precision, int64_t planes) {
   const bool px = (g->periodic & 1u) != 0;
   if (g->nx % 4 == 0 || g->nx < 17 || (g->d == 2 && px)) return;
   Geometry p = *g;
@@ -222,8 +223,11 @@ void pad_rows(Geometry* g, int precision) {
   p.n = (int64_t)p.nx * p.ny * p.nz;
   p.ilv = 1;
   p.hx = p.nx / 2;
-  const int kernel = pick_step_kernel(p, precision);
-  if (g->d == 2 ? pad_pays_2d(p, precision, kernel) : pad_pays_3d(p, precision, kernel)) *g = p;
+  Geometry whole = p;
+  (g->d == 2 ? whole.ny : whole.nz) = (int)planes;
+  whole.n = (int64_t)whole.nx * whole.ny * whole.nz;
+  const int kernel = pick_step_kernel(whole, precision);
+  if (g->d == 2 ? pad_pays_2d(whole, precision, kernel) : pad_pays_3d(whole, precision, kernel)) *g = p;
 }
 
 static const char* kernel_name(const Geometry& g, int precision, int kernel) {

@@ -38,6 +38,7 @@ class Case:
     wall_u: np.ndarray | None = None      # [n_wall_ids, d]
     force: tuple | None = None            # lattice-unit increment per step
     name: str = ""
+    planes: int | None = None             # of the undivided domain along the march axis, for a slab of it
 
     @property
     def d(self) -> int:

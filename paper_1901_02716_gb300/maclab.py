@@ -60,6 +60,7 @@ _VP = ctypes.c_void_p
 _S = ctypes.c_int32
 SIGNATURES = {
     "maclab_create": (_S, [ctypes.POINTER(maclab_config), ctypes.POINTER(_H)]),
+    "maclab_create_slab": (_S, [ctypes.POINTER(maclab_config), ctypes.c_int64, ctypes.POINTER(_H)]),
     "maclab_destroy": (_S, [_H]),
     "maclab_params": (_S, [_H, ctypes.POINTER(ctypes.c_double)]),
     "maclab_set_state": (_S, [_H, _VP, _VP, ctypes.c_int32, ctypes.c_int32]),
@@ -200,6 +201,14 @@ def maclab_create(cfg: maclab_config):
     h = _H()
     s = lib().maclab_create(ctypes.byref(cfg), ctypes.byref(h))
     _check(s, "maclab_create")
+    return h, s
+
+
+def maclab_create_slab(cfg: maclab_config, planes):
+    """One slab of a domain of ``planes`` planes along the march axis."""
+    h = _H()
+    s = lib().maclab_create_slab(ctypes.byref(cfg), int(planes), ctypes.byref(h))
+    _check(s, "maclab_create_slab")
     return h, s
 
 
@@ -512,10 +521,11 @@ class Solver:
     """One MacLAB domain on the GPU (owns a maclab handle)."""
 
     def __init__(self, lattice, dims, dx, nu, precision=F32, periodic=0, node_type=None,
-                 wall_rho=None, wall_u=None, body_force=None, rho0=1.0, stream=None):
+                 wall_rho=None, wall_u=None, body_force=None, rho0=1.0, stream=None, planes=None):
+        """planes: of the undivided domain along the march axis, where this one is a slab of it."""
         cfg, keep = make_config(lattice, dims, dx, nu, precision, periodic, node_type, wall_rho,
                                 wall_u, body_force, rho0, stream)
-        self.handle, self.create_status = maclab_create(cfg)
+        self.handle, self.create_status = maclab_create(cfg) if planes is None else maclab_create_slab(cfg, planes)
         self.lattice = lattice
         self.d = 2 if lattice == D2Q9 else 3
         self.dims = tuple(dims)
@@ -536,7 +546,7 @@ class Solver:
         bf = None if case.force is None else [f * e / dt for f in case.force]
         wu = None if case.wall_u is None else np.asarray(case.wall_u) * e
         s = cls(case.lattice, case.dims, dx, nu, precision, case.periodic, case.node_type,
-                case.wall_rho, wu, bf, stream=stream)
+                case.wall_rho, wu, bf, stream=stream, planes=case.planes)
         s.set_state(np.ascontiguousarray(case.rho, dtype=np.float64),
                     np.ascontiguousarray(case.u * e, dtype=np.float64))
         return s

@@ -12,8 +12,9 @@ exchange all those planes hold the neighbour's values; each step spoils one
 more plane from each end (the wall plane does not advance), so with depth h
 the interior stays exact for h steps and the exchange of h planes per side
 follows every h steps (depth 1: one wall plane, exchanged every step).  Every
-interior node thus sees exactly the upstream values of the undivided domain,
-and the slabs' interiors equal the undivided run bit for bit.
+interior node thus sees exactly the upstream values of the undivided domain, and
+every slab takes the library's choices for it (maclab_create_slab), so the slabs'
+interiors equal the undivided run bit for bit.
 
 This module holds no arithmetic of the method: partitioning, ghost-plane
 bookkeeping and the exchange pattern.  The stepping is done by a "stepper"
@@ -84,7 +85,7 @@ def slab_case(case: inputs.Case, start: int, stop: int, depth: int = 1) -> input
     wall_u = np.concatenate([wall_u, np.zeros((1, d))])
     dims = case.dims[:-1] + (stop - start + 2 * depth,)
     return inputs.Case(case.lattice, dims, case.periodic & ~_axis_bit(case), rho, u, nt, wall_rho,
-                       wall_u, force=case.force, name=f"{case.name}-slab{start}-{stop}")
+                       wall_u, force=case.force, name=f"{case.name}-slab{start}-{stop}", planes=n)
 
 
 @dataclasses.dataclass
