@@ -1108,13 +1108,30 @@ static maclab_status planes_args(maclab_ctx* h, int64_t p0, int64_t count, const
   return MACLAB_OK;
 }
 
+// Whether a kernel on the handle's device may read and write `p` itself: memory of that
+// device, aligned to the stored values.  (Buffers of other devices, and host memory,
+// go through the staging buffer.)
+static bool own_device_values(const maclab_ctx* h, const void* p, int32_t where) {
+  if (where != MACLAB_DEVICE || reinterpret_cast<uintptr_t>(p) % h->elem != 0) return false;
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged) && a.device == h->device;
+}
+
 maclab_status maclab_get_planes(maclab_handle h, int64_t p0, int64_t count, void* dst, int32_t where) {
   NvtxRange nvtx_range("maclab_get_planes");
   size_t pb = 0;
   maclab_status s = planes_args(h, p0, count, dst, where, &pb);
   if (s != MACLAB_OK) return s;
   DeviceGuard dg(h->device);
-  if (h->g.pad) {  // packed into the staging buffer, then one copy (dst may be on another device)
+  if (h->g.pad && own_device_values(h, dst, where)) {
+    CUDA_TRY(launch_repack(h->g, h->precision, h->buf[h->cur], dst, p0, count, true, h->stream), "get_planes repack");
+    return MACLAB_OK;
+  }
+  if (h->g.pad) {  // packed into the staging buffer, then one copy
     const size_t bytes = (size_t)(h->g.d + 1) * count * pb;
     s = ensure_staging(h, bytes);
     if (s != MACLAB_OK) return s;
@@ -1140,11 +1157,15 @@ maclab_status maclab_set_planes(maclab_handle h, int64_t p0, int64_t count, cons
   if (s != MACLAB_OK) return s;
   DeviceGuard dg(h->device);
   if (h->g.pad) {
-    const size_t bytes = (size_t)(h->g.d + 1) * count * pb;
-    s = ensure_staging(h, bytes);
-    if (s != MACLAB_OK) return s;
-    CUDA_TRY(cudaMemcpyAsync(h->d_staging, src, bytes, cudaMemcpyDefault, h->stream), "set_planes copy");
-    CUDA_TRY(launch_repack(h->g, h->precision, h->buf[h->cur], h->d_staging, p0, count, false, h->stream),
+    const bool direct = own_device_values(h, src, where);
+    if (!direct) {
+      const size_t bytes = (size_t)(h->g.d + 1) * count * pb;
+      s = ensure_staging(h, bytes);
+      if (s != MACLAB_OK) return s;
+      CUDA_TRY(cudaMemcpyAsync(h->d_staging, src, bytes, cudaMemcpyDefault, h->stream), "set_planes copy");
+    }
+    CUDA_TRY(launch_repack(h->g, h->precision, h->buf[h->cur], direct ? const_cast<void*>(src) : h->d_staging, p0, count,
+                           false, h->stream),
              "set_planes repack");
     if ((s = refresh_images(h, h->cur)) != MACLAB_OK) return s;
     if (where == MACLAB_HOST) CUDA_TRY(cudaStreamSynchronize(h->stream), "set_planes sync");
