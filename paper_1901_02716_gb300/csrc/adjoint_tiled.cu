@@ -174,8 +174,13 @@ cudaError_t launch_tiled_adjoint(const Geometry& g, int precision, const void* s
   return tiled_adjoint_t<kD3Q19, float>(g, s, state_n, state_np1, lam_np1, lam_n, force_lat, grad_force, overlap, st);
 }
 
+// adj_nu_rows where it beats the per-node kernel (us, per node and by rows): 29^3 8.3
+// and 7.4; then its blocks, one an SM, march too few planes each (33^3 8.3 and 9.3,
+// 111 x 24 x 24 8.7 and 10.1, 49^3 10.3 and 12.4), until the nodes count (53^3 12.4 and
+// 12.3, 63^3 14.5 and 13.2, 127 x 80 x 80 35 and 22).
 bool rows_nu_supported(const Geometry& g, int precision) {
   AdjShape s;
+  if (g.n > 26000 && g.n < 148000) return false;
   return precision == MACLAB_F32 && g.d == 3 && adj_shape(g, precision, &s) && s.rows;
 }
 
