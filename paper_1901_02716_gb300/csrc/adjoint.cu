@@ -635,7 +635,7 @@ static cudaError_t by_adjoint_unit(const Geometry& g, const void* a, const void*
                                    Fn&& launch) {
   Unit unit = unit_of(g, a, b, 2 * sizeof(T));
   if ((reinterpret_cast<uintptr_t>(state) | reinterpret_cast<uintptr_t>(lam)) % 16 != 0) unit = kNode;
-  return by_unit(g, unit, [&](unsigned, auto index, auto u) {
+  return by_unit(g, unit, [&](unsigned, unsigned, auto index, auto u) {
     return launch(grid256(unit == kNode ? g.n : g.n / 4), index, u);
   });
 }

@@ -120,16 +120,16 @@ size_t state_bytes(const maclab_ctx* h) { return (size_t)(h->g.d + 1) * (size_t)
 // one of the two state buffers
 size_t buffer_bytes(const maclab_ctx* h) { return (size_t)(h->g.d + 1) * (size_t)h->g.n * h->elem; }
 
-// Put the current buffer's wall values into the other one as well (wall nodes
-// are never written by the step kernels; every fluid node of a buffer is
-// written by the step that fills it, so nothing else needs to be copied).
-// And the periodic images of padded rows, wherever nodes were written from outside.
+// The periodic images of a padded buffer, wherever nodes were written from outside.
 maclab_status refresh_images(maclab_ctx* h, int buffer) {
   if (wrap_columns(h->g))
     CUDA_TRY(launch_wrap_columns(h->g, h->precision, h->buf[buffer], h->stream, 0), "periodic images");
   return MACLAB_OK;
 }
 
+// Put the current buffer's wall values into the other one as well (wall nodes
+// are never written by the step kernels; every fluid node of a buffer is
+// written by the step that fills it, so nothing else needs to be copied).
 maclab_status mirror_walls(maclab_ctx* h) {
   CUDA_TRY(launch_copy_walls(h->g, h->precision, h->d_node_type, h->buf[h->cur], h->buf[h->cur ^ 1], h->stream),
            "mirror wall values");
@@ -582,7 +582,7 @@ maclab_status maclab_set_lattice_state(maclab_handle h, const void* state, int32
       raw = h->d_staging;
     }
     CUDA_TRY(launch_repack(h->g, h->precision, h->buf[h->cur], const_cast<void*>(raw), 0, march_planes(h), false,
-                           h->stream),
+                           h->stream, h->buf[h->cur ^ 1], h->d_node_type),
              "set_lattice_state repack");
     if (maclab_status s = refresh_images(h, h->cur)) return s;
   } else {
@@ -590,9 +590,9 @@ maclab_status maclab_set_lattice_state(maclab_handle h, const void* state, int32
                              where == MACLAB_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice,
                              h->stream),
              "set_lattice_state");
+    maclab_status s = mirror_walls(h);
+    if (s != MACLAB_OK) return s;
   }
-  maclab_status s = mirror_walls(h);
-  if (s != MACLAB_OK) return s;
   h->prev_valid = false;
   if (where == MACLAB_HOST) CUDA_TRY(cudaStreamSynchronize(h->stream), "set_lattice_state sync");
   return MACLAB_OK;

@@ -383,9 +383,10 @@ cudaError_t launch_set_wall_values(const Geometry& g, int precision, const void*
                                    void* s1, cudaStream_t stream);
 // Planes [p0, p0 + count) of the march axis between the stored rows of g and the
 // raw layout of a state without padding ([field][plane][row] of g.nx - g.pad
-// nodes in their natural order); to_raw: out of the state, else into it.
+// nodes in their natural order); to_raw: out of the state, else into it, and, where
+// they are given, the wall nodes (node_type, in the state's rows) into the other buffer.
 cudaError_t launch_repack(const Geometry& g, int precision, void* state, void* raw, int64_t p0, int64_t count,
-                          bool to_raw, cudaStream_t stream);
+                          bool to_raw, cudaStream_t stream, void* other = nullptr, const uint8_t* node_type = nullptr);
 // The periodic images of a state in padded rows (wrap_columns).
 cudaError_t launch_wrap_columns(const Geometry& g, int precision, void* state, cudaStream_t stream, int overlap);
 cudaError_t launch_copy_walls(const Geometry& g, int precision, const uint8_t* node_type, const void* src,

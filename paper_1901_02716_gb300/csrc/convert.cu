@@ -125,28 +125,65 @@ __global__ void __launch_bounds__(256) set_walls_k(Geometry g, const T* __restri
   });
 }
 
-// The wall nodes of one raw state into the other buffer.
-template <typename S>
+// The wall nodes of one raw state into the other buffer.  W: nodes a thread looks at,
+// four where the fields are whole quads (one by one the look alone took longer than
+// copying a whole 16-bit state: 128^3 BF16 16.1 us a maclab_set_lattice_state, 12.3).
+template <typename S, int W>
 __global__ void __launch_bounds__(256) copy_walls_k(int d, int64_t N, const uint8_t* __restrict__ node_type,
                                                     const S* __restrict__ src, S* __restrict__ dst) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
-    if (node_type[i] != 0)
-      for (int f = 0; f <= d; ++f) dst[f * N + i] = src[f * N + i];
+  const int64_t i = W * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
+  if (i >= N) return;
+  if constexpr (W == 4) {
+    const uchar4 k = *reinterpret_cast<const uchar4*>(node_type + i);
+    const bool wall[4] = {k.x != 0, k.y != 0, k.z != 0, k.w != 0};
+    if (!(wall[0] | wall[1] | wall[2] | wall[3])) return;
+    Four<S> v[4];
+#pragma unroll
+    for (int f = 0; f < 4; ++f)
+      if (f <= d) v[f] = *reinterpret_cast<const Four<S>*>(src + f * N + i);
+#pragma unroll
+    for (int f = 0; f < 4; ++f)
+      if (f <= d) {
+        if (wall[0] & wall[1] & wall[2] & wall[3]) {
+          *reinterpret_cast<Four<S>*>(dst + f * N + i) = v[f];
+        } else {
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            if (wall[c]) dst[f * N + i + c] = v[f].v[c];
+        }
+      }
+  } else {
+    if (node_type[i] == 0) return;
+    for (int f = 0; f <= d; ++f) dst[f * N + i] = src[f * N + i];
+  }
+}
+
+template <typename S>
+static cudaError_t copy_walls_t(const Geometry& g, const uint8_t* nt, const void* src, void* dst, cudaStream_t st) {
+  if (g.n % 4 == 0)
+    copy_walls_k<S, 4><<<(unsigned)((g.n / 4 + 255) / 256), 256, 0, st>>>(g.d, g.n, nt, (const S*)src, (S*)dst);
+  else
+    copy_walls_k<S, 1><<<(unsigned)((g.n + 255) / 256), 256, 0, st>>>(g.d, g.n, nt, (const S*)src, (S*)dst);
+  return cudaGetLastError();
 }
 
 // Rows of planes [p0, p0 + count) between padded storage and the raw layout
-// (kQuad1 units of the rows; `rows` rows a field).
+// (kQuad1 units of the rows; `rows` rows a field).  Into the state, quads with walls
+// (node_type, of the state's rows) go to the other buffer as well where it is given.
 template <typename S, typename I, bool TO_RAW>
 __global__ void __launch_bounds__(256) repack_k(Geometry g, int64_t row0, int64_t rows, S* __restrict__ state,
-                                                S* __restrict__ raw) {
+                                                S* __restrict__ raw, S* __restrict__ other,
+                                                const uint8_t* __restrict__ node_type) {
   const int64_t N = g.n, NU = rows * (g.nx - g.pad);
   Geometry part = g;  // the planes' rows only
   part.n = rows * g.nx;
   for_units<I, kQuad1>(part, [&](int64_t i, int64_t j, int x) {
+    const int64_t at = row0 * g.nx + i;
+    const bool walls = !TO_RAW && other && *reinterpret_cast<const uint32_t*>(node_type + at) != 0;
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
       if (f > g.d) continue;
-      Four<S>* const q = reinterpret_cast<Four<S>*>(state + f * N + row0 * g.nx + i);
+      Four<S>* const q = reinterpret_cast<Four<S>*>(state + f * N + at);
       if constexpr (TO_RAW) {
         const Four<S> v = *q;
         st_user<kQuad1, S>(g, raw + f * NU, j, x, v.v);
@@ -154,6 +191,7 @@ __global__ void __launch_bounds__(256) repack_k(Geometry g, int64_t row0, int64_
         Four<S> v;
         ld_user<kQuad1, S>(g, raw + f * NU, j, x, v.v);
         *q = v;
+        if (walls) *reinterpret_cast<Four<S>*>(other + f * N + at) = v;
       }
     }
   });
@@ -187,9 +225,9 @@ __global__ void __launch_bounds__(256) get_physical_k(Geometry g, const S* __res
 template <typename S, typename T, bool FAST>
 static cudaError_t set_t(const Geometry& g, const void* rho, const void* u, const UnitMap& m, const uint8_t* nt,
                          const double* wl, int nw, void* s0, void* s1, cudaStream_t st) {
-  return by_unit(g, unit_of(g, rho, u, 2 * sizeof(T)), [&](unsigned grid, auto index, auto unit) {
+  return by_unit(g, unit_of(g, rho, u, 2 * sizeof(T)), [&](unsigned grid, unsigned threads, auto index, auto unit) {
     set_physical_k<S, T, FAST, decltype(index), decltype(unit)::value>
-        <<<grid, 256, 0, st>>>(g, (const T*)rho, (const T*)u, m, nt, wl, nw, (S*)s0, (S*)s1);
+        <<<grid, threads, 0, st>>>(g, (const T*)rho, (const T*)u, m, nt, wl, nw, (S*)s0, (S*)s1);
     return cudaGetLastError();
   });
 }
@@ -219,9 +257,9 @@ cudaError_t launch_set_physical(const Geometry& g, int precision, const void* rh
 
 template <typename S, typename T, bool FAST>
 static cudaError_t get_t(const Geometry& g, const void* state, const UnitMap& m, void* rho, void* u, cudaStream_t st) {
-  return by_unit(g, unit_of(g, rho, u, 2 * sizeof(T)), [&](unsigned grid, auto index, auto unit) {
+  return by_unit(g, unit_of(g, rho, u, 2 * sizeof(T)), [&](unsigned grid, unsigned threads, auto index, auto unit) {
     get_physical_k<S, T, FAST, decltype(index), decltype(unit)::value>
-        <<<grid, 256, 0, st>>>(g, (const S*)state, m, (T*)rho, (T*)u);
+        <<<grid, threads, 0, st>>>(g, (const S*)state, m, (T*)rho, (T*)u);
     return cudaGetLastError();
   });
 }
@@ -251,9 +289,9 @@ cudaError_t launch_get_physical(const Geometry& g, int precision, const void* st
 template <typename S, typename T, bool FAST>
 static cudaError_t walls_t(const Geometry& g, const void* rho, const void* u, const UnitMap& m, const uint8_t* nt,
                            void* s0, void* s1, cudaStream_t st) {
-  return by_unit(g, unit_of(g, rho, u, 2 * sizeof(T)), [&](unsigned grid, auto index, auto unit) {
+  return by_unit(g, unit_of(g, rho, u, 2 * sizeof(T)), [&](unsigned grid, unsigned threads, auto index, auto unit) {
     set_walls_k<S, T, FAST, decltype(index), decltype(unit)::value>
-        <<<grid, 256, 0, st>>>(g, (const T*)rho, (const T*)u, m, nt, (S*)s0, (S*)s1);
+        <<<grid, threads, 0, st>>>(g, (const T*)rho, (const T*)u, m, nt, (S*)s0, (S*)s1);
     return cudaGetLastError();
   });
 }
@@ -284,27 +322,28 @@ cudaError_t launch_set_wall_values(const Geometry& g, int precision, const void*
 
 template <typename S>
 static cudaError_t repack_t(const Geometry& g, void* state, void* raw, int64_t row0, int64_t rows, bool to_raw,
-                            cudaStream_t st) {
+                            void* other, const uint8_t* nt, cudaStream_t st) {
   const unsigned grid = grid_for(rows * g.nx / 4);
   S* const s = (S*)state;
   S* const r = (S*)raw;
+  S* const o = nt ? (S*)other : nullptr;
   if (small_index(g.n)) {
-    if (to_raw) repack_k<S, uint32_t, true><<<grid, 256, 0, st>>>(g, row0, rows, s, r);
-    else repack_k<S, uint32_t, false><<<grid, 256, 0, st>>>(g, row0, rows, s, r);
+    if (to_raw) repack_k<S, uint32_t, true><<<grid, 256, 0, st>>>(g, row0, rows, s, r, o, nt);
+    else repack_k<S, uint32_t, false><<<grid, 256, 0, st>>>(g, row0, rows, s, r, o, nt);
   } else {
-    if (to_raw) repack_k<S, int64_t, true><<<grid, 256, 0, st>>>(g, row0, rows, s, r);
-    else repack_k<S, int64_t, false><<<grid, 256, 0, st>>>(g, row0, rows, s, r);
+    if (to_raw) repack_k<S, int64_t, true><<<grid, 256, 0, st>>>(g, row0, rows, s, r, o, nt);
+    else repack_k<S, int64_t, false><<<grid, 256, 0, st>>>(g, row0, rows, s, r, o, nt);
   }
   return cudaGetLastError();
 }
 
 cudaError_t launch_repack(const Geometry& g, int precision, void* state, void* raw, int64_t p0, int64_t count,
-                          bool to_raw, cudaStream_t st) {
+                          bool to_raw, cudaStream_t st, void* other, const uint8_t* nt) {
   const int64_t plane_rows = g.d == 3 ? g.ny : 1;
   switch (storage_bytes(precision)) {
-    case 8: return repack_t<double>(g, state, raw, p0 * plane_rows, count * plane_rows, to_raw, st);
-    case 4: return repack_t<float>(g, state, raw, p0 * plane_rows, count * plane_rows, to_raw, st);
-    case 2: return repack_t<uint16_t>(g, state, raw, p0 * plane_rows, count * plane_rows, to_raw, st);
+    case 8: return repack_t<double>(g, state, raw, p0 * plane_rows, count * plane_rows, to_raw, other, nt, st);
+    case 4: return repack_t<float>(g, state, raw, p0 * plane_rows, count * plane_rows, to_raw, other, nt, st);
+    case 2: return repack_t<uint16_t>(g, state, raw, p0 * plane_rows, count * plane_rows, to_raw, other, nt, st);
   }
   return cudaErrorInvalidValue;
 }
@@ -342,14 +381,12 @@ cudaError_t launch_wrap_columns(const Geometry& g, int precision, void* state, c
 cudaError_t launch_copy_walls(const Geometry& g, int precision, const uint8_t* nt, const void* src, void* dst,
                               cudaStream_t st) {
   if (!nt) return cudaSuccess;
-  const unsigned grid = grid_for(g.n);
   switch (storage_bytes(precision)) {
-    case 8: copy_walls_k<double><<<grid, 256, 0, st>>>(g.d, g.n, nt, (const double*)src, (double*)dst); break;
-    case 4: copy_walls_k<float><<<grid, 256, 0, st>>>(g.d, g.n, nt, (const float*)src, (float*)dst); break;
-    case 2: copy_walls_k<uint16_t><<<grid, 256, 0, st>>>(g.d, g.n, nt, (const uint16_t*)src, (uint16_t*)dst); break;
-    default: return cudaErrorInvalidValue;
+    case 8: return copy_walls_t<double>(g, nt, src, dst, st);
+    case 4: return copy_walls_t<float>(g, nt, src, dst, st);
+    case 2: return copy_walls_t<uint16_t>(g, nt, src, dst, st);
   }
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_fill_walls(const Geometry& g, int precision, const uint8_t* nt, const double* wl,
