@@ -155,7 +155,7 @@ __device__ __forceinline__ void row_update_2d(const typename Pair<C>::P (&st)[3]
       }
     }
   }
-  if constexpr (!kDoubleBuffer) __syncthreads();
+  __syncthreads();  // the row's slots are the next row's (one buffer, whatever the planes use)
 }
 
 }  // namespace maclab
