@@ -176,16 +176,19 @@ maclab_status maclab_step_raw(maclab_handle h, const void *in, void *out);
 /* Step kernels.  MACLAB_KERNEL_AUTO lets the library choose (the default);
  * MACLAB_KERNEL_REFERENCE is the simple one-thread-per-node gather, kept as the
  * GPU-side yardstick; MACLAB_KERNEL_TILED is the staged, vectorised kernel;
- * MACLAB_KERNEL_FOLDED is its D3Q19 FP32 form without halo-row threads (the
- * tile's edge rows fold their halo rows in; needs ny divisible by the tile's
- * rows); MACLAB_KERNEL_SEGMENT is the batched D2Q9 kernel run on one domain
+ * MACLAB_KERNEL_FOLDED is its D3Q19 form with FP32 or 16-bit storage without
+ * halo-row threads (the tile's edge rows fold their halo rows in; needs ny
+ * divisible by the tile's rows; the default for 16-bit storage where it applies,
+ * and for rows of 132 to 512 nodes); MACLAB_KERNEL_SEGMENT is the batched D2Q9 kernel run on one domain
  * (a warp per 30-quad row segment, x exchange by warp shuffles; with two
  * steps per launch the rows are staged four ahead in the warp's own shared
  * memory; nx % 4 == 0; the tile's tz is its rows per work item, by default as
  * few as make one wave of resident warps, and ty the time steps per launch, 1
  * or 2, default 2 with FP32 storage and, with FP64 storage, below 200,000 quads,
  * see maclab_batch_set_depth), the default for D2Q9 grids with nx % 4 == 0 that the
- * block kernel does not take (below).  All compute Eqs.
+ * block kernel does not take (below); its one-step form also takes the single steps
+ * that are left of a run, and those of the block kernel's default FP32 grids of more
+ * than 131,072 node pairs.  All compute Eqs.
  * (4)-(5) with the same terms per node (the folded kernel sums them in
  * another order; the segment and tiled kernels give identical bits).
  * MACLAB_KERNEL_ROWS2 is the D3Q19 kernel with two rows per thread (FP32,
@@ -207,13 +210,16 @@ maclab_status maclab_step_raw(maclab_handle h, const void *in, void *out);
  * a one-step launch (the previous state is step n - 1).  Its sums run in the
  * tiled kernel's order: identical bits.  The default for FP32 D2Q9 grids of
  * fewer than 524,288 node pairs and FP64 ones of up to 131,072 (512^2).
- * The default also takes these kernels where a choice by hand is refused: an x
- * axis of at least 17 nodes whose width is not a multiple of 4 is stored in rows
- * padded to one (D2Q9: closed axes; D3Q19 with FP32 or 16-bit storage: closed from
- * 50,000 nodes on, periodic from 150,000; the raw state keeps its (d + 1) * N
- * values); with D2Q9 the block kernel takes a periodic x axis of any width of at
- * least 32 nodes; and the two-rows and folded kernels run on row counts that their
- * tiles do not divide (at least one tile of rows). */
+ * The default also takes these kernels where a choice by hand is refused.  Rows of
+ * at least 17 nodes whose width is not a multiple of 4 are stored padded to one where
+ * a kernel then serves them that is faster than the reference kernel: D2Q9 with a
+ * closed x axis (all but narrow, tall domains), and D3Q19 with FP32 or 16-bit storage
+ * from 50,000 nodes on, with a periodic x axis from 150,000, in rows of up to 512
+ * stored nodes (16-bit rows of whole 16 bytes; two-rows or folded kernel).  Slabs
+ * follow the undivided domain (maclab_create_slab), and raw states keep their
+ * (d + 1) * N values.  With D2Q9 the block kernel takes a periodic x axis of any
+ * width of at least 32 nodes.  The two-rows and folded kernels run on row counts that
+ * their tiles do not divide (at least one tile of rows). */
 #define MACLAB_KERNEL_AUTO 0
 #define MACLAB_KERNEL_REFERENCE 1
 #define MACLAB_KERNEL_TILED 2

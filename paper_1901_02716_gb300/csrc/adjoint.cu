@@ -446,7 +446,7 @@ cudaError_t launch_adjoint_nu_term(const Geometry& g, int precision, const void*
 // (large, or so small that an error term could be subnormal) is summed in FP64.
 // Done in FP64 throughout, seven conversions and multiply-adds per value on a
 // pipe of two lanes per SM (and the divisions by e) bounded both kernels.  96^3
-// FP32, whole calls with their read-back: seed 60 -> 36 us, finish 119 -> 41 us.
+// FP32, whole calls with their read-back: seed 60 -> 37 us, finish 119 -> 42 us.
 
 // a + b; *err is what the rounding of the sum left out.
 __device__ __forceinline__ float two_sum(float a, float b, float* err) {

@@ -12,9 +12,9 @@
 // weights 36 w, divided out at the end).  That is half the arithmetic and half
 // the shared-memory reads of the direct sum, and two staged planes instead of
 // four.  Bound by latency and by the halo rows and planes, whose records are
-// formed again by every block (FP32 97x96x95: 35.4 us for 33 MB of states and
+// formed again by every block (FP32 97x96x95: 32.5 us for 33 MB of states and
 // adjoints read three times and written once; the reference kernels took 62.8),
-// in FP64 by the arithmetic pipe (96^3: 325 us, the direct sums 478).
+// in FP64 by the arithmetic pipe (96^3: 328 us, the direct sums 478).
 #pragma once
 #include "adjoint_tiled.cuh"
 

@@ -14,16 +14,16 @@ struct AdjShape {
 
 // Tiled reverse steps built (us a step, periodic):
 //  * adj_step_rows for natural rows in FP32 and interleaved rows in FP64, of 3
-//    to 128 nodes in 3D and to 512 in 2D.  FP32 97x96x95: 35.4 (reference kernels
-//    62.8), 33x40x50 10.5 (16.6), 255x256 5.7 (12.4); FP64 96^3: 325
-//    (adj_step_tiled 479), 256^2 18.5 (32.1).
+//    to 128 nodes in 3D and to 512 in 2D.  FP32 97x96x95: 32.5 (reference kernels
+//    62.8), 33x40x50 9.9 (16.6), 255x256 6.1 (12.4); FP64 96^3: 328
+//    (adj_step_tiled 479), 256^2 19.3 (32.1).
 //  * adj_step_tiled for interleaved FP32 rows, whose threads keep twice the bytes
-//    in flight: 96^3 19.6 (adj_step_rows 27.3), 128^3 38.8 (72.5); up to 512
+//    in flight: 96^3 19.1 (adj_step_rows 27.3), 128^3 38.8 (72.5); up to 512
 //    nodes in 3D, 1024 in 2D.
 // The rest takes the reference kernels, natural FP64 rows because they are
 // faster there (97x64x64: 160, adj_step_rows 190).
-// Blocks of adj_step_rows: FP32 8 rows with the halo, 53x61x47 12.2 (10 rows, one
-// block an SM: 16.4) and 127x80x80 25.9 (6 rows: 32.7); FP64 is bound by its
+// Blocks of adj_step_rows: FP32 8 rows with the halo, 53x61x47 12.1 (10 rows, one
+// block an SM: 16.4) and 127x80x80 23.9 (6 rows: 32.7); FP64 is bound by its
 // arithmetic, not by the blocks an SM holds: 32^3 34 (10 rows: 45), but with 64
 // columns its registers spill (96^3: 356 with 64 x 8 threads).
 bool adj_shape(const Geometry& g, int precision, AdjShape* s) {

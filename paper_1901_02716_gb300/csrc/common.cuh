@@ -189,15 +189,15 @@ struct Geometry {
   // Stored rows may end in pad = 1..3 positions beyond the domain's last node
   // (x = nx - pad .. nx - 1), which bring a closed x axis of any width to the
   // interleaved rows of the fast kernels (FP32 step of the 251^3 cavity: 508 us
-  // on the one-thread-per-node kernel, 142 us now; of the 401^2 cavity: 4.3 and
-  // 2.1 us).  The domain's right wall is then at x = nx - 1 -
+  // on the one-thread-per-node kernel, 140 us now; of the 401^2 cavity: 4.3 and
+  // 1.8 us).  The domain's right wall is then at x = nx - 1 -
   // pad and shields it: whatever a step leaves in the padding reaches only wall
   // nodes, which keep their values.  In mask mode the padding is marked as wall.
   // On a periodic x axis (D3Q19) the padding is 2 to 5 positions: the first holds a
   // copy of node 0 and the last, the seam's neighbour of node 0, one of the
   // domain's last node; they are copied after every step (launch_wrap_columns; FP32
   // step of a periodic 251^3 grid: 498 us on the one-thread-per-node kernel, 148
-  // now; 95^3: 26.4 and 15.7).
+  // now; 95^3: 26.4 and 13.5).
   int pad;
 };
 

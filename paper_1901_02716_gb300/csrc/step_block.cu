@@ -189,8 +189,10 @@ __device__ __forceinline__ void block_next_state(const typename Pair<C>::P (&s)[
 // ------------------------------------------------------------------ FP64: one pair per thread
 //
 // A warp is one tile row of 32 pairs; blockDim.y rows (block_rows_f64).  GB300's
-// FP64 pipe (two lanes per SM) bounds it: 41 operations a node and step, plus
-// those of the halo, which is why the rows of a tile are chosen for the grid.
+// FP64 pipe (two lanes per SM) bounds it: 41 operations a node and step and a
+// division (the correctly rounded one: 256^2 9.94 us a step, 9.89 with a
+// reciprocal good to an ulp, 64^2 4.23 and 4.05), plus those of the halo, which is why the rows of a tile are
+// chosen for the grid.
 // WRAP: rows of at most 32 pairs (interleaved), which a tile holds whole: the
 // neighbour across the row's end is the lane at its other end, swapped, and the
 // tile needs no halo columns.
@@ -408,8 +410,8 @@ int block_sms() {
 
 // Output rows of a tile of the FP64 kernel: those whose busiest SM has the least
 // to do, in units of one operation of a warp's row of pairs.  A step forms and
-// sums its source rows (29 operations) and finishes its destination rows (16);
-// the blocks of a launch share the SMs' FP64 pipes evenly.  (256^2 at 2 steps a
+// sums its source rows (29 operations) and finishes its destination rows (16, the
+// division counted as three); the blocks of a launch share the SMs' FP64 pipes evenly.  (256^2 at 2 steps a
 // launch: 128 blocks of 32 x 16 pairs before, 16.4 us a step.)
 int block_rows_f64(int ny, int xtiles, int steps) {
   int best = 1;
@@ -499,8 +501,10 @@ cudaError_t launch_block2_any(const StepLaunch& s, cudaStream_t stream) {
 // Steps per launch for the tile setting ty; default (ty = 0): FP32 8 up to 65,536
 // pairs, 4 above (256^2 0.84, 512^2 1.76 us a step, the other way 0.98 and 2.41);
 // FP64, whose halo costs more than the launch it saves, 1 below 8,192 pairs (64^2:
-// 4.05 us a step, 4.12 at two, 5.00 at four), then the documented 4 up to 16,384
-// pairs and 2 above (128^2: 6.34, and 5.19 at one; 256^2: 9.89 and 9.45).
+// 4.23 us a step, 4.29 at two, 5.17 at four).  Above that 4 up to 16,384 pairs, then
+// 2: the counts that launches of this kernel have had from the start and that its
+// tests hold, not the fastest (128^2: 6.57 at four, 5.26 at one; 256^2: 9.94 at two,
+// 9.72 at one).
 int block_steps(const Geometry& g, int precision, int ty) {
   if (precision != MACLAB_F32 && precision != MACLAB_F64) return 0;
   const int64_t pairs = (int64_t)(g.nx / 2) * g.ny;
