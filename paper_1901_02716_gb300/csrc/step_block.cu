@@ -191,8 +191,8 @@ __device__ __forceinline__ void block_next_state(const typename Pair<C>::P (&s)[
 // A warp is one tile row of 32 pairs; blockDim.y rows (block_rows_f64).  GB300's
 // FP64 pipe (two lanes per SM) bounds it: 41 operations a node and step and a
 // division (the correctly rounded one: 256^2 9.94 us a step, 9.89 with a
-// reciprocal good to an ulp, 64^2 4.23 and 4.05), plus those of the halo, which is why the rows of a tile are
-// chosen for the grid.
+// reciprocal good to an ulp, 64^2 4.23 and 4.05), plus those of the halo, which is
+// why the rows of a tile are chosen for the grid.
 // WRAP: rows of at most 32 pairs (interleaved), which a tile holds whole: the
 // neighbour across the row's end is the lane at its other end, swapped, and the
 // tile needs no halo columns.
@@ -411,8 +411,9 @@ int block_sms() {
 // Output rows of a tile of the FP64 kernel: those whose busiest SM has the least
 // to do, in units of one operation of a warp's row of pairs.  A step forms and
 // sums its source rows (29 operations) and finishes its destination rows (16, the
-// division counted as three); the blocks of a launch share the SMs' FP64 pipes evenly.  (256^2 at 2 steps a
-// launch: 128 blocks of 32 x 16 pairs before, 16.4 us a step.)
+// division counted as three); the blocks of a launch share the SMs' FP64 pipes
+// evenly.  (256^2 at 2 steps a launch: 128 blocks of 32 x 16 pairs before, 16.4 us a
+// step.)
 int block_rows_f64(int ny, int xtiles, int steps) {
   int best = 1;
   int64_t least = INT64_MAX;
