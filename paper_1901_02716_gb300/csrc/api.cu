@@ -703,11 +703,19 @@ static maclab_status segment_persist_prepare(maclab_ctx* h) {
 // form (ty 3) its wait lists.  With two steps per launch a list of its own serves
 // single steps: cut for one step, it has wider segments and rows that fill one
 // wave of the one-step kernel's warps (1024^2: 5.6 us a single step, 7.1 on the
-// two-step list).
+// two-step list).  The block kernel can do without (single_step): no list is built for
+// it while the caller captures its stream, nor where memory for one is refused.
 static maclab_status segment_prepare(maclab_ctx* h) {
   if (!segment_single(h)) return MACLAB_OK;
   const int runs = h->kernel == MACLAB_KERNEL_SEGMENT;
-  if (!h->d_seg_items || h->seg_runs != runs || h->seg_ty != h->ty || h->seg_tz != h->tz) {
+  if (!h->d_seg_items || h->seg_runs != runs || (runs && (h->seg_ty != h->ty || h->seg_tz != h->tz))) {
+    if (!runs) {
+      cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+      if (cudaStreamIsCapturing(h->stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return MACLAB_OK;
+      }
+    }
     const int depth = runs ? segment_depth(h->g, h->precision, h->ty) : 1;
     int rows1 = segment_rows(h->g, h->precision, 1, 0);
     if (runs && h->tz > 0) rows1 = depth == 1 ? h->tz : std::min(h->tz, rows1);
@@ -715,7 +723,7 @@ static maclab_status segment_prepare(maclab_ctx* h) {
       if (cudaMalloc(&h->d_seg_inst, batch_inst_bytes()) != cudaSuccess) {
         cudaGetLastError();
         h->d_seg_inst = nullptr;
-        return fail(MACLAB_ERR_OOM, "segment descriptor allocation failed");
+        return runs ? fail(MACLAB_ERR_OOM, "segment descriptor allocation failed") : MACLAB_OK;
       }
     }
     std::vector<unsigned char> inst(batch_inst_bytes());
@@ -728,7 +736,7 @@ static maclab_status segment_prepare(maclab_ctx* h) {
     void* d = nullptr;
     if (cudaMalloc(&d, items.size() * sizeof(int)) != cudaSuccess) {
       cudaGetLastError();
-      return fail(MACLAB_ERR_OOM, "segment work list allocation failed");
+      return runs ? fail(MACLAB_ERR_OOM, "segment work list allocation failed") : MACLAB_OK;
     }
     CUDA_TRY(cudaMemcpyAsync(h->d_seg_inst, inst.data(), inst.size(), cudaMemcpyHostToDevice, h->stream),
              "segment descriptor upload");
